@@ -146,7 +146,7 @@ __device__ __forceinline__ void reflector(double alpha, double s, double* beta, 
     *scale = (alpha >= 0.0 ? rq : -rq) * rq;
 }
 
-// householder() for M <= 32 rows: lanes are rows within aligned segments of
+// householder() for few rows (at most 32, used up to 16): lanes are rows within aligned segments of
 // S = pow2_at_least(M) lanes, so one warp instruction serves 32/S columns of
 // the trailing update; every warp forms the reflector itself (no broadcast
 // through shared memory), and the column's scaled v is stored after the
@@ -184,7 +184,7 @@ __device__ __forceinline__ void householder_small(double* A, double* tau, int M,
     __syncthreads();
 }
 
-// form_q() for M <= 32 rows (segment layout as in householder_small).
+// form_q() for few rows (segment layout as in householder_small).
 __device__ __forceinline__ void form_q_small(const double* A, const double* tau, double* Q, int M, int k) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarps();
     const int S = pow2_at_least(M), G = 32 / S;
@@ -209,84 +209,137 @@ __device__ __forceinline__ void form_q_small(const double* A, const double* tau,
     }
 }
 
+// Segments of 8 lanes: a warp works on four columns (or column pairs) at once,
+// lane sl of a segment on the rows i = sl mod 8.  On this GPU an SMSP issues one
+// FP64 warp instruction per 64 cycles however many lanes it serves, so what a
+// routine costs is its FP64 warp instructions: a 32-lane dot product of n rows
+// takes n/32 + 5 of them per column, four 8-lane ones n/8 + 3 together.
+__device__ __forceinline__ double seg8_sum(double v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
+}
+
+// One warp: reflector of column j (rows j .. M-1), v scaled in place (v_j = 1
+// implicit), R(j, j) and tau[j] stored.
+__device__ __forceinline__ void reflect_column(double* A, double* tau, int M, int j, int lane) {
+    double* x = A + (int64_t)j * M;
+    double s = 0.0;
+    for (int i = j + 1 + lane; i < M; i += 32) s = fma(x[i], x[i], s);
+    s = warp_sum(s);
+    const double alpha = x[j];
+    double tj = 0.0, scale = 0.0, beta = alpha;
+    if (s != 0.0) reflector(alpha, s, &beta, &tj, &scale);
+    if (tj != 0.0)
+        for (int i = j + 1 + lane; i < M; i += 32) x[i] *= scale;
+    __syncwarp();   // every lane has read x[j]
+    if (lane == 0) {
+        x[j] = beta;
+        tau[j] = tj;
+    }
+    __syncwarp();
+}
+
+// The columns c0 + 4 w + segment, stepping 4 nw, of A: a_c -= tau_j (v_j^T a_c) v_j.
+__device__ __forceinline__ void reflect_segments(double* A, double tj, int M, int N, int j, int c0, int w, int nw,
+                                                 int lane) {
+    const int sl = lane & 7;
+    const double* v = A + (int64_t)j * M;
+    for (int cb = c0 + 4 * w; cb < N; cb += 4 * nw) {
+        const int c = cb + (lane >> 3);
+        double* a = A + (int64_t)(c < N ? c : cb) * M;
+        const double a_j = a[j];
+        double d = 0.0;
+        for (int i = j + 1 + sl; i < M; i += 8) d = fma(v[i], a[i], d);
+        d = seg8_sum(d) + a_j;
+        const double tw = tj * d;
+        if (c < N) {
+            if (sl == 0) a[j] = a_j - tw;
+            for (int i = j + 1 + sl; i < M; i += 8) a[i] = fma(-tw, v[i], a[i]);
+        }
+    }
+}
+
 // Householder factorisation of A (M x N, column-major, ld M) in place: R in the
 // upper trapezoid, v_j below the diagonal (v_j = 1 implicit), tau[j].
 // H = I - tau v v^T, beta = -sign(alpha) ||x||, tau = (beta - alpha)/beta,
-// v = x/(alpha - beta).  sh: 2 shared doubles.
+// v = x/(alpha - beta).
+//
+// One barrier per column: while the other warps apply H_j to the columns beyond
+// j + 1, warp 0 applies it to column j + 1 and forms H_{j+1} at once (its chain
+// of about 35 dependent FP64 instructions is what bounds a small QR).  Warps that
+// share warp 0's scheduler (4, 8, ...) stay out of the updates of small
+// matrices, where they would lengthen that chain.
 __device__ __forceinline__ void householder(double* A, double* tau, int M, int N, double* red, double* sh) {
-    if (M <= 32) {
+    if (M <= 16) {
         householder_small(A, tau, M, N);
         return;
     }
     const int k = M < N ? M : N;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarps();
+    int w = warp - 1, nwork = nw - 1;
+    if (nw == 1) {
+        w = 0;
+        nwork = 1;
+    } else if (nw >= 6 && (int64_t)M * N <= 64 * 64) {
+        w = (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
+        nwork = (nw >> 2) * 3 + ((nw & 3) ? (nw & 3) - 1 : 0);
+    }
+    if (warp == 0) reflect_column(A, tau, M, 0, lane);
+    __syncthreads();
     for (int j = 0; j < k; ++j) {
-        double s = 0.0;
-        for (int i = j + 1 + threadIdx.x; i < M; i += nthreads()) {
-            const double v = A[(int64_t)j * M + i];
-            s += v * v;
-        }
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) {
-            const double alpha = A[(int64_t)j * M + j];
-            if (s == 0.0) {
-                sh[0] = 0.0;
-                sh[1] = 0.0;
-            } else {
-                const double nrm = sqrt(alpha * alpha + s);
-                const double beta = alpha >= 0.0 ? -nrm : nrm;
-                sh[0] = (beta - alpha) / beta;
-                sh[1] = 1.0 / (alpha - beta);
-                A[(int64_t)j * M + j] = beta;
+        const double tj = tau[j];
+        if (warp == 0 && j + 1 < N) {
+            if (tj != 0.0) {
+                const double* v = A + (int64_t)j * M;
+                double* a = A + (int64_t)(j + 1) * M;
+                const double a_j = a[j];
+                double d = 0.0;
+                for (int i = j + 1 + lane; i < M; i += 32) d = fma(v[i], a[i], d);
+                d = warp_sum(d) + a_j;
+                const double tw = tj * d;
+                if (lane == 0) a[j] = a_j - tw;
+                for (int i = j + 1 + lane; i < M; i += 32) a[i] = fma(-tw, v[i], a[i]);
+                __syncwarp();
             }
-            tau[j] = sh[0];
+            if (j + 1 < k) reflect_column(A, tau, M, j + 1, lane);
         }
-        __syncthreads();
-        const double tj = sh[0], scale = sh[1];
-        if (tj != 0.0) {
-            for (int i = j + 1 + threadIdx.x; i < M; i += nthreads()) A[(int64_t)j * M + i] *= scale;
-            __syncthreads();
-            for (int c = j + 1 + warp; c < N; c += nwarps()) {
-                // read A(j, c) before the warp-synchronous reduction: lane 0 rewrites it after
-                const double a_jc = A[(int64_t)c * M + j];
-                double w = 0.0;
-                for (int i = j + 1 + lane; i < M; i += 32) w += A[(int64_t)j * M + i] * A[(int64_t)c * M + i];
-                w = warp_sum(w) + a_jc;
-                const double tw = tj * w;
-                if (lane == 0) A[(int64_t)c * M + j] -= tw;
-                for (int i = j + 1 + lane; i < M; i += 32) A[(int64_t)c * M + i] -= tw * A[(int64_t)j * M + i];
-            }
-        }
+        if (w >= 0 && tj != 0.0) reflect_segments(A, tj, M, N, j, j + 2, w, nwork, lane);
         __syncthreads();
     }
 }
 
 // Q (M x k, column-major) = H_0 ... H_{k-1} applied to the first k columns of I.
+// Column c needs H_c ... H_0 only and no other column of Q: every 8-lane segment
+// takes a column through all its reflectors without a barrier (each lane keeps
+// to the rows i = sl mod 8), longest columns first.
 __device__ __forceinline__ void form_q(const double* A, const double* tau, double* Q, int M, int k) {
-    if (M <= 32) {
+    if (M <= 16) {
         form_q_small(A, tau, Q, M, k);
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t e = threadIdx.x; e < (int64_t)M * k; e += nthreads()) {
-        const int i = (int)(e % M), c = (int)(e / M);
-        Q[e] = i == c ? 1.0 : 0.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
+    for (int cb = 4 * warp; cb < k; cb += 4 * nwarps()) {
+        const int c = k - 1 - (cb + (lane >> 3));
+        const bool own = c >= 0;
+        double* q = Q + (int64_t)(own ? c : 0) * M;
+        if (own)
+            for (int i = sl; i < M; i += 8) q[i] = i == c ? 1.0 : 0.0;
+        for (int j = k - 1 - cb; j >= 0; --j) {
+            const double tj = tau[j];
+            if (tj == 0.0) continue;
+            const double* v = A + (int64_t)j * M;
+            const int i0 = j + ((sl - j) & 7);
+            double d = 0.0;
+            if (own && c >= j)
+                for (int i = i0; i < M; i += 8) d = fma(i == j ? 1.0 : v[i], q[i], d);
+            const double tw = tj * seg8_sum(d);
+            if (own && c >= j)
+                for (int i = i0; i < M; i += 8) q[i] = fma(-tw, i == j ? 1.0 : v[i], q[i]);
+        }
     }
     __syncthreads();
-    for (int j = k - 1; j >= 0; --j) {
-        const double tj = tau[j];
-        if (tj == 0.0) continue;
-        for (int c = j + warp; c < k; c += nwarps()) {
-            const double q_jc = Q[(int64_t)c * M + j];
-            double w = 0.0;
-            for (int i = j + 1 + lane; i < M; i += 32) w += A[(int64_t)j * M + i] * Q[(int64_t)c * M + i];
-            w = warp_sum(w) + q_jc;
-            const double tw = tj * w;
-            if (lane == 0) Q[(int64_t)c * M + j] -= tw;
-            for (int i = j + 1 + lane; i < M; i += 32) Q[(int64_t)c * M + i] -= tw * A[(int64_t)j * M + i];
-        }
-        __syncthreads();
-    }
 }
 
 __device__ __forceinline__ int rr_player(int pos, int round, int n2) {
@@ -586,6 +639,388 @@ __device__ __forceinline__ void svd_assemble_direct(const double* B, const doubl
             for (int i = lane; i < M; i += 32) US[(int64_t)i * ldus + r] = -US[(int64_t)i * ldus + r];
         }
     }
+}
+
+// x 2^sh as a float (truncated; 0 below 2^-126, saturated above, NaN for a
+// non-finite x), by integer operations: FP64 conversions would occupy the FP64 pipe.
+__device__ __forceinline__ float to_float_scaled(double x, int sh) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7ff), e = ex - 1023 + 127 + sh;
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned u = ex == 0x7ff ? 0x7fc00000u : e <= 0 ? 0u : (e >= 255 ? 0x7f7fffffu : ((unsigned)e << 23) | m);
+    return __uint_as_float(u | (hi & 0x80000000u));
+}
+// A finite float as a double, by integer operations (FP32 subnormals become 0).
+__device__ __forceinline__ double to_double(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xff;
+    const unsigned hi = e ? ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3) : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), e ? (int)(u << 29) : 0);
+}
+__device__ __forceinline__ float seg8_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
+}
+// tan of the angle that makes columns of squared norms a, b (d = b - a) and
+// inner product g (g2 = 2 g) orthogonal; d and g2 scaled so that the larger is near 1.
+__device__ __forceinline__ float jacobi_tan(float d, float g2) {
+    const float w = fmaf(d, d, g2 * g2);
+    const float r = w * rsqrtf(w);
+    const float sz = (d == 0.0f || ((d > 0.0f) == (g2 > 0.0f))) ? 1.0f : -1.0f;
+    return sz * __fdividef(fabsf(g2), fabsf(d) + r);
+}
+
+// The pair of segment u (of 4 per warp) in `round` of a round-robin over k columns.
+__device__ __forceinline__ bool seg_pair(int u, int round, int k, int* p, int* q) {
+    const int n2 = k + (k & 1);
+    if (u >= n2 / 2) return false;
+    int a = rr_player(u, round, n2), b = rr_player(n2 - 1 - u, round, n2);
+    if (a > b) {
+        const int t = a;
+        a = b;
+        b = t;
+    }
+    *p = a;
+    *q = b;
+    return b < k;
+}
+
+// FP32 one-sided Jacobi of G (k x k, column-major, ||G||_F ~ 1, overwritten), the
+// rotations accumulated in V (identity on entry): one pair per 8-lane segment.
+// Tolerance 4 sqrt(k) eps_32; a sweep rotating at most 1/32 of the pairs ends.
+template <int R>
+__device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, int* s_cnt) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
+    const int n2 = k + (k & 1);
+    const float tol = 4.0f * sqrtf((float)k) * FLT_EPSILON;
+    for (int sweep = 0; sweep < 20; ++sweep) {
+        if (threadIdx.x == 0) *s_cnt = 0;
+        int cnt = 0;
+        for (int round = 0; round < n2 - 1; ++round) {
+            for (int ub = 4 * warp; ub < n2 / 2; ub += 4 * nwarps()) {
+                int p = 0, q = 0;
+                const bool on = seg_pair(ub + (lane >> 3), round, k, &p, &q);
+                float xp[R], xq[R];
+                float a = 0.0f, b = 0.0f, g = 0.0f;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = sl + 8 * r;
+                    const bool in = on && i < k;
+                    xp[r] = in ? G[p * k + i] : 0.0f;
+                    xq[r] = in ? G[q * k + i] : 0.0f;
+                    a = fmaf(xp[r], xp[r], a);
+                    b = fmaf(xq[r], xq[r], b);
+                    g = fmaf(xp[r], xq[r], g);
+                }
+                a = seg8_sum(a);
+                b = seg8_sum(b);
+                g = seg8_sum(g);
+                const bool rot = fminf(a, b) > 1e-36f && fabsf(g) > tol * (a * rsqrtf(a)) * (b * rsqrtf(b));
+                if (rot) {
+                    const float d = b - a, g2 = g + g;
+                    const float m = __fdividef(1.0f, fmaxf(fabsf(d), fabsf(g2)));
+                    const float t = jacobi_tan(d * m, g2 * m);
+                    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int i = sl + 8 * r;
+                        if (i < k) {
+                            G[p * k + i] = c * xp[r] - sn * xq[r];
+                            G[q * k + i] = sn * xp[r] + c * xq[r];
+                            const float vp = V[p * k + i], vq = V[q * k + i];
+                            V[p * k + i] = c * vp - sn * vq;
+                            V[q * k + i] = sn * vp + c * vq;
+                        }
+                    }
+                    cnt += sl == 0;
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+        }
+        if (cnt) atomicAdd(s_cnt, cnt);
+        __syncthreads();
+        const int total = *s_cnt;
+        __syncthreads();
+        if (64 * total <= k * (k - 1)) break;
+    }
+}
+
+// FP64 one-sided Jacobi of G (k x k, column-major, ||G||_F in [1/2, 1)) rotating
+// the columns of V along: one pair per 8-lane segment, the columns' squared norms
+// tracked in nrm (recomputed every sweep), the tests and angles in FP32 (only the
+// inner product, the norms and the rotation itself need FP64).  A rotation by a
+// small angle is applied as x_p - alpha x_q, x_q + beta x_p (two FMAs per row
+// instead of four operations): that is the rotation times 1 / cos, and the cosines
+// are gathered per column in del (column = (1 + del) x stored; alpha and beta
+// carry the ratio of the two scales, terms below 2^-57 dropped).  Larger angles
+// (and columns with |del| >= 2^-30) take the full rotation, which clears del.
+// Stopping rule: |g| > k eps sqrt(a b), min(a, b) > (k eps)^2 ||G||_F^2.
+template <int R>
+__device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, double fro,
+                                                    int* s_rot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
+    const int n2 = k + (k & 1);
+    const float tol = (float)k * 2.220446e-16f * 0x1p48f;   // compared with g 2^48
+    const float tiny = (float)k * 2.220446e-16f * (float)k * 2.220446e-16f * to_float_scaled(fro, 0);
+    for (int j = threadIdx.x; j < k; j += nthreads()) del[j] = 0.0f;
+    __syncthreads();
+    for (int sweep = 0; sweep < kMaxSweeps && k > 1; ++sweep) {
+        if (threadIdx.x == 0) *s_rot = 0;
+        for (int jb = 4 * warp; jb < k; jb += 4 * nwarps()) {
+            const int j = jb + (lane >> 3);
+            double a = 0.0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = sl + 8 * r;
+                const double x = (j < k && i < k) ? G[j * k + i] : 0.0;
+                a = fma(x, x, a);
+            }
+            a = seg8_sum(a);
+            if (j < k && sl == 0) nrm[j] = a;
+        }
+        __syncthreads();
+        for (int round = 0; round < n2 - 1; ++round) {
+            for (int ub = 4 * warp; ub < n2 / 2; ub += 4 * nwarps()) {
+                int p = 0, q = 0;
+                const bool on = seg_pair(ub + (lane >> 3), round, k, &p, &q);
+                double xp[R], xq[R];
+                double g = 0.0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = sl + 8 * r;
+                    const bool in = on && i < k;
+                    xp[r] = in ? G[p * k + i] : 0.0;
+                    xq[r] = in ? G[q * k + i] : 0.0;
+                    g = fma(xp[r], xq[r], g);
+                }
+                g = seg8_sum(g);
+                const double a = nrm[p], b = nrm[q];
+                const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0);
+                const bool rot = on && fminf(af, bf) > tiny &&
+                                 fabsf(to_float_scaled(g, 48)) > tol * (af * rsqrtf(af)) * (bf * rsqrtf(bf));
+                if (!__any_sync(0xffffffffu, rot)) continue;
+                // angle: d = b - a and 2 g scaled by the larger exponent
+                const double d = b - a;
+                const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
+                const int sh = 1023 - (ed > eg ? ed : eg);
+                const float t = rot ? jacobi_tan(to_float_scaled(d, sh), to_float_scaled(g, sh + 1)) : 0.0f;
+                const float dp = del[p], dq = del[q];
+                const bool small = fabsf(t) < 0x1p-14f && fabsf(dp) < 0x1p-30f && fabsf(dq) < 0x1p-30f;
+                const double td = to_double(t);
+                double fp = 1.0, fq = 1.0;                            // p' = fp x_p - sq x_q
+                double sq = fma(td, to_double(dq - dp), td);          // q' = fq x_q + sp x_p
+                double sp = fma(td, to_double(dp - dq), td);
+                if (__any_sync(0xffffffffu, rot && !small)) {
+                    if (!small) {
+                        const double c = rsqrt(fma(td, td, 1.0)), s = c * td;
+                        const double ep = to_double(dp), eq = to_double(dq);
+                        fp = fma(c, ep, c);
+                        fq = fma(c, eq, c);
+                        sq = fma(s, eq, s);
+                        sp = fma(s, ep, s);
+                    }
+                    if (rot) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const int i = sl + 8 * r;
+                            if (i < k) {
+                                G[p * k + i] = fma(-sq, xq[r], fp * xp[r]);
+                                G[q * k + i] = fma(sp, xp[r], fq * xq[r]);
+                                const double vp = V[p * k + i], vq = V[q * k + i];
+                                V[p * k + i] = fma(-sq, vq, fp * vp);
+                                V[q * k + i] = fma(sp, vp, fq * vq);
+                            }
+                        }
+                    }
+                } else if (rot) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int i = sl + 8 * r;
+                        if (i < k) {
+                            G[p * k + i] = fma(-sq, xq[r], xp[r]);
+                            G[q * k + i] = fma(sp, xp[r], xq[r]);
+                            const double vp = V[p * k + i], vq = V[q * k + i];
+                            V[p * k + i] = fma(-sq, vq, vp);
+                            V[q * k + i] = fma(sp, vp, vq);
+                        }
+                    }
+                }
+                __syncwarp();   // every lane of the segment has read nrm and del
+                if (rot && sl == 0) {
+                    nrm[p] = fma(-td, g, a);
+                    nrm[q] = fma(td, g, b);
+                    const float h = 0.5f * t * t;
+                    del[p] = small ? dp - h : 0.0f;
+                    del[q] = small ? dq - h : 0.0f;
+                    *s_rot = 1;
+                }
+            }
+            __syncthreads();
+        }
+        const int rot = *s_rot;
+        __syncthreads();
+        if (!rot) break;
+    }
+}
+
+// One-sided Jacobi of G (k x k, column-major, 16 < k <= 64) as jacobi(): G ends as
+// U diag(Sraw), V accumulates the rotations.  The FP64 sweeps are few because an
+// FP32 Jacobi of G comes first (FP32 arithmetic runs at 64 times the FP64 rate
+// here): its rotations P, orthogonal to about 1e-6, are orthogonalised in FP64 as
+// Qp = P (I - E/2 + 3/8 E^2) with E = P^T P - I (a second pass when E is not below
+// 2e-6, since the dropped terms are of order E^3), and the FP64 Jacobi starts from
+// G Qp with V = Qp: two sweeps with rotations and one without.  Where the FP32
+// iteration gives nothing (non-finite entries) it starts from G and I.
+// scr: k^2 shared doubles; del: k shared doubles.
+template <int R>
+__device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int k, double* scr, double* del,
+                                           double* red, int* s_int) {
+    constexpr int kOwn = 8;   // outputs of a k x k product per thread: k^2 <= 8 blockDim (64 k <= blockDim at k <= 64)
+    const int T = nthreads(), kk = k * k;
+    double f = 0.0;
+    for (int e = threadIdx.x; e < kk; e += T) f = fma(G[e], G[e], f);
+    f = block_sum(f, red);
+    // exact scaling to ||G||_F in [1/2, 1)
+    int ex = 0;
+    if (f > 0.0 && f < DBL_MAX) frexp(sqrt(f), &ex);
+    const double sc = ldexp(1.0, -ex);
+    const double fro = f * sc * sc;
+    float* Gf = (float*)scr;
+    float* Vf = Gf + kk;
+    for (int e = threadIdx.x; e < kk; e += T) {
+        const double x = G[e] * sc;
+        G[e] = x;
+        Gf[e] = (float)x;
+        Vf[e] = e % k == e / k ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    jacobi_f32_segments<R>(Gf, Vf, k, s_int);
+    // V row-major <- P
+    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[e]);
+    bool ok = true;
+    for (int pass = 0; pass < 3; ++pass) {
+        __syncthreads();
+        if (threadIdx.x == 0) *s_int = 0;
+        float mx = 0.0f;
+        __syncthreads();
+        for (int e = threadIdx.x; e < kk; e += T) {
+            const int i = e % k, j = e / k;
+            double acc = i == j ? -1.0 : 0.0;
+            for (int r = 0; r < k; ++r) acc = fma(V[r * k + i], V[r * k + j], acc);
+            scr[e] = acc;
+            const float af = fabsf(to_float_scaled(acc, 0));
+            mx = af <= mx ? mx : (af == af ? af : FLT_MAX);
+        }
+        atomicMax(s_int, (int)__float_as_uint(mx));
+        __syncthreads();
+        const float emax = __uint_as_float((unsigned)*s_int);
+        if (!(emax < 1e-2f)) {
+            ok = false;
+            break;
+        }
+        double own[kOwn];
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) {
+                const int i = e % k, j = e / k;
+                double acc = 0.0;
+                for (int m = 0; m < k; ++m) acc = fma(scr[m * k + i], scr[j * k + m], acc);
+                own[n] = fma(0.5, scr[e], -0.375 * acc);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) scr[e] = own[n];
+        }
+        __syncthreads();
+        // P (I - F): row i of V (row-major) times the symmetric F
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) {
+                const int c = e % k, i = e / k;
+                double acc = 0.0;
+                for (int j = 0; j < k; ++j) acc = fma(V[i * k + j], scr[j * k + c], acc);
+                own[n] = V[e] - acc;
+            }
+        }
+        __syncthreads();
+        const bool last = emax < 2e-6f;
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) V[last ? (e % k) * k + e / k : e] = own[n];   // column-major at the end
+        }
+        if (last) break;
+        ok = pass < 2;
+    }
+    __syncthreads();
+    if (ok) {
+        double own[kOwn];
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) {
+                const int i = e % k, c = e / k;
+                double acc = 0.0;
+                for (int j = 0; j < k; ++j) acc = fma(G[j * k + i], V[c * k + j], acc);
+                own[n] = acc;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int n = 0; n < kOwn; ++n) {
+            const int e = threadIdx.x + n * T;
+            if (e < kk) G[e] = own[n];
+        }
+    } else {
+        for (int e = threadIdx.x; e < kk; e += T) V[e] = e % k == e / k ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    float* dl = (float*)del;
+    jacobi_f64_segments<R>(G, V, Sraw, dl, k, fro, s_int);
+    // the columns' scales, and the norms of the result
+    const double up = ldexp(1.0, ex);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
+    for (int jb = 4 * warp; jb < k; jb += 4 * nwarps()) {
+        const int j = jb + (lane >> 3);
+        double a = 0.0;
+        if (j < k) {
+            const double s1 = 1.0 + to_double(dl[j]);
+            for (int i = sl; i < k; i += 8) {
+                const double x = G[j * k + i] * s1;
+                a = fma(x, x, a);
+                G[j * k + i] = x * up;
+                V[j * k + i] *= s1;
+            }
+        }
+        a = seg8_sum(a);
+        if (j < k && sl == 0) Sraw[j] = sqrt_via_rsqrt(a) * up;
+    }
+    __syncthreads();
+}
+
+// jacobi_pre() for the sizes it serves (16 < k <= 64 and enough threads), else jacobi().
+__device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k, double* red, int* s_rot);
+__device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
+                                            double* red, int* s_rot) {
+    if (k > 16 && k <= 64 && k * k <= 8 * nthreads()) {
+        if (k <= 24)
+            jacobi_pre<3>(G, V, Sraw, k, scr, del, red, s_rot);
+        else if (k <= 32)
+            jacobi_pre<4>(G, V, Sraw, k, scr, del, red, s_rot);
+        else if (k <= 40)
+            jacobi_pre<5>(G, V, Sraw, k, scr, del, red, s_rot);
+        else
+            jacobi_pre<8>(G, V, Sraw, k, scr, del, red, s_rot);
+        return;
+    }
+    jacobi(G, V, Sraw, k, red, s_rot);
 }
 
 // One-sided (Hestenes) Jacobi on the columns of G (k x k, column-major) with the

@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
     }
     dev::form_q(B, tau, Q, len, k);
     __syncthreads();
-    dev::jacobi(G, V, Sraw, k, red, &s_rot);
+    dev::jacobi_auto(G, V, Sraw, k, B, tau, red, &s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
@@ -388,7 +388,7 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     }
     dev::form_q(B, tau, Q, len, k);
     __syncthreads();
-    dev::jacobi(G, V, Sraw, k, red, s_rot);
+    dev::jacobi_auto(G, V, Sraw, k, B, tau, red, s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
