@@ -221,91 +221,137 @@ __device__ __forceinline__ double seg8_sum(double v) {
     return v;
 }
 
-// One warp: reflector of column j (rows j .. M-1), v scaled in place (v_j = 1
-// implicit), R(j, j) and tau[j] stored.
-__device__ __forceinline__ void reflect_column(double* A, double* tau, int M, int j, int lane) {
+// x 2^sh as a float (truncated; 0 below 2^-126, saturated above, NaN for a
+// non-finite x), by integer operations: FP64 conversions would occupy the FP64 pipe.
+__device__ __forceinline__ float to_float_scaled(double x, int sh) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7ff), e = ex - 1023 + 127 + sh;
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned u = ex == 0x7ff ? 0x7fc00000u : e <= 0 ? 0u : (e >= 255 ? 0x7f7fffffu : ((unsigned)e << 23) | m);
+    return __uint_as_float(u | (hi & 0x80000000u));
+}
+// A finite float as a double, by integer operations (FP32 subnormals become 0).
+__device__ __forceinline__ double to_double(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xff;
+    const unsigned hi = e ? ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3) : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), e ? (int)(u << 29) : 0);
+}
+// 1/sqrt(w) for normal w > 0: Halley's iteration from an FP32 seed (22 bits or
+// more), whose relative error after one step is of order 2^-63; five FP64
+// instructions.  Exponents outside FP32's comfortable range, zeros and non-finite
+// values go through the library function.
+__device__ __forceinline__ double rsqrt_halley(double w) {
+    const int e = (__double2hiint(w) >> 20) & 0x7ff;
+    if (__double2hiint(w) < 0 || e < 2 || e > 2045) return rsqrt(w);
+    const int h = (e - 1023) >> 1;   // w = 4^h u, u in [1, 4)
+    const double u = __hiloint2double(__double2hiint(w) - (h << 21), __double2loint(w));
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_scaled(u, 0)));
+    const double y0 = to_double(y);
+    const double r = fma(-(u * y0), y0, 1.0);
+    const double z = fma(y0 * r, fma(0.375, r, 0.5), y0);
+    return __hiloint2double(__double2hiint(z) - (h << 20), __double2loint(z));
+}
+// 1/q for normal q > 0 by the same kind of step: y0 (1 + r + r^2), r = 1 - q y0.
+__device__ __forceinline__ double recip_newton(double q) {
+    const int e = (__double2hiint(q) >> 20) & 0x7ff;
+    if (__double2hiint(q) < 0 || e < 2 || e > 2040) return 1.0 / q;
+    const int h = e - 1023;
+    const double u = __hiloint2double(__double2hiint(q) - (h << 20), __double2loint(q));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_scaled(u, 0)));
+    const double y0 = to_double(y);
+    const double r = fma(-u, y0, 1.0);
+    const double z = fma(y0, fma(r, r, r), y0);
+    return __hiloint2double(__double2hiint(z) - (h << 20), __double2loint(z));
+}
+
+// One warp: reflector of column j (rows j .. M-1): H = I - tau v v^T with v = x
+// below row j (left in place, no scaling pass), v_j = alpha - beta = sign(alpha)
+// (|alpha| + n), n = ||(alpha, x)||, tau = 1 / (n (n + |alpha|)).  tau[j] and
+// vd[j] = v_j are stored; R(j, j) = beta replaces the diagonal entry.
+__device__ __forceinline__ void reflect_column(double* A, double* tau, double* vd, int M, int j, int lane) {
     double* x = A + (int64_t)j * M;
     double s = 0.0;
     for (int i = j + 1 + lane; i < M; i += 32) s = fma(x[i], x[i], s);
     s = warp_sum(s);
     const double alpha = x[j];
-    double tj = 0.0, scale = 0.0, beta = alpha;
-    if (s != 0.0) reflector(alpha, s, &beta, &tj, &scale);
-    if (tj != 0.0)
-        for (int i = j + 1 + lane; i < M; i += 32) x[i] *= scale;
     __syncwarp();   // every lane has read x[j]
     if (lane == 0) {
-        x[j] = beta;
+        double tj = 0.0;
+        if (s != 0.0) {
+            const double w = fma(alpha, alpha, s);
+            const double rn = rsqrt_halley(w);
+            const double n = w * rn, q = fabs(alpha) + n;
+            tj = rn * recip_newton(q);
+            x[j] = alpha >= 0.0 ? -n : n;
+            vd[j] = alpha >= 0.0 ? q : -q;
+        }
         tau[j] = tj;
     }
     __syncwarp();
 }
 
 // The columns c0 + 4 w + segment, stepping 4 nw, of A: a_c -= tau_j (v_j^T a_c) v_j.
-__device__ __forceinline__ void reflect_segments(double* A, double tj, int M, int N, int j, int c0, int w, int nw,
-                                                 int lane) {
+__device__ __forceinline__ void reflect_segments(double* A, double tj, double vj, int M, int N, int j, int c0, int w,
+                                                 int nw, int lane) {
     const int sl = lane & 7;
     const double* v = A + (int64_t)j * M;
     for (int cb = c0 + 4 * w; cb < N; cb += 4 * nw) {
         const int c = cb + (lane >> 3);
         double* a = A + (int64_t)(c < N ? c : cb) * M;
         const double a_j = a[j];
-        double d = 0.0;
+        double d = sl == 0 ? vj * a_j : 0.0;
         for (int i = j + 1 + sl; i < M; i += 8) d = fma(v[i], a[i], d);
-        d = seg8_sum(d) + a_j;
-        const double tw = tj * d;
+        const double tw = tj * seg8_sum(d);
         if (c < N) {
-            if (sl == 0) a[j] = a_j - tw;
+            if (sl == 0) a[j] = fma(-tw, vj, a_j);
             for (int i = j + 1 + sl; i < M; i += 8) a[i] = fma(-tw, v[i], a[i]);
         }
     }
 }
 
 // Householder factorisation of A (M x N, column-major, ld M) in place: R in the
-// upper trapezoid, v_j below the diagonal (v_j = 1 implicit), tau[j].
-// H = I - tau v v^T, beta = -sign(alpha) ||x||, tau = (beta - alpha)/beta,
-// v = x/(alpha - beta).
+// upper trapezoid, the reflectors' vectors below the diagonal and in vd (their
+// diagonal entries), tau[j]; form_q() reads them.
 //
 // One barrier per column: while the other warps apply H_j to the columns beyond
 // j + 1, warp 0 applies it to column j + 1 and forms H_{j+1} at once (its chain
 // of about 35 dependent FP64 instructions is what bounds a small QR).  Warps that
-// share warp 0's scheduler (4, 8, ...) stay out of the updates of small
-// matrices, where they would lengthen that chain.
-__device__ __forceinline__ void householder(double* A, double* tau, int M, int N, double* red, double* sh) {
+// share warp 0's scheduler (4, 8, ...) stay out of the updates while these are
+// shorter than that chain, which they would lengthen.
+__device__ __forceinline__ void householder(double* A, double* tau, double* vd, int M, int N) {
     if (M <= 16) {
         householder_small(A, tau, M, N);
         return;
     }
     const int k = M < N ? M : N;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarps();
-    int w = warp - 1, nwork = nw - 1;
-    if (nw == 1) {
-        w = 0;
-        nwork = 1;
-    } else if (nw >= 6 && (int64_t)M * N <= 64 * 64) {
-        w = (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
-        nwork = (nw >> 2) * 3 + ((nw & 3) ? (nw & 3) - 1 : 0);
-    }
-    if (warp == 0) reflect_column(A, tau, M, 0, lane);
+    const int w_all = nw == 1 ? 0 : warp - 1, n_all = nw == 1 ? 1 : nw - 1;
+    const int w_off = (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
+    const int n_off = (nw >> 2) * 3 + ((nw & 3) ? (nw & 3) - 1 : 0);
+    if (warp == 0) reflect_column(A, tau, vd, M, 0, lane);
     __syncthreads();
     for (int j = 0; j < k; ++j) {
-        const double tj = tau[j];
+        const double tj = tau[j], vj = vd[j];
         if (warp == 0 && j + 1 < N) {
             if (tj != 0.0) {
                 const double* v = A + (int64_t)j * M;
                 double* a = A + (int64_t)(j + 1) * M;
                 const double a_j = a[j];
-                double d = 0.0;
+                double d = lane == 0 ? vj * a_j : 0.0;
                 for (int i = j + 1 + lane; i < M; i += 32) d = fma(v[i], a[i], d);
-                d = warp_sum(d) + a_j;
-                const double tw = tj * d;
-                if (lane == 0) a[j] = a_j - tw;
+                const double tw = tj * warp_sum(d);
+                if (lane == 0) a[j] = fma(-tw, vj, a_j);
                 for (int i = j + 1 + lane; i < M; i += 32) a[i] = fma(-tw, v[i], a[i]);
                 __syncwarp();
             }
-            if (j + 1 < k) reflect_column(A, tau, M, j + 1, lane);
+            if (j + 1 < k) reflect_column(A, tau, vd, M, j + 1, lane);
         }
-        if (w >= 0 && tj != 0.0) reflect_segments(A, tj, M, N, j, j + 2, w, nwork, lane);
+        // FP64 instructions of the other columns' updates against the chain's
+        const bool off = nw >= 6 && (N - j) * ((M - j) / 4 + 4) <= 4 * 120;
+        const int w = off ? w_off : w_all;
+        if (w >= 0 && tj != 0.0) reflect_segments(A, tj, vj, M, N, j, j + 2, w, off ? n_off : n_all, lane);
         __syncthreads();
     }
 }
@@ -314,7 +360,7 @@ __device__ __forceinline__ void householder(double* A, double* tau, int M, int N
 // Column c needs H_c ... H_0 only and no other column of Q: every 8-lane segment
 // takes a column through all its reflectors without a barrier (each lane keeps
 // to the rows i = sl mod 8), longest columns first.
-__device__ __forceinline__ void form_q(const double* A, const double* tau, double* Q, int M, int k) {
+__device__ __forceinline__ void form_q(const double* A, const double* tau, const double* vd, double* Q, int M, int k) {
     if (M <= 16) {
         form_q_small(A, tau, Q, M, k);
         return;
@@ -329,14 +375,15 @@ __device__ __forceinline__ void form_q(const double* A, const double* tau, doubl
         for (int j = k - 1 - cb; j >= 0; --j) {
             const double tj = tau[j];
             if (tj == 0.0) continue;
+            const double vj = vd[j];
             const double* v = A + (int64_t)j * M;
             const int i0 = j + ((sl - j) & 7);
             double d = 0.0;
             if (own && c >= j)
-                for (int i = i0; i < M; i += 8) d = fma(i == j ? 1.0 : v[i], q[i], d);
+                for (int i = i0; i < M; i += 8) d = fma(i == j ? vj : v[i], q[i], d);
             const double tw = tj * seg8_sum(d);
             if (own && c >= j)
-                for (int i = i0; i < M; i += 8) q[i] = fma(-tw, i == j ? 1.0 : v[i], q[i]);
+                for (int i = i0; i < M; i += 8) q[i] = fma(-tw, i == j ? vj : v[i], q[i]);
         }
     }
     __syncthreads();
@@ -641,104 +688,129 @@ __device__ __forceinline__ void svd_assemble_direct(const double* B, const doubl
     }
 }
 
-// x 2^sh as a float (truncated; 0 below 2^-126, saturated above, NaN for a
-// non-finite x), by integer operations: FP64 conversions would occupy the FP64 pipe.
-__device__ __forceinline__ float to_float_scaled(double x, int sh) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int ex = (int)((hi >> 20) & 0x7ff), e = ex - 1023 + 127 + sh;
-    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
-    const unsigned u = ex == 0x7ff ? 0x7fc00000u : e <= 0 ? 0u : (e >= 255 ? 0x7f7fffffu : ((unsigned)e << 23) | m);
-    return __uint_as_float(u | (hi & 0x80000000u));
-}
-// A finite float as a double, by integer operations (FP32 subnormals become 0).
-__device__ __forceinline__ double to_double(float f) {
-    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xff;
-    const unsigned hi = e ? ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3) : 0u;
-    return __hiloint2double((int)(hi | (u & 0x80000000u)), e ? (int)(u << 29) : 0);
-}
 __device__ __forceinline__ float seg8_sum(float v) {
     v += __shfl_xor_sync(0xffffffffu, v, 4);
     v += __shfl_xor_sync(0xffffffffu, v, 2);
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     return v;
 }
+// Leading dimension of G and V in jacobi_auto(): at 16 < k <= 64 columns are padded
+// with zero rows to an odd multiple of 8, so that the 8-lane segments of a warp,
+// which work on neighbouring columns, meet distinct banks (64-byte pieces of
+// columns 64 bytes apart modulo 128), and whole segments of rows need no bounds check.
+__host__ __device__ constexpr int jacobi_ld(int k) {
+    return k <= 16 || k > 64 ? k : k <= 24 ? 24 : k <= 40 ? 40 : k <= 56 ? 56 : 72;
+}
+
+__device__ __forceinline__ float rsqrt_fast(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 // tan of the angle that makes columns of squared norms a, b (d = b - a) and
 // inner product g (g2 = 2 g) orthogonal; d and g2 scaled so that the larger is near 1.
 __device__ __forceinline__ float jacobi_tan(float d, float g2) {
     const float w = fmaf(d, d, g2 * g2);
-    const float r = w * rsqrtf(w);
-    const float sz = (d == 0.0f || ((d > 0.0f) == (g2 > 0.0f))) ? 1.0f : -1.0f;
-    return sz * __fdividef(fabsf(g2), fabsf(d) + r);
+    const float r = w * rsqrt_fast(w);
+    const float t = __fdividef(fabsf(g2), fabsf(d) + r);
+    return __uint_as_float(__float_as_uint(t) | ((__float_as_uint(d) ^ __float_as_uint(g2)) & 0x80000000u));
 }
 
-// The pair of segment u (of 4 per warp) in `round` of a round-robin over k columns.
-__device__ __forceinline__ bool seg_pair(int u, int round, int k, int* p, int* q) {
-    const int n2 = k + (k & 1);
-    if (u >= n2 / 2) return false;
-    int a = rr_player(u, round, n2), b = rr_player(n2 - 1 - u, round, n2);
-    if (a > b) {
-        const int t = a;
-        a = b;
-        b = t;
+// Round-robin over k columns, one pair per 8-lane segment u: the pair of a round
+// follows from the one before (position 0 stands still, the others move on by one).
+struct SegPair {
+    int a, b, n2, k;
+    bool fixed;
+    __device__ __forceinline__ SegPair(int u, int k_) : n2(k_ + (k_ & 1)), k(k_) {
+        fixed = u == 0;
+        a = u;
+        b = u < n2 / 2 ? n2 - 1 - u : n2;   // out of range: never valid
     }
-    *p = a;
-    *q = b;
-    return b < k;
-}
+    __device__ __forceinline__ bool get(int* p, int* q) const {
+        const bool on = b < n2 && a < k && b < k;
+        *p = on ? min(a, b) : 0;
+        *q = on ? max(a, b) : 0;
+        return on;
+    }
+    __device__ __forceinline__ void next() {
+        if (!fixed) a = a == n2 - 1 ? 1 : a + 1;
+        if (b < n2) b = b == n2 - 1 ? 1 : b + 1;
+    }
+};
+
+// Barrier 1 among the first n threads of the CTA (a multiple of 32).
+__device__ __forceinline__ void bar_first(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
 // FP32 one-sided Jacobi of G (k x k, column-major, ||G||_F ~ 1, overwritten), the
 // rotations accumulated in V (identity on entry): one pair per 8-lane segment.
-// Tolerance 4 sqrt(k) eps_32; a sweep rotating at most 1/32 of the pairs ends.
+// Bound by the latency of a round (loads, three shuffles, two reciprocal square
+// roots, stores, a barrier of the working warps).  Tolerance 4 sqrt(k) eps_32; a
+// sweep rotating at most 1/32 of the pairs ends.  Needs 4 warps per 32 columns.
 template <int R>
-__device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, int* s_cnt) {
+__device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, int ld, int* s_cnt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
     const int n2 = k + (k & 1);
+    const int nact = (n2 / 2 + 3) / 4;
     const float tol = 4.0f * sqrtf((float)k) * FLT_EPSILON;
     for (int sweep = 0; sweep < 20; ++sweep) {
         if (threadIdx.x == 0) *s_cnt = 0;
         int cnt = 0;
-        for (int round = 0; round < n2 - 1; ++round) {
-            for (int ub = 4 * warp; ub < n2 / 2; ub += 4 * nwarps()) {
-                int p = 0, q = 0;
-                const bool on = seg_pair(ub + (lane >> 3), round, k, &p, &q);
-                float xp[R], xq[R];
+        if (warp < nact) {
+            SegPair pr(4 * warp + (lane >> 3), k);
+            for (int round = 0; round < n2 - 1; ++round, pr.next()) {
+                int p, q;
+                const bool on = pr.get(&p, &q);
+                float* Gp = G + p * ld;
+                float* Gq = G + q * ld;
+                float* Vp = V + p * ld;
+                float* Vq = V + q * ld;
+                float xp[R], xq[R], vp[R], vq[R];
                 float a = 0.0f, b = 0.0f, g = 0.0f;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const int i = sl + 8 * r;
-                    const bool in = on && i < k;
-                    xp[r] = in ? G[p * k + i] : 0.0f;
-                    xq[r] = in ? G[q * k + i] : 0.0f;
+                    xp[r] = Gp[i];
+                    xq[r] = Gq[i];
                     a = fmaf(xp[r], xp[r], a);
                     b = fmaf(xq[r], xq[r], b);
                     g = fmaf(xp[r], xq[r], g);
                 }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = sl + 8 * r;
+                    vp[r] = Vp[i];
+                    vq[r] = Vq[i];
+                }
                 a = seg8_sum(a);
                 b = seg8_sum(b);
                 g = seg8_sum(g);
-                const bool rot = fminf(a, b) > 1e-36f && fabsf(g) > tol * (a * rsqrtf(a)) * (b * rsqrtf(b));
+                // cos and sin of the rotation from cos(2 theta) = |d| / sqrt(d^2 + 4 g^2)
+                const float d = b - a, g2 = g + g;
+                const unsigned mb = max(__float_as_uint(fabsf(d)), __float_as_uint(fabsf(g2))) >> 23;
+                const float sc = __uint_as_float((254u - min(mb, 253u)) << 23);
+                const float dn = d * sc, gn = g2 * sc;
+                const float ri = rsqrt_fast(fmaf(dn, dn, gn * gn));
+                const float c2 = fmaf(0.5f, fabsf(dn) * ri, 0.5f);
+                const float rc = rsqrt_fast(c2);
+                const float c = c2 * rc;
+                const float h = 0.5f * gn * ri * rc;
+                const float sn = __uint_as_float(__float_as_uint(h) ^ (__float_as_uint(d) & 0x80000000u));
+                const bool rot = on && fminf(a, b) > 1e-30f && fabsf(g) > tol * (a * rsqrt_fast(a)) * (b * rsqrt_fast(b));
                 if (rot) {
-                    const float d = b - a, g2 = g + g;
-                    const float m = __fdividef(1.0f, fmaxf(fabsf(d), fabsf(g2)));
-                    const float t = jacobi_tan(d * m, g2 * m);
-                    const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = c * t;
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const int i = sl + 8 * r;
-                        if (i < k) {
-                            G[p * k + i] = c * xp[r] - sn * xq[r];
-                            G[q * k + i] = sn * xp[r] + c * xq[r];
-                            const float vp = V[p * k + i], vq = V[q * k + i];
-                            V[p * k + i] = c * vp - sn * vq;
-                            V[q * k + i] = sn * vp + c * vq;
-                        }
+                        Gp[i] = c * xp[r] - sn * xq[r];
+                        Gq[i] = sn * xp[r] + c * xq[r];
+                        Vp[i] = c * vp[r] - sn * vq[r];
+                        Vq[i] = sn * vp[r] + c * vq[r];
                     }
                     cnt += sl == 0;
                 }
-                __syncwarp();
+                bar_first(32 * nact);
             }
-            __syncthreads();
         }
+        __syncthreads();
         if (cnt) atomicAdd(s_cnt, cnt);
         __syncthreads();
         const int total = *s_cnt;
@@ -746,6 +818,14 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
         if (64 * total <= k * (k - 1)) break;
     }
 }
+
+// Rotation of one pair as the G warps hand it to the V warps.
+struct SegRot {
+    double fp, sq, sp, fq;   // x_p' = fp x_p - sq x_q, x_q' = sp x_p + fq x_q
+    int p, q;
+    int mode;                // 0: none, 1: fp = fq = 1, 2: full
+    int pad;
+};
 
 // FP64 one-sided Jacobi of G (k x k, column-major, ||G||_F in [1/2, 1)) rotating
 // the columns of V along: one pair per 8-lane segment, the columns' squared norms
@@ -757,11 +837,15 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
 // carry the ratio of the two scales, terms below 2^-57 dropped).  Larger angles
 // (and columns with |del| >= 2^-30) take the full rotation, which clears del.
 // Stopping rule: |g| > k eps sqrt(a b), min(a, b) > (k eps)^2 ||G||_F^2.
+// The first nact warps work on G; the next nact rotate V one round behind them,
+// which fills the FP64 pipe while the G warps wait for loads, shuffles and
+// angles.  ring: 2 x 32 rotations.  Needs 2 nact warps.
 template <int R>
-__device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, double fro,
-                                                    int* s_rot) {
+__device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, int ld, double fro,
+                                                    SegRot* ring, int* s_rot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
     const int n2 = k + (k & 1);
+    const int nact = (n2 / 2 + 3) / 4;
     const float tol = (float)k * 2.220446e-16f * 0x1p48f;   // compared with g 2^48
     const float tiny = (float)k * 2.220446e-16f * (float)k * 2.220446e-16f * to_float_scaled(fro, 0);
     for (int j = threadIdx.x; j < k; j += nthreads()) del[j] = 0.0f;
@@ -774,43 +858,53 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const int i = sl + 8 * r;
-                const double x = (j < k && i < k) ? G[j * k + i] : 0.0;
+                const double x = j < k ? G[j * ld + i] : 0.0;
                 a = fma(x, x, a);
             }
             a = seg8_sum(a);
             if (j < k && sl == 0) nrm[j] = a;
         }
         __syncthreads();
-        for (int round = 0; round < n2 - 1; ++round) {
-            for (int ub = 4 * warp; ub < n2 / 2; ub += 4 * nwarps()) {
-                int p = 0, q = 0;
-                const bool on = seg_pair(ub + (lane >> 3), round, k, &p, &q);
+        if (warp < nact) {
+            const int u = 4 * warp + (lane >> 3);
+            SegPair pr(u, k);
+            int any = 0;
+            for (int round = 0; round < n2 - 1; ++round, pr.next()) {
+                int p, q;
+                const bool on = pr.get(&p, &q);
+                double* Gp = G + p * ld;
+                double* Gq = G + q * ld;
                 double xp[R], xq[R];
                 double g = 0.0;
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     const int i = sl + 8 * r;
-                    const bool in = on && i < k;
-                    xp[r] = in ? G[p * k + i] : 0.0;
-                    xq[r] = in ? G[q * k + i] : 0.0;
+                    xp[r] = Gp[i];
+                    xq[r] = Gq[i];
                     g = fma(xp[r], xq[r], g);
                 }
-                g = seg8_sum(g);
                 const double a = nrm[p], b = nrm[q];
-                const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0);
-                const bool rot = on && fminf(af, bf) > tiny &&
-                                 fabsf(to_float_scaled(g, 48)) > tol * (af * rsqrtf(af)) * (bf * rsqrtf(bf));
-                if (!__any_sync(0xffffffffu, rot)) continue;
-                // angle: d = b - a and 2 g scaled by the larger exponent
-                const double d = b - a;
-                const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
-                const int sh = 1023 - (ed > eg ? ed : eg);
-                const float t = rot ? jacobi_tan(to_float_scaled(d, sh), to_float_scaled(g, sh + 1)) : 0.0f;
                 const float dp = del[p], dq = del[q];
+                const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0);
+                const float lim = tol * (af * rsqrt_fast(af)) * (bf * rsqrt_fast(bf));
+                const double d = b - a;
+                g = seg8_sum(g);
+                const bool rot = on && fminf(af, bf) > tiny && fabsf(to_float_scaled(g, 48)) > lim;
+                SegRot* out = ring + (round & 1) * 32 + u;
+                if (!__any_sync(0xffffffffu, rot)) {
+                    if (sl == 0) out->mode = 0;
+                    bar_first(64 * nact);
+                    continue;
+                }
+                any = 1;
+                // angle: d and 2 g scaled by the larger exponent
+                const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
+                const int sh = 1023 - max(ed, eg);
+                const float t = rot ? jacobi_tan(to_float_scaled(d, sh), to_float_scaled(g, sh + 1)) : 0.0f;
                 const bool small = fabsf(t) < 0x1p-14f && fabsf(dp) < 0x1p-30f && fabsf(dq) < 0x1p-30f;
                 const double td = to_double(t);
-                double fp = 1.0, fq = 1.0;                            // p' = fp x_p - sq x_q
-                double sq = fma(td, to_double(dq - dp), td);          // q' = fq x_q + sp x_p
+                double fp = 1.0, fq = 1.0;
+                double sq = fma(td, to_double(dq - dp), td);
                 double sp = fma(td, to_double(dp - dq), td);
                 if (__any_sync(0xffffffffu, rot && !small)) {
                     if (!small) {
@@ -825,40 +919,70 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
 #pragma unroll
                         for (int r = 0; r < R; ++r) {
                             const int i = sl + 8 * r;
-                            if (i < k) {
-                                G[p * k + i] = fma(-sq, xq[r], fp * xp[r]);
-                                G[q * k + i] = fma(sp, xp[r], fq * xq[r]);
-                                const double vp = V[p * k + i], vq = V[q * k + i];
-                                V[p * k + i] = fma(-sq, vq, fp * vp);
-                                V[q * k + i] = fma(sp, vp, fq * vq);
-                            }
+                            Gp[i] = fma(-sq, xq[r], fp * xp[r]);
+                            Gq[i] = fma(sp, xp[r], fq * xq[r]);
                         }
                     }
                 } else if (rot) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const int i = sl + 8 * r;
-                        if (i < k) {
-                            G[p * k + i] = fma(-sq, xq[r], xp[r]);
-                            G[q * k + i] = fma(sp, xp[r], xq[r]);
-                            const double vp = V[p * k + i], vq = V[q * k + i];
-                            V[p * k + i] = fma(-sq, vq, vp);
-                            V[q * k + i] = fma(sp, vp, vq);
+                        Gp[i] = fma(-sq, xq[r], xp[r]);
+                        Gq[i] = fma(sp, xp[r], xq[r]);
+                    }
+                }
+                if (sl == 0) {
+                    out->mode = rot ? (small ? 1 : 2) : 0;
+                    if (rot) {
+                        out->fp = fp;
+                        out->sq = sq;
+                        out->sp = sp;
+                        out->fq = fq;
+                        out->p = p;
+                        out->q = q;
+                        nrm[p] = fma(-td, g, a);
+                        nrm[q] = fma(td, g, b);
+                        const float h = 0.5f * t * t;
+                        del[p] = small ? dp - h : 0.0f;
+                        del[q] = small ? dq - h : 0.0f;
+                    }
+                }
+                bar_first(64 * nact);
+            }
+            if (any && lane == 0) *s_rot = 1;
+        } else if (warp < 2 * nact) {
+            const int u = 4 * (warp - nact) + (lane >> 3);
+            for (int round = 0; round < n2 - 1; ++round) {
+                bar_first(64 * nact);
+                const SegRot* in = ring + (round & 1) * 32 + u;
+                const int mode = in->mode;
+                if (!__any_sync(0xffffffffu, mode != 0)) continue;
+                if (mode) {
+                    const double fp = in->fp, sq = in->sq, sp = in->sp, fq = in->fq;
+                    double* Vp = V + in->p * ld;
+                    double* Vq = V + in->q * ld;
+                    if (mode == 1) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const int i = sl + 8 * r;
+                            const double vp = Vp[i], vq = Vq[i];
+                            Vp[i] = fma(-sq, vq, vp);
+                            Vq[i] = fma(sp, vp, vq);
+                        }
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const int i = sl + 8 * r;
+                            const double vp = Vp[i], vq = Vq[i];
+                            Vp[i] = fma(-sq, vq, fp * vp);
+                            Vq[i] = fma(sp, vp, fq * vq);
                         }
                     }
                 }
-                __syncwarp();   // every lane of the segment has read nrm and del
-                if (rot && sl == 0) {
-                    nrm[p] = fma(-td, g, a);
-                    nrm[q] = fma(td, g, b);
-                    const float h = 0.5f * t * t;
-                    del[p] = small ? dp - h : 0.0f;
-                    del[q] = small ? dq - h : 0.0f;
-                    *s_rot = 1;
-                }
+                __syncwarp();
             }
-            __syncthreads();
         }
+        __syncthreads();
         const int rot = *s_rot;
         __syncthreads();
         if (!rot) break;
@@ -873,14 +997,15 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
 // 2e-6, since the dropped terms are of order E^3), and the FP64 Jacobi starts from
 // G Qp with V = Qp: two sweeps with rotations and one without.  Where the FP32
 // iteration gives nothing (non-finite entries) it starts from G and I.
-// scr: k^2 shared doubles; del: k shared doubles.
+// G and V have leading dimension jacobi_ld(k), the rows from k on zero in G on entry.
+// scr: k jacobi_ld(k) shared doubles; del: k shared doubles.
 template <int R>
 __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int k, double* scr, double* del,
-                                           double* red, int* s_int) {
+                                           SegRot* ring, double* red, int* s_int) {
     constexpr int kOwn = 8;   // outputs of a k x k product per thread: k^2 <= 8 blockDim (64 k <= blockDim at k <= 64)
-    const int T = nthreads(), kk = k * k;
+    const int T = nthreads(), kk = k * k, ld = jacobi_ld(k), kl = k * ld;
     double f = 0.0;
-    for (int e = threadIdx.x; e < kk; e += T) f = fma(G[e], G[e], f);
+    for (int e = threadIdx.x; e < kl; e += T) f = fma(G[e], G[e], f);
     f = block_sum(f, red);
     // exact scaling to ||G||_F in [1/2, 1)
     int ex = 0;
@@ -888,28 +1013,32 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     const double sc = ldexp(1.0, -ex);
     const double fro = f * sc * sc;
     float* Gf = (float*)scr;
-    float* Vf = Gf + kk;
-    for (int e = threadIdx.x; e < kk; e += T) {
+    float* Vf = Gf + kl;
+    for (int e = threadIdx.x; e < kl; e += T) {
         const double x = G[e] * sc;
         G[e] = x;
         Gf[e] = (float)x;
-        Vf[e] = e % k == e / k ? 1.0f : 0.0f;
+        Vf[e] = e % ld == e / ld ? 1.0f : 0.0f;
     }
     __syncthreads();
-    jacobi_f32_segments<R>(Gf, Vf, k, s_int);
+    jacobi_f32_segments<R>(Gf, Vf, k, ld, s_int);
     // V row-major <- P
-    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[e]);
+    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ld + e % k]);
     bool ok = true;
     for (int pass = 0; pass < 3; ++pass) {
         __syncthreads();
         if (threadIdx.x == 0) *s_int = 0;
         float mx = 0.0f;
         __syncthreads();
-        for (int e = threadIdx.x; e < kk; e += T) {
-            const int i = e % k, j = e / k;
+        for (int e = threadIdx.x; e < k * (k + 1) / 2; e += T) {
+            // row i, column j <= i of the symmetric E
+            int i = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+            i += (i + 1) * (i + 2) / 2 <= e;
+            i -= i * (i + 1) / 2 > e;
+            const int j = e - i * (i + 1) / 2;
             double acc = i == j ? -1.0 : 0.0;
             for (int r = 0; r < k; ++r) acc = fma(V[r * k + i], V[r * k + j], acc);
-            scr[e] = acc;
+            scr[i * k + j] = scr[j * k + i] = acc;
             const float af = fabsf(to_float_scaled(acc, 0));
             mx = af <= mx ? mx : (af == af ? af : FLT_MAX);
         }
@@ -925,10 +1054,12 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
             if (e < kk) {
+                // E^2 in FP32: it is below 1e-12 of the result at the last pass
                 const int i = e % k, j = e / k;
-                double acc = 0.0;
-                for (int m = 0; m < k; ++m) acc = fma(scr[m * k + i], scr[j * k + m], acc);
-                own[n] = fma(0.5, scr[e], -0.375 * acc);
+                float acc = 0.0f;
+                for (int m = 0; m < k; ++m)
+                    acc = fmaf(to_float_scaled(scr[m * k + i], 16), to_float_scaled(scr[j * k + m], 16), acc);
+                own[n] = fma(0.5, scr[e], -0.375 * 0x1p-32 * to_double(acc));
             }
         }
         __syncthreads();
@@ -954,7 +1085,7 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) V[last ? (e % k) * k + e / k : e] = own[n];   // column-major at the end
+            if (e < kk) V[last ? (e % k) * ld + e / k : e] = own[n];   // column-major at the end
         }
         if (last) break;
         ok = pass < 2;
@@ -968,7 +1099,7 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             if (e < kk) {
                 const int i = e % k, c = e / k;
                 double acc = 0.0;
-                for (int j = 0; j < k; ++j) acc = fma(G[j * k + i], V[c * k + j], acc);
+                for (int j = 0; j < k; ++j) acc = fma(G[j * ld + i], V[c * ld + j], acc);
                 own[n] = acc;
             }
         }
@@ -976,14 +1107,15 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) G[e] = own[n];
+            if (e < kk) G[(e / k) * ld + e % k] = own[n];
         }
     } else {
-        for (int e = threadIdx.x; e < kk; e += T) V[e] = e % k == e / k ? 1.0 : 0.0;
+        for (int e = threadIdx.x; e < kl; e += T) V[e] = e % ld == e / ld ? 1.0 : 0.0;
     }
+    for (int e = threadIdx.x; e < k * (ld - k); e += T) V[(e / (ld - k)) * ld + k + e % (ld - k)] = 0.0;
     __syncthreads();
     float* dl = (float*)del;
-    jacobi_f64_segments<R>(G, V, Sraw, dl, k, fro, s_int);
+    jacobi_f64_segments<R>(G, V, Sraw, dl, k, ld, fro, ring, s_int);
     // the columns' scales, and the norms of the result
     const double up = ldexp(1.0, ex);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
@@ -993,10 +1125,10 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
         if (j < k) {
             const double s1 = 1.0 + to_double(dl[j]);
             for (int i = sl; i < k; i += 8) {
-                const double x = G[j * k + i] * s1;
+                const double x = G[j * ld + i] * s1;
                 a = fma(x, x, a);
-                G[j * k + i] = x * up;
-                V[j * k + i] *= s1;
+                G[j * ld + i] = x * up;
+                V[j * ld + i] *= s1;
             }
         }
         a = seg8_sum(a);
@@ -1005,19 +1137,23 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     __syncthreads();
 }
 
-// jacobi_pre() for the sizes it serves (16 < k <= 64 and enough threads), else jacobi().
+// jacobi_pre() for 16 < k <= 64 (blockDim >= 16 k, as block_for() gives), else
+// jacobi().  G and V: leading dimension jacobi_ld(k).
 __device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k, double* red, int* s_rot);
 __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
                                             double* red, int* s_rot) {
-    if (k > 16 && k <= 64 && k * k <= 8 * nthreads()) {
+    __shared__ SegRot ring[64];
+    if (k > 16 && k <= 64) {
         if (k <= 24)
-            jacobi_pre<3>(G, V, Sraw, k, scr, del, red, s_rot);
+            jacobi_pre<3>(G, V, Sraw, k, scr, del, ring, red, s_rot);
         else if (k <= 32)
-            jacobi_pre<4>(G, V, Sraw, k, scr, del, red, s_rot);
+            jacobi_pre<4>(G, V, Sraw, k, scr, del, ring, red, s_rot);
         else if (k <= 40)
-            jacobi_pre<5>(G, V, Sraw, k, scr, del, red, s_rot);
+            jacobi_pre<5>(G, V, Sraw, k, scr, del, ring, red, s_rot);
+        else if (k <= 56)
+            jacobi_pre<7>(G, V, Sraw, k, scr, del, ring, red, s_rot);
         else
-            jacobi_pre<8>(G, V, Sraw, k, scr, del, red, s_rot);
+            jacobi_pre<8>(G, V, Sraw, k, scr, del, ring, red, s_rot);
         return;
     }
     jacobi(G, V, Sraw, k, red, s_rot);
@@ -1107,9 +1243,9 @@ __device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k
 // descending, ties by index), US = U diag(S) (M x k row-major) and Vt (k x N
 // row-major, row strides ldus / ldvt) with the largest-|.| entry of every Vt
 // row positive.  perm: k ints.
-__device__ __forceinline__ void svd_assemble(const double* G, const double* QV, const double* Sraw, int* perm,
-                                             double* S, double* US, double* Vt, int M, int N, int k, int len,
-                                             int wide, int ldus, int ldvt) {
+__device__ __forceinline__ void svd_assemble(const double* G, int ldg, const double* QV, const double* Sraw,
+                                             int* perm, double* S, double* US, double* Vt, int M, int N, int k,
+                                             int len, int wide, int ldus, int ldvt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < k; i += nthreads()) {
         const double si = Sraw[i];
@@ -1124,7 +1260,7 @@ __device__ __forceinline__ void svd_assemble(const double* G, const double* QV, 
     for (int64_t e = threadIdx.x; e < (int64_t)M * k; e += nthreads()) {
         const int i = (int)(e / k), r = (int)(e % k);
         const int p = perm[r];
-        US[(int64_t)i * ldus + r] = wide ? G[(int64_t)p * k + i] : Sraw[p] * QV[(int64_t)p * len + i];
+        US[(int64_t)i * ldus + r] = wide ? G[(int64_t)p * ldg + i] : Sraw[p] * QV[(int64_t)p * len + i];
     }
     for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += nthreads()) {
         const int r = (int)(e / N), c = (int)(e % N);
@@ -1134,7 +1270,7 @@ __device__ __forceinline__ void svd_assemble(const double* G, const double* QV, 
             v = QV[(int64_t)p * len + c];
         } else {
             const double sp = Sraw[p];
-            v = sp > 0.0 ? G[(int64_t)p * k + c] / sp : 0.0;
+            v = sp > 0.0 ? G[(int64_t)p * ldg + c] / sp : 0.0;
         }
         Vt[(int64_t)r * ldvt + c] = v;
     }

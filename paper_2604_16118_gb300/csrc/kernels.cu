@@ -100,25 +100,26 @@ __global__ void __launch_bounds__(kSmallGemmThreads) k_gemm_small(const GemmOut*
 // tau = (beta - alpha)/beta, v = x/(alpha - beta).
 __global__ void __launch_bounds__(kThreads) k_qr(const QrTask* __restrict__ tasks) {
     extern __shared__ double sm[];
-    __shared__ double red[33];
-    __shared__ double sh[2];
     const QrTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = M < N ? M : N;
     double* A = tk.smem ? sm : tk.A;
     double* Q = tk.smem ? sm + (int64_t)M * N : tk.Q;
     double* tau = tk.smem ? sm + (int64_t)M * N + (int64_t)M * k : tk.tau;
+    double* vd = tk.smem ? tau + k : tk.R;   // the reflectors' diagonals, until Q is formed
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (tk.smem) {
         for (int64_t e = threadIdx.x; e < (int64_t)M * N; e += kThreads) A[e] = tk.A[e];
         __syncthreads();
     }
-    dev::householder(A, tau, M, N, red, sh);
+    dev::householder(A, tau, vd, M, N);
+    dev::form_q(A, tau, vd, Q, M, k);
+    __syncthreads();
     // R (k x N row-major) from the upper trapezoid
     for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += kThreads) {
         const int r = (int)(e / N), c = (int)(e % N);
         tk.R[e] = c >= r ? A[(int64_t)c * M + r] : 0.0;
     }
-    dev::form_q(A, tau, Q, M, k);
+    __syncthreads();
     // diag(R) >= 0 (R is in global memory; every thread sees the final R after the barrier)
     for (int j = warp; j < k; j += kWarps) {
         const double rjj = A[(int64_t)j * M + j];
@@ -177,7 +178,7 @@ struct SvdFin {
 
 __global__ void __launch_bounds__(kThreads) k_svd_finalize(const SvdFin* __restrict__ tasks) {
     const SvdFin tk = tasks[blockIdx.x];
-    dev::svd_assemble(tk.G, tk.QVt, tk.Sraw, tk.perm, tk.S, tk.US, tk.Vt, tk.M, tk.N, tk.k, tk.len, tk.wide, tk.k, tk.N);
+    dev::svd_assemble(tk.G, tk.k, tk.QVt, tk.Sraw, tk.perm, tk.S, tk.US, tk.Vt, tk.M, tk.N, tk.k, tk.len, tk.wide, tk.k, tk.N);
 }
 
 __global__ void __launch_bounds__(kThreads) k_sumsq(const double* const* __restrict__ xs,
@@ -461,7 +462,7 @@ void launch_qr(Context* ctx, const std::vector<QrTask>& tasks_in, int kind) {
         if (need <= kSmemBudget) {
             t.smem = 1;
             small.push_back(t);
-            smem_max = std::max(smem_max, need);
+            smem_max = std::max(smem_max, need + sizeof(double) * (size_t)std::min(t.M, t.N));
         } else {
             t.smem = 0;
             large.push_back(t);
@@ -478,7 +479,7 @@ void launch_qr(Context* ctx, const std::vector<QrTask>& tasks_in, int kind) {
                 const size_t need = sizeof(double) * ((size_t)t.M * t.N + (size_t)t.M * std::min(t.M, t.N) +
                                                       (size_t)std::min(t.M, t.N));
                 t.smem = need <= kSmemBudget ? 1 : 0;
-                if (t.smem) smem_max = std::max(smem_max, need);
+                if (t.smem) smem_max = std::max(smem_max, need + sizeof(double) * (size_t)std::min(t.M, t.N));
                 (t.smem ? small : large).push_back(t);
             }
         }

@@ -45,7 +45,7 @@ struct QrTask {
     double* R;
     double* tau;
     int M, N;
-    int smem = 0;     // set by launch_qr
+    int smem = 0;     // set by launch_qr (1: one CTA in shared memory) and by launch_qr_cluster (reflectors pulled at a time)
 };
 
 // SVD of an M x N matrix A, k = min(M, N), given in G: A column-major when
@@ -93,6 +93,9 @@ constexpr int kClusterJacobiMax = 336;
 // Jacobi problems from this size on go to the cluster kernel: below it one SM's
 // FP64 units suffice for the latency of a round.
 constexpr int kClusterJacobiMin = 32;
+// Sectors of the per-site right sweep with at most this many kept columns run whole
+// (QR, Jacobi, assembly) in one CTA when they fit its shared memory.
+constexpr int kSvdSiteMax = 64;
 bool launch_jacobi_cluster(Context* ctx, const std::vector<JacTask>& tasks);
 // FP32 one-sided Jacobi of the same tasks as a preconditioner: reads G (FP64,
 // unchanged), writes to V the accumulated FP32 rotations as FP64 (orthogonal to

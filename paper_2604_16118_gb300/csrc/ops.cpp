@@ -555,11 +555,11 @@ void right_sweep_sitewise(Context* ctx, TruncJob& J) {
         }
         double* S_all = s.dbl((size_t)std::max<int64_t>(stot, 1));
         // sectors of this bond: small ones in the fused one-CTA kernel, the others
-        // (k >= kClusterJacobiMin, or too large for it) by QR + Jacobi on clusters
+        // (k > kSvdSiteMax, or too large for it) by QR + Jacobi on clusters
         std::vector<int> site_sec, gen_sec;
         for (int ni = 0; ni < nn; ++ni) {
             if (kk[ni] == 0) continue;
-            if (kk[ni] < kClusterJacobiMin && svd_site_fits(bn.dim[ni], c0[ni] + c1[ni]))
+            if (kk[ni] <= kSvdSiteMax && svd_site_fits(bn.dim[ni], c0[ni] + c1[ni]))
                 site_sec.push_back(ni);
             else
                 gen_sec.push_back(ni);

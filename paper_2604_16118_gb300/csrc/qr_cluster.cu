@@ -4,15 +4,21 @@
 // FP64 units of C SMs (one SM retires one FP64 warp instruction per 16 cycles
 // on this GPU, which bounds a one-CTA QR).
 //
-// Column j: its owner forms the reflector H_j = I - tau v v^T (v_j = 1,
-// beta = -sign(alpha) ||x||, the reflector() of dev::householder_small) and
-// scales v in place; after one cluster barrier every CTA copies v_j and tau_j
-// from the owner's shared memory and applies H_j to its own columns p > j.
-// Q = H_0 ... H_{k-1} applied to the first k columns of I is formed
-// afterwards by every CTA for its own Q columns without further barriers (the
-// reflectors no longer change).  diag(R) >= 0: row j of R and column j of Q
-// change sign when beta_j < 0.  Output as QrTask of k_qr: Q (M x k,
-// column-major), R (k x N, row-major).
+// What bounds it is the chain from one reflector to the next (two reductions, a
+// reciprocal square root and a reciprocal, the hand-over to the other CTAs), so
+// that chain runs ahead: in step j the owner of column j + 1 applies H_j to that
+// column first, forms H_{j+1} = I - tau v v^T (v = the column below row j + 1,
+// unscaled, v_{j+1} = sign(alpha) (|alpha| + n), tau = 1 / (n (n + |alpha|))) and
+// writes v, tau and v_{j+1} straight into every CTA's shared memory, while all
+// other warps of the cluster apply H_j to the columns beyond.  One cluster
+// barrier per column ends the step.  A column of a trailing update is worked on by
+// 8, 16 or 32 lanes, the fewer the more columns a CTA holds (fewer reduction
+// steps per column), so that all four schedulers stay busy.
+// Q = H_0 ... H_{k-1} applied to the first k columns of I is formed afterwards
+// by every CTA for its own Q columns, the reflectors pulled from their owners a
+// few at a time.  diag(R) >= 0: row j of R and column j of Q change sign when
+// beta_j < 0.  Output as QrTask of k_qr: Q (M x k, column-major), R (k x N,
+// row-major).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -25,126 +31,244 @@ namespace cg = cooperative_groups;
 namespace bsm {
 namespace {
 
-constexpr int kQcThreads = 512;
+constexpr int kQcThreads = 256;
 constexpr int kQcWarps = kQcThreads / 32;
 constexpr size_t kQcSmemMax = 220 * 1024;
+constexpr int kQcLongRows = 256;   // from this many rows on four warps share a column's chain
 
-// shared memory of one CTA: its A and Q columns, one copy of v, tau and beta of every column
+// shared memory of one CTA: its A and Q columns, one pulled reflector, tau and the reflectors' diagonals
 size_t qc_smem(int M, int N, int C) {
     const int k = std::min(M, N);
     const size_t na = (size_t)(N + C - 1) / C, nq = (size_t)(k + C - 1) / C;
     return sizeof(double) * ((na + nq + 1) * (size_t)M + 2 * (size_t)k);
 }
+// The kernel pulls up to 8 reflectors at a time where shared memory has room for more than one.
+constexpr int kQcPull = 8;
+int qc_pull(int M, int N, int C) {
+    const size_t base = qc_smem(M, N, C);
+    if (base >= kQcSmemMax) return 1;
+    return (int)std::min<size_t>(kQcPull, 1 + (kQcSmemMax - base) / (sizeof(double) * (size_t)M));
+}
+
+template <int L>
+__device__ __forceinline__ double seg_sum_of(double v) {
+#pragma unroll
+    for (int o = L >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Local columns lp (global rank + lp C), lp0 <= lp < n, lp != skip: a -= tau (v^T a) v
+// over the rows j .. M-1 (v_j = vj), L lanes per column, by worker w of nw.
+template <int L>
+__device__ __forceinline__ void qc_update(double* Al, const double* v, double tj, double vj, int M, int j, int lp0,
+                                          int n, int skip, int w, int nw, int lane) {
+    const int sl = lane & (L - 1);
+    for (int cb = lp0 + w * (32 / L); cb < n; cb += nw * (32 / L)) {
+        const int lp = cb + lane / L;
+        const bool on = lp < n && lp != skip;
+        double* a = Al + (size_t)(on ? lp : lp0) * M;
+        double d = sl == 0 ? vj * a[j] : 0.0;
+        for (int i = j + 1 + sl; i < M; i += L) d = fma(v[i], a[i], d);
+        const double tw = tj * seg_sum_of<L>(d);
+        if (on) {
+            if (sl == 0) a[j] = fma(-tw, vj, a[j]);
+            for (int i = j + 1 + sl; i < M; i += L) a[i] = fma(-tw, v[i], a[i]);
+        }
+    }
+}
+
+// This CTA's columns of Q, L lanes each, through the reflectors j0 + n - 1 .. j0 held in vb (rows from j on).
+template <int L, int C>
+__device__ __forceinline__ void qc_form(double* Ql, const double* vb, const double* taus, const double* vds, int M,
+                                        int j0, int n, int q_loc, int rank, int warp, int lane) {
+    const int sl = lane & (L - 1);
+    for (int cb = warp * (32 / L); cb < q_loc; cb += kQcWarps * (32 / L)) {
+        const int lq = cb + lane / L;
+        const int p = lq < q_loc ? rank + lq * C : -1;
+        double* q = Ql + (size_t)(lq < q_loc ? lq : 0) * M;
+        for (int b = n - 1; b >= 0; --b) {
+            const int j = j0 + b;
+            const double tj = taus[j];
+            if (tj == 0.0) continue;
+            const double vj = vds[j];
+            const double* v = vb + (size_t)b * M;
+            const int i0 = j + ((sl - j) & (L - 1));
+            double d = 0.0;
+            if (p >= j)
+                for (int i = i0; i < M; i += L) d = fma(i == j ? vj : v[i], q[i], d);
+            const double tw = tj * seg_sum_of<L>(d);
+            if (p >= j)
+                for (int i = i0; i < M; i += L) q[i] = fma(-tw, i == j ? vj : v[i], q[i]);
+        }
+    }
+}
 
 template <int C>
 __global__ void __launch_bounds__(kQcThreads) k_qr_cluster(const QrTask* __restrict__ tasks) {
     extern __shared__ double qc_sm[];
-    __shared__ double red[33];
+    __shared__ double part[2][4];
+    __shared__ double s_alpha;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const QrTask tk = tasks[blockIdx.x / C];
     const int M = tk.M, N = tk.N, k = M < N ? M : N;
     const int na = (N + C - 1) / C, nq = (k + C - 1) / C;
     double* Al = qc_sm;                          // local column lp = global column rank + lp C
-    double* Ql = Al + (size_t)na * M;
-    double* vb = Ql + (size_t)nq * M;            // copy of the current reflector
-    double* taus = vb + M;                       // tau_j of the columns this CTA owns (by j)
-    double* betas = taus + k;                    // R(j, j) before the sign rule, owned columns
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* Ql = Al + (size_t)na * M;            // while A is factorised: two reflectors in flight
+    double* taus = Ql + (size_t)nq * M;          // tau_j and v_j(j) of every column
+    double* vds = taus + k;                      // (tau_j = 0: -R(j, j)); beta_j < 0 exactly when vds[j] > 0
+    double* vb = vds + k;                        // pulled reflectors
+    const int n_pull = tk.smem;
+    const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_loc = rank < N ? (N - 1 - rank) / C + 1 : 0;
-    for (int64_t e = threadIdx.x; e < (int64_t)n_loc * M; e += kQcThreads) {
+    const int nch = M >= kQcLongRows ? 4 : 1;    // warps of the chain
+    for (int64_t e = tid; e < (int64_t)n_loc * M; e += kQcThreads) {
         const int lp = (int)(e / M), i = (int)(e % M);
         Al[e] = tk.A[(int64_t)(rank + lp * C) * M + i];
     }
-    __syncthreads();
+    cluster.sync();   // every CTA runs before the first reflector is written into it
+    // sum over the chain's warps; slot: two reductions in a row use different slots
+    auto chain_sum = [&](double v, int slot) {
+        v = dev::warp_sum(v);
+        if (nch == 1) return v;
+        if (lane == 0) part[slot][warp] = v;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        return (part[slot][0] + part[slot][1]) + (part[slot][2] + part[slot][3]);
+    };
+    // H_{j-1} applied to column j (j > 0), H_j formed and handed to every CTA
+    auto chain = [&](int j) {
+        double* x = Al + (size_t)(j / C) * M;
+        const int t0 = tid, step = 32 * nch;
+        double tw = 0.0, vj = 0.0;
+        const double* v = Ql + (size_t)((j - 1) & 1) * M;
+        if (j > 0) {
+            const double tj = taus[j - 1];
+            vj = vds[j - 1];
+            if (tj != 0.0) {
+                double d = t0 == 0 ? vj * x[j - 1] : 0.0;
+                for (int i = j + t0; i < M; i += step) d = fma(v[i], x[i], d);
+                tw = tj * chain_sum(d, 0);
+                if (t0 == 0) x[j - 1] = fma(-tw, vj, x[j - 1]);
+            }
+        }
+        double s = 0.0, alpha = 0.0;
+        double* dst = Ql + (size_t)(j & 1) * M;
+        for (int i = j + t0; i < M; i += step) {
+            const double y = tw != 0.0 ? fma(-tw, v[i], x[i]) : x[i];
+            x[i] = y;
+            if (i == j) {
+                alpha = y;
+                continue;
+            }
+            s = fma(y, y, s);
+#pragma unroll
+            for (int c = 0; c < C; ++c) cluster.map_shared_rank(dst, c)[i] = y;
+        }
+        if (nch > 1 && t0 == 0) s_alpha = alpha;   // visible after the reduction's barrier
+        s = chain_sum(s, 1);
+        alpha = nch > 1 ? s_alpha : __shfl_sync(0xffffffffu, alpha, 0);
+        double tj = 0.0, vd = -alpha;
+        if (s != 0.0) {
+            const double w = fma(alpha, alpha, s);
+            const double rn = dev::rsqrt_halley(w);
+            const double n = w * rn, q = fabs(alpha) + n;
+            tj = rn * dev::recip_newton(q);
+            vd = alpha >= 0.0 ? q : -q;
+            if (t0 == 0) x[j] = alpha >= 0.0 ? -n : n;
+        }
+        if (t0 < C) {
+            cluster.map_shared_rank(taus, t0)[j] = tj;
+            cluster.map_shared_rank(vds, t0)[j] = vd;
+        }
+    };
+    if (rank == 0 && warp < nch) chain(0);
+    cluster.sync();
     for (int j = 0; j < k; ++j) {
-        const int owner = j % C;
-        if (rank == owner) {
-            double* col = Al + (size_t)(j / C) * M;
-            double s = 0.0;
-            for (int i = j + 1 + threadIdx.x; i < M; i += kQcThreads) s += col[i] * col[i];
-            s = dev::block_sum(s, red);
-            const double alpha = col[j];
-            double tj = 0.0, scale = 0.0, beta = alpha;
-            if (s != 0.0) dev::reflector(alpha, s, &beta, &tj, &scale);
-            if (tj != 0.0)
-                for (int i = j + 1 + threadIdx.x; i < M; i += kQcThreads) col[i] *= scale;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                col[j] = beta;
-                taus[j] = tj;
-                betas[j] = beta;
+        const double tj = taus[j], vj = vds[j];
+        const bool own = j + 1 < k && rank == (j + 1) % C;
+        if (own && warp < nch) {
+            chain(j + 1);
+        } else if (tj != 0.0) {
+            // in the owner's CTA the other warps, without those on the chain's scheduler when it has one
+            int w = warp, nw = kQcWarps;
+            if (own && nch == 1) {
+                w = (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
+                nw = kQcWarps / 4 * 3;
+            } else if (own) {
+                w = warp - nch;
+                nw = kQcWarps - nch;
+            }
+            const int lp0 = j + 1 <= rank ? 0 : (j + 1 - rank + C - 1) / C;
+            const int left = n_loc - lp0, skip = own ? (j + 1) / C : -1;
+            const double* v = Ql + (size_t)(j & 1) * M;
+            if (w >= 0 && left > 0) {
+                if (left <= 4)
+                    qc_update<32>(Al, v, tj, vj, M, j, lp0, n_loc, skip, w, nw, lane);
+                else if (left <= 8)
+                    qc_update<16>(Al, v, tj, vj, M, j, lp0, n_loc, skip, w, nw, lane);
+                else
+                    qc_update<8>(Al, v, tj, vj, M, j, lp0, n_loc, skip, w, nw, lane);
             }
         }
         cluster.sync();
-        const double* ocol = cluster.map_shared_rank(Al + (size_t)(j / C) * M, owner);
-        const double tj = *cluster.map_shared_rank(taus + j, owner);
-        if (tj != 0.0) {
-            for (int i = j + 1 + threadIdx.x; i < M; i += kQcThreads) vb[i] = ocol[i];
-            __syncthreads();
-            // local columns p > j
-            const int lp0 = (j + 1 - rank + C - 1) / C > 0 ? (j + 1 - rank + C - 1) / C : 0;
-            for (int lp = lp0 + warp; lp < n_loc; lp += kQcWarps) {
-                double* a = Al + (size_t)lp * M;
-                const double a_j = a[j];
-                double w = 0.0;
-                for (int i = j + 1 + lane; i < M; i += 32) w += vb[i] * a[i];
-                w = dev::warp_sum(w) + a_j;
-                const double tw = tj * w;
-                if (lane == 0) a[j] = a_j - tw;
-                for (int i = j + 1 + lane; i < M; i += 32) a[i] -= tw * vb[i];
-            }
-        }
-        __syncthreads();
     }
     // Q: this CTA's columns p < k (p = rank + lq C), from the identity, reflectors backwards
     const int q_loc = rank < k ? (k - 1 - rank) / C + 1 : 0;
-    for (int64_t e = threadIdx.x; e < (int64_t)q_loc * M; e += kQcThreads) {
+    for (int64_t e = tid; e < (int64_t)q_loc * M; e += kQcThreads) {
         const int lq = (int)(e / M), i = (int)(e % M);
         Ql[e] = i == rank + lq * C ? 1.0 : 0.0;
     }
-    __syncthreads();
-    for (int j = k - 1; j >= 0; --j) {
-        const int owner = j % C;
-        const double tj = *cluster.map_shared_rank(taus + j, owner);
-        if (tj == 0.0) continue;
-        const double* ocol = cluster.map_shared_rank(Al + (size_t)(j / C) * M, owner);
-        for (int i = j + 1 + threadIdx.x; i < M; i += kQcThreads) vb[i] = ocol[i];
-        __syncthreads();
-        const int lq0 = (j - rank + C - 1) / C > 0 ? (j - rank + C - 1) / C : 0;
-        for (int lq = lq0 + warp; lq < q_loc; lq += kQcWarps) {
-            double* q = Ql + (size_t)lq * M;
-            const double q_j = q[j];
-            double w = 0.0;
-            for (int i = j + 1 + lane; i < M; i += 32) w += vb[i] * q[i];
-            w = dev::warp_sum(w) + q_j;
-            const double tw = tj * w;
-            if (lane == 0) q[j] = q_j - tw;
-            for (int i = j + 1 + lane; i < M; i += 32) q[i] -= tw * vb[i];
+    const int half = n_pull >= 2 ? n_pull / 2 : 1;
+    auto pull = [&](int j1, double* dst) {   // reflectors max(0, j1 - half) .. j1 - 1
+        const int j0 = max(0, j1 - half);
+        for (int e = tid; e < (j1 - j0) * M; e += kQcThreads) {
+            const int b = e / M, i = e % M, j = j0 + b;
+            if (i > j) dst[e] = cluster.map_shared_rank(Al + (size_t)(j / C) * M, j % C)[i];
         }
+    };
+    pull(k, vb);
+    __syncthreads();
+    for (int j1 = k, it = 0; j1 > 0; j1 -= half, ++it) {
+        const int j0 = max(0, j1 - half);
+        const double* cur = vb + (n_pull >= 2 ? (size_t)(it & 1) * half * M : 0);
+        double* nxt = vb + (n_pull >= 2 ? (size_t)((it + 1) & 1) * half * M : 0);
+        if (n_pull >= 2) pull(j0, nxt);
+        if (q_loc <= 4)
+            qc_form<32, C>(Ql, cur, taus, vds, M, j0, j1 - j0, q_loc, rank, warp, lane);
+        else if (q_loc <= 8)
+            qc_form<16, C>(Ql, cur, taus, vds, M, j0, j1 - j0, q_loc, rank, warp, lane);
+        else
+            qc_form<8, C>(Ql, cur, taus, vds, M, j0, j1 - j0, q_loc, rank, warp, lane);
         __syncthreads();
+        if (n_pull < 2) {
+            pull(j0, nxt);
+            __syncthreads();
+        }
     }
     // R (row-major k x N) from this CTA's A columns and Q columns, with the sign rule
-    for (int64_t e = threadIdx.x; e < (int64_t)n_loc * k; e += kQcThreads) {
+    for (int64_t e = tid; e < (int64_t)n_loc * k; e += kQcThreads) {
         const int lp = (int)(e / k), r = (int)(e % k);
         const int c = rank + lp * C;
-        const double sg = *cluster.map_shared_rank(betas + r, r % C) < 0.0 ? -1.0 : 1.0;
-        tk.R[(int64_t)r * N + c] = c >= r ? sg * Al[(size_t)lp * M + r] : 0.0;
+        tk.R[(int64_t)r * N + c] = c >= r ? (vds[r] > 0.0 ? -1.0 : 1.0) * Al[(size_t)lp * M + r] : 0.0;
     }
-    for (int64_t e = threadIdx.x; e < (int64_t)q_loc * M; e += kQcThreads) {
+    for (int64_t e = tid; e < (int64_t)q_loc * M; e += kQcThreads) {
         const int lq = (int)(e / M), i = (int)(e % M);
         const int p = rank + lq * C;
-        tk.Q[(int64_t)p * M + i] = (betas[p] < 0.0 ? -1.0 : 1.0) * Ql[e];
+        tk.Q[(int64_t)p * M + i] = (vds[p] > 0.0 ? -1.0 : 1.0) * Ql[e];
     }
     // no CTA leaves while another may still read its shared memory
     cluster.sync();
 }
 
 template <int C>
-bool launch_qc(Context* ctx, const std::vector<QrTask>& tasks) {
+bool launch_qc(Context* ctx, const std::vector<QrTask>& tasks_in) {
     size_t smem = 0;
-    for (const QrTask& t : tasks) smem = std::max(smem, qc_smem(t.M, t.N, C));
-    if (smem > kQcSmemMax) return false;
+    std::vector<QrTask> tasks = tasks_in;
+    for (QrTask& t : tasks) {
+        if (qc_smem(t.M, t.N, C) > kQcSmemMax) return false;
+        t.smem = qc_pull(t.M, t.N, C);   // reflectors pulled at a time
+        smem = std::max(smem, qc_smem(t.M, t.N, C) + sizeof(double) * (size_t)(t.smem - 1) * t.M);
+    }
     static bool attr = false;
     if (!attr) {
         BSM_CUDA(cudaFuncSetAttribute(k_qr_cluster<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQcSmemMax));

@@ -31,8 +31,8 @@ size_t cut_smem(const CutTask& c) {
 }
 
 size_t svd_smem(int M, int N) {
-    const size_t k = (size_t)std::min(M, N), len = (size_t)std::max(M, N);
-    return sizeof(double) * (2 * len * k + 2 * k * k + 3 * k);
+    const size_t k = (size_t)std::min(M, N), len = (size_t)std::max(M, N), ld = (size_t)dev::jacobi_ld((int)k);
+    return sizeof(double) * ((std::max(len, ld) + len) * k + 2 * k * ld + 3 * k);
 }
 
 // Global loads of data that other CTAs of the same launch may have written
@@ -90,7 +90,7 @@ __device__ void left_rank1(const LeftTask& tk, const LeftSrc* __restrict__ srcs,
 
 template <bool CG>
 __device__ void left_body(const LeftTask& tk, const LeftSrc* __restrict__ srcs, const LeftX* __restrict__ xs,
-                          double* sm, double* red, double* sh) {
+                          double* sm, double* red) {
     const int M = tk.M, N = tk.N, k = tk.k;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* A = sm;
@@ -130,12 +130,13 @@ __device__ void left_body(const LeftTask& tk, const LeftSrc* __restrict__ srcs, 
         left_rank1<CG>(tk, srcs, xs, A, red);
         return;
     }
-    dev::householder(A, tau, M, N, red, sh);
+    dev::householder(A, tau, R, M, N);   // R's first k entries hold the reflectors' diagonals until Q is formed
+    dev::form_q(A, tau, R, Q, M, k);
+    __syncthreads();
     for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += nthreads()) {
         const int r = (int)(e / N), c = (int)(e % N);
         R[e] = c >= r ? A[(int64_t)c * M + r] : 0.0;
     }
-    dev::form_q(A, tau, Q, M, k);
     __syncthreads();
     for (int j = warp; j < k; j += nwarps()) {
         if (A[(int64_t)j * M + j] < 0.0) {
@@ -167,24 +168,23 @@ __global__ void __launch_bounds__(kSweepThreads) k_left_site(const LeftTask* __r
                                                         const LeftX* __restrict__ xs) {
     extern __shared__ double sm[];
     __shared__ double red[33];
-    __shared__ double sh[2];
-    left_body<false>(tasks[blockIdx.x], srcs, xs, sm, red, sh);
+    left_body<false>(tasks[blockIdx.x], srcs, xs, sm, red);
 }
 
 __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* __restrict__ tasks,
                                                        const SvdPart* __restrict__ parts) {
     extern __shared__ double sm[];
     __shared__ double red[33];
-    __shared__ double sh[2];
     __shared__ int s_rot;
     const SvdSiteTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = tk.k, len = tk.len;
     double* B = sm;                               // QR input (len x k), later Q V
-    double* Q = B + (int64_t)len * k;
+    const int ld = dev::jacobi_ld(k);
+    double* Q = B + (int64_t)max(len, ld) * k;
     double* tau = Q + (int64_t)len * k;
     double* G = tau + k;
-    double* V = G + (int64_t)k * k;
-    double* Sraw = V + (int64_t)k * k;
+    double* V = G + (int64_t)k * ld;
+    double* Sraw = V + (int64_t)k * ld;
     int* perm = (int*)(Sraw + k);
     for (int p = tk.p_beg; p < tk.p_end; ++p) {
         const SvdPart pt = parts[p];
@@ -197,23 +197,23 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
         }
     }
     __syncthreads();
-    dev::householder(B, tau, len, k, red, sh);
+    dev::householder(B, tau, Sraw, len, k);
     // G = R^T (column-major): G(i, j) = R(j, i), nonzero for i >= j
-    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += nthreads()) {
-        const int j = (int)(e / k), i = (int)(e % k);
-        G[e] = i >= j ? B[(int64_t)i * len + j] : 0.0;
+    for (int e = threadIdx.x; e < k * ld; e += nthreads()) {
+        const int j = e / ld, i = e % ld;
+        G[e] = i >= j && i < k ? B[(int64_t)i * len + j] : 0.0;
     }
-    dev::form_q(B, tau, Q, len, k);
+    dev::form_q(B, tau, Sraw, Q, len, k);
     __syncthreads();
     dev::jacobi_auto(G, V, Sraw, k, B, tau, red, &s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
-        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * k + j], acc);
+        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * ld + j], acc);
         B[e] = acc;
     }
     __syncthreads();
-    dev::svd_assemble(G, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, tk.wide, k, N);
+    dev::svd_assemble(G, ld, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, tk.wide, k, N);
 }
 
 __global__ void __launch_bounds__(kThreads) k_right_apply(const RTask* __restrict__ tasks,
@@ -319,7 +319,7 @@ __device__ void right_rank1(const DynTask& tk, const double* v, int len, int wid
 
 template <bool CG>
 __device__ void right_body(const DynTask& tk, double* sm, double* red,
-                           double* sh, int* s_rot, int* s_cols) {
+                           int* s_rot, int* s_cols) {
     const int np = tk.p_end - tk.p_beg;
     if (threadIdx.x < 2) {
         int c = 0;
@@ -337,11 +337,12 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     }
     const int k = M < N ? M : N, len = M < N ? N : M, wide = M < N ? 1 : 0;
     double* B = sm;
-    double* Q = B + (int64_t)len * k;
+    const int ld = dev::jacobi_ld(k);
+    double* Q = B + (int64_t)max(len, ld) * k;
     double* tau = Q + (int64_t)len * k;
     double* G = tau + k;
-    double* V = G + (int64_t)k * k;
-    double* Sraw = V + (int64_t)k * k;
+    double* V = G + (int64_t)k * ld;
+    double* Sraw = V + (int64_t)k * ld;
     int* perm = (int*)(Sraw + k);
     int coff = 0;
     for (int p = 0; p < np; ++p) {
@@ -381,32 +382,31 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
         if (threadIdx.x == 0) *tk.kact = k;
         return;
     }
-    dev::householder(B, tau, len, k, red, sh);
-    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += nthreads()) {
-        const int j = (int)(e / k), i = (int)(e % k);
-        G[e] = i >= j ? B[(int64_t)i * len + j] : 0.0;
+    dev::householder(B, tau, Sraw, len, k);
+    for (int e = threadIdx.x; e < k * ld; e += nthreads()) {
+        const int j = e / ld, i = e % ld;
+        G[e] = i >= j && i < k ? B[(int64_t)i * len + j] : 0.0;
     }
-    dev::form_q(B, tau, Q, len, k);
+    dev::form_q(B, tau, Sraw, Q, len, k);
     __syncthreads();
     dev::jacobi_auto(G, V, Sraw, k, B, tau, red, s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
-        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * k + j], acc);
+        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * ld + j], acc);
         B[e] = acc;
     }
     __syncthreads();
-    dev::svd_assemble(G, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, wide, tk.kpad, tk.ncols_pad);
+    dev::svd_assemble(G, ld, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, wide, tk.kpad, tk.ncols_pad);
     if (threadIdx.x == 0) *tk.kact = k;
 }
 
 __global__ void __launch_bounds__(kSweepThreads) k_right_dyn(const DynTask* __restrict__ tasks) {
     extern __shared__ double sm[];
     __shared__ double red[33];
-    __shared__ double sh[2];
     __shared__ int s_rot;
     __shared__ int s_cols[2];
-    right_body<false>(tasks[blockIdx.x], sm, red, sh, &s_rot, s_cols);
+    right_body<false>(tasks[blockIdx.x], sm, red, &s_rot, s_cols);
 }
 
 // Pooled cut of one bond (one CTA): stable descending order with ties by
@@ -566,12 +566,11 @@ __global__ void __launch_bounds__(kSweepThreads) k_left_sweep(const LeftTask* __
                                                          GridSync* gs) {
     extern __shared__ double sm[];
     __shared__ double red[33];
-    __shared__ double sh[2];
     __shared__ int s_flag;
     for (int p = 0; p < n_phase; ++p) {
         for (int ti = phase_beg[p] + (int)blockIdx.x; ti < phase_beg[p + 1]; ti += (int)gridDim.x) {
             __syncthreads();
-            left_body<true>(tasks[ti], srcs, xs, sm, red, sh);
+            left_body<true>(tasks[ti], srcs, xs, sm, red);
         }
         if (p + 1 < n_phase && !phase_end(gs, (unsigned)p, &s_flag)) return;
     }
@@ -595,7 +594,6 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
                                                           int pb_off, GridSync* gs) {
     extern __shared__ double sm[];
     __shared__ double red[33];
-    __shared__ double sh[2];
     __shared__ int s_rot;
     __shared__ int s_cols[2];
     __shared__ int s_n;
@@ -622,7 +620,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
             __syncthreads();
             const bool first = ti == pb[p] + (int)blockIdx.x;
             const DynTask& tk = first ? s_task[p & 1] : tasks[ti];
-            right_body<true>(tk, sm, red, sh, &s_rot, s_cols);
+            right_body<true>(tk, sm, red, &s_rot, s_cols);
             // the CTA that completes the last task of this truncation's bond runs its cut
             __syncthreads();
             const CutTask& ct = cuts[tk.cut];
