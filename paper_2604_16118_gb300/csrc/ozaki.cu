@@ -11,10 +11,8 @@
 // integers below 2^14; the pairs of one d (at most 8) over 128 values of k stay
 // below 2^24, so the FP32 accumulator of the tensor-core product (tcgen05.mma
 // kind::f16, BF16 operands, accumulators in tensor memory) is exact, the
-// diagonals are combined exactly in 64-bit integers, and only the FP64
-// recombination rounds.
-#include <cuda_bf16.h>
-
+// diagonals are combined exactly in 64-bit integers, and the result is rounded
+// once.
 #include <algorithm>
 
 #include "kernels.h"
@@ -28,70 +26,145 @@ void launched(Context* ctx) {
     BSM_CUDA(cudaGetLastError());
 }
 
-// One row of op(A) or one column of B: its exponent and its digit slices.
-struct OzRow {
-    const double* src;
-    int64_t stride;        // element k at src[k * stride]
-    int len, Kp;           // K and K rounded up to 16
-    int* exp;
-    __nv_bfloat16* dst;    // slice 0 of the row; slice p at dst + p * slice_stride
-    int64_t slice_stride;
-};
-
-// One warp per row: e = the smallest integer with max |x| < 2^e, then the S
-// digits of x 2^-e (d = trunc(r 2^7), r <- r 2^7 - d, exact), zeros for k >= K.
-__global__ void k_oz_rows(const OzRow* __restrict__ rows, int n_rows, int S) {
-    const int lane = threadIdx.x & 31;
-    const int w = (int)blockIdx.x * (blockDim.x >> 5) + (int)(threadIdx.x >> 5);
-    if (w >= n_rows) return;
-    const OzRow rw = rows[w];
-    double mx = 0.0;
-    for (int k = lane; k < rw.len; k += 32) mx = fmax(mx, fabs(rw.src[(int64_t)k * rw.stride]));
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    int ex = 0;
-    if (mx > 0.0) frexp(mx, &ex);   // mx = m 2^ex, 0.5 <= m < 1
-    if (lane == 0) *rw.exp = ex;
-    for (int k = lane; k < rw.Kp; k += 32) {
-        double rem = k < rw.len ? ldexp(rw.src[(int64_t)k * rw.stride], -ex) : 0.0;
-        for (int p = 0; p < S; ++p) {
-            rem *= 128.0;                 // exact (power of two)
-            const double d = trunc(rem);
-            rem -= d;                     // exact
-            rw.dst[p * rw.slice_stride + k] = __double2bfloat16(d);   // |d| <= 127: exact
-        }
-    }
-}
-
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 fills zeros.
-__device__ __forceinline__ void cp16(void* smem, const void* gmem, int src_bytes) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(a), "l"(gmem), "r"(src_bytes));
-}
-
-constexpr int kOzKStep = 32;       // Kp is a multiple of this (slice rows padded with zeros)
+constexpr int kOzKStep = 32;       // k values of one staged chunk; Kp is a multiple of it (zeros from K on)
 constexpr int kOzMaxS = 8;
 constexpr int kOzM = 128;          // tile rows: the M of one tcgen05.mma (cta_group::1)
 constexpr int kOzN = 64;           // tile columns: its N, and the tensor-memory columns of one diagonal
-constexpr int kOzK = 16;           // k values per staged chunk: the K of one kind::f16 MMA
-constexpr int kOzThreads = 128;    // warp w reads tensor-memory lanes 32 w .. 32 w + 31
-constexpr int kOzSbo = 8 * kOzK * 2;                  // bytes between 8-row groups of a slice tile
-constexpr int kOzSliceA = kOzM * kOzK * 2;            // bytes of one A slice tile (128 x 16 bf16)
-constexpr int kOzSliceB = kOzN * kOzK * 2;            // bytes of one B slice tile (64 x 16 bf16)
+constexpr int kOzSbo = 8 * kOzKStep * 2;              // bytes between 8-row groups of a slice tile
+constexpr int kOzSliceA = kOzM * kOzKStep * 2;        // bytes of one A slice tile (128 x 32 bf16)
+constexpr int kOzSliceB = kOzN * kOzKStep * 2;        // bytes of one B slice tile (64 x 32 bf16)
+constexpr int kOzGroup = 128 / kOzKStep;              // chunks whose FP32 sums of slice products stay exact
+constexpr int kOzEpiWarps = 8;
+constexpr int kOzThreads = 32 * (2 + kOzEpiWarps);    // producer warp, MMA warp, epilogue warps
 constexpr uint32_t kOzIdesc = tc::idesc_bf16(kOzM, kOzN);
 
-// byte offset of (row r, k) in a K-major slice tile without swizzle: 8-row x
-// 16-byte core matrices, the two core matrices of a row group along k 128
-// bytes apart, row groups kOzSbo bytes apart
-__device__ __forceinline__ uint32_t oz_off(int r, int k) {
-    return (uint32_t)((r >> 3) * kOzSbo + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
+// One factor of a product, read as n rows of K values (rows of op(A), columns of
+// B: row r, value k at src[r rs + k ks], one of the strides 1), and its slices:
+// blocks of `blk` rows x 32 k values, all S slices of a block one after the
+// other, each in the canonical K-major operand layout (8-row x 16-byte core
+// matrices, the four core matrices of a row group along k 128 bytes apart, row
+// groups kOzSbo apart), so that a chunk of a tile is one contiguous copy.
+struct OzSide {
+    const double* src;
+    int64_t rs, ks;
+    int n, K, nkc, blk;
+    int64_t dst;         // bytes from the slice buffer to block (0, 0)
+    int row0;            // first row in the maxima and exponent arrays
+    int max0, cut0;      // first CTA of this factor in k_oz_max / k_oz_slice
+};
+
+__device__ __forceinline__ int oz_find(const OzSide* __restrict__ sides, int n, int cta, bool cut) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((cut ? sides[mid].cut0 : sides[mid].max0) <= cta) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Largest magnitudes of the rows (bit patterns of non-negative doubles, ordered
+// like their values; mx zeroed before).  Rows contiguous in k: one warp per row,
+// eight rows per CTA.  Rows contiguous across: 32 rows x 512 k values per CTA.
+constexpr int kOzMaxK = 512;
+__global__ void __launch_bounds__(256) k_oz_max(const OzSide* __restrict__ sides, int n_sides,
+                                                unsigned long long* __restrict__ mx) {
+    const OzSide sd = sides[oz_find(sides, n_sides, (int)blockIdx.x, false)];
+    const int u = (int)blockIdx.x - sd.max0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFull;
+    const unsigned long long* src = (const unsigned long long*)sd.src;
+    unsigned long long m = 0ull;
+    if (sd.ks == 1) {
+        const int r = 8 * u + warp;
+        if (r >= sd.n) return;
+        for (int k = lane; k < sd.K; k += 32) m = max(m, src[(int64_t)r * sd.rs + k] & kAbs);
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) mx[sd.row0 + r] = m;
+        return;
+    }
+    __shared__ unsigned long long part[8][32];
+    const int nb = (sd.n + 31) / 32;
+    const int r = 32 * (u % nb) + lane, k0 = (u / nb) * kOzMaxK;
+    if (r < sd.n)
+        for (int k = k0 + warp; k < min(sd.K, k0 + kOzMaxK); k += 8) m = max(m, src[r * sd.rs + k * sd.ks] & kAbs);
+    part[warp][lane] = m;
+    __syncthreads();
+    if (warp == 0 && r < sd.n) {
+        for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
+        atomicMax(&mx[sd.row0 + r], m);
+    }
+}
+
+// Exponents and slices.  e = the smallest integer with max |x| < 2^e; |x| 2^-e is
+// a 56-bit fraction F (FP64 magnitudes have 53 bits; what lies below is cut, as
+// digit by digit truncation does) whose 7-bit digits, with the sign of x, are the
+// slices: integer operations only (an FP64 digit costs four FP64 instructions,
+// 0.4 ms at n = 2048 on this GPU).  A warp writes 8 rows x 32 k values: lane
+// (kg, r) the eight values k = 8 kg .. 8 kg + 7 of row r as one 16-byte store per
+// slice, 512 contiguous bytes per warp.  Eight warps of a CTA cover eight chunks of
+// k (rows contiguous in k) or eight row groups (rows contiguous across).
+__global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sides, int n_sides, int S,
+                                                  const unsigned long long* __restrict__ mx, int* __restrict__ exps,
+                                                  unsigned char* __restrict__ buf) {
+    const OzSide sd = sides[oz_find(sides, n_sides, (int)blockIdx.x, true)];
+    const int u = (int)blockIdx.x - sd.cut0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int rg, kc;
+    if (sd.ks == 1) {
+        const int nk8 = (sd.nkc + 7) / 8;
+        rg = u / nk8;
+        kc = 8 * (u % nk8) + warp;
+    } else {
+        const int ng = ((sd.n + 7) / 8 + 7) / 8;
+        rg = 8 * (u % ng) + warp;
+        kc = u / ng;
+    }
+    if (kc >= sd.nkc || 8 * rg >= sd.n) return;
+    const int r = 8 * rg + (lane & 7), kg = lane >> 3;
+    const bool on = r < sd.n;
+    const unsigned long long top = on ? mx[sd.row0 + r] : 0ull;
+    int e = 0;
+    if (top != 0ull) frexp(__longlong_as_double((long long)top), &e);   // max = m 2^e, 0.5 <= m < 1
+    if (on && kc == 0 && kg == 0) exps[sd.row0 + r] = e;
+    unsigned long long F[8];
+    uint32_t neg = 0u;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int k = kOzKStep * kc + 8 * kg + t;
+        F[t] = 0ull;
+        if (on && k < sd.K) {
+            const unsigned long long b = ((const unsigned long long*)sd.src)[r * sd.rs + k * sd.ks];
+            const int ef = (int)((b >> 52) & 0x7ff);
+            const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (ef ? 1ull << 52 : 0ull);
+            const int sh = (ef ? ef : 1) - 1023 - e + 4;   // |x| = m 2^(ef - 1075), F = |x| 2^(56 - e)
+            F[t] = sh >= 0 ? m << min(sh, 3) : (sh > -64 ? m >> -sh : 0ull);
+            neg |= (uint32_t)(b >> 63) << t;
+        }
+    }
+    const int row = 8 * rg, blk = row / sd.blk;
+    const int64_t slice = (int64_t)sd.blk * kOzKStep * 2;
+    unsigned char* dst = buf + sd.dst + ((int64_t)blk * sd.nkc + kc) * S * slice + (row % sd.blk) / 8 * kOzSbo +
+                         kg * 128 + (lane & 7) * 16;
+    for (int p = 0; p < S; ++p) {
+        uint32_t w[4];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const uint32_t d = (uint32_t)(F[t] >> (49 - 7 * p)) & 127u;
+            // d as a float (2^23 + d - 2^23), whose upper half is the BF16 value
+            uint32_t h = __float_as_uint(__uint_as_float(0x4B000000u | d) - 8388608.0f) >> 16;
+            if (d) h |= ((neg >> t) & 1u) << 15;
+            if (t & 1) w[t >> 1] |= h << 16;
+            else w[t >> 1] = h;
+        }
+        *(uint4*)(dst + p * slice) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
 }
 
 // One product of a group, C = alpha op(A) B, with its slices and exponents.
 struct OzProd {
     double* C;
-    int M, N, Kp, ldc;
+    int M, N, nkc, ldc;
     double alpha;
-    int64_t a_off, b_off;   // slice 0 of op(A) (M x Kp) and of B^T (N x Kp) in the slice buffers
+    int64_t a_off, b_off;   // bytes from the slice buffer to the blocks of op(A) (128 rows) and of B (64 columns)
     int e_off, f_off;       // row exponents of op(A), column exponents of B
 };
 
@@ -99,59 +172,87 @@ struct OzTile {
     int prod, m0, n0;
 };
 
+// (hi 2^64 + lo) 2^sc rounded to nearest even, by integer operations.
+__device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, int sc) {
+    const bool neg = hi < 0;
+    unsigned long long h = (unsigned long long)hi;
+    if (neg) {
+        h = ~h;
+        lo = ~lo + 1ull;
+        h += lo == 0ull;
+    }
+    if ((h | lo) == 0ull) return 0.0;
+    const int lz = h ? __clzll((long long)h) : 64 + __clzll((long long)lo);
+    unsigned long long top, rest;
+    if (lz >= 64) {
+        top = lo << (lz - 64);
+        rest = 0ull;
+    } else {
+        top = lz ? (h << lz) | (lo >> (64 - lz)) : h;
+        rest = lo << lz;
+    }
+    unsigned long long m = top >> 11;
+    const unsigned r = (unsigned)top & 0x7ffu;
+    if (r > 0x400u || (r == 0x400u && (rest != 0ull || (m & 1ull)))) ++m;
+    const int E = 127 - lz + sc;   // exponent of the leading bit
+    if (E < -1022 || E > 1022) return ldexp(neg ? -(double)m : (double)m, E - 52);
+    // m = 2^53 after a carry raises the exponent by one: the addition does it
+    const unsigned long long b = ((unsigned long long)(E + 1022) << 52) + m;
+    return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
+}
+
 // C (M x N, row-major, ldc) = alpha sum_d 2^{e_i + f_j - 7(d + 2)} sum_{p + q = d + 2} A_p B_q
-// (slices numbered from 1).  One CTA per 128 x 64 output tile:
-//  - k chunks of 16 values of every A and B slice are staged by cp.async into
-//    two buffers (the next chunk loads while the tensor cores work on this one);
-//  - one thread issues one tcgen05.mma.kind::f16 (BF16 operands, FP32
-//    accumulation) per slice pair (p, q), p + q <= S + 1, into the tensor-memory
-//    accumulator of its diagonal d (64 columns each) and commits the chunk to
-//    the buffer's mbarrier;
+// (slices numbered from 1).  A persistent CTA per SM takes 128 x 64 output tiles:
+//  - one thread copies chunks of 32 k values of every slice (96 KB at S = 8: two
+//    contiguous pieces, cp.async.bulk) into a ring of stages;
+//  - one thread issues a tcgen05.mma.kind::f16 (BF16 operands, FP32 accumulation)
+//    per slice pair (p, q), p + q <= S + 1, and 16 values of k, into the
+//    tensor-memory accumulator of its diagonal d = p + q - 2 (64 columns each),
+//    diagonals in descending order;
 //  - every 128 values of k (where the FP32 sums of integer slice products are
-//    still exact) the warps read the accumulators with tcgen05.ld and combine
-//    the diagonals exactly in two 64-bit integers (four diagonals each: below
-//    2^46); the leading group is summed exactly in a 64-bit integer in shared
-//    memory over all of k, the trailing one (2^-28 of its weight) in FP64; the
-//    next chunk restarts the tensor-memory sums.  The shared accumulators of
-//    (row r, column c) sit at r 64 + (c xor (r mod 32)), so the 32 rows a warp
-//    updates together fall on distinct banks.
-// Every mbarrier wait is bounded; a CTA that gives up sets *err, waits
-// boundedly for its MMAs, frees its tensor memory and returns.
+//    still exact) eight warps read a diagonal as soon as its last product is done
+//    and add it, shifted to its weight, to two exact 64-bit integers per entry in
+//    registers (four diagonals each, below 2^46 per 128 values of k), and the next
+//    products of that diagonal may restart it: the tensor cores wait only for the
+//    first of the eight reads;
+//  - at the end of a tile the two integers are combined and rounded once.
+// Bound by the MMAs' shared-memory operand reads (128 x 16 + 64 x 16 BF16 per MMA,
+// 48 cycles at 128 bytes per cycle, against 32 cycles of multiplication): a wider
+// tile has no room in tensor memory beside eight diagonals.
+// Every mbarrier wait is bounded; whoever gives up sets *err and leaves, the
+// others run out of their own waits, and the tensor memory is freed after a
+// bounded wait for the MMAs and copies in flight.
 template <int S>
-__global__ void __launch_bounds__(kOzThreads) k_oz_gemm(const OzProd* __restrict__ prods,
-                                                        const OzTile* __restrict__ tiles,
-                                                        const __nv_bfloat16* __restrict__ Aslices,
-                                                        const __nv_bfloat16* __restrict__ Bslices,
-                                                        const int* __restrict__ exps, int* err) {
+constexpr int oz_stages() {
+    return S * (kOzSliceA + kOzSliceB) * 4 <= 200 * 1024 ? 4 : 2;
+}
+
+template <int S>
+__global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restrict__ prods,
+                                                           const OzTile* __restrict__ tiles, int n_tiles,
+                                                           const unsigned char* __restrict__ slices,
+                                                           const int* __restrict__ exps, int* err) {
     constexpr uint32_t kCols = S * kOzN <= 64 ? 64 : S * kOzN <= 128 ? 128 : S * kOzN <= 256 ? 256 : 512;
-    constexpr int kBuf = S * (kOzSliceA + kOzSliceB);
+    constexpr int kStages = oz_stages<S>();
+    constexpr uint32_t kBytesA = S * kOzSliceA, kBytesB = S * kOzSliceB, kStage = kBytesA + kBytesB;
     extern __shared__ __align__(1024) unsigned char oz_smem[];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bars[2 * kStages + 2 * S + 1];
     __shared__ uint32_t tmem_slot;
-    __shared__ int gave_up;
-    unsigned char* base = (unsigned char*)(((uintptr_t)oz_smem + 1023) & ~(uintptr_t)1023);
-    long long* acc0 = (long long*)(base + 2 * kBuf);    // exact sums of the leading group (weight 2^-35)
-    double* acc1 = (double*)(acc0 + kOzM * kOzN);        // sums of the trailing group, already scaled
-    auto sw = [](int r, int c) { return r * kOzN + (c ^ (r & 31)); };
+    const uint32_t base = (tc::smem_addr(oz_smem) + 1023u) & ~1023u;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const OzTile tl = tiles[blockIdx.x];
-    const OzProd pd = prods[tl.prod];
-    const int M = pd.M, N = pd.N, Kp = pd.Kp;
-    const __nv_bfloat16* As = Aslices + pd.a_off;
-    const __nv_bfloat16* Bs = Bslices + pd.b_off;
-    const int64_t sa = (int64_t)M * Kp, sb = (int64_t)N * Kp;
-    const uint32_t bar0 = tc::smem_addr(&bar[0]), bar1 = tc::smem_addr(&bar[1]);
+    auto full = [&](int s) { return tc::smem_addr(&bars[s]); };                          // a stage's copies landed
+    auto empty = [&](int s) { return tc::smem_addr(&bars[kStages + s]); };               // its MMAs are done
+    auto dfull = [&](int d) { return tc::smem_addr(&bars[2 * kStages + d]); };           // a diagonal's sums are done
+    auto dempty = [&](int d) { return tc::smem_addr(&bars[2 * kStages + S + d]); };      // they have been read
+    const uint32_t drain = tc::smem_addr(&bars[2 * kStages + 2 * S]);
     if (tid == 0) {
-        gave_up = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar1));
+        for (int i = 0; i < 2 * kStages + 2 * S + 1; ++i) {
+            const uint32_t count = i >= 2 * kStages + S && i < 2 * kStages + 2 * S ? kOzEpiWarps : 1;
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc::smem_addr(&bars[i])), "r"(count));
+        }
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    for (int e = tid; e < kOzM * kOzN; e += kOzThreads) {
-        acc0[e] = 0;
-        acc1[e] = 0.0;
-    }
-    if (warp == 0) {
+    if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          tc::smem_addr(&tmem_slot)),
                      "r"(kCols));
@@ -161,140 +262,164 @@ __global__ void __launch_bounds__(kOzThreads) k_oz_gemm(const OzProd* __restrict
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_slot;
-    // stage chunk c (k = 16 c .. 16 c + 15) of every slice into buffer b
-    auto stage = [&](int b, int c) {
-        unsigned char* bb = base + b * kBuf;
-        const int k0 = c * kOzK;
-        constexpr int nA = S * kOzM * 2, nB = S * kOzN * 2;   // 16-byte pieces
-        for (int i = tid; i < nA + nB; i += kOzThreads) {
-            const bool isB = i >= nA;
-            const int j = isB ? i - nA : i;
-            const int R = isB ? kOzN : kOzM;
-            const int p = j / (R * 2), r = (j / 2) % R, piece = j & 1;
-            const int row = (isB ? tl.n0 : tl.m0) + r;
-            const bool ok = row < (isB ? N : M);
-            const __nv_bfloat16* src = (isB ? Bs + p * sb : As + p * sa) + (ok ? (int64_t)row * Kp + k0 + piece * 8 : 0);
-            unsigned char* dst = bb + (isB ? S * kOzSliceA + p * kOzSliceB : p * kOzSliceA) + oz_off(r, piece * 8);
-            cp16(dst, src, ok ? 16 : 0);
-        }
-        asm volatile("cp.async.commit_group;\n" ::);
-    };
-    const int n_chunks = Kp / kOzK;
-    constexpr int kFlushChunks = 128 / kOzK;   // exact FP32 sums cover 128 values of k
-    uint32_t fresh = (1u << S) - 1u;           // diagonals whose next MMA starts a new sum (thread 0)
-    int last = -1;                             // last committed chunk
-    if (n_chunks > 0) stage(0, 0);
-    for (int c = 0; c < n_chunks; ++c) {
-        const int buf = c & 1;
-        if (c + 1 < n_chunks) {
-            if (c >= 1) {
-                // the MMAs of chunk c - 1 read the buffer the next chunk goes to
-                if (!tc::mbar_wait(buf ? bar0 : bar1, ((c - 1) >> 1) & 1)) {
-                    if (tid == 0) atomicExch(&gave_up, 1);
+    bool ok = true;
+    if (warp == 0) {
+        if (lane == 0) {
+            uint32_t it = 0;   // chunks issued: stage it % kStages, use it / kStages of its barriers
+            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+                const OzTile tl = tiles[t];
+                const OzProd& pd = prods[tl.prod];
+                const int nkc = pd.nkc;
+                const unsigned char* a = slices + pd.a_off + (int64_t)(tl.m0 / kOzM) * nkc * kBytesA;
+                const unsigned char* b = slices + pd.b_off + (int64_t)(tl.n0 / kOzN) * nkc * kBytesB;
+                for (int c = 0; c < nkc; ++c, ++it) {
+                    const int s = it % kStages;
+                    if (it >= kStages && !tc::mbar_wait(empty(s), (it / kStages - 1) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t dst = base + s * kStage;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(kStage)
+                                 : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            dst),
+                        "l"(a + (int64_t)c * kBytesA), "r"(kBytesA), "r"(full(s))
+                        : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            dst + kBytesA),
+                        "l"(b + (int64_t)c * kBytesB), "r"(kBytesB), "r"(full(s))
+                        : "memory");
                 }
-                __syncthreads();
-                if (gave_up) break;
             }
-            stage(buf ^ 1, c + 1);
-            asm volatile("cp.async.wait_group 1;\n" ::);
-        } else {
-            asm volatile("cp.async.wait_group 0;\n" ::);
+            // copies in flight land before the CTA may end
+            for (uint32_t i = it > kStages ? it - kStages : 0; i < it; ++i)
+                tc::mbar_wait(full(i % kStages), (i / kStages) & 1);
         }
-        // the copies of this thread landed; make every thread's copies visible to
-        // the tensor cores' (async) proxy
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t sA = tc::smem_addr(base + buf * kBuf), sB = sA + S * kOzSliceA;
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            uint32_t it = 0, g = 0;   // g: groups of 128 values of k (uses of every diagonal)
+            for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+                const int nkc = prods[tiles[t].prod].nkc;
+                for (int c = 0; c < nkc && ok; ++c, ++it) {
+                    const int s = it % kStages;
+                    const bool first = c % kOzGroup == 0, last = c % kOzGroup == kOzGroup - 1 || c + 1 == nkc;
+                    if (!tc::mbar_wait(full(s), (it / kStages) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint64_t da = tc::desc_sbo(base + s * kStage, kOzSbo);
+                    const uint64_t db = tc::desc_sbo(base + s * kStage + kBytesA, kOzSbo);
 #pragma unroll
-            for (int p = 1; p <= S; ++p)
+                    for (int d = S - 1; d >= 0; --d) {
+                        if (first && g > 0) {
+                            if (!tc::mbar_wait(dempty(d), (g - 1) & 1)) {
+                                ok = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;");
+                        }
 #pragma unroll
-                for (int q = 1; p + q <= S + 1; ++q) {
-                    const int d = p + q - 2;
-                    tc::mma_bf16(tmem + (uint32_t)(d * kOzN), tc::desc_sbo(sA + (p - 1) * kOzSliceA, kOzSbo),
-                                 tc::desc_sbo(sB + (q - 1) * kOzSliceB, kOzSbo), kOzIdesc, (fresh >> d) & 1u ? 0u : 1u);
-                    fresh &= ~(1u << d);
+                        for (int p = 0; p <= d; ++p)
+#pragma unroll
+                            for (int kk = 0; kk < kOzKStep / 16; ++kk)
+                                tc::mma_bf16(tmem + (uint32_t)(d * kOzN), da + ((p * kOzSliceA + kk * 256) >> 4),
+                                             db + (((d - p) * kOzSliceB + kk * 256) >> 4), kOzIdesc,
+                                             first && p == 0 && kk == 0 ? 0u : 1u);
+                        if (last)
+                            asm volatile(
+                                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                    dfull(d))
+                                : "memory");
+                    }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     empty(s))
+                                 : "memory");
+                    if (last) ++g;
                 }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             buf ? bar1 : bar0)
+            }
+            // every MMA and every earlier commit has happened before the CTA ends
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain)
                          : "memory");
+            ok = tc::mbar_wait(drain, 0) && ok;
         }
-        last = c;
-        if ((c + 1) % kFlushChunks == 0 || c + 1 == n_chunks) {
-            // the sums of this group of chunks: wait for its last commit (which
-            // covers every earlier MMA of the issuing thread)
-            if (!tc::mbar_wait(buf ? bar1 : bar0, (c >> 1) & 1)) {
-                if (tid == 0) atomicExch(&gave_up, 1);
-            }
-            __syncthreads();
-            if (gave_up) break;
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const int r = warp * 32 + lane;
-            for (int c0 = 0; c0 < kOzN; c0 += 16) {
-                long long i0[16], i1[16];
+        __syncwarp();
+    } else {
+        const int quad = warp & 3, half = (warp - 2) >> 2;   // tensor-memory lanes 32 quad .., columns 32 half ..
+        uint32_t g = 0;
+        for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+            const OzTile tl = tiles[t];
+            const OzProd pd = prods[tl.prod];
+            const int n_groups = (pd.nkc + kOzGroup - 1) / kOzGroup;
+            long long i0[32], i1[32];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) i0[j] = i1[j] = 0;
+            for (int j = 0; j < 32; ++j) i0[j] = i1[j] = 0;
+            for (int q = 0; q < n_groups && ok; ++q, ++g) {
 #pragma unroll
-                for (int d = 0; d < S; ++d) {
-                    uint32_t v[16];
-                    tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(d * kOzN + c0), v);
+                for (int d = S - 1; d >= 0; --d) {
+                    if (!__all_sync(0xffffffffu, tc::mbar_wait(dfull(d), g & 1))) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    uint32_t v[32];
+                    tc::ld_32x32b_x32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(d * kOzN + half * 32), v);
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(dempty(d)) : "memory");
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const long long x = __float2int_rz(__uint_as_float(v[j]));   // an exact integer below 2^24
+                    for (int j = 0; j < 32; ++j) {
+                        const int x = __float2int_rz(__uint_as_float(v[j]));   // an exact integer below 2^24
                         if (d < 4)
-                            i0[j] += x << (7 * (3 - d));
+                            i0[j] += (long long)x * (1 << (7 * (3 - d)));
                         else
-                            i1[j] += x << (7 * (7 - d));
+                            i1[j] += (long long)x * (1 << (7 * (7 - d)));
                     }
                 }
+            }
+            if (!ok) break;
+            // diagonal d carries 2^-7(d + 2): C = (i0 2^28 + i1) 2^(e + f - 63)
+            const int row = tl.m0 + quad * 32 + lane, c0 = tl.n0 + half * 32;
+            if (row < pd.M) {
+                const int e = exps[pd.e_off + row] - 63;
+                const int* f = exps + pd.f_off;
+                double* out = pd.C + (int64_t)row * pd.ldc;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    // diagonal d carries 2^-7(d + 2): group 0 (d <= 3) 2^-35 i0, group 1 (d >= 4) 2^-63 i1
-                    const int idx = sw(r, c0 + j);
-                    acc0[idx] += i0[j];
-                    if (S > 4) acc1[idx] = fma((double)i1[j], 0x1p-63, acc1[idx]);
+                for (int j = 0; j < 32; ++j) {
+                    if (c0 + j < pd.N) {
+                        const unsigned long long l0 = (unsigned long long)i0[j] << 28;
+                        const unsigned long long lo = l0 + (unsigned long long)i1[j];
+                        const long long hi = (i0[j] >> 36) + (i1[j] >> 63) + (lo < l0 ? 1 : 0);
+                        const double v = oz_round(hi, lo, e + f[c0 + j]);
+                        out[c0 + j] = pd.alpha == 1.0 ? v : pd.alpha * v;
+                    }
                 }
             }
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncthreads();
-            if (tid == 0) fresh = (1u << S) - 1u;
         }
     }
-    if (!gave_up) {
-        const int* e = exps + pd.e_off;
-        const int* f = exps + pd.f_off;
-        for (int idx = tid; idx < kOzM * kOzN; idx += kOzThreads) {
-            const int rr = idx / kOzN, cc = idx % kOzN;
-            const int gr = tl.m0 + rr, gc = tl.n0 + cc;
-            if (gr < M && gc < N) {
-                const int a = sw(rr, cc);
-                const double v = fma((double)acc0[a], 0x1p-35, acc1[a]);
-                pd.C[(int64_t)gr * pd.ldc + gc] = pd.alpha * ldexp(ldexp(v, e[gr]), f[gc]);
-            }
-        }
-    } else {
-        if (tid == 0) atomicExch(err, 1);
-        asm volatile("cp.async.wait_group 0;\n" ::);
-        // MMAs may still be in flight: a bounded wait for the last commit before
-        // the tensor memory they write is released
-        if (last >= 0) tc::mbar_wait((last & 1) ? bar1 : bar0, (last >> 1) & 1);
-    }
+    if (!ok) atomicExch(err, 1);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
 template <int S>
-void launch_oz_gemm(Context* ctx, int n_tiles, const OzProd* prods, const OzTile* tiles, const __nv_bfloat16* As,
-                    const __nv_bfloat16* Bs, const int* exps) {
-    const size_t smem = 2 * (size_t)S * (kOzSliceA + kOzSliceB) + 16 * (size_t)kOzM * kOzN + 1024;
+void launch_oz_gemm(Context* ctx, int n_tiles, const OzProd* prods, const OzTile* tiles, const unsigned char* slices,
+                    const int* exps) {
+    const size_t smem = (size_t)oz_stages<S>() * S * (kOzSliceA + kOzSliceB) + 1024;
     static bool attr = false;
     if (!attr) {
         BSM_CUDA(cudaFuncSetAttribute(k_oz_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = true;
     }
-    k_oz_gemm<S><<<n_tiles, kOzThreads, smem, ctx->stream>>>(prods, tiles, As, Bs, exps, ctx->err_word());
+    int nsm = 0;
+    BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+    k_oz_gemm<S><<<std::min(n_tiles, nsm), kOzThreads, smem, ctx->stream>>>(prods, tiles, n_tiles, slices, exps,
+                                                                            ctx->err_word());
 }
 
 }  // namespace
@@ -302,61 +427,70 @@ void launch_oz_gemm(Context* ctx, int n_tiles, const OzProd* prods, const OzTile
 void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S) {
     BSM_REQUIRE(S >= 1 && S <= kOzMaxS, BSMPS_ERR_INVALID_ARG, "emulated GEMM: 1 <= slices <= 8");
     std::vector<OzProd> prods;
+    std::vector<OzSide> sides;
     std::vector<OzTile> tiles;
-    int64_t a_tot = 0, b_tot = 0;
-    int ex_tot = 0;
+    int64_t bytes = 0;
+    int rows = 0, max_ctas = 0, cut_ctas = 0;
     double fl = 0.0;
+    auto side = [&](const double* src, int64_t rs, int64_t ks, int n, int K, int nkc, int blk) {
+        OzSide sd{src, rs, ks, n, K, nkc, blk, bytes, rows, max_ctas, cut_ctas};
+        bytes += (int64_t)((n + blk - 1) / blk) * nkc * S * blk * kOzKStep * 2;
+        rows += n;
+        const int groups = (n + 7) / 8;
+        if (ks == 1) {
+            max_ctas += groups;
+            cut_ctas += groups * ((nkc + 7) / 8);
+        } else {
+            max_ctas += ((n + 31) / 32) * std::max(1, (K + kOzMaxK - 1) / kOzMaxK);
+            cut_ctas += ((groups + 7) / 8) * nkc;
+        }
+        sides.push_back(sd);
+        return sd;
+    };
     for (const OzGemm& g : gs) {
         BSM_REQUIRE(g.M >= 0 && g.N >= 0 && g.K >= 0, BSMPS_ERR_INVALID_ARG, "emulated GEMM: sizes >= 0");
-        // the exact 64-bit sum of the leading diagonals (below 2^46 per 128 values of k) stays below 2^63
+        // the exact 64-bit sums of the diagonals (below 2^46 per 128 values of k) stay below 2^63
         BSM_REQUIRE(g.K < (1 << 24), BSMPS_ERR_INVALID_ARG, "emulated GEMM: K < 2^24");
         if (g.M == 0 || g.N == 0) continue;
-        const int Kp = (g.K + kOzKStep - 1) / kOzKStep * kOzKStep;
-        OzProd pd{g.C, g.M, g.N, Kp, g.ldc, g.alpha, a_tot, b_tot, ex_tot, ex_tot + g.M};
-        a_tot += (int64_t)S * g.M * Kp;
-        b_tot += (int64_t)S * g.N * Kp;
-        ex_tot += g.M + g.N;
+        const int nkc = (g.K + kOzKStep - 1) / kOzKStep;
+        // (a stride-1 row of one value each counts as contiguous in k)
+        const OzSide a = side(g.A, g.lda, 1, g.M, g.K, nkc, kOzM);
+        const OzSide b = side(g.B, 1, g.ldb, g.N, g.K, nkc, kOzN);
         for (int m0 = 0; m0 < g.M; m0 += kOzM)
             for (int n0 = 0; n0 < g.N; n0 += kOzN) tiles.push_back({(int)prods.size(), m0, n0});
-        prods.push_back(pd);
+        prods.push_back({g.C, g.M, g.N, nkc, g.ldc, g.alpha, a.dst, b.dst, a.row0, b.row0});
         fl += 2.0 * g.M * (double)g.N * g.K;
     }
     if (prods.empty()) return;
     Scratch s(ctx);
-    __nv_bfloat16* As = (__nv_bfloat16*)ctx->alloc(sizeof(__nv_bfloat16) * (size_t)(a_tot + 8));
-    s.ptrs.push_back(As);
-    __nv_bfloat16* Bs = (__nv_bfloat16*)ctx->alloc(sizeof(__nv_bfloat16) * (size_t)(b_tot + 8));
-    s.ptrs.push_back(Bs);
-    int* exps = (int*)ctx->alloc(sizeof(int) * (size_t)ex_tot);
+    unsigned char* slices = (unsigned char*)ctx->alloc((size_t)bytes + 128);
+    s.ptrs.push_back(slices);
+    unsigned long long* mx = (unsigned long long*)ctx->alloc(sizeof(unsigned long long) * (size_t)rows);
+    s.ptrs.push_back(mx);
+    int* exps = (int*)ctx->alloc(sizeof(int) * (size_t)rows);
     s.ptrs.push_back(exps);
-    // rows of op(A) and columns of B, with their exponent slots and slice rows
-    std::vector<OzRow> rows;
-    size_t pi = 0;
-    for (const OzGemm& g : gs) {
-        if (g.M == 0 || g.N == 0) continue;
-        const OzProd& pd = prods[pi++];
-        for (int r = 0; r < g.M; ++r)
-            rows.push_back({g.A + (int64_t)r * g.lda, 1, g.K, pd.Kp,
-                            exps + pd.e_off + r, As + pd.a_off + (int64_t)r * pd.Kp, (int64_t)g.M * pd.Kp});
-        for (int c = 0; c < g.N; ++c)
-            rows.push_back({g.B + c, (int64_t)g.ldb, g.K, pd.Kp, exps + pd.f_off + c, Bs + pd.b_off + (int64_t)c * pd.Kp,
-                            (int64_t)g.N * pd.Kp});
-    }
-    const OzRow* d_rows = s.up(rows);
+    const OzSide* d_sides = s.up(sides);
     const OzProd* d_prods = s.up(prods);
     const OzTile* d_tiles = s.up(tiles);
-    k_oz_rows<<<((int)rows.size() + 7) / 8, 256, 0, ctx->stream>>>(d_rows, (int)rows.size(), S);
+    BSM_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)rows, ctx->stream));
+    k_oz_max<<<max_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), mx);
     launched(ctx);
+    if (cut_ctas > 0) {
+        k_oz_slice<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), S, mx, exps, slices);
+        launched(ctx);
+    } else {
+        BSM_CUDA(cudaMemsetAsync(exps, 0, sizeof(int) * (size_t)rows, ctx->stream));   // K = 0: C = 0
+    }
     const int nt = (int)tiles.size();
     switch (S) {
-        case 1: launch_oz_gemm<1>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 2: launch_oz_gemm<2>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 3: launch_oz_gemm<3>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 4: launch_oz_gemm<4>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 5: launch_oz_gemm<5>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 6: launch_oz_gemm<6>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        case 7: launch_oz_gemm<7>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
-        default: launch_oz_gemm<8>(ctx, nt, d_prods, d_tiles, As, Bs, exps); break;
+        case 1: launch_oz_gemm<1>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 2: launch_oz_gemm<2>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 3: launch_oz_gemm<3>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 4: launch_oz_gemm<4>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 5: launch_oz_gemm<5>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 6: launch_oz_gemm<6>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        case 7: launch_oz_gemm<7>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        default: launch_oz_gemm<8>(ctx, nt, d_prods, d_tiles, slices, exps); break;
     }
     launched(ctx);
     ctx->flops += fl;
