@@ -5,7 +5,9 @@
 // 5th-generation tensor cores (tcgen05.mma kind::tf32, FP32 accumulation in
 // tensor memory): the BF16 weights are exact in TF32, and the activations and
 // back-propagated errors enter the products rounded to TF32 (nearest, ties
-// away from zero).
+// away from zero).  Every result is stored once in the layouts in which the next
+// products read it (operand images), so that the products move their operands
+// with bulk copies only.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -23,6 +25,8 @@ struct bsmps_mlp_s {
     int64_t n_params = 0;
     float* master = nullptr;          // FP32 parameters (device)
     __nv_bfloat16* wbf = nullptr;     // BF16 copy of the parameters (device)
+    float* img = nullptr;             // the BF16 weights as FP32 operand images (device), zero padded
+    std::vector<int64_t> w1_off, w2_off;   // per layer: W (rows = outputs) and W^T (rows = inputs), in floats
     float* m1 = nullptr;              // Adam first moment
     float* m2 = nullptr;              // Adam second moment
     float* grad = nullptr;
@@ -34,195 +38,238 @@ namespace {
 
 constexpr int kT = 256;
 
-// One product of the network on the tensor cores:
-//     C(m, n) = epi( sum_k a(m, k) b(n, k) ),   m < M, n < N, k < K,
-// a and b read through element strides from FP32 or BF16 arrays and rounded to
-// TF32; epi adds bias[n] (BF16) and applies ReLU, or keeps the entry only where
-// mask(m, n) > 0 (the derivative of the ReLU that produced mask), else nothing.
+// Operand image of a matrix of n rows x K values (FP32, already rounded to TF32):
+// blocks of 128 rows x 32 values (16 KB, K-major with 128-byte swizzle), the blocks
+// of a row range contiguous along K, so that a chunk of a tile is one bulk copy.
+// Values of k >= K are zero (the products run over whole chunks); rows >= n hold
+// anything (they reach only entries that are not stored).
+constexpr int kImgRows = 128, kImgK = 32;
+constexpr int64_t kImgBlock = kImgRows * kImgK;   // floats
+__host__ __device__ __forceinline__ int img_chunks(int K) { return (K + kImgK - 1) / kImgK; }
+inline int64_t img_size(int n, int K) { return (int64_t)((n + kImgRows - 1) / kImgRows) * img_chunks(K) * kImgBlock; }
+__device__ __forceinline__ int64_t img_at(int r, int k, int nkc) {
+    return ((int64_t)(r / kImgRows) * nkc + k / kImgK) * kImgBlock + (r % kImgRows) * kImgK +
+           ((((k >> 2) & 7) ^ (r & 7)) << 2) + (k & 3);
+}
+__device__ __forceinline__ float tf32_round(float f) { return __uint_as_float(tc::tf32_bits(f)); }
+
+// One product of the network on the tensor cores, C(m, n) = epi( sum_k a(m, k) b(n, k) ),
+// both factors given as operand images over nkc chunks of 32 values of k.  Outputs:
+//  - part: raw sums of a k range to part[z] (row-major), summed by k_mlp_reduce;
+//  - y: row-major FP32 (the network's output);
+//  - i1, i2: the operand images of the result (rows = m; rows = n), rounded to TF32
+//    as the next products read them.
+// epi adds bias[n] (BF16) and applies ReLU, or keeps the entry only where the image
+// mask (rows = m) is positive (the derivative of the ReLU that produced it).
 struct MlpGemm {
-    const void* A;
-    int64_t sam, sak;
-    int a_bf16;
-    const void* B;
-    int64_t sbn, sbk;
-    int b_bf16;
-    float* C;
-    int64_t scm, scn;
+    const float* A;
+    const float* B;
+    int M, N, K, nkc;   // nkc: chunks of K
     const __nv_bfloat16* bias;
-    const float* mask;
     int relu;
-    int M, N, K;
+    const float* mask;
+    float* y;
+    float *i1, *i2;
+    float* part;
 };
 
 constexpr int kMlpM = 128;         // rows of a tile (the M of one tcgen05.mma)
-constexpr int kMlpN = 64;          // columns of a tile (its N, and the tensor-memory columns)
-constexpr int kMlpK = 32;          // k values per staged chunk (4 MMAs of K = 8)
+constexpr int kMlpN = 128;         // columns of a tile (its N, and the tensor-memory columns)
+constexpr int kMlpStages = 4;
+constexpr uint32_t kMlpOperand = kImgBlock * 4;       // bytes of one operand block
+constexpr uint32_t kMlpStage = 2 * kMlpOperand;
 constexpr int kMlpThreads = 128;   // warp w reads tensor-memory lanes 32 w .. 32 w + 31
 constexpr uint32_t kMlpIdesc = tc::idesc_tf32(kMlpM, kMlpN);
 
-__device__ __forceinline__ float mlp_load(const void* p, int bf16, int64_t i) {
-    return bf16 ? __bfloat162float(((const __nv_bfloat16*)p)[i]) : ((const float*)p)[i];
-}
-
-// One CTA per 128 x 64 output tile and k range (blockIdx.z of gridDim.z, each
-// a multiple of 32 long): 4 warps stage 32-wide k chunks of a and b in the
-// canonical K-major layout (the index order follows whichever of the two
-// strides is 1, so the loads coalesce) into two buffers, so that staging chunk
-// i + 1 overlaps the MMAs of chunk i; one thread issues the MMAs and commits
-// them to the buffer's mbarrier (bounded waits; a CTA that gives up sets *err,
-// waits boundedly for its MMAs and frees its tensor memory).  With one k range
-// the epilogue (tcgen05.ld) applies bias / ReLU / mask and stores C; with
-// several, every CTA stores its raw tile to part[z] and k_mlp_reduce sums the
-// ranges in order and applies the epilogue.
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, int k_len, float* part, int* err) {
+// One CTA per 128 x 128 output tile and range of chunks (blockIdx.z): one thread
+// streams the blocks through four stages by bulk copies, another issues four MMAs
+// per chunk; no thread touches an operand (staging them through registers, strided
+// and rounded on the way, took 0.86 ms for the products of a batch of 8192).  All
+// four warps run the epilogue.  What is left is latency: at 8 chunks a tile's copies
+// and its epilogue (two images) are longer than its 32 MMAs.  Waits are bounded; a CTA that
+// gives up sets *err and frees its tensor memory after its MMAs and copies.
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, int chunks, int* err) {
     extern __shared__ __align__(1024) unsigned char mlp_smem[];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bars[2 * kMlpStages + 1];
     __shared__ uint32_t tmem_slot;
-    __shared__ int gave_up;
-    unsigned char* base = (unsigned char*)(((uintptr_t)mlp_smem + 1023) & ~(uintptr_t)1023);
-    constexpr int kBuf = (kMlpM + kMlpN) * kMlpK * 4;
-    const int m0 = blockIdx.x * kMlpM, n0 = blockIdx.y * kMlpN;
-    const int kb = blockIdx.z * k_len, ke = min(g.K, kb + k_len);
+    const uint32_t base = (tc::smem_addr(mlp_smem) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t bar0 = tc::smem_addr(&bar[0]), bar1 = tc::smem_addr(&bar[1]);
+    const int m0 = blockIdx.x * kMlpM, n0 = blockIdx.y * kMlpN;
+    const int c0 = blockIdx.z * chunks, nc = min(chunks, g.nkc - c0);   // >= 1
+    auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
+    auto empty = [&](int s) { return tc::smem_addr(&bars[kMlpStages + s]); };
+    const uint32_t done = tc::smem_addr(&bars[2 * kMlpStages]);
     if (threadIdx.x == 0) {
-        gave_up = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar1));
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        for (int i = 0; i < 2 * kMlpStages + 1; ++i) tc::mbar_init(tc::smem_addr(&bars[i]), 1);
+        tc::mbar_init_fence();
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         tc::smem_addr(&tmem_slot)),
-                     "r"(kMlpN));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    if (warp == 1) tc::tmem_alloc(&tmem_slot, kMlpN);
+    tc::fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tc::fence_after();
     const uint32_t tmem = tmem_slot;
-    int n_chunks = 0;   // chunks committed; chunk i used buffer i & 1 and is commit i >> 1 of its mbarrier
-    for (int k0 = kb; k0 < ke; k0 += kMlpK, ++n_chunks) {
-        const int buf = n_chunks & 1;
-        if (n_chunks >= 2) {
-            // the MMAs of chunk n_chunks - 2 (the last user of this buffer) are done
-            if (!tc::mbar_wait(buf ? bar1 : bar0, ((n_chunks - 2) >> 1) & 1)) {
-                if (threadIdx.x == 0) atomicExch(&gave_up, 1);
+    bool ok = true;
+    if (warp == 0) {
+        if (lane == 0) {
+            const float* a = g.A + ((int64_t)blockIdx.x * g.nkc + c0) * kImgBlock;
+            const float* b = g.B + ((int64_t)blockIdx.y * g.nkc + c0) * kImgBlock;
+            int c = 0;
+            for (; c < nc; ++c) {
+                const int s = c % kMlpStages;
+                if (c >= kMlpStages && !tc::mbar_wait(empty(s), (c / kMlpStages - 1) & 1)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t dst = base + s * kMlpStage;
+                tc::mbar_expect(full(s), kMlpStage);
+                tc::bulk_load(dst, a + c * kImgBlock, kMlpOperand, full(s));
+                tc::bulk_load(dst + kMlpOperand, b + c * kImgBlock, kMlpOperand, full(s));
             }
-            __syncthreads();
-            if (gave_up) break;
+            // copies in flight land before the CTA may end
+            for (int i = c > kMlpStages ? c - kMlpStages : 0; i < c; ++i)
+                tc::mbar_wait(full(i % kMlpStages), (i / kMlpStages) & 1);
         }
-        unsigned char* a_s = base + buf * kBuf;
-        unsigned char* b_s = a_s + kMlpM * kMlpK * 4;
-        for (int idx = threadIdx.x; idx < kMlpM * kMlpK; idx += kMlpThreads) {
-            const int r = g.sak == 1 ? idx / kMlpK : idx % kMlpM;
-            const int k = g.sak == 1 ? idx % kMlpK : idx / kMlpM;
-            const int gm = m0 + r, gk = k0 + k;
-            const float v = (gm < g.M && gk < ke) ? mlp_load(g.A, g.a_bf16, gm * g.sam + gk * g.sak) : 0.0f;
-            *(uint32_t*)(a_s + tc::off(r, k)) = tc::tf32_bits(v);
-        }
-        for (int idx = threadIdx.x; idx < kMlpN * kMlpK; idx += kMlpThreads) {
-            const int n = g.sbk == 1 ? idx / kMlpK : idx % kMlpN;
-            const int k = g.sbk == 1 ? idx % kMlpK : idx / kMlpN;
-            const int gn = n0 + n, gk = k0 + k;
-            const float v = (gn < g.N && gk < ke) ? mlp_load(g.B, g.b_bf16, gn * g.sbn + gk * g.sbk) : 0.0f;
-            *(uint32_t*)(b_s + tc::off(n, k)) = tc::tf32_bits(v);
-        }
-        // generic-proxy writes become visible to the tensor cores' (async) proxy
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint32_t sa = tc::smem_addr(a_s), sb = tc::smem_addr(b_s);
-            for (int kk = 0; kk < kMlpK / 8; ++kk) {
-                const uint32_t step = (uint32_t)kk * 256u;   // two core matrices along k per MMA
-                tc::mma_tf32(tmem, tc::desc(sa + step), tc::desc(sb + step), kMlpIdesc,
-                             (n_chunks == 0 && kk == 0) ? 0u : 1u);
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             buf ? bar1 : bar0)
-                         : "memory");
-        }
-    }
-    // the last chunk's commit covers every earlier MMA of this thread
-    const int last = n_chunks - 1;
-    if (!gave_up && n_chunks > 0) {
-        if (!tc::mbar_wait((last & 1) ? bar1 : bar0, (last >> 1) & 1)) {
-            if (threadIdx.x == 0) atomicExch(&gave_up, 1);
-        }
-        __syncthreads();
-        if (!gave_up) asm volatile("tcgen05.fence::after_thread_sync;");
-    }
-    if (!gave_up) {
-        const int row = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < kMlpN; c0 += 16) {
-            uint32_t v[16];
-            if (n_chunks > 0) {
-                tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-            } else {
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            for (int c = 0; c < nc; ++c) {
+                const int s = c % kMlpStages;
+                if (!tc::mbar_wait(full(s), (c / kMlpStages) & 1)) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after();
+                const uint64_t a = tc::desc_sw128(base + s * kMlpStage), b = a + (kMlpOperand >> 4);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = 0u;
+                for (int kk = 0; kk < kImgK / 8; ++kk)   // 32 bytes along k per MMA
+                    tc::mma_tf32(tmem, a + 2 * kk, b + 2 * kk, kMlpIdesc, c == 0 && kk == 0 ? 0u : 1u);
+                tc::commit(empty(s));
             }
+            tc::commit(done);   // covers every MMA and every earlier commit
+            ok = tc::mbar_wait(done, 0) && ok;
+        }
+        __syncwarp();
+    }
+    ok = __all_sync(0xffffffffu, tc::mbar_wait(done, 0) && ok);
+    tc::fence_after();
+    const int row = m0 + warp * 32 + lane;
+    const int nk1 = img_chunks(g.N), nk2 = img_chunks(g.M);   // chunks of the result's images
+    for (int cc = 0; ok && cc < kMlpN; cc += 16) {
+        uint32_t v[16];
+        tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cc, v);
+        const int col = n0 + cc;
+        if (g.part) {
             if (row < g.M) {
+                float* o = g.part + ((int64_t)blockIdx.z * g.M + row) * g.N + col;
+                if ((g.N & 3) == 0 && ((uintptr_t)g.part & 15) == 0) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int col = n0 + c0 + j;
-                    if (col >= g.N) continue;
-                    float acc = __uint_as_float(v[j]);
-                    if (part) {
-                        part[((int64_t)blockIdx.z * g.M + row) * g.N + col] = acc;
-                        continue;
-                    }
-                    if (g.bias) acc += __bfloat162float(g.bias[col]);
-                    if (g.relu) acc = fmaxf(acc, 0.0f);
-                    const int64_t ci = row * g.scm + col * g.scn;
-                    if (g.mask && !(g.mask[ci] > 0.0f)) acc = 0.0f;
-                    g.C[ci] = acc;
+                    for (int j = 0; j < 16; j += 4)
+                        if (col + j < g.N) *(uint4*)(o + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (col + j < g.N) o[j] = __uint_as_float(v[j]);
                 }
             }
+            continue;
         }
-    } else {
-        if (threadIdx.x == 0) atomicExch(err, 1);
-        // MMAs of this CTA may still be in flight: a bounded wait for the last
-        // commit before the tensor memory they write is released
-        if (n_chunks > 0) tc::mbar_wait((last & 1) ? bar1 : bar0, (last >> 1) & 1);
+        float w[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            float acc = __uint_as_float(v[j]);
+            if (g.bias && col + j < g.N) acc += __bfloat162float(g.bias[col + j]);
+            if (g.relu) acc = fmaxf(acc, 0.0f);
+            w[j] = acc;
+        }
+        if (g.mask && col < nk1 * kImgK) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+                const float4 h = *(const float4*)(g.mask + img_at(row, col + j, nk1));
+                if (!(h.x > 0.0f)) w[j] = 0.0f;
+                if (!(h.y > 0.0f)) w[j + 1] = 0.0f;
+                if (!(h.z > 0.0f)) w[j + 2] = 0.0f;
+                if (!(h.w > 0.0f)) w[j + 3] = 0.0f;
+            }
+        }
+        if (g.y) {
+            if (row < g.M)
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (col + j < g.N) g.y[(int64_t)row * g.N + col + j] = w[j];
+            continue;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) w[j] = row < g.M && col + j < g.N ? tf32_round(w[j]) : 0.0f;
+        if (col < nk1 * kImgK)
+#pragma unroll
+            for (int j = 0; j < 16; j += 4)
+                *(float4*)(g.i1 + img_at(row, col + j, nk1)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+        if (g.i2 && row < nk2 * kImgK)
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (col + j < g.N) g.i2[img_at(col + j, row, nk2)] = w[j];
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    if (!ok) atomicExch(err, 1);
+    tc::fence_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMlpN));
+    if (warp == 1) tc::tmem_free(tmem, kMlpN);
 }
 
-// C(m, n) = epi( sum_z part[z](m, n) ), the k ranges summed in order.
-__global__ void k_mlp_reduce(const MlpGemm g, const float* __restrict__ part, int n_parts) {
+// C = sum_z part[z], the k ranges summed in order.
+__global__ void k_mlp_reduce(const float* __restrict__ part, float* __restrict__ C, int64_t n, int n_parts) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)g.M * g.N) return;
-    const int m = (int)(e / g.N), n = (int)(e % g.N);
-    float acc = 0.0f;
-    for (int z = 0; z < n_parts; ++z) acc += part[(int64_t)z * g.M * g.N + e];
-    if (g.bias) acc += __bfloat162float(g.bias[n]);
-    if (g.relu) acc = fmaxf(acc, 0.0f);
-    const int64_t ci = m * g.scm + n * g.scn;
-    if (g.mask && !(g.mask[ci] > 0.0f)) acc = 0.0f;
-    g.C[ci] = acc;
-}
-
-// dY of the loss 1/(B out) sum (Y - T)^2, and the per-element squared error.
-__global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, float* __restrict__ dY,
-                      float* __restrict__ sq, int n, float scale) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
-    const float d = Y[e] - T[e];
-    dY[e] = 2.0f * scale * d;
-    sq[e] = d * d;
+    float acc = 0.0f;
+#pragma unroll 8
+    for (int z = 0; z < n_parts; ++z) acc += part[(int64_t)z * n + e];
+    C[e] = acc;
 }
 
-// db[o] = sum_b dY[b, o] (TF32-rounded dY, as the weight-gradient product reads it), one CTA per o.
-__global__ void k_mlp_bgrad(const float* __restrict__ dY, float* __restrict__ db, int B, int out) {
+// The operand images of a row-major matrix X (n x K): rows of X, and (i2 not
+// null) rows of X^T over n.  32 x 32 tiles through shared memory.
+__global__ void __launch_bounds__(256) k_mlp_pack(const float* __restrict__ X, int n, int K, float* __restrict__ i1,
+                                                  float* __restrict__ i2) {
+    __shared__ float t[32][33];
+    const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int nk1 = img_chunks(K), nk2 = img_chunks(n);
+    for (int i = y; i < 32; i += 8) {
+        const int r = r0 + i, k = k0 + x;
+        const float v = r < n && k < K ? tf32_round(X[(int64_t)r * K + k]) : 0.0f;
+        t[i][x] = v;
+        if (r < n) i1[img_at(r, k, nk1)] = v;
+    }
+    if (!i2) return;
+    __syncthreads();
+    for (int i = y; i < 32; i += 8)
+        if (k0 + i < K) i2[img_at(k0 + i, r0 + x, nk2)] = t[x][i];
+}
+
+// dY of the loss 1/(B out) sum (Y - T)^2 as operand images (rows = batch, rows =
+// outputs; rounded to TF32), and the per-element squared error.
+__global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, float* __restrict__ d1,
+                      float* __restrict__ d2, float* __restrict__ sq, int B, int out, float scale) {
+    const int nk1 = img_chunks(out), nk2 = img_chunks(B);
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (int)(e / (nk1 * kImgK)), o = (int)(e % (nk1 * kImgK));
+    if (b >= nk2 * kImgK) return;
+    float v = 0.0f;
+    if (b < B && o < out) {
+        const float d = Y[(int64_t)b * out + o] - T[(int64_t)b * out + o];
+        v = tf32_round(2.0f * scale * d);
+        sq[(int64_t)b * out + o] = d * d;
+    }
+    if (b < B) d1[img_at(b, o, nk1)] = v;
+    if (o < out) d2[img_at(o, b, nk2)] = v;
+}
+
+// db[o] = sum_b dY[b, o] (rounded as the weight-gradient product reads it), one
+// CTA per o; the image's rows are contiguous runs of 32 values of b (zeros beyond B).
+__global__ void k_mlp_bgrad(const float* __restrict__ d2, float* __restrict__ db, int B) {
     __shared__ float red[32];
-    const int o = blockIdx.x;
+    const int o = blockIdx.x, nk2 = img_chunks(B);
+    const float* row = d2 + (int64_t)(o / kImgRows) * nk2 * kImgBlock + (o % kImgRows) * kImgK;
     float acc = 0.0f;
-    for (int b = threadIdx.x; b < B; b += blockDim.x)
-        acc += __uint_as_float(tc::tf32_bits(dY[(int64_t)b * out + o]));
+    for (int b = threadIdx.x; b < nk2 * kImgK; b += blockDim.x) acc += row[(int64_t)(b / kImgK) * kImgBlock + b % kImgK];
     for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -233,10 +280,30 @@ __global__ void k_mlp_bgrad(const float* __restrict__ dY, float* __restrict__ db
     }
 }
 
-// Adam (beta1 = 0.9, beta2 = 0.999, eps = 1e-8) on the FP32 masters, then the BF16 copy.
+// Where parameter e lies: the weight images of its layer.
+constexpr int kMaxLayers = 16;
+struct MlpLayers {
+    int n;
+    int64_t w_off[kMaxLayers], w1[kMaxLayers], w2[kMaxLayers];
+    int in[kMaxLayers], out[kMaxLayers];
+};
+__device__ __forceinline__ void store_bf16(const MlpLayers& L, float* img, __nv_bfloat16* pb, int64_t e, float q) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(q);
+    pb[e] = h;
+    for (int l = 0; l < L.n; ++l) {
+        const int64_t d = e - L.w_off[l];
+        if (d < 0 || d >= (int64_t)L.in[l] * L.out[l]) continue;
+        const int o = (int)(d / L.in[l]), i = (int)(d % L.in[l]);
+        const float w = __bfloat162float(h);
+        img[L.w1[l] + img_at(o, i, img_chunks(L.in[l]))] = w;
+        img[L.w2[l] + img_at(i, o, img_chunks(L.out[l]))] = w;
+    }
+}
+
+// Adam (beta1 = 0.9, beta2 = 0.999, eps = 1e-8) on the FP32 masters, then the BF16 copy and its images.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m1,
-                       float* __restrict__ m2, __nv_bfloat16* __restrict__ pb, int64_t n, float lr, float c1,
-                       float c2) {
+                       float* __restrict__ m2, __nv_bfloat16* __restrict__ pb, float* __restrict__ img,
+                       const MlpLayers L, int64_t n, float lr, float c1, float c2) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     const float gg = g[e];
@@ -246,12 +313,13 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     m2[e] = v;
     const float q = p[e] - lr * (a / c1) / (sqrtf(v / c2) + 1e-8f);
     p[e] = q;
-    pb[e] = __float2bfloat16_rn(q);
+    store_bf16(L, img, pb, e, q);
 }
 
-__global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ pb, int64_t n) {
+__global__ void k_to_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ pb, float* __restrict__ img,
+                          const MlpLayers L, int64_t n) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) pb[e] = __float2bfloat16_rn(p[e]);
+    if (e < n) store_bf16(L, img, pb, e, p[e]);
 }
 
 unsigned grid(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
@@ -261,55 +329,91 @@ void done(Context* ctx) {
     BSM_CUDA(cudaGetLastError());
 }
 
-struct Acts {
-    std::vector<float*> h;   // h[0] = input, h[l+1] = output of layer l
-};
+MlpLayers layers_of(const bsmps_mlp_s* net) {
+    MlpLayers L{};
+    L.n = (int)net->widths.size() - 1;
+    for (int l = 0; l < L.n; ++l) {
+        L.w_off[l] = net->w_off[l];
+        L.w1[l] = net->w1_off[l];
+        L.w2[l] = net->w2_off[l];
+        L.in[l] = net->widths[l];
+        L.out[l] = net->widths[l + 1];
+    }
+    return L;
+}
 
-// One product: tiles of 128 x 64; the k range split over gridDim.z CTAs per
-// tile (partials reduced in order by k_mlp_reduce) when the tiles alone would
-// leave most SMs idle.
-void launch_mlp_gemm(Context* ctx, const MlpGemm& g, Scratch& s) {
-    if (g.M <= 0 || g.N <= 0) return;
-    const int smem = 2 * (kMlpM + kMlpN) * kMlpK * 4 + 1024;   // two buffers, aligned to 1024 bytes
+float* floats(Scratch& s, int64_t n) { return (float*)s.dbl((size_t)(n + 1) / 2); }
+
+// One product.  grad != null: the k range is split over gridDim.z CTAs per tile
+// (partials reduced in order into grad) as far as the tiles alone leave SMs idle.
+void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr) {
+    const int smem = kMlpStages * (int)kMlpStage + 1024;
     static bool attr = false;
     if (!attr) {
         BSM_CUDA(cudaFuncSetAttribute(k_mlp_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         attr = true;
     }
-    const int64_t tiles = (int64_t)((g.M + kMlpM - 1) / kMlpM) * ((g.N + kMlpN - 1) / kMlpN);
-    const int chunks = (g.K + kMlpK - 1) / kMlpK;
-    int splits = 1;
-    while (tiles * splits < 2 * 148 && chunks / (splits * 2) >= 4) splits *= 2;
-    const int k_len = ((chunks + splits - 1) / splits) * kMlpK;
-    splits = std::max(1, (g.K + k_len - 1) / k_len);
-    float* part = splits > 1 ? (float*)s.dbl(((size_t)splits * g.M * g.N + 1) / 2) : nullptr;
-    const dim3 grid_tc((unsigned)((g.M + kMlpM - 1) / kMlpM), (unsigned)((g.N + kMlpN - 1) / kMlpN),
-                       (unsigned)splits);
+    const int tm = (g.M + kMlpM - 1) / kMlpM, tn = (g.N + kMlpN - 1) / kMlpN;
+    int chunks = g.nkc;
+    if (grad) {
+        // one wave of CTAs (one per SM at 128 KB of stages), at least four chunks each
+        const int splits = std::max(1, std::min(148 / std::max(1, tm * tn), g.nkc / 4));
+        chunks = (g.nkc + splits - 1) / splits;
+    }
+    const int parts = (g.nkc + chunks - 1) / chunks;
+    if (grad) g.part = parts > 1 ? floats(s, (int64_t)parts * g.M * g.N) : grad;
     const double fl = 2.0 * g.M * (double)g.N * g.K;
-    const double by = 4.0 * ((double)g.M * g.K + (double)g.N * g.K + (double)g.M * g.N);
+    const double by = 4.0 * ((double)(g.M + g.N) * g.K + (double)g.M * g.N);
     ProfScope ps(ctx, KK_MLP, fl, by);
-    k_mlp_gemm_tc<<<grid_tc, kMlpThreads, smem, ctx->stream>>>(g, k_len, part, ctx->err_word());
+    k_mlp_gemm_tc<<<dim3((unsigned)tm, (unsigned)tn, (unsigned)parts), kMlpThreads, smem, ctx->stream>>>(
+        g, chunks, ctx->err_word());
     done(ctx);
-    if (part) {
-        k_mlp_reduce<<<grid((int64_t)g.M * g.N), kT, 0, ctx->stream>>>(g, part, splits);
+    if (parts > 1) {
+        const int64_t n = (int64_t)g.M * g.N;
+        k_mlp_reduce<<<grid(n), kT, 0, ctx->stream>>>(g.part, grad, n, parts);
         done(ctx);
     }
     ps.done();
 }
 
-// forward pass of a batch already on the device; returns the activations
-Acts forward(Context* ctx, bsmps_mlp_s* net, const float* x_dev, int B, Scratch& s) {
+// Forward pass of a batch: y (B x out, row-major, device); with `keep`, the images
+// of every layer's input (rows = batch, rows = features) for the backward pass.
+struct Acts {
+    std::vector<float*> h1, h2;
+    float* y = nullptr;
+};
+Acts forward(Context* ctx, bsmps_mlp_s* net, const float* x_host, int B, Scratch& s, bool keep) {
     const int nl = (int)net->widths.size() - 1;
     Acts a;
-    a.h.push_back(const_cast<float*>(x_dev));
+    const int in0 = net->widths[0];
+    float* x = (float*)ctx->upload_raw(x_host, sizeof(float) * (size_t)B * in0);
+    s.ptrs.push_back(x);
+    a.h1.push_back(floats(s, img_size(B, in0)));
+    a.h2.push_back(keep ? floats(s, img_size(in0, B)) : nullptr);
+    k_mlp_pack<<<dim3((unsigned)img_chunks(B), (unsigned)img_chunks(in0)), 256, 0, ctx->stream>>>(x, B, in0, a.h1[0],
+                                                                                                  a.h2[0]);
+    done(ctx);
     for (int l = 0; l < nl; ++l) {
         const int in = net->widths[l], out = net->widths[l + 1];
-        float* y = (float*)s.dbl(((size_t)B * out + 1) / 2 + 1);
-        // Y[b, o] = sum_i X[b, i] W[o, i] + bias[o]: a = X (B x in), b(n = o, k = i) = W[o, i]
-        MlpGemm g{a.h.back(), in, 1, 0, net->wbf + net->w_off[l], in, 1, 1, y, out, 1,
-                  net->wbf + net->b_off[l], nullptr, l + 1 < nl ? 1 : 0, B, out, in};
+        // Y[b, o] = sum_i X[b, i] W[o, i] + bias[o]
+        MlpGemm g{};
+        g.A = a.h1[l];
+        g.B = net->img + net->w1_off[l];
+        g.M = B;
+        g.N = out;
+        g.K = in;
+        g.nkc = img_chunks(in);
+        g.bias = net->wbf + net->b_off[l];
+        if (l + 1 < nl) {
+            g.relu = 1;
+            a.h1.push_back(floats(s, img_size(B, out)));
+            a.h2.push_back(keep ? floats(s, img_size(out, B)) : nullptr);
+            g.i1 = a.h1.back();
+            g.i2 = a.h2.back();
+        } else {
+            g.y = a.y = floats(s, (int64_t)B * out);
+        }
         launch_mlp_gemm(ctx, g, s);
-        a.h.push_back(y);
     }
     return a;
 }
@@ -317,31 +421,46 @@ Acts forward(Context* ctx, bsmps_mlp_s* net, const float* x_dev, int B, Scratch&
 // loss and gradient into net->grad (device)
 float loss_grad(Context* ctx, bsmps_mlp_s* net, const float* x_host, const float* t_host, int B) {
     const int nl = (int)net->widths.size() - 1;
-    const int in0 = net->widths[0], outL = net->widths[nl];
+    const int outL = net->widths[nl];
     Scratch s(ctx);
-    std::vector<float> xv(x_host, x_host + (size_t)B * in0), tv(t_host, t_host + (size_t)B * outL);
-    float* xd = s.up(xv);
-    float* td = s.up(tv);
-    Acts a = forward(ctx, net, xd, B, s);
+    float* td = (float*)ctx->upload_raw(t_host, sizeof(float) * (size_t)B * outL);
+    s.ptrs.push_back(td);
+    Acts a = forward(ctx, net, x_host, B, s, true);
     const int n = B * outL;
-    float* dY = (float*)s.dbl((size_t)n / 2 + 1);
-    float* sq = (float*)s.dbl((size_t)n / 2 + 1);
-    k_mse<<<grid(n), kT, 0, ctx->stream>>>(a.h.back(), td, dY, sq, n, 1.0f / (float)n);
+    float* d1 = floats(s, img_size(B, outL));
+    float* d2 = floats(s, img_size(outL, B));
+    float* sq = floats(s, n);
+    k_mse<<<grid((int64_t)img_chunks(B) * kImgK * img_chunks(outL) * kImgK), kT, 0, ctx->stream>>>(
+        a.y, td, d1, d2, sq, B, outL, 1.0f / (float)n);
     done(ctx);
     for (int l = nl - 1; l >= 0; --l) {
         const int in = net->widths[l], out = net->widths[l + 1];
-        // dW[o, i] = sum_b dY[b, o] X[b, i]: a(m = o, k = b) = dY[b, o], b(n = i, k = b) = X[b, i]
-        MlpGemm gw{dY, 1, out, 0, a.h[l], 1, in, 0, net->grad + net->w_off[l], in, 1, nullptr, nullptr, 0,
-                   out, in, B};
-        launch_mlp_gemm(ctx, gw, s);
-        k_mlp_bgrad<<<(unsigned)out, kT, 0, ctx->stream>>>(dY, net->grad + net->b_off[l], B, out);
+        // dW[o, i] = sum_b dY[b, o] X[b, i]
+        MlpGemm gw{};
+        gw.A = d2;
+        gw.B = a.h2[l];
+        gw.M = out;
+        gw.N = in;
+        gw.K = B;
+        gw.nkc = img_chunks(B);
+        launch_mlp_gemm(ctx, gw, s, net->grad + net->w_off[l]);
+        k_mlp_bgrad<<<(unsigned)out, kT, 0, ctx->stream>>>(d2, net->grad + net->b_off[l], B);
         done(ctx);
         if (l > 0) {
-            // dX[b, i] = (sum_o dY[b, o] W[o, i]) [X[b, i] > 0]: a = dY (B x out), b(n = i, k = o) = W[o, i]
-            float* dX = (float*)s.dbl(((size_t)B * in) / 2 + 1);
-            MlpGemm gx{dY, out, 1, 0, net->wbf + net->w_off[l], 1, in, 1, dX, in, 1, nullptr, a.h[l], 0, B, in, out};
+            // dX[b, i] = (sum_o dY[b, o] W[o, i]) [X[b, i] > 0]
+            MlpGemm gx{};
+            gx.A = d1;
+            gx.B = net->img + net->w2_off[l];
+            gx.M = B;
+            gx.N = in;
+            gx.K = out;
+            gx.nkc = img_chunks(out);
+            gx.mask = a.h1[l];
+            gx.i1 = floats(s, img_size(B, in));
+            gx.i2 = floats(s, img_size(in, B));
             launch_mlp_gemm(ctx, gx, s);
-            dY = dX;
+            d1 = gx.i1;
+            d2 = gx.i2;
         }
     }
     std::vector<float> sh((size_t)n);
@@ -409,13 +528,23 @@ bsmps_status bsmps_mlp_create(bsmps_ctx c, int n_layers, const int* widths, cons
         BSM_REQUIRE(n_params == off, BSMPS_ERR_INVALID_ARG, "mlp_create: params must hold every weight and bias");
         BSM_CUDA(cudaMalloc(&net->master, sizeof(float) * off));
         BSM_CUDA(cudaMalloc(&net->wbf, sizeof(__nv_bfloat16) * off));
+        int64_t images = 0;
+        for (int l = 0; l < n_layers; ++l) {
+            net->w1_off.push_back(images);
+            images += bsm::img_size(widths[l + 1], widths[l]);
+            net->w2_off.push_back(images);
+            images += bsm::img_size(widths[l], widths[l + 1]);
+        }
+        BSM_CUDA(cudaMalloc(&net->img, sizeof(float) * images));
+        BSM_CUDA(cudaMemsetAsync(net->img, 0, sizeof(float) * images, ctx->stream));
         BSM_CUDA(cudaMalloc(&net->m1, sizeof(float) * off));
         BSM_CUDA(cudaMalloc(&net->m2, sizeof(float) * off));
         BSM_CUDA(cudaMalloc(&net->grad, sizeof(float) * off));
         BSM_CUDA(cudaMemcpy(net->master, params, sizeof(float) * off, cudaMemcpyHostToDevice));
         BSM_CUDA(cudaMemset(net->m1, 0, sizeof(float) * off));
         BSM_CUDA(cudaMemset(net->m2, 0, sizeof(float) * off));
-        bsm::k_to_bf16<<<bsm::grid(off), bsm::kT, 0, ctx->stream>>>(net->master, net->wbf, off);
+        bsm::k_to_bf16<<<bsm::grid(off), bsm::kT, 0, ctx->stream>>>(net->master, net->wbf, net->img,
+                                                                        bsm::layers_of(net), off);
         bsm::done(ctx);
         ctx->sync();
         *out = net;
@@ -424,6 +553,7 @@ bsmps_status bsmps_mlp_create(bsmps_ctx c, int n_layers, const int* widths, cons
     if (net) {
         cudaFree(net->master);
         cudaFree(net->wbf);
+        cudaFree(net->img);
         cudaFree(net->m1);
         cudaFree(net->m2);
         cudaFree(net->grad);
@@ -452,11 +582,9 @@ bsmps_status bsmps_mlp_forward(bsmps_mlp m, const float* x, int B, float* y) {
         bsm::Context* ctx = ctx_of(m);
         BSM_REQUIRE(x && y && B > 0, BSMPS_ERR_INVALID_ARG, "mlp_forward: x, y and B > 0 required");
         bsm::Scratch s(ctx);
-        std::vector<float> xv(x, x + (size_t)B * m->widths[0]);
-        float* xd = s.up(xv);
-        bsm::Acts a = bsm::forward(ctx, m, xd, B, s);
+        bsm::Acts a = bsm::forward(ctx, m, x, B, s, false);
         const int out = m->widths.back();
-        BSM_CUDA(cudaMemcpyAsync(y, a.h.back(), sizeof(float) * B * out, cudaMemcpyDeviceToHost, ctx->stream));
+        BSM_CUDA(cudaMemcpyAsync(y, a.y, sizeof(float) * B * out, cudaMemcpyDeviceToHost, ctx->stream));
         ctx->sync();
     });
 }
@@ -483,7 +611,8 @@ bsmps_status bsmps_mlp_train_step(bsmps_mlp m, const float* x, const float* t, i
         const float c1 = 1.0f - std::pow(0.9f, (float)m->step);
         const float c2 = 1.0f - std::pow(0.999f, (float)m->step);
         bsm::k_adam<<<bsm::grid(m->n_params), bsm::kT, 0, ctx->stream>>>(m->master, m->grad, m->m1, m->m2, m->wbf,
-                                                                          m->n_params, lr, c1, c2);
+                                                                          m->img, bsm::layers_of(m), m->n_params, lr,
+                                                                          c1, c2);
         bsm::done(ctx);
         if (loss) *loss = l;
     });
@@ -494,6 +623,7 @@ bsmps_status bsmps_mlp_destroy(bsmps_mlp m) {
     cudaSetDevice(m->ctx->device);
     cudaFree(m->master);
     cudaFree(m->wbf);
+    cudaFree(m->img);
     cudaFree(m->m1);
     cudaFree(m->m2);
     cudaFree(m->grad);

@@ -3,19 +3,23 @@
 // (2012); integer slices as in Uchino, Ozaki, Imamura 2024).  Not part of the
 // paper: an FP64 path for the large contractions of the solver.
 //
-// Row i of A is scaled by 2^-e_i (e_i the smallest integer with
-// max_j |a_ij| < 2^e_i), column j of B by 2^-f_j; the scaled values are cut
-// into S digits of 7 bits plus sign (d = trunc(r 2^7), r <- r 2^7 - d), each an
-// integer in [-127, 127] and exact in bf16.  C = sum over slice pairs (p, q)
-// with p + q = d <= S + 1 of 2^{e_i + f_j - 7d} A_p B_q.  A slice product sums
-// integers below 2^14; the pairs of one d (at most 8) over 128 values of k stay
-// below 2^24, so the FP32 accumulator of the tensor-core product (tcgen05.mma
+// Row i of A is scaled by 2^-(e_i + 1) (e_i the smallest integer with
+// max_j |a_ij| < 2^e_i), column j of B by 2^-(f_j + 1); the scaled values, below
+// 1/2 in magnitude, are cut into S balanced digits of base 128 (integers in
+// [-64, 64], exact in bf16; what lies below the last digit is rounded, so that
+// the remainder is at most 2^(e_i - 7S)).  C = sum over slice pairs (p, q) with
+// p + q = d <= S + 1 of 2^{e_i + f_j + 2 - 7d} A_p B_q.  A slice product sums
+// integers up to 2^12; the pairs of one d (at most 8) over 128 values of k stay
+// within 2^22, so the FP32 accumulator of the tensor-core product (tcgen05.mma
 // kind::f16, BF16 operands, accumulators in tensor memory) is exact, the
 // diagonals are combined exactly in 64-bit integers, and the result is rounded
-// once.
+// once.  (Balanced digits instead of seven bits and a sign: sums within 2^22 turn
+// into integers by one FP32 addition, where a conversion instruction takes 32
+// cycles per warp and scheduler and bound the kernel: 740 us at n = 2048 before.)
 #include <algorithm>
 
 #include "kernels.h"
+#include "row_scan.cuh"
 #include "tc_common.cuh"
 
 namespace bsm {
@@ -41,63 +45,18 @@ constexpr uint32_t kOzIdesc = tc::idesc_bf16(kOzM, kOzN);
 // One factor of a product, read as n rows of K values (rows of op(A), columns of
 // B: row r, value k at src[r rs + k ks], one of the strides 1), and its slices:
 // blocks of `blk` rows x 32 k values, all S slices of a block one after the
-// other, each in the canonical K-major operand layout (8-row x 16-byte core
-// matrices, the four core matrices of a row group along k 128 bytes apart, row
-// groups kOzSbo apart), so that a chunk of a tile is one contiguous copy.
-struct OzSide {
-    const double* src;
-    int64_t rs, ks;
-    int n, K, nkc, blk;
+// other, each in the K-major operand layout with 64-byte swizzle (rows of 32
+// values, 8-row groups kOzSbo apart), so that a chunk of a tile is one contiguous
+// copy.
+struct OzSide : ScanSide {
+    int nkc, blk;
     int64_t dst;         // bytes from the slice buffer to block (0, 0)
-    int row0;            // first row in the maxima and exponent arrays
-    int max0, cut0;      // first CTA of this factor in k_oz_max / k_oz_slice
+    int cut0;            // first CTA of this factor in k_oz_slice
 };
 
-__device__ __forceinline__ int oz_find(const OzSide* __restrict__ sides, int n, int cta, bool cut) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((cut ? sides[mid].cut0 : sides[mid].max0) <= cta) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Largest magnitudes of the rows (bit patterns of non-negative doubles, ordered
-// like their values; mx zeroed before).  Rows contiguous in k: one warp per row,
-// eight rows per CTA.  Rows contiguous across: 32 rows x 512 k values per CTA.
-constexpr int kOzMaxK = 512;
-__global__ void __launch_bounds__(256) k_oz_max(const OzSide* __restrict__ sides, int n_sides,
-                                                unsigned long long* __restrict__ mx) {
-    const OzSide sd = sides[oz_find(sides, n_sides, (int)blockIdx.x, false)];
-    const int u = (int)blockIdx.x - sd.max0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFull;
-    const unsigned long long* src = (const unsigned long long*)sd.src;
-    unsigned long long m = 0ull;
-    if (sd.ks == 1) {
-        const int r = 8 * u + warp;
-        if (r >= sd.n) return;
-        for (int k = lane; k < sd.K; k += 32) m = max(m, src[(int64_t)r * sd.rs + k] & kAbs);
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) mx[sd.row0 + r] = m;
-        return;
-    }
-    __shared__ unsigned long long part[8][32];
-    const int nb = (sd.n + 31) / 32;
-    const int r = 32 * (u % nb) + lane, k0 = (u / nb) * kOzMaxK;
-    if (r < sd.n)
-        for (int k = k0 + warp; k < min(sd.K, k0 + kOzMaxK); k += 8) m = max(m, src[r * sd.rs + k * sd.ks] & kAbs);
-    part[warp][lane] = m;
-    __syncthreads();
-    if (warp == 0 && r < sd.n) {
-        for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
-        atomicMax(&mx[sd.row0 + r], m);
-    }
-}
-
-// Exponents and slices.  e = the smallest integer with max |x| < 2^e; |x| 2^-e is
-// a 56-bit fraction F (FP64 magnitudes have 53 bits; what lies below is cut, as
-// digit by digit truncation does) whose 7-bit digits, with the sign of x, are the
+// Exponents and slices.  e = the smallest integer with max |x| < 2^e; x 2^-(e+1)
+// is a 56-bit signed fraction X (rounded to nearest where the 53 bits of x reach
+// below it), for S < 8 rounded to 7 S bits, whose balanced base-128 digits are the
 // slices: integer operations only (an FP64 digit costs four FP64 instructions,
 // 0.4 ms at n = 2048 on this GPU).  A warp writes 8 rows x 32 k values: lane
 // (kg, r) the eight values k = 8 kg .. 8 kg + 7 of row r as one 16-byte store per
@@ -106,7 +65,13 @@ __global__ void __launch_bounds__(256) k_oz_max(const OzSide* __restrict__ sides
 __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sides, int n_sides, int S,
                                                   const unsigned long long* __restrict__ mx, int* __restrict__ exps,
                                                   unsigned char* __restrict__ buf) {
-    const OzSide sd = sides[oz_find(sides, n_sides, (int)blockIdx.x, true)];
+    int f = 0;   // the last factor whose CTAs start at or before this one
+    for (int hi = n_sides - 1; f < hi;) {
+        const int mid = (f + hi + 1) >> 1;
+        if (sides[mid].cut0 <= (int)blockIdx.x) f = mid;
+        else hi = mid - 1;
+    }
+    const OzSide sd = sides[f];
     const int u = (int)blockIdx.x - sd.cut0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int rg, kc;
     if (sd.ks == 1) {
@@ -125,33 +90,37 @@ __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sid
     int e = 0;
     if (top != 0ull) frexp(__longlong_as_double((long long)top), &e);   // max = m 2^e, 0.5 <= m < 1
     if (on && kc == 0 && kg == 0) exps[sd.row0 + r] = e;
-    unsigned long long F[8];
-    uint32_t neg = 0u;
+    long long X[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const int k = kOzKStep * kc + 8 * kg + t;
-        F[t] = 0ull;
+        X[t] = 0;
         if (on && k < sd.K) {
             const unsigned long long b = ((const unsigned long long*)sd.src)[r * sd.rs + k * sd.ks];
             const int ef = (int)((b >> 52) & 0x7ff);
             const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (ef ? 1ull << 52 : 0ull);
-            const int sh = (ef ? ef : 1) - 1023 - e + 4;   // |x| = m 2^(ef - 1075), F = |x| 2^(56 - e)
-            F[t] = sh >= 0 ? m << min(sh, 3) : (sh > -64 ? m >> -sh : 0ull);
-            neg |= (uint32_t)(b >> 63) << t;
+            const int sh = (ef ? ef : 1) - 1023 - e + 3;   // |x| = m 2^(ef - 1075), |X| = |x| 2^(55 - e)
+            unsigned long long f = 0ull;
+            if (sh >= 0) f = m << min(sh, 63);   // (beyond 2 for subnormal x only)
+            else if (sh > -55) f = (m + (1ull << (-sh - 1))) >> -sh;
+            if (S < kOzMaxS) f = (f + (1ull << (7 * (kOzMaxS - S) - 1))) >> (7 * (kOzMaxS - S));
+            X[t] = (b >> 63) ? -(long long)f : (long long)f;
         }
     }
     const int row = 8 * rg, blk = row / sd.blk;
     const int64_t slice = (int64_t)sd.blk * kOzKStep * 2;
     unsigned char* dst = buf + sd.dst + ((int64_t)blk * sd.nkc + kc) * S * slice + (row % sd.blk) / 8 * kOzSbo +
-                         kg * 128 + (lane & 7) * 16;
-    for (int p = 0; p < S; ++p) {
+                         (lane & 7) * 64 + (kg ^ ((lane >> 1) & 3)) * 16;
+    for (int p = S - 1; p >= 0; --p) {
         uint32_t w[4];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            const uint32_t d = (uint32_t)(F[t] >> (49 - 7 * p)) & 127u;
-            // d as a float (2^23 + d - 2^23), whose upper half is the BF16 value
-            uint32_t h = __float_as_uint(__uint_as_float(0x4B000000u | d) - 8388608.0f) >> 16;
-            if (d) h |= ((neg >> t) & 1u) << 15;
+            // the lowest digit, in [-64, 63] (the first one takes what is left, at most 64)
+            const int d = p ? (((int)X[t] + 64) & 127) - 64 : (int)X[t];
+            X[t] = (X[t] - d) >> 7;
+            // d as a float (1.5 2^23 + d - 1.5 2^23), whose upper half is the BF16 value
+            const uint32_t h =
+                __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)d) - 12582912.0f) >> 16;
             if (t & 1) w[t >> 1] |= h << 16;
             else w[t >> 1] = h;
         }
@@ -201,7 +170,7 @@ __device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, 
     return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
 }
 
-// C (M x N, row-major, ldc) = alpha sum_d 2^{e_i + f_j - 7(d + 2)} sum_{p + q = d + 2} A_p B_q
+// C (M x N, row-major, ldc) = alpha sum_d 2^{e_i + f_j + 2 - 7(d + 2)} sum_{p + q = d + 2} A_p B_q
 // (slices numbered from 1).  A persistent CTA per SM takes 128 x 64 output tiles:
 //  - one thread copies chunks of 32 k values of every slice (96 KB at S = 8: two
 //    contiguous pieces, cp.async.bulk) into a ring of stages;
@@ -212,7 +181,7 @@ __device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, 
 //  - every 128 values of k (where the FP32 sums of integer slice products are
 //    still exact) eight warps read a diagonal as soon as its last product is done
 //    and add it, shifted to its weight, to two exact 64-bit integers per entry in
-//    registers (four diagonals each, below 2^46 per 128 values of k), and the next
+//    registers (four diagonals each, below 2^44 per 128 values of k), and the next
 //    products of that diagonal may restart it: the tensor cores wait only for the
 //    first of the eight reads;
 //  - at the end of a tile the two integers are combined and rounded once.
@@ -248,19 +217,14 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
     if (tid == 0) {
         for (int i = 0; i < 2 * kStages + 2 * S + 1; ++i) {
             const uint32_t count = i >= 2 * kStages + S && i < 2 * kStages + 2 * S ? kOzEpiWarps : 1;
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(tc::smem_addr(&bars[i])), "r"(count));
+            tc::mbar_init(tc::smem_addr(&bars[i]), count);
         }
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tc::mbar_init_fence();
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         tc::smem_addr(&tmem_slot)),
-                     "r"(kCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    if (warp == 1) tc::tmem_alloc(&tmem_slot, kCols);
+    tc::fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tc::fence_after();
     const uint32_t tmem = tmem_slot;
     bool ok = true;
     if (warp == 0) {
@@ -279,18 +243,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                         break;
                     }
                     const uint32_t dst = base + s * kStage;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(kStage)
-                                 : "memory");
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            dst),
-                        "l"(a + (int64_t)c * kBytesA), "r"(kBytesA), "r"(full(s))
-                        : "memory");
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            dst + kBytesA),
-                        "l"(b + (int64_t)c * kBytesB), "r"(kBytesB), "r"(full(s))
-                        : "memory");
+                    tc::mbar_expect(full(s), kStage);
+                    tc::bulk_load(dst, a + (int64_t)c * kBytesA, kBytesA, full(s));
+                    tc::bulk_load(dst + kBytesA, b + (int64_t)c * kBytesB, kBytesB, full(s));
                 }
             }
             // copies in flight land before the CTA may end
@@ -310,9 +265,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                         ok = false;
                         break;
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint64_t da = tc::desc_sbo(base + s * kStage, kOzSbo);
-                    const uint64_t db = tc::desc_sbo(base + s * kStage + kBytesA, kOzSbo);
+                    tc::fence_after();
+                    const uint64_t da = tc::desc_sw64(base + s * kStage);
+                    const uint64_t db = tc::desc_sw64(base + s * kStage + kBytesA);
 #pragma unroll
                     for (int d = S - 1; d >= 0; --d) {
                         if (first && g > 0) {
@@ -320,30 +275,24 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                                 ok = false;
                                 break;
                             }
-                            asm volatile("tcgen05.fence::after_thread_sync;");
+                            tc::fence_after();
                         }
 #pragma unroll
                         for (int p = 0; p <= d; ++p)
 #pragma unroll
                             for (int kk = 0; kk < kOzKStep / 16; ++kk)
-                                tc::mma_bf16(tmem + (uint32_t)(d * kOzN), da + ((p * kOzSliceA + kk * 256) >> 4),
-                                             db + (((d - p) * kOzSliceB + kk * 256) >> 4), kOzIdesc,
+                                tc::mma_bf16(tmem + (uint32_t)(d * kOzN), da + ((p * kOzSliceA + kk * 32) >> 4),
+                                             db + (((d - p) * kOzSliceB + kk * 32) >> 4), kOzIdesc,
                                              first && p == 0 && kk == 0 ? 0u : 1u);
                         if (last)
-                            asm volatile(
-                                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                    dfull(d))
-                                : "memory");
+                            tc::commit(dfull(d));
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     empty(s))
-                                 : "memory");
+                    tc::commit(empty(s));
                     if (last) ++g;
                 }
             }
             // every MMA and every earlier commit has happened before the CTA ends
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain)
-                         : "memory");
+            tc::commit(drain);
             ok = tc::mbar_wait(drain, 0) && ok;
         }
         __syncwarp();
@@ -364,28 +313,35 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                         ok = false;
                         break;
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;");
-                    uint32_t v[32];
-                    tc::ld_32x32b_x32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(d * kOzN + half * 32), v);
-                    asm volatile("tcgen05.fence::before_thread_sync;");
-                    __syncwarp();
-                    if (lane == 0)
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(dempty(d)) : "memory");
+                    tc::fence_after();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int x = __float2int_rz(__uint_as_float(v[j]));   // an exact integer below 2^24
-                        if (d < 4)
-                            i0[j] += (long long)x * (1 << (7 * (3 - d)));
-                        else
-                            i1[j] += (long long)x * (1 << (7 * (7 - d)));
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t v[16];
+                        tc::ld_32x32b_x16(
+                            tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(d * kOzN + half * 32 + 16 * h), v);
+                        if (h == 1) {
+                            tc::fence_before();
+                            __syncwarp();
+                            if (lane == 0)
+                                tc::mbar_arrive(dempty(d));
+                        }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            // an integer within 2^22: its bits in the sum with 1.5 2^23, less 0x4B400000
+                            const int x = (int)__float_as_uint(__uint_as_float(v[j]) + 12582912.0f) - 0x4B400000;
+                            if (d < 4)
+                                i0[16 * h + j] += (long long)x * (1 << (7 * (3 - d)));
+                            else
+                                i1[16 * h + j] += (long long)x * (1 << (7 * (7 - d)));
+                        }
                     }
                 }
             }
             if (!ok) break;
-            // diagonal d carries 2^-7(d + 2): C = (i0 2^28 + i1) 2^(e + f - 63)
+            // diagonal d carries 2^(2 - 7(d + 2)): C = (i0 2^28 + i1) 2^(e + f - 61)
             const int row = tl.m0 + quad * 32 + lane, c0 = tl.n0 + half * 32;
             if (row < pd.M) {
-                const int e = exps[pd.e_off + row] - 63;
+                const int e = exps[pd.e_off + row] - 61;
                 const int* f = exps + pd.f_off;
                 double* out = pd.C + (int64_t)row * pd.ldc;
 #pragma unroll
@@ -402,9 +358,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
         }
     }
     if (!ok) atomicExch(err, 1);
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tc::fence_before();
     __syncthreads();
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+    if (warp == 1) tc::tmem_free(tmem, kCols);
 }
 
 template <int S>
@@ -433,23 +389,18 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S)
     int rows = 0, max_ctas = 0, cut_ctas = 0;
     double fl = 0.0;
     auto side = [&](const double* src, int64_t rs, int64_t ks, int n, int K, int nkc, int blk) {
-        OzSide sd{src, rs, ks, n, K, nkc, blk, bytes, rows, max_ctas, cut_ctas};
+        const OzSide sd{{src, rs, ks, n, K, rows, max_ctas}, nkc, blk, bytes, cut_ctas};
         bytes += (int64_t)((n + blk - 1) / blk) * nkc * S * blk * kOzKStep * 2;
         rows += n;
         const int groups = (n + 7) / 8;
-        if (ks == 1) {
-            max_ctas += groups;
-            cut_ctas += groups * ((nkc + 7) / 8);
-        } else {
-            max_ctas += ((n + 31) / 32) * std::max(1, (K + kOzMaxK - 1) / kOzMaxK);
-            cut_ctas += ((groups + 7) / 8) * nkc;
-        }
+        max_ctas += scan_ctas(ks, n, K);
+        cut_ctas += ks == 1 ? groups * ((nkc + 7) / 8) : ((groups + 7) / 8) * nkc;
         sides.push_back(sd);
         return sd;
     };
     for (const OzGemm& g : gs) {
         BSM_REQUIRE(g.M >= 0 && g.N >= 0 && g.K >= 0, BSMPS_ERR_INVALID_ARG, "emulated GEMM: sizes >= 0");
-        // the exact 64-bit sums of the diagonals (below 2^46 per 128 values of k) stay below 2^63
+        // the exact 64-bit sums of the diagonals (below 2^44 per 128 values of k) stay below 2^63
         BSM_REQUIRE(g.K < (1 << 24), BSMPS_ERR_INVALID_ARG, "emulated GEMM: K < 2^24");
         if (g.M == 0 || g.N == 0) continue;
         const int nkc = (g.K + kOzKStep - 1) / kOzKStep;
@@ -473,7 +424,7 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S)
     const OzProd* d_prods = s.up(prods);
     const OzTile* d_tiles = s.up(tiles);
     BSM_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)rows, ctx->stream));
-    k_oz_max<<<max_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), mx);
+    k_row_max<OzSide><<<max_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), mx);
     launched(ctx);
     if (cut_ctas > 0) {
         k_oz_slice<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), S, mx, exps, slices);

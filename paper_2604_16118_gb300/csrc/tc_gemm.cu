@@ -27,6 +27,7 @@
 #include <cstdint>
 
 #include "kernels.h"
+#include "row_scan.cuh"
 #include "tc_common.cuh"
 
 namespace bsm {
@@ -279,6 +280,222 @@ finish:
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcN));
 }
 
+// ---- one large product: operands split once, then a pipelined GEMM ----
+//
+// The grouped kernel above splits the operands of every tile again (each value of
+// A once per 64 columns of C) and scans them for the scales first; for one product
+// of 3000 x 1100 x 700 that took 800 us.  Here k_row_max finds the scales, k_tc_split
+// writes the TF32 parts once, in operand layout (128 rows x 32 k values per block,
+// 128-byte swizzle: the high parts, then the low parts), and k_gemm_split streams
+// blocks by bulk copies through a ring of stages: the same products in the same
+// order per entry.
+
+// One factor with its split blocks and power-of-two exponents (alpha folded into A).
+struct SplitSide : ScanSide {
+    int nkc;
+    double alpha;
+    int is_b;
+    int64_t dst;   // bytes from the buffer to block (0, 0)
+    int cut0;      // first CTA in k_tc_split
+};
+
+constexpr int kSpTile = 128;                          // rows and columns of a tile
+constexpr uint32_t kSpPart = kSpTile * kTcK * 4;      // bytes of the high (or low) parts of a block
+constexpr uint32_t kSpStage = 4 * kSpPart;            // A and B blocks of one chunk
+constexpr int kSpStages = 3;
+constexpr int kSpThreads = 192;                       // producer warp, MMA warp, four epilogue warps
+constexpr uint32_t kSpIdesc = tc::idesc_tf32(kSpTile, kSpTile);
+
+// One warp writes 8 rows x 32 k values: a lane four values of k (16 bytes of each part) twice.
+__global__ void __launch_bounds__(256) k_tc_split(const SplitSide* __restrict__ sides,
+                                                  const unsigned long long* __restrict__ mx, int* __restrict__ exps,
+                                                  unsigned char* __restrict__ buf) {
+    const SplitSide sd = sides[(int)blockIdx.x >= sides[1].cut0 ? 1 : 0];
+    const int u = (int)blockIdx.x - sd.cut0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int rg, kc;
+    if (sd.ks == 1) {
+        const int nk8 = (sd.nkc + 7) / 8;
+        rg = u / nk8;
+        kc = 8 * (u % nk8) + warp;
+    } else {
+        const int ng = ((sd.n + 7) / 8 + 7) / 8;
+        rg = 8 * (u % ng) + warp;
+        kc = u / ng;
+    }
+    if (kc >= sd.nkc || 8 * rg >= sd.n) return;
+    unsigned char* dst = buf + sd.dst + ((int64_t)(8 * rg / kSpTile) * sd.nkc + kc) * (2 * kSpPart) +
+                         (8 * rg % kSpTile) / 8 * 1024;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        // rows contiguous in k: eight lanes along k; rows contiguous across: eight lanes along the rows
+        const int rr = sd.ks == 1 ? (lane >> 3) + 4 * h : lane & 7;
+        const int kg = sd.ks == 1 ? lane & 7 : (lane >> 3) + 4 * h;
+        const int r = 8 * rg + rr;
+        const unsigned long long top = r < sd.n ? mx[sd.row0 + r] : 0ull;
+        // (the columns of B have no factor; their largest bit pattern decides as it is)
+        const double mxa = __longlong_as_double((long long)top) * fabs(sd.alpha);
+        const int sc = sd.is_b ? pow2_exponent(top)
+                                             : mxa > 0.0 ? pow2_exponent((unsigned long long)__double_as_longlong(mxa)) : 0;
+        if (r < sd.n && kc == 0 && kg == 0) exps[sd.row0 + r] = sc;
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int k = kTcK * kc + 4 * kg + t;
+            hi[t] = lo[t] = 0u;
+            if (r < sd.n && k < sd.K)
+                split_scaled(
+                    (unsigned long long)__double_as_longlong(sd.alpha * sd.src[(int64_t)r * sd.rs + k * sd.ks]), sc,
+                    &hi[t], &lo[t]);
+        }
+        unsigned char* o = dst + rr * 128 + (kg ^ rr) * 16;
+        *(uint4*)o = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *(uint4*)(o + kSpPart) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+}
+
+// C tile (128 x 128 per CTA): one thread streams the chunks (64 KB each) into three
+// stages, one issues 12 MMAs per chunk (A_lo B_hi, A_hi B_lo, A_hi B_hi per 8 values of k),
+// four warps read the accumulators and store FP64.  Waits bounded as above.
+__global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, int nkc, int e_a, int e_b,
+                                                              const unsigned char* __restrict__ A,
+                                                              const unsigned char* __restrict__ B,
+                                                              const int* __restrict__ exps, int* err) {
+    extern __shared__ __align__(1024) unsigned char sp_smem[];
+    __shared__ __align__(8) uint64_t bars[2 * kSpStages + 1];
+    __shared__ uint32_t tmem_slot;
+    const uint32_t base = (smem_addr(sp_smem) + 1023u) & ~1023u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m0 = blockIdx.x * kSpTile, n0 = blockIdx.y * kSpTile;
+    auto full = [&](int s) { return smem_addr(&bars[s]); };
+    auto empty = [&](int s) { return smem_addr(&bars[kSpStages + s]); };
+    const uint32_t done = smem_addr(&bars[2 * kSpStages]);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2 * kSpStages + 1; ++i) tc::mbar_init(smem_addr(&bars[i]), 1);
+        tc::mbar_init_fence();
+    }
+    if (warp == 1) tc::tmem_alloc(&tmem_slot, kSpTile);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tmem_slot;
+    bool ok = true;
+    if (warp == 0) {
+        if (lane == 0) {
+            const unsigned char* a = A + (int64_t)blockIdx.x * nkc * (2 * kSpPart);
+            const unsigned char* b = B + (int64_t)blockIdx.y * nkc * (2 * kSpPart);
+            int c = 0;
+            for (; c < nkc; ++c) {
+                const int s = c % kSpStages;
+                if (c >= kSpStages && !mbar_wait(empty(s), (c / kSpStages - 1) & 1)) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t dst = base + s * kSpStage;
+                tc::mbar_expect(full(s), kSpStage);
+                tc::bulk_load(dst, a + (int64_t)c * (2 * kSpPart), 2 * kSpPart, full(s));
+                tc::bulk_load(dst + 2 * kSpPart, b + (int64_t)c * (2 * kSpPart), 2 * kSpPart, full(s));
+            }
+            // copies in flight land before the CTA may end
+            for (int i = c > kSpStages ? c - kSpStages : 0; i < c; ++i)
+                mbar_wait(full(i % kSpStages), (i / kSpStages) & 1);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            for (int c = 0; c < nkc; ++c) {
+                const int s = c % kSpStages;
+                if (!mbar_wait(full(s), (c / kSpStages) & 1)) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after();
+                const uint64_t a_hi = tc::desc_sw128(base + s * kSpStage), a_lo = a_hi + (kSpPart >> 4);
+                const uint64_t b_hi = a_hi + (2 * kSpPart >> 4), b_lo = a_hi + (3 * kSpPart >> 4);
+#pragma unroll
+                for (int kk = 0; kk < kTcK / 8; ++kk) {
+                    const uint64_t step = (uint64_t)kk * 2;   // 32 bytes along k
+                    tc::mma_tf32(tmem, a_lo + step, b_hi + step, kSpIdesc, c == 0 && kk == 0 ? 0u : 1u);
+                    tc::mma_tf32(tmem, a_hi + step, b_lo + step, kSpIdesc, 1u);
+                    tc::mma_tf32(tmem, a_hi + step, b_hi + step, kSpIdesc, 1u);
+                }
+                tc::commit(empty(s));
+            }
+            tc::commit(done);   // covers every MMA and every earlier commit
+            ok = mbar_wait(done, 0) && ok;
+        }
+        __syncwarp();
+    } else {
+        ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
+        tc::fence_after();
+        const int quad = warp & 3, row = m0 + quad * 32 + lane;
+        const int e = row < o.M ? exps[e_a + row] : 0;
+        for (int c0 = 0; ok && c0 < kSpTile; c0 += 16) {
+            uint32_t v[16];
+            tc::ld_32x32b_x16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, v);
+            if (row < o.M) {
+                double* cr = o.C + (int64_t)row * o.ldc;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int col = n0 + c0 + j;
+                    if (col < o.N) {
+                        const double acc = scale_out(v[j], e + exps[e_b + col]);
+                        cr[col] = o.beta == 0.0 ? acc : o.beta * cr[col] + acc;
+                    }
+                }
+            }
+        }
+    }
+    if (!ok) atomicExch(err, 1);
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 1) tc::tmem_free(tmem, kSpTile);
+}
+
+void launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kind) {
+    const int nkc = (in.K + kTcK - 1) / kTcK;
+    std::vector<SplitSide> sides;
+    int64_t bytes = 0;
+    int rows = 0, max_ctas = 0, cut_ctas = 0;
+    auto side = [&](const double* src, int64_t rs, int64_t ks, int n, double alpha, int is_b) {
+        sides.push_back({{src, rs, ks, n, in.K, rows, max_ctas}, nkc, alpha, is_b, bytes, cut_ctas});
+        bytes += (int64_t)((n + kSpTile - 1) / kSpTile) * nkc * (2 * kSpPart);
+        rows += n;
+        const int groups = (n + 7) / 8;
+        max_ctas += scan_ctas(ks, n, in.K);
+        cut_ctas += ks == 1 ? groups * ((nkc + 7) / 8) : ((groups + 7) / 8) * nkc;
+    };
+    side(in.A, in.lda, 1, o.M, in.alpha, 0);
+    side(in.B, 1, in.ldb, o.N, 1.0, 1);
+    const double fl = 2.0 * o.M * (double)o.N * in.K;
+    const double by = 8.0 * ((double)o.M * in.K + (double)in.K * o.N + o.M * (double)o.N * (o.beta == 0.0 ? 1.0 : 2.0));
+    ctx->flops += fl;
+    Scratch s(ctx);
+    unsigned char* buf = (unsigned char*)ctx->alloc((size_t)bytes);
+    s.ptrs.push_back(buf);
+    unsigned long long* mx = (unsigned long long*)ctx->alloc(sizeof(unsigned long long) * (size_t)rows);
+    s.ptrs.push_back(mx);
+    int* exps = (int*)ctx->alloc(sizeof(int) * (size_t)rows);
+    s.ptrs.push_back(exps);
+    const SplitSide* d_sides = s.up(sides);
+    const int smem = kSpStages * (int)kSpStage + 1024;
+    static bool attr = false;
+    if (!attr) {
+        BSM_CUDA(cudaFuncSetAttribute(k_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        attr = true;
+    }
+    BSM_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)rows, ctx->stream));
+    ProfScope ps(ctx, kind, fl, by);
+    k_row_max<SplitSide><<<max_ctas, 256, 0, ctx->stream>>>(d_sides, 2, mx);
+    check_launch(ctx);
+    k_tc_split<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, mx, exps, buf);
+    check_launch(ctx);
+    const dim3 grid((unsigned)((o.M + kSpTile - 1) / kSpTile), (unsigned)((o.N + kSpTile - 1) / kSpTile));
+    k_gemm_split<<<grid, kSpThreads, smem, ctx->stream>>>(o, nkc, sides[0].row0, sides[1].row0, buf + sides[0].dst,
+                                                          buf + sides[1].dst, exps, ctx->err_word());
+    check_launch(ctx);
+    ps.done();
+}
+
 }  // namespace
 
 bool gemm_tf32x3_eligible(const std::vector<GemmOut>& outs, const std::vector<GemmIn>& ins) {
@@ -290,6 +507,16 @@ bool gemm_tf32x3_eligible(const std::vector<GemmOut>& outs, const std::vector<Ge
 
 void launch_gemm_tf32x3(Context* ctx, const std::vector<GemmOut>& outs, const std::vector<GemmIn>& ins, int kind) {
     if (outs.empty()) return;
+    // One product with one contribution (bsmps_gemm_tf32x3, whole iterates): split once.  Below
+    // 2^17 multiplications its three launches cost more than the grouped kernel's repeated splits
+    // save; the grouped launches of the zip-up stay on the grouped kernel (the scales there span
+    // several contributions).
+    if (outs.size() == 1 && outs[0].end == outs[0].beg + 1 && !ins[outs[0].beg].transA && outs[0].M > 0 &&
+        outs[0].N > 0 && ins[outs[0].beg].K > 0 &&
+        (double)outs[0].M * outs[0].N * ins[outs[0].beg].K >= (double)(1 << 17)) {
+        launch_gemm_split(ctx, outs[0], ins[outs[0].beg], kind);
+        return;
+    }
     std::vector<TcTile> tiles;
     double fl = 0.0, by = 0.0;
     for (int o = 0; o < (int)outs.size(); ++o) {
