@@ -463,10 +463,11 @@ BSMPS_API bsmps_status bsmps_eigensolve_step(bsmps_ctx ctx, bsmps_mpo W, const b
  *   - Scaling: each row of A and each column of B is scaled by a power of two
  *     below which all its entries lie.
  *   - Slices: the scaled values are cut into `slices` (1..8) digits of 7 bits
- *     plus sign, each exact in bf16.
- *   - Products: slice pairs (p, q) with p + q <= slices + 1 are multiplied
- *     exactly (FP32 accumulation of integers below 2^24, 128 values of k at a
- *     time) and summed in float64.
+ *     (balanced digits, each exact in bf16; the 56 bits of 8 slices as 7 digits of
+ *     8 bits, which keeps the bound below).
+ *   - Products: slice pairs (p, q) whose weights lie above the last digit's are
+ *     multiplied exactly (FP32 accumulation of integers below 2^24, 128 values of
+ *     k at a time), summed exactly and rounded once.
  * Error bound per entry, in units of K 2^{e_i + f_j}:
  * 2^{1 - 7 slices} + sum_{d > slices+1} (2 slices - d + 1) 2^{14 - 7d}
  * + slices 2^{-52}.  With 8 slices this is within a few units of float64

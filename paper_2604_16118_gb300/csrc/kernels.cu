@@ -46,17 +46,78 @@ struct GemmTile {
 constexpr int kTile = dev::kGemmTile;
 constexpr int kSmallGemmThreads = 128;
 
+// Contributions that read the same B block (untransposed): their A blocks are summed first,
+// sum_c alpha_c A_c B = (sum_c alpha_c A_c) B.  In the zip-up contraction every output has at
+// most two B blocks (one per occupation of the site) and as many contributions as operator
+// entries, so the products shrink from one per entry to two.
+__device__ __forceinline__ bool same_b(const GemmIn& x, const GemmIn& y) {
+    return x.B == y.B && x.K == y.K && x.ldb == y.ldb && !x.transA && !y.transA;
+}
+
+// One run in[0 .. n) of such contributions added to the tile's accumulators (thread mapping and
+// staging as dev::gemm_tile_accumulate; the sum is formed while A is staged).
+__device__ __forceinline__ void tile_accumulate_run(const GemmIn* in, int n, int M, int N, int m0, int n0,
+                                                    double (*As)[kTile + 1], double (*Bs)[kTile + 1], double acc[4]) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int K = in[0].K, ldb = in[0].ldb, gn = n0 + tx;
+    const double* B = in[0].B;
+    for (int k0 = 0; k0 < K; k0 += kTile) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int mm = ty + 8 * r, gm = m0 + mm, gk = k0 + tx;
+            if (m0 + 8 * r >= M) break;
+            double v = 0.0;
+            if (gm < M && gk < K) {
+#pragma unroll 4
+                for (int u = 0; u < n; ++u) v = fma(in[u].alpha, in[u].A[(int64_t)gm * in[u].lda + gk], v);
+            }
+            As[tx][mm] = v;
+        }
+        const int kk_end = min(kTile, K - k0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int kk = ty + 8 * r;
+            if (kk < kk_end) Bs[kk][tx] = gn < N ? B[(int64_t)(k0 + kk) * ldb + gn] : 0.0;
+        }
+        __syncthreads();
+        for (int kk = 0; kk < kk_end; ++kk) {
+            const double b = Bs[kk][tx];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (m0 + ty + 8 * r < M) acc[r] = fma(As[kk][ty + 8 * r], b, acc[r]);
+        }
+        __syncthreads();
+    }
+}
+
 // 32 x 32 output tile per CTA; thread (ty, tx) owns rows ty + 8 r (r < 4), column tx.
+constexpr int kGemmIns = 64;   // descriptors staged at a time
 __global__ void __launch_bounds__(kThreads) k_gemm(const GemmOut* __restrict__ outs,
                                                    const GemmIn* __restrict__ ins,
                                                    const GemmTile* __restrict__ tiles) {
     __shared__ double As[kTile][kTile + 1];   // [k][m]
     __shared__ double Bs[kTile][kTile + 1];   // [k][n]
+    __shared__ GemmIn s_in[kGemmIns];
     const GemmTile tl = tiles[blockIdx.x];
     const GemmOut o = outs[tl.out];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int c = o.beg; c < o.end; ++c) dev::gemm_tile_accumulate(ins[c], o.M, o.N, tl.m0, tl.n0, As, Bs, acc);
+    for (int cb = o.beg; cb < o.end; cb += kGemmIns) {
+        const int n = min(kGemmIns, o.end - cb);
+        constexpr int kWords = (int)(sizeof(GemmIn) / sizeof(long long));
+        for (int i = threadIdx.x; i < n * kWords; i += kThreads) ((long long*)s_in)[i] = ((const long long*)(ins + cb))[i];
+        __syncthreads();
+        for (int u = 0; u < n;) {
+            int v = u + 1;
+            while (v < n && same_b(s_in[v], s_in[u])) ++v;
+            if (s_in[u].transA)
+                dev::gemm_tile_accumulate(s_in[u], o.M, o.N, tl.m0, tl.n0, As, Bs, acc);
+            else
+                tile_accumulate_run(s_in + u, v - u, o.M, o.N, tl.m0, tl.n0, As, Bs, acc);
+            u = v;
+        }
+        __syncthreads();   // the descriptors are replaced
+    }
     const int gn = tl.n0 + tx;
     if (gn >= o.N) return;
 #pragma unroll
@@ -246,6 +307,53 @@ struct ZeroChunk {
 __global__ void __launch_bounds__(kThreads) k_zero(const ZeroChunk* __restrict__ chunks) {
     const ZeroChunk c = chunks[blockIdx.x];
     for (int64_t e = threadIdx.x; e < c.n; e += kThreads) c.p[e] = 0.0;
+}
+
+// Up to kFlatCores cores per launch, their pointers in the kernel's arguments (no task upload).
+constexpr int kFlatCores = 120;
+struct FlatCores {
+    double* core[kFlatCores];
+    int64_t beg[kFlatCores + 1];   // offsets in the flat array
+    int n;
+};
+
+__global__ void __launch_bounds__(kThreads) k_flat_cores(const FlatCores fc, double* __restrict__ flat, int to_cores) {
+    for (int64_t e = fc.beg[0] + (int64_t)blockIdx.x * kThreads + threadIdx.x; e < fc.beg[fc.n];
+         e += (int64_t)gridDim.x * kThreads) {
+        int lo = 0, hi = fc.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (fc.beg[mid] <= e) lo = mid;
+            else hi = mid - 1;
+        }
+        double* c = fc.core[lo] + (e - fc.beg[lo]);
+        if (to_cores) *c = flat[e];
+        else flat[e] = *c;
+    }
+}
+
+void launch_flat_cores(Context* ctx, const std::vector<double*>& core, const std::vector<int64_t>& n, double* flat,
+                       bool to_cores) {
+    configure_carveout();
+    int64_t off = 0;
+    for (size_t t = 0; t < core.size();) {
+        FlatCores fc{};
+        for (; t < core.size() && fc.n < kFlatCores; ++t) {
+            if (n[t] > 0) {
+                fc.core[fc.n] = core[t];
+                fc.beg[fc.n++] = off;
+            }
+            off += n[t];
+        }
+        fc.beg[fc.n] = off;
+        if (fc.n == 0) continue;
+        const int64_t total = off - fc.beg[0];
+        const unsigned ctas = (unsigned)std::min<int64_t>((total + 4 * kThreads - 1) / (4 * kThreads), 1024);
+        ProfScope ps(ctx, KK_COPY, 0.0, 16.0 * (double)total);
+        k_flat_cores<<<ctas, kThreads, 0, ctx->stream>>>(fc, flat, to_cores ? 1 : 0);
+        check_launch(ctx);
+        ps.done();
+    }
 }
 
 void launch_zero(Context* ctx, const std::vector<double*>& ptr, const std::vector<int64_t>& n, int kind) {

@@ -125,6 +125,10 @@ void launch_copy(Context* ctx, const std::vector<CopyTask>& tasks, int kind = KK
 // Sets n[i] doubles at ptr[i] to zero, all regions in one launch.
 void launch_zero(Context* ctx, const std::vector<double*>& ptr, const std::vector<int64_t>& n,
                  int kind = KK_COPY);
+// Copies between the cores (n[t] doubles at core[t], one buffer each) and their
+// concatenation `flat`: into the cores (to_cores) or out of them.
+void launch_flat_cores(Context* ctx, const std::vector<double*>& core, const std::vector<int64_t>& n, double* flat,
+                       bool to_cores);
 // Counts a launch and raises the launch error, if any.
 void check_launch(Context* ctx);
 // The same grouped GEMM on the tensor cores in split precision (3xTF32, FP32
@@ -309,24 +313,32 @@ int check_grid_wait(Context* ctx, int skip_cta);
 struct EnvGroupPhase {
     int64_t base[4], stride[4];
     int mem_beg, n_mem;   // members: member_fac[mem_beg .. mem_beg + n_mem)
-    double shift;         // added to the weight of inputs with shift_flag
+    double shift;         // added to the weights that ask for it
 };
+// Output C (M x N, row-major) = sum over runs beg .. end.
 struct EnvOutT {
-    int M, N, ldc, beg, end;
+    int M, N, beg, end;
     int gp;    // its group-phase entry
     int cbuf;
     int64_t coff;
 };
-struct EnvInT {
-    const double* A;   // real pointer when abuf < 0
-    const double* B;   // real pointer when bbuf < 0
-    int64_t aoff, boff;
-    int abuf, bbuf;
-    int K, lda, ldb, transA;
+// One run: op(A) (K values of k) times a sum of right factors.
+//  - site product T = E X (even phases): A is the M x K block at offset `off` of
+//    the environment buffer (abuf), the right factor the K x N block at ptr;
+//  - environment update E' = sum X_a^T T (odd phases): A^T is the K x M block at
+//    ptr, the right factor sum_c w_c T_c over cons cbeg .. cend (blocks of T, K x N,
+//    combined before they are multiplied: one product per block of a instead of one
+//    per operator entry).
+struct EnvRunT {
+    const double* ptr;
+    int64_t off;
+    int abuf, K;
+    int cbeg, cend, site;
+};
+struct EnvConT {
+    int64_t off;       // block of T
     double w;
-    int shift_flag;
-    int so, si;        // factor rows: fa[so], fb[si] of the member (so < 0: no factors)
-    int site;
+    int fac, pad;      // bit 0: s_out, bit 1: s_in (factor rows fa[s_out], fb[s_in] of the member), bit 2: add the shift
 };
 struct EnvTileT {
     int out, m0, n0, member;
@@ -335,8 +347,8 @@ struct EnvTileT {
 struct EnvMemberFac {
     int row[4];
 };
-bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvInT>& ins,
-                        const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
+bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
+                        const std::vector<EnvConT>& cons, const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
                         const std::vector<EnvGroupPhase>& gph, const std::vector<EnvMemberFac>& mfac,
                         const std::vector<double>& ftab, int K, double* const base[4],
                         const std::vector<const double*>& finals, const std::vector<int>& final_beg, double* res,

@@ -38,26 +38,29 @@ Mps* new_mps(Context* ctx, const Layout& L, bool zero) {
 
 static MpsPtr make_mps(Context* ctx, const Layout& L, bool zero) { return MpsPtr(new_mps(ctx, L, zero)); }
 
+// The flat layout of an iterate and its cores (one buffer per core) meet in one
+// staging buffer: one host copy and one kernel instead of a copy per core (a
+// small copy from or to pageable memory costs 10 to 20 us).
 void mps_upload(Mps* x, const double* host) {
-    int64_t off = 0;
-    for (int t = 0; t < x->lay.K; ++t) {
-        const int64_t n = x->lay.core_size[t];
-        if (n > 0)
-            BSM_CUDA(cudaMemcpyAsync(x->core[t], host + off, (size_t)n * sizeof(double),
-                                     cudaMemcpyHostToDevice, x->ctx->stream));
-        off += n;
+    const int64_t n = x->lay.total();
+    if (n > 0) {
+        Scratch s(x->ctx);
+        double* flat = s.dbl((size_t)n);
+        BSM_CUDA(cudaMemcpyAsync(flat, host, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, x->ctx->stream));
+        launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, true);
     }
     x->ctx->sync();
 }
 
 void mps_download(const Mps* x, double* host) {
-    int64_t off = 0;
-    for (int t = 0; t < x->lay.K; ++t) {
-        const int64_t n = x->lay.core_size[t];
-        if (n > 0)
-            BSM_CUDA(cudaMemcpyAsync(host + off, x->core[t], (size_t)n * sizeof(double),
-                                     cudaMemcpyDeviceToHost, x->ctx->stream));
-        off += n;
+    const int64_t n = x->lay.total();
+    if (n > 0) {
+        Scratch s(x->ctx);
+        double* flat = s.dbl((size_t)n);
+        launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, false);
+        BSM_CUDA(cudaMemcpyAsync(host, flat, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, x->ctx->stream));
+        x->ctx->sync();
+        return;
     }
     x->ctx->sync();
 }
@@ -1481,7 +1484,8 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
         int64_t off;   // within a member's share of the E buffer
     };
     std::vector<EnvOutT> outs;
-    std::vector<EnvInT> ins;
+    std::vector<EnvRunT> runs;
+    std::vector<EnvConT> cons;
     std::vector<EnvTileT> tiles;
     std::vector<EnvGroupPhase> gph;
     std::vector<int> phase_beg{0};
@@ -1506,86 +1510,57 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
         gph.push_back(e);
         return (int)gph.size() - 1;
     };
+    // one operator entry acting on one environment block: the block of E' it adds to
+    // (right sectors of a and b), the block of a it multiplies, its T block and entry
     struct Contrib {
-        uint64_t key;
-        int seq, ti, ab, ei;
-        int so, si;
+        uint64_t key;   // ra 2^42 + rb 2^21 + ab
+        int ti, ei;
     };
     struct TBlk {
-        int env, sigma, rows, cols, bb;
+        int env, rows, cols, bb;
         int64_t off;   // within a member's share of the T buffer
     };
+    std::vector<Contrib> cs;
     for (int t = 0; t < K; ++t) {
         const int eid = t == 0 ? 3 : 1 + (t % 2);   // buffer of E at bond t
         const int nid = 1 + ((t + 1) % 2);          // buffer of E at bond t + 1
         std::vector<std::vector<TBlk>> T(G);
-        std::vector<int64_t> T_size(G, 0);
-        std::vector<std::vector<Contrib>> contrib(G);
-        // ---- structure of the site, once per group ----
-        for (int g = 0; g < G; ++g) {
-            const Layout& A = probs[rep[g]].a->lay;
-            const Layout& B = probs[rep[g]].b->lay;
-            const std::vector<int> blook = block_lookup(B, t);
-            const std::vector<int> alook = block_lookup(A, t);
-            std::vector<std::array<int, 2>> tidx(E[g].size(), {-1, -1});
-            for (int e = 0; e < (int)E[g].size(); ++e)
-                for (int si = 0; si < 2; ++si) {
-                    const int bb = blook[E[g][e].ib * 2 + si];
-                    if (bb < 0) continue;
-                    tidx[e][si] = (int)T[g].size();
-                    const Block& bk = B.blocks[t][bb];
-                    T[g].push_back({e, si, E[g][e].rows, bk.cols, bb, T_size[g]});
-                    T_size[g] += (int64_t)E[g][e].rows * bk.cols;
-                }
-            const Mpo& W = *ops[g];
-            const int nch = W.bond_dim(t);
-            std::vector<std::vector<int>> by_chan(nch);
-            for (int e = 0; e < (int)E[g].size(); ++e) by_chan[E[g][e].c].push_back(e);
-            int seq = 0;
-            for (int ei = 0; ei < (int)W.entries[t].size(); ++ei) {
-                const MpoEntry& me = W.entries[t][ei];
-                if (me.a >= nch || by_chan[me.a].empty()) continue;
-                for (int e : by_chan[me.a]) {
-                    const int ab = alook[E[g][e].ia * 2 + me.so];
-                    const int ti = tidx[e][me.si];
-                    if (ab < 0 || ti < 0) continue;
-                    const int bb = blook[E[g][e].ib * 2 + me.si];
-                    const uint64_t ra = (uint64_t)A.blocks[t][ab].ri, rb = (uint64_t)B.blocks[t][bb].ri;
-                    const uint64_t key = ((uint64_t)me.b << 42) | (ra << 21) | rb;
-                    contrib[g].push_back({key, seq++, ti, ab, ei, me.so, me.si});
-                }
-            }
-            std::sort(contrib[g].begin(), contrib[g].end(), [](const Contrib& x, const Contrib& y) {
-                return x.key != y.key ? x.key < y.key : x.seq < y.seq;
-            });
-        }
+        std::vector<std::vector<std::array<int, 2>>> tidx(G);   // (environment block, s_in) -> T block
+        std::vector<int64_t> T_size(G, 0), T_base(G, 0);
         // ---- stage 1: T = E X_b (templates once per group) ----
         int64_t tot_T = 0;
-        std::vector<int64_t> T_base(G, 0);
         for (int g = 0; g < G; ++g) {
+            const Mps* b = probs[rep[g]].b;
+            const Layout& B = b->lay;
+            const std::vector<int> blook = block_lookup(B, t);
+            tidx[g].assign(E[g].size(), {-1, -1});
+            const int gp = group_phase(g);
+            for (int e = 0; e < (int)E[g].size(); ++e)
+                for (int si = 0; si < 2; ++si) {
+                    const EBlk& eb = E[g][e];
+                    const int bb = blook[eb.ib * 2 + si];
+                    if (bb < 0) continue;
+                    const Block& bk = B.blocks[t][bb];
+                    tidx[g][e][si] = (int)T[g].size();
+                    T[g].push_back({e, eb.rows, bk.cols, bb, T_size[g]});
+                    const int o = (int)outs.size(), r = (int)runs.size();
+                    outs.push_back({eb.rows, bk.cols, r, r + 1, gp, 0, T_size[g]});
+                    runs.push_back({b->core[t] + bk.off, eb.off, eid, eb.cols, 0, 1, t});
+                    T_size[g] += (int64_t)eb.rows * bk.cols;
+                    add_tiles(o, (int)members[g].size());
+                }
             T_base[g] = tot_T;
             tot_T += (int64_t)members[g].size() * T_size[g];
-            const int gp = group_phase(g);
             gph[gp].base[0] = T_base[g];
             gph[gp].stride[0] = T_size[g];
             if (eid != 3) {
                 gph[gp].base[eid] = E_base[g];
                 gph[gp].stride[eid] = E_size[g];
             }
-            const Mps* b = probs[rep[g]].b;
-            for (const TBlk& tb : T[g]) {
-                const EBlk& eb = E[g][tb.env];
-                const Block& bk = b->lay.blocks[t][tb.bb];
-                const int o = (int)outs.size();
-                outs.push_back({tb.rows, tb.cols, tb.cols, (int)ins.size(), (int)ins.size() + 1, gp, 0, tb.off});
-                ins.push_back({nullptr, b->core[t] + bk.off, eb.off, 0, eid, -1, eb.cols, eb.cols, bk.cols, 0, 1.0,
-                               0, -1, -1, t});
-                add_tiles(o, (int)members[g].size());
-            }
         }
         maxT = std::max(maxT, tot_T);
         phase_beg.push_back((int)tiles.size());
-        // ---- stage 2: E'(d, ra, rb) = sum alpha X_a^T T ----
+        // ---- stage 2: E'(d, ra, rb) = sum over blocks of a of X_a^T (sum of alpha T) ----
         std::vector<std::vector<EBlk>> En(G);
         std::vector<int64_t> En_size(G, 0), En_base(G, 0);
         int64_t tot_E = 0;
@@ -1595,45 +1570,59 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
             const Layout& B = probs[rep[g]].b->lay;
             const Mpo& W = *ops[g];
             const bool real_op = probs[rep[g]].W != nullptr;
-            const std::vector<Contrib>& cs = contrib[g];
-            // blocks of E' first (their sizes fix the member stride)
-            for (size_t i = 0; i < cs.size();) {
-                size_t j = i;
-                while (j < cs.size() && cs[j].key == cs[i].key) ++j;
-                const int d = (int)(cs[i].key >> 42), ra = (int)((cs[i].key >> 21) & 0x1fffff),
-                          rb = (int)(cs[i].key & 0x1fffff);
-                const int rows = A.bonds[t + 1].dim[ra], cols = B.bonds[t + 1].dim[rb];
-                En[g].push_back({d, ra, rb, rows, cols, En_size[g]});
-                En_size[g] += (int64_t)rows * cols;
-                i = j;
+            const std::vector<int> alook = block_lookup(A, t);
+            const int nch = W.bond_dim(t), nd = W.bond_dim(t + 1), n_ent = (int)W.entries[t].size();
+            std::vector<std::vector<int>> by_chan(nch), by_d(nd);   // environment blocks / entries of a channel
+            for (int e = 0; e < (int)E[g].size(); ++e) by_chan[E[g][e].c].push_back(e);
+            for (int ei = 0; ei < n_ent; ++ei) {
+                const MpoEntry& me = W.entries[t][ei];
+                if (me.a < nch && me.b < nd && !by_chan[me.a].empty()) by_d[me.b].push_back(ei);
+            }
+            const int gp = group_phase(g);
+            for (int d = 0; d < nd; ++d) {
+                cs.clear();
+                for (const int ei : by_d[d]) {
+                    const MpoEntry& me = W.entries[t][ei];
+                    for (const int e : by_chan[me.a]) {
+                        const int ab = alook[E[g][e].ia * 2 + me.so], ti = tidx[g][e][me.si];
+                        if (ab < 0 || ti < 0) continue;
+                        const uint64_t ra = (uint64_t)A.blocks[t][ab].ri, rb = (uint64_t)B.blocks[t][T[g][ti].bb].ri;
+                        cs.push_back({(ra << 42) | (rb << 21) | (uint64_t)ab, ti, ei});
+                    }
+                }
+                std::stable_sort(cs.begin(), cs.end(),
+                                 [](const Contrib& x, const Contrib& y) { return x.key < y.key; });
+                for (size_t i = 0; i < cs.size();) {
+                    const int ra = (int)(cs[i].key >> 42), rb = (int)((cs[i].key >> 21) & 0x1fffff);
+                    const uint64_t block = cs[i].key >> 21;
+                    const int rows = A.bonds[t + 1].dim[ra], cols = B.bonds[t + 1].dim[rb];
+                    const int o = (int)outs.size();
+                    outs.push_back({rows, cols, (int)runs.size(), 0, gp, nid, En_size[g]});
+                    En[g].push_back({d, ra, rb, rows, cols, En_size[g]});
+                    En_size[g] += (int64_t)rows * cols;
+                    while (i < cs.size() && (cs[i].key >> 21) == block) {
+                        const uint64_t key = cs[i].key;
+                        const Block& abk = A.blocks[t][(int)(key & 0x1fffff)];
+                        const int cbeg = (int)cons.size();
+                        for (; i < cs.size() && cs[i].key == key; ++i) {
+                            const int ei = cs[i].ei;
+                            const MpoEntry& me = W.entries[t][ei];
+                            const int sf =
+                                real_op && t == 0 && (ei == W.shift_entry[0] || ei == W.shift_entry[1]) ? 4 : 0;
+                            cons.push_back({T[g][cs[i].ti].off, me.w, me.so | (me.si << 1) | sf, 0});
+                        }
+                        runs.push_back({a_->core[t] + abk.off, 0, -1, abk.rows, cbeg, (int)cons.size(), t});
+                    }
+                    outs[o].end = (int)runs.size();
+                    add_tiles(o, (int)members[g].size());
+                }
             }
             En_base[g] = tot_E;
             tot_E += (int64_t)members[g].size() * En_size[g];
-            const int gp = group_phase(g);
             gph[gp].base[0] = T_base[g];
             gph[gp].stride[0] = T_size[g];
             gph[gp].base[nid] = En_base[g];
             gph[gp].stride[nid] = En_size[g];
-            size_t q = 0;
-            for (size_t i = 0; i < cs.size(); ++q) {
-                size_t j = i;
-                while (j < cs.size() && cs[j].key == cs[i].key) ++j;
-                const EBlk& nb = En[g][q];
-                const int o = (int)outs.size();
-                outs.push_back({nb.rows, nb.cols, nb.cols, (int)ins.size(), 0, gp, nid, nb.off});
-                for (size_t u = i; u < j; ++u) {
-                    const Contrib& c = cs[u];
-                    const MpoEntry& me = W.entries[t][c.ei];
-                    const int sf = real_op && t == 0 && (c.ei == W.shift_entry[0] || c.ei == W.shift_entry[1]);
-                    const TBlk& tb = T[g][c.ti];
-                    const Block& abk = A.blocks[t][c.ab];
-                    ins.push_back({a_->core[t] + abk.off, nullptr, 0, tb.off, -1, 0, abk.rows, abk.cols, tb.cols, 1,
-                                   me.w, sf, c.so, c.si, t});
-                }
-                outs[o].end = (int)ins.size();
-                add_tiles(o, (int)members[g].size());
-                i = j;
-            }
         }
         maxE = std::max(maxE, tot_E);
         phase_beg.push_back((int)tiles.size());
@@ -1668,7 +1657,7 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
             finals.push_back(base[fid] + E_base[g] + (int64_t)member_index[p] * E_size[g] + eb.off);
         final_beg.push_back((int)finals.size());
     }
-    if (!launch_env_sweep_t(ctx, outs, ins, tiles, phase_beg, gph, mfac, ftab, K, base, finals, final_beg, res,
+    if (!launch_env_sweep_t(ctx, outs, runs, cons, tiles, phase_beg, gph, mfac, ftab, K, base, finals, final_beg, res,
                             gs)) {
         BSM_REQUIRE(!grams, BSMPS_ERR_RANK_CAP, "Gram matrices need the persistent environment sweep");
         return dot_batch_sitewise(ctx, probs);

@@ -5,17 +5,16 @@
 //
 // Row i of A is scaled by 2^-(e_i + 1) (e_i the smallest integer with
 // max_j |a_ij| < 2^e_i), column j of B by 2^-(f_j + 1); the scaled values, below
-// 1/2 in magnitude, are cut into S balanced digits of base 128 (integers in
-// [-64, 64], exact in bf16; what lies below the last digit is rounded, so that
-// the remainder is at most 2^(e_i - 7S)).  C = sum over slice pairs (p, q) with
-// p + q = d <= S + 1 of 2^{e_i + f_j + 2 - 7d} A_p B_q.  A slice product sums
-// integers up to 2^12; the pairs of one d (at most 8) over 128 values of k stay
-// within 2^22, so the FP32 accumulator of the tensor-core product (tcgen05.mma
-// kind::f16, BF16 operands, accumulators in tensor memory) is exact, the
-// diagonals are combined exactly in 64-bit integers, and the result is rounded
-// once.  (Balanced digits instead of seven bits and a sign: sums within 2^22 turn
-// into integers by one FP32 addition, where a conversion instruction takes 32
-// cycles per warp and scheduler and bound the kernel: 740 us at n = 2048 before.)
+// 1/2 in magnitude, are cut into S balanced digits of b bits (integers in
+// [-2^(b-1), 2^(b-1)], exact in bf16; what lies below the last digit is rounded, so
+// that the remainder is at most 2^(e_i - b S)).  C = sum over slice pairs (p, q) with
+// p + q = d <= S + 1 of 2^{e_i + f_j + 2 - b d} A_p B_q.  The slice products of one d
+// over 128 values of k are integers below 2^24, so the FP32 accumulator of the
+// tensor-core product (tcgen05.mma kind::f16, BF16 operands, accumulators in
+// tensor memory) is exact, the diagonals are combined exactly in 64-bit integers,
+// and the result is rounded once.  b = 7, except that the full 56 bits (8 slices asked
+// for) are cut into 7 digits of 8 bits: the same remainders and the same size of
+// the first dropped pairs, with 28 products instead of 36.
 #include <algorithm>
 
 #include "kernels.h"
@@ -38,6 +37,7 @@ constexpr int kOzSbo = 8 * kOzKStep * 2;              // bytes between 8-row gro
 constexpr int kOzSliceA = kOzM * kOzKStep * 2;        // bytes of one A slice tile (128 x 32 bf16)
 constexpr int kOzSliceB = kOzN * kOzKStep * 2;        // bytes of one B slice tile (64 x 32 bf16)
 constexpr int kOzGroup = 128 / kOzKStep;              // chunks whose FP32 sums of slice products stay exact
+constexpr int kOzWays = 4;                            // diagonals whose products alternate
 constexpr int kOzEpiWarps = 8;
 constexpr int kOzThreads = 32 * (2 + kOzEpiWarps);    // producer warp, MMA warp, epilogue warps
 constexpr uint32_t kOzIdesc = tc::idesc_bf16(kOzM, kOzN);
@@ -56,13 +56,13 @@ struct OzSide : ScanSide {
 
 // Exponents and slices.  e = the smallest integer with max |x| < 2^e; x 2^-(e+1)
 // is a 56-bit signed fraction X (rounded to nearest where the 53 bits of x reach
-// below it), for S < 8 rounded to 7 S bits, whose balanced base-128 digits are the
-// slices: integer operations only (an FP64 digit costs four FP64 instructions,
-// 0.4 ms at n = 2048 on this GPU).  A warp writes 8 rows x 32 k values: lane
+// below it), rounded to b S bits, whose balanced digits are the slices: integer
+// operations only (an FP64 digit costs four FP64 instructions, 0.4 ms at n = 2048
+// on this GPU).  A warp writes 8 rows x 32 k values: lane
 // (kg, r) the eight values k = 8 kg .. 8 kg + 7 of row r as one 16-byte store per
 // slice, 512 contiguous bytes per warp.  Eight warps of a CTA cover eight chunks of
 // k (rows contiguous in k) or eight row groups (rows contiguous across).
-__global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sides, int n_sides, int S,
+__global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sides, int n_sides, int S, int bits,
                                                   const unsigned long long* __restrict__ mx, int* __restrict__ exps,
                                                   unsigned char* __restrict__ buf) {
     int f = 0;   // the last factor whose CTAs start at or before this one
@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sid
     if (top != 0ull) frexp(__longlong_as_double((long long)top), &e);   // max = m 2^e, 0.5 <= m < 1
     if (on && kc == 0 && kg == 0) exps[sd.row0 + r] = e;
     long long X[8];
+    const int drop = 56 - bits * S, half = 1 << (bits - 1);
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
         const int k = kOzKStep * kc + 8 * kg + t;
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sid
             unsigned long long f = 0ull;
             if (sh >= 0) f = m << min(sh, 63);   // (beyond 2 for subnormal x only)
             else if (sh > -55) f = (m + (1ull << (-sh - 1))) >> -sh;
-            if (S < kOzMaxS) f = (f + (1ull << (7 * (kOzMaxS - S) - 1))) >> (7 * (kOzMaxS - S));
+            if (drop > 0) f = (f + (1ull << (drop - 1))) >> drop;
             X[t] = (b >> 63) ? -(long long)f : (long long)f;
         }
     }
@@ -115,9 +116,9 @@ __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sid
         uint32_t w[4];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            // the lowest digit, in [-64, 63] (the first one takes what is left, at most 64)
-            const int d = p ? (((int)X[t] + 64) & 127) - 64 : (int)X[t];
-            X[t] = (X[t] - d) >> 7;
+            // the lowest digit, in [-half, half) (the first one takes what is left, at most half)
+            const int d = p ? (((int)X[t] + half) & (2 * half - 1)) - half : (int)X[t];
+            X[t] = (X[t] - d) >> bits;
             // d as a float (1.5 2^23 + d - 1.5 2^23), whose upper half is the BF16 value
             const uint32_t h =
                 __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)d) - 12582912.0f) >> 16;
@@ -170,9 +171,9 @@ __device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, 
     return __longlong_as_double((long long)(b | (neg ? 1ull << 63 : 0ull)));
 }
 
-// C (M x N, row-major, ldc) = alpha sum_d 2^{e_i + f_j + 2 - 7(d + 2)} sum_{p + q = d + 2} A_p B_q
+// C (M x N, row-major, ldc) = alpha sum_d 2^{e_i + f_j + 2 - b(d + 2)} sum_{p + q = d + 2} A_p B_q
 // (slices numbered from 1).  A persistent CTA per SM takes 128 x 64 output tiles:
-//  - one thread copies chunks of 32 k values of every slice (96 KB at S = 8: two
+//  - one thread copies chunks of 32 k values of every slice (84 KB at S = 7: two
 //    contiguous pieces, cp.async.bulk) into a ring of stages;
 //  - one thread issues a tcgen05.mma.kind::f16 (BF16 operands, FP32 accumulation)
 //    per slice pair (p, q), p + q <= S + 1, and 16 values of k, into the
@@ -181,7 +182,7 @@ __device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, 
 //  - every 128 values of k (where the FP32 sums of integer slice products are
 //    still exact) eight warps read a diagonal as soon as its last product is done
 //    and add it, shifted to its weight, to two exact 64-bit integers per entry in
-//    registers (four diagonals each, below 2^44 per 128 values of k), and the next
+//    registers (below 2^46 per 128 values of k), and the next
 //    products of that diagonal may restart it: the tensor cores wait only for the
 //    first of the eight reads;
 //  - at the end of a tile the two integers are combined and rounded once.
@@ -196,13 +197,26 @@ constexpr int oz_stages() {
     return S * (kOzSliceA + kOzSliceB) * 4 <= 200 * 1024 ? 4 : 2;
 }
 
-template <int S>
+// An integer below 2^24 in a float (b = 7: within 2^22) as an int: by FP32 additions, whose
+// sums with 1.5 2^23 hold it in their last bits (a conversion instruction takes 32 cycles per
+// warp and scheduler here).
+template <int B>
+__device__ __forceinline__ int oz_int(float v) {
+    constexpr float kMagic = 12582912.0f;
+    if (B == 7) return (int)__float_as_uint(v + kMagic) - 0x4B400000;
+    const float h = fmaf(v, 0.25f, kMagic);                   // v / 4, rounded
+    const float l = fmaf(h - kMagic, -4.0f, v) + kMagic;      // the rest, within 2
+    return ((int)__float_as_uint(h) - 0x4B400000) * 4 + ((int)__float_as_uint(l) - 0x4B400000);
+}
+
+template <int S, int B>
 __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restrict__ prods,
                                                            const OzTile* __restrict__ tiles, int n_tiles,
                                                            const unsigned char* __restrict__ slices,
                                                            const int* __restrict__ exps, int* err) {
     constexpr uint32_t kCols = S * kOzN <= 64 ? 64 : S * kOzN <= 128 ? 128 : S * kOzN <= 256 ? 256 : 512;
     constexpr int kStages = oz_stages<S>();
+    constexpr int kTop = B == 7 ? 7 : 6;   // last diagonal of the second integer
     constexpr uint32_t kBytesA = S * kOzSliceA, kBytesB = S * kOzSliceB, kStage = kBytesA + kBytesB;
     extern __shared__ __align__(1024) unsigned char oz_smem[];
     __shared__ __align__(8) uint64_t bars[2 * kStages + 2 * S + 1];
@@ -268,24 +282,31 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                     tc::fence_after();
                     const uint64_t da = tc::desc_sw64(base + s * kStage);
                     const uint64_t db = tc::desc_sw64(base + s * kStage + kBytesA);
+                    // consecutive MMAs go to kOzWays accumulators in turn: one accumulator takes a new
+                    // product of 64 columns only every 75 cycles, the tensor cores one every 32
 #pragma unroll
-                    for (int d = S - 1; d >= 0; --d) {
+                    for (int d1 = S - 1; d1 >= 0; d1 -= kOzWays) {
+                        const int d0 = d1 - kOzWays + 1 > 0 ? d1 - kOzWays + 1 : 0;
                         if (first && g > 0) {
-                            if (!tc::mbar_wait(dempty(d), (g - 1) & 1)) {
-                                ok = false;
-                                break;
-                            }
+#pragma unroll
+                            for (int d = d1; d >= d0; --d) ok = ok && tc::mbar_wait(dempty(d), (g - 1) & 1);
+                            if (!ok) break;
                             tc::fence_after();
                         }
 #pragma unroll
-                        for (int p = 0; p <= d; ++p)
+                        for (int p = 0; p <= d1; ++p)
 #pragma unroll
                             for (int kk = 0; kk < kOzKStep / 16; ++kk)
-                                tc::mma_bf16(tmem + (uint32_t)(d * kOzN), da + ((p * kOzSliceA + kk * 32) >> 4),
-                                             db + (((d - p) * kOzSliceB + kk * 32) >> 4), kOzIdesc,
-                                             first && p == 0 && kk == 0 ? 0u : 1u);
+#pragma unroll
+                                for (int d = d1; d >= d0; --d)
+                                    if (p <= d)
+                                        tc::mma_bf16(tmem + (uint32_t)(d * kOzN),
+                                                     da + ((p * kOzSliceA + kk * 32) >> 4),
+                                                     db + (((d - p) * kOzSliceB + kk * 32) >> 4), kOzIdesc,
+                                                     first && p == 0 && kk == 0 ? 0u : 1u);
                         if (last)
-                            tc::commit(dfull(d));
+#pragma unroll
+                            for (int d = d1; d >= d0; --d) tc::commit(dfull(d));
                     }
                     tc::commit(empty(s));
                     if (last) ++g;
@@ -327,29 +348,29 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                         }
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            // an integer within 2^22: its bits in the sum with 1.5 2^23, less 0x4B400000
-                            const int x = (int)__float_as_uint(__uint_as_float(v[j]) + 12582912.0f) - 0x4B400000;
+                            const long long x = oz_int<B>(__uint_as_float(v[j]));
                             if (d < 4)
-                                i0[16 * h + j] += (long long)x * (1 << (7 * (3 - d)));
+                                i0[16 * h + j] += x * (1 << (B * (3 - d)));
                             else
-                                i1[16 * h + j] += (long long)x * (1 << (7 * (7 - d)));
+                                i1[16 * h + j] += x * (1 << (B * (kTop - d)));
                         }
                     }
                 }
             }
             if (!ok) break;
-            // diagonal d carries 2^(2 - 7(d + 2)): C = (i0 2^28 + i1) 2^(e + f - 61)
+            // diagonal d carries 2^(2 - B(d + 2)): C = (i0 2^(B (kTop - 3)) + i1) 2^(e + f + 2 - B (kTop + 2))
+            constexpr int kUp = B * (kTop - 3);
             const int row = tl.m0 + quad * 32 + lane, c0 = tl.n0 + half * 32;
             if (row < pd.M) {
-                const int e = exps[pd.e_off + row] - 61;
+                const int e = exps[pd.e_off + row] + 2 - B * (kTop + 2);
                 const int* f = exps + pd.f_off;
                 double* out = pd.C + (int64_t)row * pd.ldc;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     if (c0 + j < pd.N) {
-                        const unsigned long long l0 = (unsigned long long)i0[j] << 28;
+                        const unsigned long long l0 = (unsigned long long)i0[j] << kUp;
                         const unsigned long long lo = l0 + (unsigned long long)i1[j];
-                        const long long hi = (i0[j] >> 36) + (i1[j] >> 63) + (lo < l0 ? 1 : 0);
+                        const long long hi = (i0[j] >> (64 - kUp)) + (i1[j] >> 63) + (lo < l0 ? 1 : 0);
                         const double v = oz_round(hi, lo, e + f[c0 + j]);
                         out[c0 + j] = pd.alpha == 1.0 ? v : pd.alpha * v;
                     }
@@ -363,25 +384,26 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
     if (warp == 1) tc::tmem_free(tmem, kCols);
 }
 
-template <int S>
+template <int S, int B = 7>
 void launch_oz_gemm(Context* ctx, int n_tiles, const OzProd* prods, const OzTile* tiles, const unsigned char* slices,
                     const int* exps) {
     const size_t smem = (size_t)oz_stages<S>() * S * (kOzSliceA + kOzSliceB) + 1024;
     static bool attr = false;
     if (!attr) {
-        BSM_CUDA(cudaFuncSetAttribute(k_oz_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BSM_CUDA(cudaFuncSetAttribute(k_oz_gemm<S, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = true;
     }
     int nsm = 0;
     BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-    k_oz_gemm<S><<<std::min(n_tiles, nsm), kOzThreads, smem, ctx->stream>>>(prods, tiles, n_tiles, slices, exps,
+    k_oz_gemm<S, B><<<std::min(n_tiles, nsm), kOzThreads, smem, ctx->stream>>>(prods, tiles, n_tiles, slices, exps,
                                                                             ctx->err_word());
 }
 
 }  // namespace
 
-void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S) {
-    BSM_REQUIRE(S >= 1 && S <= kOzMaxS, BSMPS_ERR_INVALID_ARG, "emulated GEMM: 1 <= slices <= 8");
+void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int slices_asked) {
+    BSM_REQUIRE(slices_asked >= 1 && slices_asked <= kOzMaxS, BSMPS_ERR_INVALID_ARG, "emulated GEMM: 1 <= slices <= 8");
+    const int bits = slices_asked == kOzMaxS ? 8 : 7, S = slices_asked == kOzMaxS ? 7 : slices_asked;
     std::vector<OzProd> prods;
     std::vector<OzSide> sides;
     std::vector<OzTile> tiles;
@@ -400,7 +422,7 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S)
     };
     for (const OzGemm& g : gs) {
         BSM_REQUIRE(g.M >= 0 && g.N >= 0 && g.K >= 0, BSMPS_ERR_INVALID_ARG, "emulated GEMM: sizes >= 0");
-        // the exact 64-bit sums of the diagonals (below 2^44 per 128 values of k) stay below 2^63
+        // the exact 64-bit sums of the diagonals (below 2^46 per 128 values of k) stay below 2^63
         BSM_REQUIRE(g.K < (1 << 24), BSMPS_ERR_INVALID_ARG, "emulated GEMM: K < 2^24");
         if (g.M == 0 || g.N == 0) continue;
         const int nkc = (g.K + kOzKStep - 1) / kOzKStep;
@@ -427,13 +449,13 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S)
     k_row_max<OzSide><<<max_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), mx);
     launched(ctx);
     if (cut_ctas > 0) {
-        k_oz_slice<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), S, mx, exps, slices);
+        k_oz_slice<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, (int)sides.size(), S, bits, mx, exps, slices);
         launched(ctx);
     } else {
         BSM_CUDA(cudaMemsetAsync(exps, 0, sizeof(int) * (size_t)rows, ctx->stream));   // K = 0: C = 0
     }
     const int nt = (int)tiles.size();
-    switch (S) {
+    switch (slices_asked) {
         case 1: launch_oz_gemm<1>(ctx, nt, d_prods, d_tiles, slices, exps); break;
         case 2: launch_oz_gemm<2>(ctx, nt, d_prods, d_tiles, slices, exps); break;
         case 3: launch_oz_gemm<3>(ctx, nt, d_prods, d_tiles, slices, exps); break;
@@ -441,7 +463,7 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int S)
         case 5: launch_oz_gemm<5>(ctx, nt, d_prods, d_tiles, slices, exps); break;
         case 6: launch_oz_gemm<6>(ctx, nt, d_prods, d_tiles, slices, exps); break;
         case 7: launch_oz_gemm<7>(ctx, nt, d_prods, d_tiles, slices, exps); break;
-        default: launch_oz_gemm<8>(ctx, nt, d_prods, d_tiles, slices, exps); break;
+        default: launch_oz_gemm<7, 8>(ctx, nt, d_prods, d_tiles, slices, exps); break;
     }
     launched(ctx);
     ctx->flops += fl;

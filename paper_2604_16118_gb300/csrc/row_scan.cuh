@@ -17,14 +17,14 @@ struct ScanSide {
     int max0;   // first CTA of this factor
 };
 
-constexpr int kScanK = 512;
+constexpr int kScanK = 128;
 inline int scan_ctas(int64_t ks, int n, int K) {
     return ks == 1 ? (n + 7) / 8 : ((n + 31) / 32) * std::max(1, (K + kScanK - 1) / kScanK);
 }
 
 // mx[row0 + r] = the largest |x| of row r as a bit pattern (those of non-negative
 // doubles are ordered like their values; mx zeroed before).  Rows contiguous in
-// k: one warp per row, eight rows per CTA.  Rows contiguous across: 32 rows x 512
+// k: one warp per row, eight rows per CTA.  Rows contiguous across: 32 rows x 128
 // values per CTA, whole 256-byte lines per load.  Side: ScanSide or derived from it.
 template <class Side>
 __global__ void __launch_bounds__(256) k_row_max(const Side* __restrict__ sides, int n_sides,
@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(256) k_row_max(const Side* __restrict__ sides,
     if (sd.ks == 1) {
         const int r = 8 * u + warp;
         if (r >= sd.n) return;
+#pragma unroll 8
         for (int k = lane; k < sd.K; k += 32) m = max(m, src[(int64_t)r * sd.rs + k] & kAbs);
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) mx[sd.row0 + r] = m;
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(256) k_row_max(const Side* __restrict__ sides,
     const int nb = (sd.n + 31) / 32;
     const int r = 32 * (u % nb) + lane, k0 = (u / nb) * kScanK;
     if (r < sd.n)
+#pragma unroll 8
         for (int k = k0 + warp; k < min(sd.K, k0 + kScanK); k += 8) m = max(m, src[r * sd.rs + k * sd.ks] & kAbs);
     part[warp][lane] = m;
     __syncthreads();

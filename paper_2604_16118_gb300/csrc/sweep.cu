@@ -661,9 +661,8 @@ struct Pack {
 };
 
 unsigned char* upload_pack(Scratch& s, const Pack& p) {
-    std::vector<unsigned char> h = p.host;
-    if (h.empty()) h.push_back(0);
-    return s.up(h);
+    if (p.host.empty()) return s.up(std::vector<unsigned char>(1, 0));
+    return s.up(p.host);
 }
 
 // Warps per CTA: one per Jacobi pair of the largest problem, between 1 and 8.
@@ -716,12 +715,6 @@ struct Prof {
 };
 
 
-// Environment sweep: every phase is a set of independent output tiles of
-// grouped GEMMs whose inputs may have been written in earlier phases (loads go
-// through L2); one thread per output entry, the K loop reading A and B
-// directly so that no FP64 instruction is spent on padding.
-constexpr int kEnvThreads = 128;
-
 // One phase boundary between two CTAs; CTA skip_cta returns without arriving.
 __global__ void k_grid_wait_check(int skip_cta, GridSync* gs) {
     __shared__ int s_flag;
@@ -729,8 +722,20 @@ __global__ void k_grid_wait_check(int skip_cta, GridSync* gs) {
     phase_end(gs, 0u, &s_flag);
 }
 
+// Environment sweep: every phase is a set of independent 32 x 32 output tiles whose
+// inputs may have been written in earlier phases (loads go through L2).  A CTA
+// stages 32 values of k of both factors in shared memory; the right factor of an
+// environment update is summed over its contributions while it is staged, their
+// weights resolved once per contribution by one thread each.  Bound, at small
+// blocks, by the round trips of a phase and the grid-wide wait between phases
+// (kEnvPerSm CTAs per SM: more make the wait longer than the tiles shorter).
+constexpr int kEnvThreads = 256;
+constexpr int kEnvCons = 64;    // contributions resolved at a time
+constexpr int kEnvPerSm = 4;
+
 __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __restrict__ outs,
-                                                             const EnvInT* __restrict__ ins,
+                                                             const EnvRunT* __restrict__ runs,
+                                                             const EnvConT* __restrict__ cons,
                                                              const EnvTileT* __restrict__ tiles,
                                                              const int* __restrict__ phase_beg, int n_phase,
                                                              const EnvGroupPhase* __restrict__ gph,
@@ -742,7 +747,12 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __re
                                                              const int* __restrict__ final_beg, int n_prob,
                                                              double* __restrict__ res, GridSync* gs) {
     __shared__ int s_flag;
+    __shared__ double As[32][33];   // [k][m]
+    __shared__ double Bs[32][33];   // [k][n]
+    __shared__ const double* s_ptr[kEnvCons];
+    __shared__ double s_w[kEnvCons];
     const double* bases[4] = {b0, b1, b2, b3};
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int p = 0; p < n_phase; ++p) {
         for (int ti = phase_beg[p] + (int)blockIdx.x; ti < phase_beg[p + 1]; ti += (int)gridDim.x) {
             const EnvTileT tl = tiles[ti];
@@ -750,31 +760,69 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __re
             const EnvGroupPhase g = gph[o.gp];
             const EnvMemberFac mf = mfac[g.mem_beg + tl.member];
             const int64_t mem = tl.member;
-            double* C = const_cast<double*>(bases[o.cbuf]) + g.base[o.cbuf] + mem * g.stride[o.cbuf] + o.coff;
-            const int tm = min(32, o.M - tl.m0), tn = min(32, o.N - tl.n0);
-            for (int e = threadIdx.x; e < tm * tn; e += kEnvThreads) {
-                const int m = tl.m0 + e / tn, n = tl.n0 + e % tn;
-                double acc = 0.0;
-                for (int c = o.beg; c < o.end; ++c) {
-                    const EnvInT in = ins[c];
-                    const double* A = in.abuf < 0 ? in.A : bases[in.abuf] + g.base[in.abuf] + mem * g.stride[in.abuf] + in.aoff;
-                    const double* B = in.bbuf < 0 ? in.B : bases[in.bbuf] + g.base[in.bbuf] + mem * g.stride[in.bbuf] + in.boff;
-                    double alpha = in.w;
-                    if (in.so >= 0) {
-                        alpha += in.shift_flag ? g.shift : 0.0;
-                        const int ra = mf.row[in.so], rb = mf.row[2 + in.si];
-                        if (ra >= 0) alpha *= ftab[(int64_t)ra * K + in.site];
-                        if (rb >= 0) alpha *= ftab[(int64_t)rb * K + in.site];
+            const int gn = tl.n0 + tx;
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int r = o.beg; r < o.end; ++r) {
+                const EnvRunT run = runs[r];
+                const bool upd = (p & 1) != 0;
+                const double* E = upd ? nullptr : bases[run.abuf] + g.base[run.abuf] + mem * g.stride[run.abuf] + run.off;
+                const double* T = bases[0] + g.base[0] + mem * g.stride[0];
+                for (int cb = run.cbeg; cb < run.cend; cb += kEnvCons) {
+                    const int nc = min(kEnvCons, run.cend - cb);
+                    if (upd && (int)threadIdx.x < nc) {
+                        const EnvConT c = cons[cb + threadIdx.x];
+                        double w = c.w + ((c.fac & 4) ? g.shift : 0.0);
+                        const int ra = mf.row[c.fac & 1], rb = mf.row[2 + ((c.fac >> 1) & 1)];
+                        if (ra >= 0) w *= ftab[(int64_t)ra * K + run.site];
+                        if (rb >= 0) w *= ftab[(int64_t)rb * K + run.site];
+                        s_ptr[threadIdx.x] = T + c.off;
+                        s_w[threadIdx.x] = w;
                     }
-                    double part;
-                    if (in.transA)
-                        part = dev::dot_global<true, true>(A + m, in.lda, B + n, in.ldb, in.K, 0.0);
-                    else
-                        part = dev::dot_global<true, true>(A + (int64_t)m * in.lda, 1, B + n, in.ldb, in.K, 0.0);
-                    acc = fma(alpha, part, acc);
+                    if (upd) __syncthreads();
+                    for (int k0 = 0; k0 < run.K; k0 += 32) {
+                        const int kk_end = min(32, run.K - k0);
+                        if (upd) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int kk = ty + 8 * q, gm = tl.m0 + tx;
+                                if (kk < kk_end) {
+                                    As[kk][tx] = gm < o.M ? __ldcg(run.ptr + (int64_t)(k0 + kk) * o.M + gm) : 0.0;
+                                    double v = 0.0;
+                                    if (gn < o.N) {
+                                        const int64_t at = (int64_t)(k0 + kk) * o.N + gn;
+#pragma unroll 8
+                                        for (int c = 0; c < nc; ++c) v = fma(s_w[c], __ldcg(s_ptr[c] + at), v);
+                                    }
+                                    Bs[kk][tx] = v;
+                                }
+                            }
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int mm = ty + 8 * q, gm = tl.m0 + mm;
+                                if (gm < o.M && tx < kk_end) As[tx][mm] = __ldcg(E + (int64_t)gm * run.K + k0 + tx);
+                                if (mm < kk_end)
+                                    Bs[mm][tx] = gn < o.N ? __ldcg(run.ptr + (int64_t)(k0 + mm) * o.N + gn) : 0.0;
+                            }
+                        }
+                        __syncthreads();
+                        for (int kk = 0; kk < kk_end; ++kk) {
+                            const double b = Bs[kk][tx];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                if (tl.m0 + ty + 8 * q < o.M) acc[q] = fma(As[kk][ty + 8 * q], b, acc[q]);
+                        }
+                        __syncthreads();
+                    }
                 }
-                C[(int64_t)m * o.ldc + n] = acc;
             }
+            double* C = const_cast<double*>(bases[o.cbuf]) + g.base[o.cbuf] + mem * g.stride[o.cbuf] + o.coff;
+            if (gn < o.N)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int gm = tl.m0 + ty + 8 * q;
+                    if (gm < o.M) C[(int64_t)gm * o.N + gn] = acc[q];
+                }
         }
         if (!phase_end(gs, (unsigned)p, &s_flag)) return;
     }
@@ -1182,8 +1230,8 @@ int check_grid_wait(Context* ctx, int skip_cta) {
     return h.err;
 }
 
-bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvInT>& ins,
-                        const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
+bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
+                        const std::vector<EnvConT>& cons, const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
                         const std::vector<EnvGroupPhase>& gph, const std::vector<EnvMemberFac>& mfac,
                         const std::vector<double>& ftab, int K, double* const base[4],
                         const std::vector<const double*>& finals, const std::vector<int>& final_beg, double* res,
@@ -1197,22 +1245,27 @@ bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const st
     std::vector<int> tiles_of(outs.size(), 0);   // flops per output template times its members
     for (const EnvTileT& t : tiles)
         if (t.m0 == 0 && t.n0 == 0) tiles_of[t.out] += 1;
+    // flops of the operator's terms (one product per contribution), as the contraction counts them
     for (size_t o = 0; o < outs.size(); ++o)
-        for (int c = outs[o].beg; c < outs[o].end; ++c) {
-            fl += 2.0 * outs[o].M * outs[o].N * (double)ins[c].K * tiles_of[o];
-            by += 8.0 * ((double)outs[o].M * ins[c].K + (double)ins[c].K * outs[o].N) * tiles_of[o];
+        for (int r = outs[o].beg; r < outs[o].end; ++r) {
+            const double n = runs[r].cend - runs[r].cbeg, kk = runs[r].K;
+            fl += 2.0 * outs[o].M * outs[o].N * kk * n * tiles_of[o];
+            by += 8.0 * ((double)outs[o].M * kk + n * kk * outs[o].N) * tiles_of[o];
         }
+    int nsm = 0;
+    BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     const int cap = coresident_ctas(k_env_sweep_t, kEnvThreads, 0);
     if (cap <= 0) return false;
-    const int grid = std::min(maxt, cap);
+    const int grid = std::min({maxt, cap, kEnvPerSm * nsm});
     ctx->flops += fl;
     Pack pk;
-    const size_t oo = pk.add(outs), oi = pk.add(ins), ot = pk.add(tiles), op = pk.add(phase_beg), og = pk.add(gph),
+    const size_t oo = pk.add(outs), oi = pk.add(runs), oc = pk.add(cons), ot = pk.add(tiles), op = pk.add(phase_beg), og = pk.add(gph),
                  om = pk.add(mfac), of = pk.add(ftab), ofi = pk.add(finals), ob = pk.add(final_beg);
     Scratch s(ctx);
     unsigned char* d = upload_pack(s, pk);
     const EnvOutT* a0 = (const EnvOutT*)(d + oo);
-    const EnvInT* a1 = (const EnvInT*)(d + oi);
+    const EnvRunT* a1 = (const EnvRunT*)(d + oi);
+    const EnvConT* a1c = (const EnvConT*)(d + oc);
     const EnvTileT* a2 = (const EnvTileT*)(d + ot);
     const int* a3 = (const int*)(d + op);
     int a4 = n_phase;
@@ -1229,7 +1282,7 @@ bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const st
     int a15 = n_prob;
     double* a16 = res;
     GridSync* a17 = gs;
-    void* args[] = {&a0, &a1, &a2, &a3, &a4, &a5, &a6, &a7, &a8, &a9, &a10, &a11, &a12, &a13, &a14, &a15, &a16, &a17};
+    void* args[] = {&a0, &a1, &a1c, &a2, &a3, &a4, &a5, &a6, &a7, &a8, &a9, &a10, &a11, &a12, &a13, &a14, &a15, &a16, &a17};
     Prof pr(ctx, KK_GEMM, fl, by);
     BSM_CUDA(cudaLaunchCooperativeKernel((const void*)k_env_sweep_t, dim3(grid), dim3(kEnvThreads), args, 0,
                                          ctx->stream));

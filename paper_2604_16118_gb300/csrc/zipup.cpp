@@ -125,12 +125,15 @@ struct ZipJob {
         }
         T.assign(nb, nullptr);
         for (int i = 0; i < nb; ++i) T[i] = tsize > 0 ? (double*)ctx->alloc((size_t)tsize * sizeof(double)) : nullptr;
-        // the site's MPO entries by (s', b), in entry order
+        // the site's MPO entries by (s', b), those of one s together: for a given output they all read
+        // the same block of x, so that the grouped GEMM sums their carries before it multiplies
         std::vector<std::vector<int>> by_sob((size_t)2 * wr);
-        for (int ei = 0; ei < (int)W->entries[t].size(); ++ei) {
-            const MpoEntry& e = W->entries[t][ei];
-            if (e.so >= 0 && e.so < 2 && e.b >= 0 && e.b < wr) by_sob[(size_t)e.so * wr + e.b].push_back(ei);
-        }
+        for (int si = 0; si < 2; ++si)
+            for (int ei = 0; ei < (int)W->entries[t].size(); ++ei) {
+                const MpoEntry& e = W->entries[t][ei];
+                if (e.si == si && e.so >= 0 && e.so < 2 && e.b >= 0 && e.b < wr)
+                    by_sob[(size_t)e.so * wr + e.b].push_back(ei);
+            }
         for (const TB& tb : tbs) {
             const Charge m = yb.q[tb.mi], m2 = ex[t + 1].q[tb.em];
             const int ldc = ex[t + 1].dim[tb.em];
