@@ -530,111 +530,14 @@ __device__ __forceinline__ void jacobi_small(double* G, double* V, double* Sraw,
     __syncthreads();
 }
 
-// One-sided Jacobi directly on B (rows x k, column-major, rows <= 32, k <=
-// 16) with the rotations accumulated in V (k x k): no QR step.  One pair per
-// warp; the pair's inner products reduce in aligned segments of S =
-// pow2_at_least(rows) lanes.  Threshold |g| > tol sqrt(a b) with tol = rows
-// eps, columns below the numerical-zero level (rows eps)^2 ||B||_F^2 are left
-// alone.  Sraw: column norms of the result.
-__device__ __forceinline__ void jacobi_direct(double* B, double* V, double* Sraw, int rows, int k, double* red,
-                                              int* s_rot) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double f = 0.0;
-    for (int64_t e = threadIdx.x; e < (int64_t)rows * k; e += nthreads()) {
-        const double v = B[e];
-        f += v * v;
-    }
-    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += nthreads()) V[e] = (e % k) == (e / k) ? 1.0 : 0.0;
-    f = block_sum(f, red);
-    const double tol = (double)rows * DBL_EPSILON;
-    const double tol2 = tol * tol, tiny2 = tol2 * f;
-    const int n2 = k + (k & 1);
-    const int S = pow2_at_least(rows);
-    const int i = lane % S, sg = lane / S;
-    for (int sweep = 0; sweep < kMaxSweeps && k > 1; ++sweep) {
-        if (threadIdx.x == 0) *s_rot = 0;
-        __syncthreads();
-        for (int round = 0; round < n2 - 1; ++round) {
-            for (int pi = warp; pi < n2 / 2; pi += nwarps()) {
-                int p = rr_player(pi, round, n2), q = rr_player(n2 - 1 - pi, round, n2);
-                if (p >= k || q >= k) continue;
-                if (p > q) {
-                    const int tmp = p;
-                    p = q;
-                    q = tmp;
-                }
-                const double xp = i < rows ? B[(int64_t)p * rows + i] : 0.0;
-                const double xq = i < rows ? B[(int64_t)q * rows + i] : 0.0;
-                double a, b, g;
-                if (S <= 8) {
-                    const double u = sg == 1 ? xq : xp, w = sg == 0 ? xp : xq;
-                    const double prod = seg_sum(sg < 3 ? u * w : 0.0, S);
-                    a = __shfl_sync(0xffffffffu, prod, 0);
-                    b = __shfl_sync(0xffffffffu, prod, S);
-                    g = __shfl_sync(0xffffffffu, prod, 2 * S);
-                } else if (S == 16) {
-                    const double u = sg == 0 ? xp : xq;
-                    const double ab = seg_sum(u * u, 16);
-                    const double pg = seg_sum(xp * xq, 16);
-                    a = __shfl_sync(0xffffffffu, ab, 0);
-                    b = __shfl_sync(0xffffffffu, ab, 16);
-                    g = __shfl_sync(0xffffffffu, pg, 0);
-                } else {
-                    a = warp_sum(xp * xp);
-                    b = warp_sum(xq * xq);
-                    g = warp_sum(xp * xq);
-                }
-                if (g * g > tol2 * (a * b) && nonneg_key(a) > nonneg_key(tiny2) &&
-                    nonneg_key(b) > nonneg_key(tiny2)) {
-                    double c, s;
-                    jacobi_rotation_fast(a, b, g, &c, &s);
-                    if (S <= 16) {
-                        // lanes [0, S): rows of B; lanes [S, 2S): rows of V (k <= rows <= S)
-                        const bool onB = lane < S;
-                        if ((onB && i < rows) || (!onB && lane < 2 * S && i < k)) {
-                            double* X = onB ? B : V;
-                            const int ld = onB ? rows : k;
-                            const double vp = X[(int64_t)p * ld + i], vq = X[(int64_t)q * ld + i];
-                            X[(int64_t)p * ld + i] = c * vp - s * vq;
-                            X[(int64_t)q * ld + i] = s * vp + c * vq;
-                        }
-                    } else {
-                        if (lane < rows) {
-                            B[(int64_t)p * rows + lane] = c * xp - s * xq;
-                            B[(int64_t)q * rows + lane] = s * xp + c * xq;
-                        }
-                        if (lane < k) {
-                            const double vp = V[(int64_t)p * k + lane], vq = V[(int64_t)q * k + lane];
-                            V[(int64_t)p * k + lane] = c * vp - s * vq;
-                            V[(int64_t)q * k + lane] = s * vp + c * vq;
-                        }
-                    }
-                    if (lane == 0) *s_rot = 1;
-                }
-            }
-            __syncthreads();
-        }
-        const int rot = *s_rot;
-        __syncthreads();
-        if (!rot) break;
-    }
-    const int Gc = 32 / S;
-    for (int j0 = warp * Gc; j0 < k; j0 += nwarps() * Gc) {
-        const int j = j0 + sg;
-        const double x = (j < k && i < rows) ? B[(int64_t)j * rows + i] : 0.0;
-        const double a = seg_sum(x * x, S);
-        if (j < k && i == 0) Sraw[j] = sqrt_via_rsqrt(a);
-    }
-    __syncthreads();
-}
-
-// SVD factors from jacobi_direct (B V = U diag(Sraw), B = M for a tall M, B =
+// SVD factors from a Jacobi on B itself (B V = U diag(Sraw), B = M for a tall M, B =
 // M^T for a wide M): tall: US = columns of B, Vt = rows V^T; wide: US = V
 // diag(S), Vt = (B diag(1/S))^T.  Order, tie rule and sign rule as in
 // svd_assemble.  rinv: k scratch doubles, perm: k ints.
-__device__ __forceinline__ void svd_assemble_direct(const double* B, const double* V, const double* Sraw,
-                                                    double* rinv, int* perm, double* S, double* US, double* Vt,
-                                                    int M, int N, int k, int rows, int wide, int ldus, int ldvt) {
+__device__ __forceinline__ void svd_assemble_direct(const double* B, int ldb, const double* V, int ldv,
+                                                    const double* Sraw, double* rinv, int* perm, double* S,
+                                                    double* US, double* Vt, int M, int N, int k, int wide, int ldus,
+                                                    int ldvt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < k; i += nthreads()) {
         const double si = Sraw[i];
@@ -654,12 +557,12 @@ __device__ __forceinline__ void svd_assemble_direct(const double* B, const doubl
     for (int64_t e = threadIdx.x; e < (int64_t)M * k; e += nthreads()) {
         const int i = (int)(e / k), r = (int)(e % k);
         const int p = perm[r];
-        US[(int64_t)i * ldus + r] = wide ? V[(int64_t)p * k + i] * Sraw[p] : B[(int64_t)p * rows + i];
+        US[(int64_t)i * ldus + r] = wide ? V[(int64_t)p * ldv + i] * Sraw[p] : B[(int64_t)p * ldb + i];
     }
     for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += nthreads()) {
         const int r = (int)(e / N), c = (int)(e % N);
         const int p = perm[r];
-        Vt[(int64_t)r * ldvt + c] = wide ? B[(int64_t)p * rows + c] * rinv[p] : V[(int64_t)p * k + c];
+        Vt[(int64_t)r * ldvt + c] = wide ? B[(int64_t)p * ldb + c] * rinv[p] : V[(int64_t)p * ldv + c];
     }
     for (int r = threadIdx.x; r < k; r += nthreads()) S[r] = Sraw[perm[r]];
     __syncthreads();
@@ -694,12 +597,12 @@ __device__ __forceinline__ float seg8_sum(float v) {
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     return v;
 }
-// Leading dimension of G and V in jacobi_auto(): at 16 < k <= 64 columns are padded
-// with zero rows to an odd multiple of 8, so that the 8-lane segments of a warp,
-// which work on neighbouring columns, meet distinct banks (64-byte pieces of
+// Leading dimension of columns of n rows in jacobi_pre(): at n <= 64 columns are
+// padded with zero rows to an odd multiple of 8, so that the 8-lane segments of a
+// warp, which work on neighbouring columns, meet distinct banks (64-byte pieces of
 // columns 64 bytes apart modulo 128), and whole segments of rows need no bounds check.
-__host__ __device__ constexpr int jacobi_ld(int k) {
-    return k <= 16 || k > 64 ? k : k <= 24 ? 24 : k <= 40 ? 40 : k <= 56 ? 56 : 72;
+__host__ __device__ constexpr int jacobi_ld(int n) {
+    return n > 64 ? n : n <= 8 ? 8 : n <= 24 ? 24 : n <= 40 ? 40 : n <= 56 ? 56 : 72;
 }
 
 __device__ __forceinline__ float rsqrt_fast(float x) {
@@ -741,13 +644,13 @@ struct SegPair {
 // Barrier 1 among the first n threads of the CTA (a multiple of 32).
 __device__ __forceinline__ void bar_first(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
-// FP32 one-sided Jacobi of G (k x k, column-major, ||G||_F ~ 1, overwritten), the
-// rotations accumulated in V (identity on entry): one pair per 8-lane segment.
+// FP32 one-sided Jacobi of G (k columns of 8 RG rows, ||G||_F ~ 1, overwritten), the
+// rotations accumulated in V (k columns of 8 RV rows, identity on entry): one pair per 8-lane segment.
 // Bound by the latency of a round (loads, three shuffles, two reciprocal square
 // roots, stores, a barrier of the working warps).  Tolerance 4 sqrt(k) eps_32; a
 // sweep rotating at most 1/32 of the pairs ends.  Needs 4 warps per 32 columns.
-template <int R>
-__device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, int ld, int* s_cnt) {
+template <int RG, int RV>
+__device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, int ldg, int ldv, int* s_cnt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
     const int n2 = k + (k & 1);
     const int nact = (n2 / 2 + 3) / 4;
@@ -760,14 +663,14 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
             for (int round = 0; round < n2 - 1; ++round, pr.next()) {
                 int p, q;
                 const bool on = pr.get(&p, &q);
-                float* Gp = G + p * ld;
-                float* Gq = G + q * ld;
-                float* Vp = V + p * ld;
-                float* Vq = V + q * ld;
-                float xp[R], xq[R], vp[R], vq[R];
+                float* Gp = G + p * ldg;
+                float* Gq = G + q * ldg;
+                float* Vp = V + p * ldv;
+                float* Vq = V + q * ldv;
+                float xp[RG], xq[RG], vp[RV], vq[RV];
                 float a = 0.0f, b = 0.0f, g = 0.0f;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
+                for (int r = 0; r < RG; ++r) {
                     const int i = sl + 8 * r;
                     xp[r] = Gp[i];
                     xq[r] = Gq[i];
@@ -776,7 +679,7 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
                     g = fmaf(xp[r], xq[r], g);
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
+                for (int r = 0; r < RV; ++r) {
                     const int i = sl + 8 * r;
                     vp[r] = Vp[i];
                     vq[r] = Vq[i];
@@ -798,10 +701,14 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
                 const bool rot = on && fminf(a, b) > 1e-30f && fabsf(g) > tol * (a * rsqrt_fast(a)) * (b * rsqrt_fast(b));
                 if (rot) {
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
+                    for (int r = 0; r < RG; ++r) {
                         const int i = sl + 8 * r;
                         Gp[i] = c * xp[r] - sn * xq[r];
                         Gq[i] = sn * xp[r] + c * xq[r];
+                    }
+#pragma unroll
+                    for (int r = 0; r < RV; ++r) {
+                        const int i = sl + 8 * r;
                         Vp[i] = c * vp[r] - sn * vq[r];
                         Vq[i] = sn * vp[r] + c * vq[r];
                     }
@@ -827,7 +734,7 @@ struct SegRot {
     int pad;
 };
 
-// FP64 one-sided Jacobi of G (k x k, column-major, ||G||_F in [1/2, 1)) rotating
+// FP64 one-sided Jacobi of G (rows x k, column-major, ||G||_F in [1/2, 1)) rotating
 // the columns of V along: one pair per 8-lane segment, the columns' squared norms
 // tracked in nrm (recomputed every sweep), the tests and angles in FP32 (only the
 // inner product, the norms and the rotation itself need FP64).  A rotation by a
@@ -836,18 +743,18 @@ struct SegRot {
 // are gathered per column in del (column = (1 + del) x stored; alpha and beta
 // carry the ratio of the two scales, terms below 2^-57 dropped).  Larger angles
 // (and columns with |del| >= 2^-30) take the full rotation, which clears del.
-// Stopping rule: |g| > k eps sqrt(a b), min(a, b) > (k eps)^2 ||G||_F^2.
+// Stopping rule: |g| > rows eps sqrt(a b), min(a, b) > (rows eps)^2 ||G||_F^2.
 // The first nact warps work on G; the next nact rotate V one round behind them,
 // which fills the FP64 pipe while the G warps wait for loads, shuffles and
 // angles.  ring: 2 x 32 rotations.  Needs 2 nact warps.
-template <int R>
-__device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, int ld, double fro,
-                                                    SegRot* ring, int* s_rot) {
+template <int RG, int RV>
+__device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, int rows, int ldg,
+                                                    int ldv, double fro,SegRot* ring, int* s_rot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
     const int n2 = k + (k & 1);
     const int nact = (n2 / 2 + 3) / 4;
-    const float tol = (float)k * 2.220446e-16f * 0x1p48f;   // compared with g 2^48
-    const float tiny = (float)k * 2.220446e-16f * (float)k * 2.220446e-16f * to_float_scaled(fro, 0);
+    const float tol = (float)rows * 2.220446e-16f * 0x1p48f;   // compared with g 2^48
+    const float tiny = (float)rows * 2.220446e-16f * (float)rows * 2.220446e-16f * to_float_scaled(fro, 0);
     for (int j = threadIdx.x; j < k; j += nthreads()) del[j] = 0.0f;
     __syncthreads();
     for (int sweep = 0; sweep < kMaxSweeps && k > 1; ++sweep) {
@@ -856,9 +763,9 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
             const int j = jb + (lane >> 3);
             double a = 0.0;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
+            for (int r = 0; r < RG; ++r) {
                 const int i = sl + 8 * r;
-                const double x = j < k ? G[j * ld + i] : 0.0;
+                const double x = j < k ? G[j * ldg + i] : 0.0;
                 a = fma(x, x, a);
             }
             a = seg8_sum(a);
@@ -872,12 +779,12 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
             for (int round = 0; round < n2 - 1; ++round, pr.next()) {
                 int p, q;
                 const bool on = pr.get(&p, &q);
-                double* Gp = G + p * ld;
-                double* Gq = G + q * ld;
-                double xp[R], xq[R];
+                double* Gp = G + p * ldg;
+                double* Gq = G + q * ldg;
+                double xp[RG], xq[RG];
                 double g = 0.0;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
+                for (int r = 0; r < RG; ++r) {
                     const int i = sl + 8 * r;
                     xp[r] = Gp[i];
                     xq[r] = Gq[i];
@@ -917,7 +824,7 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                     }
                     if (rot) {
 #pragma unroll
-                        for (int r = 0; r < R; ++r) {
+                        for (int r = 0; r < RG; ++r) {
                             const int i = sl + 8 * r;
                             Gp[i] = fma(-sq, xq[r], fp * xp[r]);
                             Gq[i] = fma(sp, xp[r], fq * xq[r]);
@@ -925,7 +832,7 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                     }
                 } else if (rot) {
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
+                    for (int r = 0; r < RG; ++r) {
                         const int i = sl + 8 * r;
                         Gp[i] = fma(-sq, xq[r], xp[r]);
                         Gq[i] = fma(sp, xp[r], xq[r]);
@@ -959,11 +866,11 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                 if (!__any_sync(0xffffffffu, mode != 0)) continue;
                 if (mode) {
                     const double fp = in->fp, sq = in->sq, sp = in->sp, fq = in->fq;
-                    double* Vp = V + in->p * ld;
-                    double* Vq = V + in->q * ld;
+                    double* Vp = V + in->p * ldv;
+                    double* Vq = V + in->q * ldv;
                     if (mode == 1) {
 #pragma unroll
-                        for (int r = 0; r < R; ++r) {
+                        for (int r = 0; r < RV; ++r) {
                             const int i = sl + 8 * r;
                             const double vp = Vp[i], vq = Vq[i];
                             Vp[i] = fma(-sq, vq, vp);
@@ -971,7 +878,7 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                         }
                     } else {
 #pragma unroll
-                        for (int r = 0; r < R; ++r) {
+                        for (int r = 0; r < RV; ++r) {
                             const int i = sl + 8 * r;
                             const double vp = Vp[i], vq = Vq[i];
                             Vp[i] = fma(-sq, vq, fp * vp);
@@ -989,23 +896,26 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
     }
 }
 
-// One-sided Jacobi of G (k x k, column-major, 16 < k <= 64) as jacobi(): G ends as
-// U diag(Sraw), V accumulates the rotations.  The FP64 sweeps are few because an
+// One-sided Jacobi of G (rows x k, column-major, k <= rows <= 64) as jacobi(): G ends
+// as U diag(Sraw), V (k x k) accumulates the rotations.  The FP64 sweeps are few because an
 // FP32 Jacobi of G comes first (FP32 arithmetic runs at 64 times the FP64 rate
 // here): its rotations P, orthogonal to about 1e-6, are orthogonalised in FP64 as
 // Qp = P (I - E/2 + 3/8 E^2) with E = P^T P - I (a second pass when E is not below
 // 2e-6, since the dropped terms are of order E^3), and the FP64 Jacobi starts from
 // G Qp with V = Qp: two sweeps with rotations and one without.  Where the FP32
 // iteration gives nothing (non-finite entries) it starts from G and I.
-// G and V have leading dimension jacobi_ld(k), the rows from k on zero in G on entry.
-// scr: k jacobi_ld(k) shared doubles; del: k shared doubles.
-template <int R>
-__device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int k, double* scr, double* del,
-                                           SegRot* ring, double* red, int* s_int) {
-    constexpr int kOwn = 8;   // outputs of a k x k product per thread: k^2 <= 8 blockDim (64 k <= blockDim at k <= 64)
-    const int T = nthreads(), kk = k * k, ld = jacobi_ld(k), kl = k * ld;
+// RG, RV: rows of G and V in units of 8 (8 RG >= rows, 8 RV >= k).  Leading dimensions:
+// jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of
+// max(k, 8 RV - 7) for V, so that the 8 RG (8 RV) rows a lane segment walks stay
+// within the column.  scr: jacobi_scratch(ldg, ldv, k) shared doubles; del: k of them.
+template <int RG, int RV>
+__device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int rows, int k, double* scr,
+                                           double* del, SegRot* ring, double* red, int* s_int) {
+    constexpr int kOwn = 8;   // outputs of a product per thread: rows k <= 8 blockDim (blockDim >= min(16 k, 512))
+    const int T = nthreads(), kk = k * k;
+    const int ldg = jacobi_ld(max(rows, 8 * RG - 7)), ldv = jacobi_ld(max(k, 8 * RV - 7));   // >= 8 RG, 8 RV
     double f = 0.0;
-    for (int e = threadIdx.x; e < kl; e += T) f = fma(G[e], G[e], f);
+    for (int e = threadIdx.x; e < k * ldg; e += T) f = fma(G[e], G[e], f);
     f = block_sum(f, red);
     // exact scaling to ||G||_F in [1/2, 1)
     int ex = 0;
@@ -1013,17 +923,17 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     const double sc = ldexp(1.0, -ex);
     const double fro = f * sc * sc;
     float* Gf = (float*)scr;
-    float* Vf = Gf + kl;
-    for (int e = threadIdx.x; e < kl; e += T) {
+    float* Vf = Gf + k * ldg;
+    for (int e = threadIdx.x; e < k * ldg; e += T) {
         const double x = G[e] * sc;
         G[e] = x;
         Gf[e] = (float)x;
-        Vf[e] = e % ld == e / ld ? 1.0f : 0.0f;
     }
+    for (int e = threadIdx.x; e < k * ldv; e += T) Vf[e] = e % ldv == e / ldv ? 1.0f : 0.0f;
     __syncthreads();
-    jacobi_f32_segments<R>(Gf, Vf, k, ld, s_int);
+    jacobi_f32_segments<RG, RV>(Gf, Vf, k, ldg, ldv, s_int);
     // V row-major <- P
-    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ld + e % k]);
+    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
     bool ok = true;
     for (int pass = 0; pass < 3; ++pass) {
         __syncthreads();
@@ -1085,21 +995,22 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) V[last ? (e % k) * ld + e / k : e] = own[n];   // column-major at the end
+            if (e < kk) V[last ? (e % k) * ldv + e / k : e] = own[n];   // column-major at the end
         }
         if (last) break;
         ok = pass < 2;
     }
     __syncthreads();
     if (ok) {
+        // G <- G Qp (rows k <= 8 blockDim outputs)
         double own[kOwn];
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) {
-                const int i = e % k, c = e / k;
+            if (e < rows * k) {
+                const int i = e % rows, c = e / rows;
                 double acc = 0.0;
-                for (int j = 0; j < k; ++j) acc = fma(G[j * ld + i], V[c * ld + j], acc);
+                for (int j = 0; j < k; ++j) acc = fma(G[j * ldg + i], V[c * ldv + j], acc);
                 own[n] = acc;
             }
         }
@@ -1107,15 +1018,15 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) G[(e / k) * ld + e % k] = own[n];
+            if (e < rows * k) G[(e / rows) * ldg + e % rows] = own[n];
         }
     } else {
-        for (int e = threadIdx.x; e < kl; e += T) V[e] = e % ld == e / ld ? 1.0 : 0.0;
+        for (int e = threadIdx.x; e < k * ldv; e += T) V[e] = e % ldv == e / ldv ? 1.0 : 0.0;
     }
-    for (int e = threadIdx.x; e < k * (ld - k); e += T) V[(e / (ld - k)) * ld + k + e % (ld - k)] = 0.0;
+    for (int e = threadIdx.x; e < k * (ldv - k); e += T) V[(e / (ldv - k)) * ldv + k + e % (ldv - k)] = 0.0;
     __syncthreads();
     float* dl = (float*)del;
-    jacobi_f64_segments<R>(G, V, Sraw, dl, k, ld, fro, ring, s_int);
+    jacobi_f64_segments<RG, RV>(G, V, Sraw, dl, k, rows, ldg, ldv, fro, ring, s_int);
     // the columns' scales, and the norms of the result
     const double up = ldexp(1.0, ex);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
@@ -1124,12 +1035,12 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
         double a = 0.0;
         if (j < k) {
             const double s1 = 1.0 + to_double(dl[j]);
-            for (int i = sl; i < k; i += 8) {
-                const double x = G[j * ld + i] * s1;
+            for (int i = sl; i < rows; i += 8) {
+                const double x = G[j * ldg + i] * s1;
                 a = fma(x, x, a);
-                G[j * ld + i] = x * up;
-                V[j * ld + i] *= s1;
+                G[j * ldg + i] = x * up;
             }
+            for (int i = sl; i < k; i += 8) V[j * ldv + i] *= s1;
         }
         a = seg8_sum(a);
         if (j < k && sl == 0) Sraw[j] = sqrt_via_rsqrt(a) * up;
@@ -1137,26 +1048,33 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     __syncthreads();
 }
 
-// jacobi_pre() for 16 < k <= 64 (blockDim >= 16 k, as block_for() gives), else
-// jacobi().  G and V: leading dimension jacobi_ld(k).
+// Shared doubles of jacobi_pre()'s scratch: G and V in FP32, or a k x k FP64 matrix.
+__host__ __device__ constexpr int jacobi_scratch(int ldg, int ldv, int k) {
+    const int f = (k * (ldg + ldv) + 1) / 2;
+    return f > k * k ? f : k * k;
+}
+
+// jacobi_pre() on a square G of k <= 64 columns (blockDim as block_for() gives it),
+// else jacobi().  G and V: leading dimension jacobi_ld(k).
 __device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k, double* red, int* s_rot);
 __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
-                                            double* red, int* s_rot) {
-    __shared__ SegRot ring[64];
-    if (k > 16 && k <= 64) {
-        if (k <= 24)
-            jacobi_pre<3>(G, V, Sraw, k, scr, del, ring, red, s_rot);
-        else if (k <= 32)
-            jacobi_pre<4>(G, V, Sraw, k, scr, del, ring, red, s_rot);
-        else if (k <= 40)
-            jacobi_pre<5>(G, V, Sraw, k, scr, del, ring, red, s_rot);
-        else if (k <= 56)
-            jacobi_pre<7>(G, V, Sraw, k, scr, del, ring, red, s_rot);
-        else
-            jacobi_pre<8>(G, V, Sraw, k, scr, del, ring, red, s_rot);
-        return;
-    }
-    jacobi(G, V, Sraw, k, red, s_rot);
+                                            SegRot* ring, double* red, int* s_rot) {
+    if (k <= 8)
+        jacobi_pre<1, 1>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 16)
+        jacobi_pre<2, 2>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 24)
+        jacobi_pre<3, 3>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 32)
+        jacobi_pre<4, 4>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 40)
+        jacobi_pre<5, 5>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 56)
+        jacobi_pre<7, 7>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else if (k <= 64)
+        jacobi_pre<8, 8>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+    else
+        jacobi(G, V, Sraw, k, red, s_rot);
 }
 
 // One-sided (Hestenes) Jacobi on the columns of G (k x k, column-major) with the
@@ -1248,10 +1166,11 @@ __device__ __forceinline__ void svd_assemble(const double* G, int ldg, const dou
                                              int len, int wide, int ldus, int ldvt) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < k; i += nthreads()) {
-        const double si = Sraw[i];
+        // compared as integers: a permutation also when a value is not a number
+        const long long si = nonneg_key(Sraw[i]);
         int rank = 0;
         for (int j = 0; j < k; ++j) {
-            const double sj = Sraw[j];
+            const long long sj = nonneg_key(Sraw[j]);
             rank += (sj > si || (sj == si && j < i)) ? 1 : 0;
         }
         perm[rank] = i;

@@ -54,43 +54,45 @@ __device__ __forceinline__ bool same_b(const GemmIn& x, const GemmIn& y) {
     return x.B == y.B && x.K == y.K && x.ldb == y.ldb && !x.transA && !y.transA;
 }
 
-// One run in[0 .. n) of such contributions added to the tile's accumulators (thread mapping and
-// staging as dev::gemm_tile_accumulate; the sum is formed while A is staged).
-__device__ __forceinline__ void tile_accumulate_run(const GemmIn* in, int n, int M, int N, int m0, int n0,
-                                                    double (*As)[kTile + 1], double (*Bs)[kTile + 1], double acc[4]) {
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int K = in[0].K, ldb = in[0].ldb, gn = n0 + tx;
+// One run in[0 .. n) of such contributions (n = 1 when transposed) added to a tile of tm x tn
+// entries, which the threads own flat (entry e = thread + 256 q at row em, column en: a small
+// block then fills whole warps); the sum of the A blocks is formed while they are staged.
+__device__ __forceinline__ void tile_accumulate_run(const GemmIn* in, int n, int m0, int n0, int tm, int tn,
+                                                    const int* em, const int* en, double (*As)[kTile + 1],
+                                                    double (*Bs)[kTile + 1], double acc[4]) {
+    const int K = in[0].K, ldb = in[0].ldb, tid = (int)threadIdx.x;
     const double* B = in[0].B;
     for (int k0 = 0; k0 < K; k0 += kTile) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int mm = ty + 8 * r, gm = m0 + mm, gk = k0 + tx;
-            if (m0 + 8 * r >= M) break;
-            double v = 0.0;
-            if (gm < M && gk < K) {
-#pragma unroll 4
-                for (int u = 0; u < n; ++u) v = fma(in[u].alpha, in[u].A[(int64_t)gm * in[u].lda + gk], v);
-            }
-            As[tx][mm] = v;
-        }
         const int kk_end = min(kTile, K - k0);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int kk = ty + 8 * r;
-            if (kk < kk_end) Bs[kk][tx] = gn < N ? B[(int64_t)(k0 + kk) * ldb + gn] : 0.0;
+        if (in[0].transA) {
+            for (int e = tid; e < kk_end * tm; e += kThreads) {
+                const int kk = e / tm, mm = e - kk * tm;
+                As[kk][mm] = in[0].alpha * in[0].A[(int64_t)(k0 + kk) * in[0].lda + m0 + mm];
+            }
+        } else {
+            for (int e = tid; e < tm * kk_end; e += kThreads) {
+                const int mm = e / kk_end, kk = e - mm * kk_end;
+                double v = 0.0;
+#pragma unroll 4
+                for (int u = 0; u < n; ++u)
+                    v = fma(in[u].alpha, in[u].A[(int64_t)(m0 + mm) * in[u].lda + k0 + kk], v);
+                As[kk][mm] = v;
+            }
+        }
+        for (int e = tid; e < kk_end * tn; e += kThreads) {
+            const int kk = e / tn, nn = e - kk * tn;
+            Bs[kk][nn] = B[(int64_t)(k0 + kk) * ldb + n0 + nn];
         }
         __syncthreads();
-        for (int kk = 0; kk < kk_end; ++kk) {
-            const double b = Bs[kk][tx];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                if (m0 + ty + 8 * r < M) acc[r] = fma(As[kk][ty + 8 * r], b, acc[r]);
-        }
+        for (int q = 0; q < 4; ++q)
+            if (tid + q * kThreads < tm * tn)
+                for (int kk = 0; kk < kk_end; ++kk) acc[q] = fma(As[kk][em[q]], Bs[kk][en[q]], acc[q]);
         __syncthreads();
     }
 }
 
-// 32 x 32 output tile per CTA; thread (ty, tx) owns rows ty + 8 r (r < 4), column tx.
+// 32 x 32 output tile per CTA.
 constexpr int kGemmIns = 64;   // descriptors staged at a time
 __global__ void __launch_bounds__(kThreads) k_gemm(const GemmOut* __restrict__ outs,
                                                    const GemmIn* __restrict__ ins,
@@ -100,8 +102,15 @@ __global__ void __launch_bounds__(kThreads) k_gemm(const GemmOut* __restrict__ o
     __shared__ GemmIn s_in[kGemmIns];
     const GemmTile tl = tiles[blockIdx.x];
     const GemmOut o = outs[tl.out];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int tm = min(kTile, o.M - tl.m0), tn = min(kTile, o.N - tl.n0);
+    int em[4], en[4];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int e = threadIdx.x + q * kThreads;
+        em[q] = e / tn;
+        en[q] = e - em[q] * tn;
+    }
     for (int cb = o.beg; cb < o.end; cb += kGemmIns) {
         const int n = min(kGemmIns, o.end - cb);
         constexpr int kWords = (int)(sizeof(GemmIn) / sizeof(long long));
@@ -110,24 +119,17 @@ __global__ void __launch_bounds__(kThreads) k_gemm(const GemmOut* __restrict__ o
         for (int u = 0; u < n;) {
             int v = u + 1;
             while (v < n && same_b(s_in[v], s_in[u])) ++v;
-            if (s_in[u].transA)
-                dev::gemm_tile_accumulate(s_in[u], o.M, o.N, tl.m0, tl.n0, As, Bs, acc);
-            else
-                tile_accumulate_run(s_in + u, v - u, o.M, o.N, tl.m0, tl.n0, As, Bs, acc);
+            tile_accumulate_run(s_in + u, v - u, tl.m0, tl.n0, tm, tn, em, en, As, Bs, acc);
             u = v;
         }
         __syncthreads();   // the descriptors are replaced
     }
-    const int gn = tl.n0 + tx;
-    if (gn >= o.N) return;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int gm = tl.m0 + ty + 8 * r;
-        if (gm < o.M) {
-            double* cp = o.C + (int64_t)gm * o.ldc + gn;
-            *cp = o.beta == 0.0 ? acc[r] : o.beta * (*cp) + acc[r];
+    for (int q = 0; q < 4; ++q)
+        if (threadIdx.x + q * kThreads < tm * tn) {
+            double* cp = o.C + (int64_t)(tl.m0 + em[q]) * o.ldc + tl.n0 + en[q];
+            *cp = o.beta == 0.0 ? acc[q] : o.beta * (*cp) + acc[q];
         }
-    }
 }
 
 // Small outputs (M, N <= 32): one CTA per output, one thread per output

@@ -262,22 +262,35 @@ __global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, 
     if (o < out) d2[img_at(o, b, nk2)] = v;
 }
 
-// db[o] = sum_b dY[b, o] (rounded as the weight-gradient product reads it), one
-// CTA per o; the image's rows are contiguous runs of 32 values of b (zeros beyond B).
-__global__ void k_mlp_bgrad(const float* __restrict__ d2, float* __restrict__ db, int B) {
-    __shared__ float red[32];
-    const int o = blockIdx.x, nk2 = img_chunks(B);
-    const float* row = d2 + (int64_t)(o / kImgRows) * nk2 * kImgBlock + (o % kImgRows) * kImgK;
-    float acc = 0.0f;
-#pragma unroll 8
-    for (int b = threadIdx.x; b < nk2 * kImgK; b += blockDim.x) acc += row[(int64_t)(b / kImgK) * kImgBlock + b % kImgK];
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+// db[o] = sum_b dY[b, o] (rounded as the weight-gradient product reads it), eight o
+// per CTA: their rows are a contiguous 1 KB of every block of the image (rows = o, k
+// = b, zeros beyond B), a warp's eight lanes per row, the blocks dealt to the warps.
+constexpr int kBiasThreads = 512;
+__global__ void __launch_bounds__(kBiasThreads) k_mlp_bgrad(const float* __restrict__ d2, float* __restrict__ db, int B,
+                                                            int out) {
+    __shared__ float red[kBiasThreads / 32][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o0 = 8 * blockIdx.x, nk2 = img_chunks(B);
+    const float4* src = (const float4*)(d2 + (int64_t)(o0 / kImgRows) * nk2 * kImgBlock + (o0 % kImgRows) * kImgK);
+    float s0 = 0.0f, s1 = 0.0f;   // rows lane / 8 and 4 + lane / 8
+#pragma unroll 4
+    for (int c = warp; c < nk2; c += kBiasThreads / 32) {
+        const float4 x = src[(int64_t)c * (kImgBlock / 4) + lane], y = src[(int64_t)c * (kImgBlock / 4) + 32 + lane];
+        s0 += (x.x + x.y) + (x.z + x.w);
+        s1 += (y.x + y.y) + (y.z + y.w);
+    }
+    for (int d = 4; d > 0; d >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, d);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, d);
+    }
+    if ((lane & 7) == 0) {
+        red[warp][lane >> 3] = s0;
+        red[warp][4 + (lane >> 3)] = s1;
+    }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = threadIdx.x < (int)(blockDim.x >> 5) ? red[threadIdx.x] : 0.0f;
-        for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-        if (threadIdx.x == 0) db[o] = acc;
+    if (threadIdx.x < 8 && o0 + (int)threadIdx.x < out) {
+        float acc = 0.0f;
+        for (int w = 0; w < kBiasThreads / 32; ++w) acc += red[w][threadIdx.x];
+        db[o0 + threadIdx.x] = acc;
     }
 }
 
@@ -451,7 +464,7 @@ float loss_grad(Context* ctx, bsmps_mlp_s* net, const float* x_host, const float
         gw.K = B;
         gw.nkc = img_chunks(B);
         launch_mlp_gemm(ctx, gw, s, net->grad + net->w_off[l]);
-        k_mlp_bgrad<<<(unsigned)out, kT, 0, ctx->stream>>>(d2, net->grad + net->b_off[l], B);
+        k_mlp_bgrad<<<(unsigned)((out + 7) / 8), kBiasThreads, 0, ctx->stream>>>(d2, net->grad + net->b_off[l], B, out);
         done(ctx);
         if (l > 0) {
             // dX[b, i] = (sum_o dY[b, o] W[o, i]) [X[b, i] > 0]

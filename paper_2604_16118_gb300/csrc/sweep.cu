@@ -30,9 +30,35 @@ size_t cut_smem(const CutTask& c) {
     return sizeof(double) * 2 * (size_t)c.cap_total + sizeof(int) * (2 * (size_t)c.cap_total + c.n_sec + 1);
 }
 
+// Sectors of at most this many rows and kept columns go to Jacobi without a QR step.
+constexpr int kDirectRows = 32, kDirectCols = 16;
+// Their leading dimensions by the three instances of jacobi_pre() (8, 16 or 32 rows).
+__host__ __device__ constexpr int direct_ldb(int len) { return len <= 8 ? 8 : len <= 16 ? 24 : 40; }
+__host__ __device__ constexpr int direct_ldv(int len) { return len <= 8 ? 8 : 24; }
+static_assert(direct_ldb(8) == dev::jacobi_ld(1) && direct_ldb(16) == dev::jacobi_ld(9) &&
+                  direct_ldb(32) == dev::jacobi_ld(25) && direct_ldv(8) == dev::jacobi_ld(1) &&
+                  direct_ldv(32) == dev::jacobi_ld(9),
+              "leading dimensions of jacobi_pre<1, 1>, <2, 2> and <4, 2>");
+
+// The QR input (later Q V; while the Jacobi runs its scratch), Q, G, V and three vectors; or,
+// without a QR step, the padded input, V, the scratch and three vectors.
+__host__ __device__ inline size_t svd_buf(int len, int k) {
+    const size_t a = (size_t)len * k, b = (size_t)dev::jacobi_scratch(dev::jacobi_ld(k), dev::jacobi_ld(k), k);
+    return k <= 64 && b > a ? b : a;
+}
+size_t svd_doubles(int len, int k) {
+    return svd_buf(len, k) + (size_t)len * k + 2 * (size_t)k * dev::jacobi_ld(k) + 3 * (size_t)k;
+}
+// Monotone in both sizes: the dynamic sweep sizes its memory by padded column counts and a
+// sector with fewer may take another path.
 size_t svd_smem(int M, int N) {
-    const size_t k = (size_t)std::min(M, N), len = (size_t)std::max(M, N), ld = (size_t)dev::jacobi_ld((int)k);
-    return sizeof(double) * ((std::max(len, ld) + len) * k + 2 * k * ld + 3 * k);
+    const int k = std::min(M, N), len = std::max(M, N);
+    size_t n = svd_doubles(len, k);
+    if (k > 64) n = std::max(n, svd_doubles(len, 64));
+    const int rows = std::min(len, kDirectRows), cols = std::min(k, kDirectCols), lb = direct_ldb(rows),
+              lv = direct_ldv(rows);
+    n = std::max(n, cols * (size_t)(lb + lv) + (size_t)dev::jacobi_scratch(lb, lv, cols) + 4 * (size_t)cols);
+    return sizeof(double) * n;
 }
 
 // Global loads of data that other CTAs of the same launch may have written
@@ -175,12 +201,13 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
                                                        const SvdPart* __restrict__ parts) {
     extern __shared__ double sm[];
     __shared__ double red[33];
+    __shared__ dev::SegRot ring[64];
     __shared__ int s_rot;
     const SvdSiteTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = tk.k, len = tk.len;
     double* B = sm;                               // QR input (len x k), later Q V
     const int ld = dev::jacobi_ld(k);
-    double* Q = B + (int64_t)max(len, ld) * k;
+    double* Q = B + svd_buf(len, k);
     double* tau = Q + (int64_t)len * k;
     double* G = tau + k;
     double* V = G + (int64_t)k * ld;
@@ -205,7 +232,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
     }
     dev::form_q(B, tau, Sraw, Q, len, k);
     __syncthreads();
-    dev::jacobi_auto(G, V, Sraw, k, B, tau, red, &s_rot);
+    dev::jacobi_auto(G, V, Sraw, k, B, tau, ring, red, &s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
@@ -319,7 +346,7 @@ __device__ void right_rank1(const DynTask& tk, const double* v, int len, int wid
 
 template <bool CG>
 __device__ void right_body(const DynTask& tk, double* sm, double* red,
-                           int* s_rot, int* s_cols) {
+                           int* s_rot, int* s_cols, dev::SegRot* ring) {
     const int np = tk.p_end - tk.p_beg;
     if (threadIdx.x < 2) {
         int c = 0;
@@ -338,12 +365,16 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     const int k = M < N ? M : N, len = M < N ? N : M, wide = M < N ? 1 : 0;
     double* B = sm;
     const int ld = dev::jacobi_ld(k);
-    double* Q = B + (int64_t)max(len, ld) * k;
+    double* Q = B + svd_buf(len, k);
     double* tau = Q + (int64_t)len * k;
     double* G = tau + k;
     double* V = G + (int64_t)k * ld;
     double* Sraw = V + (int64_t)k * ld;
     int* perm = (int*)(Sraw + k);
+    const bool direct = len <= kDirectRows && k <= kDirectCols;
+    const int ldb = direct ? direct_ldb(len) : len;   // (k == 1 included: one padded column)
+    if (direct)
+        for (int e = threadIdx.x; e < k * (ldb - len); e += nthreads()) B[(e / (ldb - len)) * ldb + len + e % (ldb - len)] = 0.0;
     int coff = 0;
     for (int p = 0; p < np; ++p) {
         const DynPart& pt = tk.part[p];
@@ -358,9 +389,9 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
                 v = ldd<CG>(pt.X + (int64_t)i * pt.xcols + cc);
             }
             if (wide)
-                B[(int64_t)i * N + c] = v;
+                B[(int64_t)i * ldb + c] = v;
             else
-                B[(int64_t)c * M + i] = v;
+                B[(int64_t)c * ldb + i] = v;
         }
         coff += cols;
     }
@@ -369,14 +400,22 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
         right_rank1(tk, B, len, wide, red);
         return;
     }
-    if (len <= 32 && k <= 16) {
-        // small sector: one-sided Jacobi directly on B (no QR step)
-        double* Vd = B + (int64_t)len * k;
-        double* Sr = Vd + (int64_t)k * k;
+    if (direct) {
+        // small sector: one-sided Jacobi on B itself (no QR step)
+        const int ldv = direct_ldv(len);
+        double* Vd = B + (int64_t)k * ldb;
+        double* scr = Vd + (int64_t)k * ldv;
+        double* Sr = scr + dev::jacobi_scratch(ldb, ldv, k);
         double* rinv = Sr + k;
-        int* prm = (int*)(rinv + k);
-        dev::jacobi_direct(B, Vd, Sr, len, k, red, s_rot);
-        dev::svd_assemble_direct(B, Vd, Sr, rinv, prm, tk.S, tk.US, tk.Vt, M, N, k, len, wide, tk.kpad,
+        double* dl = rinv + k;
+        int* prm = (int*)(dl + k);
+        if (len <= 8)
+            dev::jacobi_pre<1, 1>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        else if (len <= 16)
+            dev::jacobi_pre<2, 2>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        else
+            dev::jacobi_pre<4, 2>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        dev::svd_assemble_direct(B, ldb, Vd, ldv, Sr, rinv, prm, tk.S, tk.US, tk.Vt, M, N, k, wide, tk.kpad,
                                  tk.ncols_pad);
         __syncthreads();
         if (threadIdx.x == 0) *tk.kact = k;
@@ -389,7 +428,7 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     }
     dev::form_q(B, tau, Sraw, Q, len, k);
     __syncthreads();
-    dev::jacobi_auto(G, V, Sraw, k, B, tau, red, s_rot);
+    dev::jacobi_auto(G, V, Sraw, k, B, tau, ring, red, s_rot);
     for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
         const int p = (int)(e / len), i = (int)(e % len);
         double acc = 0.0;
@@ -404,9 +443,10 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
 __global__ void __launch_bounds__(kSweepThreads) k_right_dyn(const DynTask* __restrict__ tasks) {
     extern __shared__ double sm[];
     __shared__ double red[33];
+    __shared__ dev::SegRot ring[64];
     __shared__ int s_rot;
     __shared__ int s_cols[2];
-    right_body<false>(tasks[blockIdx.x], sm, red, &s_rot, s_cols);
+    right_body<false>(tasks[blockIdx.x], sm, red, &s_rot, s_cols, ring);
 }
 
 // Pooled cut of one bond (one CTA): stable descending order with ties by
@@ -598,6 +638,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
     __shared__ int s_cols[2];
     __shared__ int s_n;
     __shared__ int s_flag;
+    __shared__ dev::SegRot ring[64];
     __shared__ DynTask s_task[2];
     int* pb = (int*)((char*)sm + pb_off);
     for (int i = threadIdx.x; i <= n_phase; i += nthreads()) pb[i] = phase_beg[i];
@@ -620,7 +661,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
             __syncthreads();
             const bool first = ti == pb[p] + (int)blockIdx.x;
             const DynTask& tk = first ? s_task[p & 1] : tasks[ti];
-            right_body<true>(tk, sm, red, &s_rot, s_cols);
+            right_body<true>(tk, sm, red, &s_rot, s_cols, ring);
             // the CTA that completes the last task of this truncation's bond runs its cut
             __syncthreads();
             const CutTask& ct = cuts[tk.cut];
@@ -672,6 +713,8 @@ unsigned char* upload_pack(Scratch& s, const Pack& p) {
 // lengthen the barriers between reflectors.
 int block_for(int kmax, int max_warps = 8) { return 32 * std::max(1, std::min(max_warps, (kmax + 1) / 2)); }
 constexpr int kSvdWarps = kSweepThreads / 32;
+// The SVD kernels: at least two warps (the Jacobi's G and V warps), and enough for 8 blockDim >= k^2.
+int svd_block_for(int kmax) { return std::max(64, block_for(kmax, kSvdWarps)); }
 
 // The attributes are per function and per process: set them once per kernel.
 template <class F>
@@ -726,12 +769,13 @@ __global__ void k_grid_wait_check(int skip_cta, GridSync* gs) {
 // inputs may have been written in earlier phases (loads go through L2).  A CTA
 // stages 32 values of k of both factors in shared memory; the right factor of an
 // environment update is summed over its contributions while it is staged, their
-// weights resolved once per contribution by one thread each.  Bound, at small
+// weights resolved once per contribution by one thread each; entries are dealt out
+// flat over the tile's valid part.  Bound, at small
 // blocks, by the round trips of a phase and the grid-wide wait between phases
 // (kEnvPerSm CTAs per SM: more make the wait longer than the tiles shorter).
-constexpr int kEnvThreads = 256;
+constexpr int kEnvThreads = 128;
 constexpr int kEnvCons = 64;    // contributions resolved at a time
-constexpr int kEnvPerSm = 4;
+constexpr int kEnvPerSm = 8;
 
 __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __restrict__ outs,
                                                              const EnvRunT* __restrict__ runs,
@@ -752,77 +796,83 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __re
     __shared__ const double* s_ptr[kEnvCons];
     __shared__ double s_w[kEnvCons];
     const double* bases[4] = {b0, b1, b2, b3};
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    constexpr int kPer = 32 * 32 / kEnvThreads;   // entries of a full tile per thread
     for (int p = 0; p < n_phase; ++p) {
+        const bool upd = (p & 1) != 0;
         for (int ti = phase_beg[p] + (int)blockIdx.x; ti < phase_beg[p + 1]; ti += (int)gridDim.x) {
             const EnvTileT tl = tiles[ti];
             const EnvOutT o = outs[tl.out];
             const EnvGroupPhase g = gph[o.gp];
             const EnvMemberFac mf = mfac[g.mem_beg + tl.member];
             const int64_t mem = tl.member;
-            const int gn = tl.n0 + tx;
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            // the tile's entries, flat over its valid rows and columns (small blocks fill few lanes otherwise)
+            const int tm = min(32, o.M - tl.m0), tn = min(32, o.N - tl.n0), n_el = tm * tn;
+            int em[kPer], en[kPer];
+            double acc[kPer];
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const int e = threadIdx.x + q * kEnvThreads;
+                em[q] = e / tn;
+                en[q] = e - em[q] * tn;
+                acc[q] = 0.0;
+            }
             for (int r = o.beg; r < o.end; ++r) {
                 const EnvRunT run = runs[r];
-                const bool upd = (p & 1) != 0;
                 const double* E = upd ? nullptr : bases[run.abuf] + g.base[run.abuf] + mem * g.stride[run.abuf] + run.off;
                 const double* T = bases[0] + g.base[0] + mem * g.stride[0];
                 for (int cb = run.cbeg; cb < run.cend; cb += kEnvCons) {
                     const int nc = min(kEnvCons, run.cend - cb);
-                    if (upd && (int)threadIdx.x < nc) {
-                        const EnvConT c = cons[cb + threadIdx.x];
-                        double w = c.w + ((c.fac & 4) ? g.shift : 0.0);
-                        const int ra = mf.row[c.fac & 1], rb = mf.row[2 + ((c.fac >> 1) & 1)];
-                        if (ra >= 0) w *= ftab[(int64_t)ra * K + run.site];
-                        if (rb >= 0) w *= ftab[(int64_t)rb * K + run.site];
-                        s_ptr[threadIdx.x] = T + c.off;
-                        s_w[threadIdx.x] = w;
+                    if (upd) {
+                        if ((int)threadIdx.x < nc) {
+                            const EnvConT c = cons[cb + threadIdx.x];
+                            double w = c.w + ((c.fac & 4) ? g.shift : 0.0);
+                            const int ra = mf.row[c.fac & 1], rb = mf.row[2 + ((c.fac >> 1) & 1)];
+                            if (ra >= 0) w *= ftab[(int64_t)ra * K + run.site];
+                            if (rb >= 0) w *= ftab[(int64_t)rb * K + run.site];
+                            s_ptr[threadIdx.x] = T + c.off;
+                            s_w[threadIdx.x] = w;
+                        }
+                        __syncthreads();
                     }
-                    if (upd) __syncthreads();
                     for (int k0 = 0; k0 < run.K; k0 += 32) {
                         const int kk_end = min(32, run.K - k0);
-                        if (upd) {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int kk = ty + 8 * q, gm = tl.m0 + tx;
-                                if (kk < kk_end) {
-                                    As[kk][tx] = gm < o.M ? __ldcg(run.ptr + (int64_t)(k0 + kk) * o.M + gm) : 0.0;
-                                    double v = 0.0;
-                                    if (gn < o.N) {
-                                        const int64_t at = (int64_t)(k0 + kk) * o.N + gn;
+                        for (int e = threadIdx.x; e < kk_end * tn; e += kEnvThreads) {
+                            const int kk = e / tn, n = e - kk * tn;
+                            const int64_t at = (int64_t)(k0 + kk) * o.N + tl.n0 + n;
+                            double v = 0.0;
+                            if (upd) {
 #pragma unroll 8
-                                        for (int c = 0; c < nc; ++c) v = fma(s_w[c], __ldcg(s_ptr[c] + at), v);
-                                    }
-                                    Bs[kk][tx] = v;
-                                }
+                                for (int c = 0; c < nc; ++c) v = fma(s_w[c], __ldcg(s_ptr[c] + at), v);
+                            } else {
+                                v = __ldcg(run.ptr + at);
+                            }
+                            Bs[kk][n] = v;
+                        }
+                        if (upd) {
+                            for (int e = threadIdx.x; e < kk_end * tm; e += kEnvThreads) {
+                                const int kk = e / tm, m = e - kk * tm;
+                                As[kk][m] = __ldcg(run.ptr + (int64_t)(k0 + kk) * o.M + tl.m0 + m);
                             }
                         } else {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int mm = ty + 8 * q, gm = tl.m0 + mm;
-                                if (gm < o.M && tx < kk_end) As[tx][mm] = __ldcg(E + (int64_t)gm * run.K + k0 + tx);
-                                if (mm < kk_end)
-                                    Bs[mm][tx] = gn < o.N ? __ldcg(run.ptr + (int64_t)(k0 + mm) * o.N + gn) : 0.0;
+                            for (int e = threadIdx.x; e < kk_end * tm; e += kEnvThreads) {
+                                const int m = e / kk_end, kk = e - m * kk_end;
+                                As[kk][m] = __ldcg(E + (int64_t)(tl.m0 + m) * run.K + k0 + kk);
                             }
                         }
                         __syncthreads();
-                        for (int kk = 0; kk < kk_end; ++kk) {
-                            const double b = Bs[kk][tx];
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                if (tl.m0 + ty + 8 * q < o.M) acc[q] = fma(As[kk][ty + 8 * q], b, acc[q]);
+                        for (int q = 0; q < kPer; ++q) {
+                            if (threadIdx.x + q * kEnvThreads < n_el)
+                                for (int kk = 0; kk < kk_end; ++kk) acc[q] = fma(As[kk][em[q]], Bs[kk][en[q]], acc[q]);
                         }
                         __syncthreads();
                     }
                 }
             }
             double* C = const_cast<double*>(bases[o.cbuf]) + g.base[o.cbuf] + mem * g.stride[o.cbuf] + o.coff;
-            if (gn < o.N)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int gm = tl.m0 + ty + 8 * q;
-                    if (gm < o.M) C[(int64_t)gm * o.N + gn] = acc[q];
-                }
+            for (int q = 0; q < kPer; ++q)
+                if (threadIdx.x + q * kEnvThreads < n_el) C[(int64_t)(tl.m0 + em[q]) * o.N + tl.n0 + en[q]] = acc[q];
         }
         if (!phase_end(gs, (unsigned)p, &s_flag)) return;
     }
@@ -1042,7 +1092,7 @@ void launch_svd_site(Context* ctx, const std::vector<SvdSiteTask>& tasks, const 
     int kmax = 1;
     for (const SvdSiteTask& t : tasks) kmax = std::max(kmax, t.k);
     const cudaStream_t st = on_side ? ctx->fork_side() : ctx->stream;
-    k_svd_site<<<(unsigned)tasks.size(), block_for(kmax, kSvdWarps), smem, st>>>((const SvdSiteTask*)(d + ot),
+    k_svd_site<<<(unsigned)tasks.size(), svd_block_for(kmax), smem, st>>>((const SvdSiteTask*)(d + ot),
                                                                                  (const SvdPart*)(d + op));
     count_launch(ctx);
     pr.done();
@@ -1104,7 +1154,7 @@ int launch_right_dyn(Context* ctx, const std::vector<DynTask>& tasks_in, const s
     unsigned char* d = upload_pack(s, pk);
     Prof pr(ctx, KK_SVD, fl, by);
     allow_smem(k_right_dyn);
-    k_right_dyn<<<(unsigned)tasks.size(), block_for(kmax, kSvdWarps), smem, ctx->stream>>>((const DynTask*)(d + ot));
+    k_right_dyn<<<(unsigned)tasks.size(), svd_block_for(kmax), smem, ctx->stream>>>((const DynTask*)(d + ot));
     count_launch(ctx);
     pr.done();
     return ctx->profiling ? (int)ctx->prof.size() - 1 : -1;
@@ -1188,7 +1238,7 @@ bool launch_right_sweep(Context* ctx, const std::vector<DynTask>& tasks_in, cons
     const size_t pb_off = (smem + 15) & ~size_t(15);   // phase_beg staged behind the working set
     smem = pb_off + sizeof(int) * (size_t)(n_phase + 1);
     if (smem > kSweepSmem) return false;
-    const int threads = block_for(kmax, kSvdWarps);
+    const int threads = svd_block_for(kmax);
     allow_smem(k_right_sweep);
     const int cap = coresident_ctas(k_right_sweep, threads, smem);
     if (cap <= 0) return false;
