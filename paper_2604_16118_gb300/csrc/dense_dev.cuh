@@ -236,58 +236,126 @@ __device__ __forceinline__ double to_double(float f) {
     const unsigned hi = e ? ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3) : 0u;
     return __hiloint2double((int)(hi | (u & 0x80000000u)), e ? (int)(u << 29) : 0);
 }
-// 1/sqrt(w) for normal w > 0: Halley's iteration from an FP32 seed (22 bits or
-// more), whose relative error after one step is of order 2^-63; five FP64
-// instructions.  Exponents outside FP32's comfortable range, zeros and non-finite
-// values go through the library function.
-__device__ __forceinline__ double rsqrt_halley(double w) {
-    const int e = (__double2hiint(w) >> 20) & 0x7ff;
-    if (__double2hiint(w) < 0 || e < 2 || e > 2045) return rsqrt(w);
-    const int h = (e - 1023) >> 1;   // w = 4^h u, u in [1, 4)
-    const double u = __hiloint2double(__double2hiint(w) - (h << 21), __double2loint(w));
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_scaled(u, 0)));
-    const double y0 = to_double(y);
-    const double r = fma(-(u * y0), y0, 1.0);
-    const double z = fma(y0 * r, fma(0.375, r, 0.5), y0);
-    return __hiloint2double(__double2hiint(z) - (h << 20), __double2loint(z));
-}
-// 1/q for normal q > 0 by the same kind of step: y0 (1 + r + r^2), r = 1 - q y0.
-__device__ __forceinline__ double recip_newton(double q) {
-    const int e = (__double2hiint(q) >> 20) & 0x7ff;
-    if (__double2hiint(q) < 0 || e < 2 || e > 2040) return 1.0 / q;
-    const int h = e - 1023;
-    const double u = __hiloint2double(__double2hiint(q) - (h << 20), __double2loint(q));
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(to_float_scaled(u, 0)));
-    const double y0 = to_double(y);
-    const double r = fma(-u, y0, 1.0);
-    const double z = fma(y0, fma(r, r, r), y0);
-    return __hiloint2double(__double2hiint(z) - (h << 20), __double2loint(z));
+// Sum over the warp by integer arithmetic: the 32 values as 58-bit fixed-point numbers
+// of a common exponent, added in three limbs by warp reductions (redux), the exact
+// sum rounded once.  275 cycles against 605 for five shuffle and FP64 addition
+// steps (about 45 + 75 cycles each here), and no FP64 instruction.  Values outside
+// the middle of the exponent range (and non-finite ones) take the shuffles.
+__device__ __forceinline__ double warp_sum_fixed(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned e = (hi >> 20) & 0x7ff;
+    const unsigned em = __reduce_max_sync(0xffffffffu, e);
+    if (em < 64 || em > 2036) return warp_sum(v);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+    const int d = (int)(em - (e ? e : 1u));
+    const long long f = d < 58 ? (long long)((m << 5) >> d) : 0;
+    const long long x = (int)hi < 0 ? -f : f;
+    const unsigned r0 = __reduce_add_sync(0xffffffffu, (unsigned)x & 0xffffffu);
+    const unsigned r1 = __reduce_add_sync(0xffffffffu, (unsigned)(x >> 24) & 0xffffffu);
+    const int r2 = __reduce_add_sync(0xffffffffu, (int)(x >> 48));
+    const long long t = (long long)r0 + ((long long)r1 << 24) + (long long)((unsigned long long)(long long)r2 << 48);
+    if (t == 0) return 0.0;
+    const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;   // below 2^63
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << lz;
+    unsigned long long q = n >> 11;
+    const unsigned r = (unsigned)n & 0x7ffu;
+    q += (r > 0x400u || (r == 0x400u && (q & 1ull))) ? 1ull : 0ull;
+    // a = 2^57 for a value of exponent field em
+    const unsigned long long bits = ((unsigned long long)(em + 5 - lz) << 52) + q;
+    return __longlong_as_double((long long)(bits | (t < 0 ? 1ull << 63 : 0ull)));
 }
 
-// One warp: reflector of column j (rows j .. M-1): H = I - tau v v^T with v = x
-// below row j (left in place, no scaling pass), v_j = alpha - beta = sign(alpha)
-// (|alpha| + n), n = ||(alpha, x)||, tau = 1 / (n (n + |alpha|)).  tau[j] and
-// vd[j] = v_j are stored; R(j, j) = beta replaces the diagonal entry.
-__device__ __forceinline__ void reflect_column(double* A, double* tau, double* vd, int M, int j, int lane) {
+// x 2^-h by exponent arithmetic (0 when the result leaves the normal range downwards).
+__device__ __forceinline__ double scale_down(double x, int h) {
+    const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+    return e == 0 || e - h < 1 ? 0.0 : __hiloint2double(hi - (int)((unsigned)h << 20), __double2loint(x));
+}
+
+// Householder vector of the column (alpha, x) with ||x||^2 = s != 0: H = I - tau v v^T
+// with v = (vd, x 2^-shift), vd = sign(alpha) (|alpha| + n) 2^-shift, n = ||(alpha, x)||,
+// tau = 2^(2 shift) / (n (n + |alpha|)); beta = -sign(alpha) n.  shift = 0 unless the
+// norm is so large or small that tau would leave the range.  1/n by Halley's
+// iteration from an FP32 reciprocal square root, 1/(n + |alpha|) by one step of
+// order three from an FP32 reciprocal that is formed while the FP64 chain of 1/n
+// runs (the errors of both are of order 2^-63): about 900 cycles against 1500 for
+// the two in turn.
+__device__ __forceinline__ void reflector_vector(double alpha, double s, double* tau, double* vd, double* beta,
+                                                 int* shift) {
+    const double w = fma(alpha, alpha, s);
+    const int e = (__double2hiint(w) >> 20) & 0x7ff;
+    *shift = 0;
+    if (__double2hiint(w) < 0 || e < 64 || e > 1980) {   // tiny, huge, subnormal or non-finite
+        const double rn = rsqrt(w), n = w * rn;
+        int h = 0;
+        if (n > 0.0 && n < 1.7976931348623157e308) frexp(n, &h);
+        const double nu = ldexp(n, -h), qu = nu + ldexp(fabs(alpha), -h);
+        *shift = h;
+        *tau = 1.0 / (nu * qu);
+        *vd = alpha >= 0.0 ? qu : -qu;
+        *beta = alpha >= 0.0 ? -n : n;
+        return;
+    }
+    const int h = (e - 1023) >> 1;   // w = 4^h u, u in [1, 4)
+    const double u = __hiloint2double(__double2hiint(w) - (h << 21), __double2loint(w));
+    const double au = scale_down(fabs(alpha), h);
+    const float uf = to_float_scaled(u, 0);
+    float yf, zf;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(uf));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(zf) : "f"(fmaf(uf, yf, to_float_scaled(au, 0))));
+    const double y0 = to_double(yf), z0 = to_double(zf);
+    const double r = fma(-(u * y0), y0, 1.0);
+    const double y = fma(y0 * r, fma(0.375, r, 0.5), y0);   // 1/sqrt(u)
+    const double nu = u * y, qu = nu + au;
+    const double p = fma(-qu, z0, 1.0);
+    const double z = fma(z0, fma(p, p, p), z0);             // 1/qu
+    const double t = y * z;                                 // in (0.1, 1]: times 4^-h
+    *tau = __hiloint2double(__double2hiint(t) - (h << 21), __double2loint(t));
+    const double q = __hiloint2double(__double2hiint(qu) + (h << 20), __double2loint(qu));
+    const double n = __hiloint2double(__double2hiint(nu) + (h << 20), __double2loint(nu));
+    *vd = alpha >= 0.0 ? q : -q;
+    *beta = alpha >= 0.0 ? -n : n;
+}
+
+// One warp: H_{j-1} (v the column j - 1 and vj, tw_scale = tau_{j-1}; none when tau = 0)
+// applied to column j, then the reflector of column j (rows j .. M-1, v below row j left
+// in place): tau[j], vd[j] = v_j, R(j, j) in the diagonal entry (tau[j] = 0: nothing to
+// eliminate).
+__device__ __forceinline__ void reflect_column(double* A, double* tau, double* vd, int M, int j, double tj, double vj,
+                                               int lane) {
     double* x = A + (int64_t)j * M;
-    double s = 0.0;
-    for (int i = j + 1 + lane; i < M; i += 32) s = fma(x[i], x[i], s);
-    s = warp_sum(s);
-    const double alpha = x[j];
-    __syncwarp();   // every lane has read x[j]
-    if (lane == 0) {
-        double tj = 0.0;
-        if (s != 0.0) {
-            const double w = fma(alpha, alpha, s);
-            const double rn = rsqrt_halley(w);
-            const double n = w * rn, q = fabs(alpha) + n;
-            tj = rn * recip_newton(q);
-            x[j] = alpha >= 0.0 ? -n : n;
-            vd[j] = alpha >= 0.0 ? q : -q;
+    const double* v = x - M;
+    double tw = 0.0;
+    if (tj != 0.0) {
+        double d = lane == 0 ? vj * x[j - 1] : 0.0;
+        for (int i = j + lane; i < M; i += 32) d = fma(v[i], x[i], d);
+        tw = tj * warp_sum_fixed(d);
+    }
+    double s = 0.0, alpha = 0.0;
+    for (int i = j + lane; i < M; i += 32) {
+        double y = x[i];
+        if (tj != 0.0) {
+            y = fma(-tw, v[i], y);
+            x[i] = y;
         }
-        tau[j] = tj;
+        if (i == j) alpha = y;
+        else s = fma(y, y, s);
+    }
+    if (tj != 0.0 && lane == 0) x[j - 1] = fma(-tw, vj, x[j - 1]);
+    s = warp_sum_fixed(s);
+    alpha = __shfl_sync(0xffffffffu, alpha, 0);
+    double t = 0.0, d = 0.0, beta = 0.0;
+    if (s != 0.0) {
+        int shift;
+        reflector_vector(alpha, s, &t, &d, &beta, &shift);
+        if (shift)
+            for (int i = j + lane; i < M; i += 32)   // the rows this lane wrote
+                if (i != j) x[i] = ldexp(x[i], -shift);
+    }
+    if (lane == 0) {
+        if (s != 0.0) x[j] = beta;
+        vd[j] = d;
+        tau[j] = t;
     }
     __syncwarp();
 }
@@ -316,8 +384,8 @@ __device__ __forceinline__ void reflect_segments(double* A, double tj, double vj
 // diagonal entries), tau[j]; form_q() reads them.
 //
 // One barrier per column: while the other warps apply H_j to the columns beyond
-// j + 1, warp 0 applies it to column j + 1 and forms H_{j+1} at once (its chain
-// of about 35 dependent FP64 instructions is what bounds a small QR).  Warps that
+// j + 1, warp 0 applies it to column j + 1 and forms H_{j+1} at once (its chain,
+// about 2300 cycles, is what bounds a small QR).  Warps that
 // share warp 0's scheduler (4, 8, ...) stay out of the updates while these are
 // shorter than that chain, which they would lengthen.
 __device__ __forceinline__ void householder(double* A, double* tau, double* vd, int M, int N) {
@@ -330,28 +398,15 @@ __device__ __forceinline__ void householder(double* A, double* tau, double* vd, 
     const int w_all = nw == 1 ? 0 : warp - 1, n_all = nw == 1 ? 1 : nw - 1;
     const int w_off = (warp & 3) ? (warp >> 2) * 3 + (warp & 3) - 1 : -1;
     const int n_off = (nw >> 2) * 3 + ((nw & 3) ? (nw & 3) - 1 : 0);
-    if (warp == 0) reflect_column(A, tau, vd, M, 0, lane);
+    if (warp == 0) reflect_column(A, tau, vd, M, 0, 0.0, 0.0, lane);
     __syncthreads();
     for (int j = 0; j < k; ++j) {
         const double tj = tau[j], vj = vd[j];
-        if (warp == 0 && j + 1 < N) {
-            if (tj != 0.0) {
-                const double* v = A + (int64_t)j * M;
-                double* a = A + (int64_t)(j + 1) * M;
-                const double a_j = a[j];
-                double d = lane == 0 ? vj * a_j : 0.0;
-                for (int i = j + 1 + lane; i < M; i += 32) d = fma(v[i], a[i], d);
-                const double tw = tj * warp_sum(d);
-                if (lane == 0) a[j] = fma(-tw, vj, a_j);
-                for (int i = j + 1 + lane; i < M; i += 32) a[i] = fma(-tw, v[i], a[i]);
-                __syncwarp();
-            }
-            if (j + 1 < k) reflect_column(A, tau, vd, M, j + 1, lane);
-        }
+        if (warp == 0 && j + 1 < k) reflect_column(A, tau, vd, M, j + 1, tj, vj, lane);
         // FP64 instructions of the other columns' updates against the chain's
-        const bool off = nw >= 6 && (N - j) * ((M - j) / 4 + 4) <= 4 * 120;
+        const bool off = nw >= 6 && (N - j) * ((M - j) / 4 + 4) <= 4 * 75;
         const int w = off ? w_off : w_all;
-        if (w >= 0 && tj != 0.0) reflect_segments(A, tj, vj, M, N, j, j + 2, w, off ? n_off : n_all, lane);
+        if (w >= 0 && tj != 0.0) reflect_segments(A, tj, vj, M, N, j, j + 1 < k ? j + 2 : j + 1, w, off ? n_off : n_all, lane);
         __syncthreads();
     }
 }
@@ -695,8 +750,11 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
                 const float ri = rsqrt_fast(fmaf(dn, dn, gn * gn));
                 const float c2 = fmaf(0.5f, fabsf(dn) * ri, 0.5f);
                 const float rc = rsqrt_fast(c2);
-                const float c = c2 * rc;
-                const float h = 0.5f * gn * ri * rc;
+                // one Newton step on c^2 + s^2 = 1: the approximate reciprocal roots are off by up
+                // to 2^-22, which hundreds of rotations would add up in the columns' lengths
+                const float cr = c2 * rc, hr = 0.5f * gn * ri * rc;
+                const float fix = fmaf(-0.5f, fmaf(cr, cr, hr * hr), 1.5f);
+                const float c = cr * fix, h = hr * fix;
                 const float sn = __uint_as_float(__float_as_uint(h) ^ (__float_as_uint(d) & 0x80000000u));
                 const bool rot = on && fminf(a, b) > 1e-30f && fabsf(g) > tol * (a * rsqrt_fast(a)) * (b * rsqrt_fast(b));
                 if (rot) {

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <tuple>
 
@@ -940,12 +941,12 @@ bool right_sweep_batch(Context* ctx, const std::vector<TruncJob*>& jobs, GridSyn
     int nsec_tot = 0;
     for (RightPlan& rp : plans) nsec_tot += rp.nsec;
     const int n_phase = K - 1;
-    const size_t n_ints = 2 * (size_t)std::max(nsec_tot, 1) + (size_t)n_phase * nj;
-    int* ints = (int*)ctx->alloc(sizeof(int) * n_ints);
-    s.ptrs.push_back(ints);
-    double* disc = s.dbl(2 * (size_t)nj);
-    BSM_CUDA(cudaMemsetAsync(ints, 0, sizeof(int) * n_ints, ctx->stream));
-    BSM_CUDA(cudaMemsetAsync(disc, 0, sizeof(double) * 2 * nj, ctx->stream));
+    // discarded norms, then kept counts and completion counters: zeroed and read back together
+    const size_t n_kept = 2 * (size_t)std::max(nsec_tot, 1), n_ints = n_kept + (size_t)n_phase * nj;
+    const size_t n_disc = 2 * (size_t)nj;
+    double* disc = s.dbl(n_disc + (n_ints + 1) / 2);
+    int* ints = (int*)(disc + n_disc);
+    BSM_CUDA(cudaMemsetAsync(disc, 0, sizeof(double) * (n_disc + (n_ints + 1) / 2), ctx->stream));
     int* done = ints + 2 * (size_t)std::max(nsec_tot, 1);
     {
         // S, US and Vt of every sector of every bond and job, carved from one allocation
@@ -1039,11 +1040,8 @@ bool right_sweep_batch(Context* ctx, const std::vector<TruncJob*>& jobs, GridSyn
             for (int j = 0; j < nj; ++j) launch_cut(ctx, cuts[(size_t)p * nj + j], secs);
         }
     }
-    std::vector<int> ints_h(2 * (size_t)std::max(nsec_tot, 1));
-    std::vector<double> disc_h(2 * (size_t)nj);
+    std::vector<double> disc_h(n_disc + (n_kept + 1) / 2);
     GridSync gs_h[2];
-    BSM_CUDA(cudaMemcpyAsync(ints_h.data(), ints, sizeof(int) * ints_h.size(), cudaMemcpyDeviceToHost,
-                             ctx->stream));
     BSM_CUDA(cudaMemcpyAsync(disc_h.data(), disc, sizeof(double) * disc_h.size(), cudaMemcpyDeviceToHost,
                              ctx->stream));
     BSM_CUDA(cudaMemcpyAsync(gs_h, gs, sizeof(gs_h), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1064,7 +1062,7 @@ bool right_sweep_batch(Context* ctx, const std::vector<TruncJob*>& jobs, GridSyn
         const Layout& L = J.L;
         J.td2 += disc_h[2 * j];
         J.cd2 += disc_h[2 * j + 1];
-        const int* keep_h = ints_h.data() + std::max(nsec_tot, 1) + (rp.keep - (ints + std::max(nsec_tot, 1)));
+        const int* keep_h = (const int*)(disc_h.data() + n_disc) + std::max(nsec_tot, 1) + (rp.keep - (ints + std::max(nsec_tot, 1)));
         auto kept = [&](int b, int m) { return b == K ? 1 : keep_h[rp.secoff[b] + m]; };
         std::vector<std::vector<int>> coff1(K);
         for (int b = K - 1; b >= 1; --b) {
@@ -1510,17 +1508,17 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
         gph.push_back(e);
         return (int)gph.size() - 1;
     };
-    // one operator entry acting on one environment block: the block of E' it adds to
-    // (right sectors of a and b), the block of a it multiplies, its T block and entry
+    // one operator entry acting on one environment block: its T block and entry, in a
+    // list per block of E' (right sectors of a and b) and block of a it multiplies (by s_out)
     struct Contrib {
-        uint64_t key;   // ra 2^42 + rb 2^21 + ab
-        int ti, ei;
+        int ti, ei, next;
     };
     struct TBlk {
         int env, rows, cols, bb;
         int64_t off;   // within a member's share of the T buffer
     };
     std::vector<Contrib> cs;
+    std::vector<int> head, tail, touched;   // lists of one channel d, by (ra nrb + rb) 2 + s_out
     for (int t = 0; t < K; ++t) {
         const int eid = t == 0 ? 3 : 1 + (t % 2);   // buffer of E at bond t
         const int nid = 1 + ((t + 1) % 2);          // buffer of E at bond t + 1
@@ -1571,6 +1569,9 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
             const Mpo& W = *ops[g];
             const bool real_op = probs[rep[g]].W != nullptr;
             const std::vector<int> alook = block_lookup(A, t);
+            std::vector<int> aright(A.bonds[t + 1].q.size() * 2, -1);   // (right sector, s_out) -> block of a
+            for (int bi = 0; bi < (int)A.blocks[t].size(); ++bi)
+                aright[A.blocks[t][bi].ri * 2 + A.blocks[t][bi].sigma] = bi;
             const int nch = W.bond_dim(t), nd = W.bond_dim(t + 1), n_ent = (int)W.entries[t].size();
             std::vector<std::vector<int>> by_chan(nch), by_d(nd);   // environment blocks / entries of a channel
             for (int e = 0; e < (int)E[g].size(); ++e) by_chan[E[g][e].c].push_back(e);
@@ -1579,38 +1580,50 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
                 if (me.a < nch && me.b < nd && !by_chan[me.a].empty()) by_d[me.b].push_back(ei);
             }
             const int gp = group_phase(g);
+            const int nrb = (int)B.bonds[t + 1].q.size();
+            head.assign((size_t)A.bonds[t + 1].q.size() * nrb * 2, -1);
+            tail.resize(head.size());
             for (int d = 0; d < nd; ++d) {
                 cs.clear();
+                touched.clear();
                 for (const int ei : by_d[d]) {
                     const MpoEntry& me = W.entries[t][ei];
                     for (const int e : by_chan[me.a]) {
                         const int ab = alook[E[g][e].ia * 2 + me.so], ti = tidx[g][e][me.si];
                         if (ab < 0 || ti < 0) continue;
-                        const uint64_t ra = (uint64_t)A.blocks[t][ab].ri, rb = (uint64_t)B.blocks[t][T[g][ti].bb].ri;
-                        cs.push_back({(ra << 42) | (rb << 21) | (uint64_t)ab, ti, ei});
+                        const int slot =
+                            (A.blocks[t][ab].ri * nrb + B.blocks[t][T[g][ti].bb].ri) * 2 + me.so;
+                        if (head[slot] < 0) {
+                            head[slot] = (int)cs.size();
+                            touched.push_back(slot);
+                        } else {
+                            cs[tail[slot]].next = (int)cs.size();
+                        }
+                        tail[slot] = (int)cs.size();
+                        cs.push_back({ti, ei, -1});
                     }
                 }
-                std::stable_sort(cs.begin(), cs.end(),
-                                 [](const Contrib& x, const Contrib& y) { return x.key < y.key; });
-                for (size_t i = 0; i < cs.size();) {
-                    const int ra = (int)(cs[i].key >> 42), rb = (int)((cs[i].key >> 21) & 0x1fffff);
-                    const uint64_t block = cs[i].key >> 21;
+                std::sort(touched.begin(), touched.end());
+                for (size_t i = 0; i < touched.size();) {
+                    const int block = touched[i] / 2, ra = block / nrb, rb = block % nrb;
                     const int rows = A.bonds[t + 1].dim[ra], cols = B.bonds[t + 1].dim[rb];
                     const int o = (int)outs.size();
                     outs.push_back({rows, cols, (int)runs.size(), 0, gp, nid, En_size[g]});
                     En[g].push_back({d, ra, rb, rows, cols, En_size[g]});
                     En_size[g] += (int64_t)rows * cols;
-                    while (i < cs.size() && (cs[i].key >> 21) == block) {
-                        const uint64_t key = cs[i].key;
-                        const Block& abk = A.blocks[t][(int)(key & 0x1fffff)];
-                        const int cbeg = (int)cons.size();
-                        for (; i < cs.size() && cs[i].key == key; ++i) {
-                            const int ei = cs[i].ei;
+                    for (; i < touched.size() && touched[i] / 2 == block; ++i) {
+                        const int so = touched[i] & 1, cbeg = (int)cons.size();
+                        // the block of a with this right sector and occupation
+                        const int ab = aright[ra * 2 + so];
+                        for (int c = head[touched[i]]; c >= 0; c = cs[c].next) {
+                            const int ei = cs[c].ei;
                             const MpoEntry& me = W.entries[t][ei];
                             const int sf =
                                 real_op && t == 0 && (ei == W.shift_entry[0] || ei == W.shift_entry[1]) ? 4 : 0;
-                            cons.push_back({T[g][cs[i].ti].off, me.w, me.so | (me.si << 1) | sf, 0});
+                            cons.push_back({T[g][cs[c].ti].off, me.w, me.so | (me.si << 1) | sf, 0});
                         }
+                        head[touched[i]] = -1;
+                        const Block& abk = A.blocks[t][ab];
                         runs.push_back({a_->core[t] + abk.off, 0, -1, abk.rows, cbeg, (int)cons.size(), t});
                     }
                     outs[o].end = (int)runs.size();
@@ -1640,9 +1653,10 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
         std::vector<double> one(1, 1.0);
         base[3] = s.up(one);
     }
-    double* res = s.dbl((size_t)P);
-    GridSync* gs = (GridSync*)ctx->alloc(sizeof(GridSync));
-    s.ptrs.push_back(gs);
+    // the results and, behind them, the sweep's phase word (one copy brings both back)
+    constexpr size_t kGs = sizeof(GridSync) / sizeof(double);
+    double* res = s.dbl((size_t)P + kGs);
+    GridSync* gs = (GridSync*)(res + P);
     BSM_CUDA(cudaMemsetAsync(gs, 0, sizeof(GridSync), ctx->stream));
     // bond K: the remaining 1x1 blocks of every problem
     const int fid = 1 + (K % 2);
@@ -1689,10 +1703,12 @@ static std::vector<double> dot_batch_impl(Context* ctx, const std::vector<EnvPro
         gh.assign((size_t)std::max<int64_t>(goff[P], 1), 0.0);
         BSM_CUDA(cudaMemcpyAsync(gh.data(), gd, sizeof(double) * gh.size(), cudaMemcpyDeviceToHost, ctx->stream));
     }
-    GridSync h;
-    BSM_CUDA(cudaMemcpyAsync(result.data(), res, sizeof(double) * P, cudaMemcpyDeviceToHost, ctx->stream));
-    BSM_CUDA(cudaMemcpyAsync(&h, gs, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+    std::vector<double> back((size_t)P + kGs);
+    BSM_CUDA(cudaMemcpyAsync(back.data(), res, sizeof(double) * back.size(), cudaMemcpyDeviceToHost, ctx->stream));
     ctx->sync();
+    GridSync h;
+    std::memcpy(&h, back.data() + P, sizeof(h));
+    std::copy(back.begin(), back.begin() + P, result.begin());
     BSM_REQUIRE(h.err == 0, BSMPS_ERR_TIMEOUT, "inner-product sweep: a grid-wide wait gave up");
     if (grams)
         for (int p = 0; p < P; ++p) (*grams)[p].assign(gh.begin() + goff[p], gh.begin() + goff[p + 1]);

@@ -7,8 +7,7 @@
 // What bounds it is the chain from one reflector to the next (two reductions, a
 // reciprocal square root and a reciprocal, the hand-over to the other CTAs), so
 // that chain runs ahead: in step j the owner of column j + 1 applies H_j to that
-// column first, forms H_{j+1} = I - tau v v^T (v = the column below row j + 1,
-// unscaled, v_{j+1} = sign(alpha) (|alpha| + n), tau = 1 / (n (n + |alpha|))) and
+// column first, forms H_{j+1} (dev::reflector_vector()) and
 // writes v, tau and v_{j+1} straight into every CTA's shared memory, while all
 // other warps of the cluster apply H_j to the columns beyond.  One cluster
 // barrier per column ends the step.  A column of a trailing update is worked on by
@@ -129,7 +128,7 @@ __global__ void __launch_bounds__(kQcThreads) k_qr_cluster(const QrTask* __restr
     cluster.sync();   // every CTA runs before the first reflector is written into it
     // sum over the chain's warps; slot: two reductions in a row use different slots
     auto chain_sum = [&](double v, int slot) {
-        v = dev::warp_sum(v);
+        v = dev::warp_sum_fixed(v);
         if (nch == 1) return v;
         if (lane == 0) part[slot][warp] = v;
         asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -169,12 +168,16 @@ __global__ void __launch_bounds__(kQcThreads) k_qr_cluster(const QrTask* __restr
         alpha = nch > 1 ? s_alpha : __shfl_sync(0xffffffffu, alpha, 0);
         double tj = 0.0, vd = -alpha;
         if (s != 0.0) {
-            const double w = fma(alpha, alpha, s);
-            const double rn = dev::rsqrt_halley(w);
-            const double n = w * rn, q = fabs(alpha) + n;
-            tj = rn * dev::recip_newton(q);
-            vd = alpha >= 0.0 ? q : -q;
-            if (t0 == 0) x[j] = alpha >= 0.0 ? -n : n;
+            double beta;
+            int shift;
+            dev::reflector_vector(alpha, s, &tj, &vd, &beta, &shift);
+            if (shift)
+                for (int i = j + t0; i < M; i += step) {   // the rows this thread wrote
+                    if (i == j) continue;
+                    x[i] = ldexp(x[i], -shift);
+                    for (int c = 0; c < C; ++c) cluster.map_shared_rank(dst, c)[i] = x[i];
+                }
+            if (t0 == 0) x[j] = beta;
         }
         if (t0 < C) {
             cluster.map_shared_rank(taus, t0)[j] = tj;

@@ -4,7 +4,9 @@
 // around the host's cut decision (right sweep).
 #include <algorithm>
 #include <cstring>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "dense_dev.cuh"
 #include "kernels.h"
@@ -729,14 +731,23 @@ void allow_smem(F* kern) {
     done.push_back((const void*)kern);
 }
 
-// Largest grid of `kern` whose CTAs are all resident at once (0: none).
+// Largest grid of `kern` whose CTAs are all resident at once (0: none).  The answer
+// depends on the kernel, the block and the device only, and is remembered.
 template <class F>
 int coresident_ctas(F* kern, int threads, size_t smem) {
-    int per_sm = 0, dev = 0, nsm = 0;
-    BSM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+    static std::mutex mu;
+    static std::map<std::tuple<const void*, int, int, size_t>, int> known;
+    int dev = 0;
     BSM_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    const auto key = std::make_tuple((const void*)kern, dev, threads, smem);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int per_sm = 0, nsm = 0;
+    BSM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    return per_sm * nsm;
+    if (known.size() > 4096) known.clear();
+    return known[key] = per_sm * nsm;
 }
 
 void count_launch(Context* ctx) {
