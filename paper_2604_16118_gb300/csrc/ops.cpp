@@ -879,7 +879,7 @@ struct RightPlan {
 // Jobs with a sector of this many kept columns or more leave the persistent
 // right sweep (one CTA per sector) for the per-site sweep, whose larger SVDs run
 // on thread-block clusters: one SM's FP64 rate bounds a one-CTA Jacobi.
-constexpr int kPersistentSvdMax = 40;
+constexpr int kPersistentSvdMax = 65;
 
 bool plan_right_sizes(const TruncJob& J, RightPlan& rp) {
     const Layout& L = J.L;
