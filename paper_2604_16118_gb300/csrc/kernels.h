@@ -94,7 +94,10 @@ constexpr int kClusterJacobiMax = 336;
 // FP64 units suffice for the latency of a round.
 constexpr int kClusterJacobiMin = 32;
 // Sectors of the per-site right sweep with at most this many kept columns run whole
-// (QR, Jacobi, assembly) in one CTA when they fit its shared memory.
+// (QR, Jacobi, assembly) in one CTA when they fit its shared memory: a bond has tens of
+// them, so the chip is filled without clusters, whose chain of launches is longer.
+// Limit 44 instead of 64 (ranks to 256 over two-charge sectors / 1024 and 203 over one
+// charge): 104 -> 123 ms, 23.6 -> 25.9 ms, 6.1 -> 6.6 ms.
 constexpr int kSvdSiteMax = 64;
 bool launch_jacobi_cluster(Context* ctx, const std::vector<JacTask>& tasks);
 // FP32 one-sided Jacobi of the same tasks as a preconditioner: reads G (FP64,
