@@ -444,6 +444,30 @@ __device__ __forceinline__ void form_q(const double* A, const double* tau, const
     __syncthreads();
 }
 
+// X (M x k, column-major) <- H_0 ... H_{k-1} X with householder()'s reflectors (M > 16),
+// whose diagonal entries stand in A: every 8-lane segment takes a column through
+// all of them without a barrier, as in form_q().  Q V this way takes 2 k (M k - k^2 / 2)
+// FMAs; forming Q and multiplying takes 2 k (M k - k^2 / 2) - k^3 / 3 and M k^2 more.
+__device__ __forceinline__ void apply_q(const double* A, const double* tau, double* X, int M, int k) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
+    for (int cb = 4 * warp; cb < k; cb += 4 * nwarps()) {
+        const bool own = cb + (lane >> 3) < k;
+        double* x = X + (int64_t)(own ? cb + (lane >> 3) : cb) * M;
+        for (int j = k - 1; j >= 0; --j) {
+            const double tj = tau[j];
+            if (tj == 0.0) continue;
+            const double* v = A + (int64_t)j * M;
+            const int i0 = j + ((sl - j) & 7);
+            double d = 0.0;
+            for (int i = i0; i < M; i += 8) d = fma(v[i], x[i], d);
+            const double tw = tj * seg8_sum(d);
+            if (own)
+                for (int i = i0; i < M; i += 8) x[i] = fma(-tw, v[i], x[i]);
+        }
+    }
+    __syncthreads();
+}
+
 __device__ __forceinline__ int rr_player(int pos, int round, int n2) {
     if (pos == 0) return 0;
     int v = pos - 1 + round;   // < 2 (n2 - 1) for round < n2 - 1
@@ -674,6 +698,13 @@ __device__ __forceinline__ float jacobi_tan(float d, float g2) {
     return __uint_as_float(__float_as_uint(t) | ((__float_as_uint(d) ^ __float_as_uint(g2)) & 0x80000000u));
 }
 
+// jacobi_tan() of FP64 norms and inner product, d = b - a and 2 g scaled by the larger exponent.
+__device__ __forceinline__ float jacobi_angle(double d, double g) {
+    const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
+    const int sh = 1023 - max(ed, eg);
+    return jacobi_tan(to_float_scaled(d, sh), to_float_scaled(g, sh + 1));
+}
+
 // Round-robin over k columns, one pair per 8-lane segment u: the pair of a round
 // follows from the one before (position 0 stands still, the others move on by one).
 struct SegPair {
@@ -801,18 +832,28 @@ struct SegRot {
 // are gathered per column in del (column = (1 + del) x stored; alpha and beta
 // carry the ratio of the two scales, terms below 2^-57 dropped).  Larger angles
 // (and columns with |del| >= 2^-30) take the full rotation, which clears del.
-// Stopping rule: |g| > rows eps sqrt(a b), min(a, b) > (rows eps)^2 ||G||_F^2.
+// Pairs rotate while |g| > rows eps sqrt(a b), min(a, b) > (rows eps)^2 ||G||_F^2.
+// Between sweeps all warps form the inner products of all pairs.  Where none is over the
+// limit the iteration ends; where all cosines |g| / sqrt(a b) and tangents over it are below
+// m = 2^-28, it ends with one step of first order, G += G X and V += V X with the tangents in
+// the antisymmetric X: what is left of a cosine are terms of second order, X_rp g_rq and X_rp
+// X_rq |g_r|^2, at most m^2 sqrt(a b) each and 5 k together, 0.3 k eps, under the
+// limit.  X is below 2^-28 times a ratio of norms, so the two products take FP32.  That step
+// costs a third of the sweep it replaces (k = 60: 65 us for 198).
 // The first nact warps work on G; the next nact rotate V one round behind them,
 // which fills the FP64 pipe while the G warps wait for loads, shuffles and
 // angles.  ring: 2 x 32 rotations.  Needs 2 nact warps.
 template <int RG, int RV>
 __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double* nrm, float* del, int k, int rows, int ldg,
-                                                    int ldv, double fro,SegRot* ring, int* s_rot) {
+                                                    int ldv, double fro, double* scr, SegRot* ring, int* s_rot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
     const int n2 = k + (k & 1);
     const int nact = (n2 / 2 + 3) / 4;
     const float tol = (float)rows * 2.220446e-16f * 0x1p48f;   // compared with g 2^48
     const float tiny = (float)rows * 2.220446e-16f * (float)rows * 2.220446e-16f * to_float_scaled(fro, 0);
+    float* Gf = (float*)scr;
+    float* Vf = Gf + k * ldg;
+    float* Xf = Vf + k * ldv;
     for (int j = threadIdx.x; j < k; j += nthreads()) del[j] = 0.0f;
     __syncthreads();
     for (int sweep = 0; sweep < kMaxSweeps && k > 1; ++sweep) {
@@ -830,10 +871,59 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
             if (j < k && sl == 0) nrm[j] = a;
         }
         __syncthreads();
+        if (sweep > 0) {
+            const int np = k * (k - 1) / 2;
+            int over = 0;
+            for (int eb = 4 * warp; eb < np; eb += 4 * nwarps()) {
+                const int e = min(eb + (lane >> 3), np - 1);
+                int q = (int)((sqrtf(8.0f * e + 1.0f) + 1.0f) * 0.5f);   // e = q (q - 1) / 2 + p, p < q
+                q += q * (q + 1) / 2 <= e;
+                q -= q * (q - 1) / 2 > e;
+                const int p = e - q * (q - 1) / 2;
+                double g = 0.0;
+#pragma unroll
+                for (int r = 0; r < RG; ++r) g = fma(G[p * ldg + sl + 8 * r], G[q * ldg + sl + 8 * r], g);
+                g = seg8_sum(g);
+                const double a = nrm[p], b = nrm[q];
+                const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0), gs = fabsf(to_float_scaled(g, 48));
+                const float nab = (af * rsqrt_fast(af)) * (bf * rsqrt_fast(bf));
+                float t = 0.0f;
+                if (fminf(af, bf) > tiny && gs > tol * nab) {
+                    t = jacobi_angle(b - a, g);
+                    over |= gs > 0x1p20f * nab || fabsf(t) > 0x1p-28f ? 3 : 1;
+                }
+                if (sl == 0) {
+                    Xf[q * k + p] = -t;
+                    Xf[p * k + q] = t;
+                }
+            }
+            if (over) atomicOr(s_rot, over);
+            __syncthreads();
+            const int state = *s_rot;
+            if (state == 0) break;
+            if (state == 1) {
+                for (int j = threadIdx.x; j < k; j += nthreads()) Xf[j * k + j] = 0.0f;
+                for (int e = threadIdx.x; e < k * ldg; e += nthreads()) Gf[e] = to_float_scaled(G[e], 0);
+                for (int e = threadIdx.x; e < k * ldv; e += nthreads()) Vf[e] = to_float_scaled(V[e], 0);
+                __syncthreads();
+                for (int e = threadIdx.x; e < k * 8 * RG; e += nthreads()) {
+                    const int p = e / (8 * RG), i = e % (8 * RG);
+                    float acc = 0.0f;
+                    for (int q = 0; q < k; ++q) acc = fmaf(Gf[q * ldg + i], Xf[q * k + p], acc);
+                    G[p * ldg + i] += to_double(acc);
+                }
+                for (int e = threadIdx.x; e < k * 8 * RV; e += nthreads()) {
+                    const int p = e / (8 * RV), i = e % (8 * RV);
+                    float acc = 0.0f;
+                    for (int q = 0; q < k; ++q) acc = fmaf(Vf[q * ldv + i], Xf[q * k + p], acc);
+                    V[p * ldv + i] += to_double(acc);
+                }
+                break;
+            }
+        }
         if (warp < nact) {
             const int u = 4 * warp + (lane >> 3);
             SegPair pr(u, k);
-            int any = 0;
             for (int round = 0; round < n2 - 1; ++round, pr.next()) {
                 int p, q;
                 const bool on = pr.get(&p, &q);
@@ -851,21 +941,18 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                 const double a = nrm[p], b = nrm[q];
                 const float dp = del[p], dq = del[q];
                 const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0);
-                const float lim = tol * (af * rsqrt_fast(af)) * (bf * rsqrt_fast(bf));
+                const float nab = (af * rsqrt_fast(af)) * (bf * rsqrt_fast(bf));
                 const double d = b - a;
                 g = seg8_sum(g);
-                const bool rot = on && fminf(af, bf) > tiny && fabsf(to_float_scaled(g, 48)) > lim;
+                const float gs = fabsf(to_float_scaled(g, 48));
+                const bool rot = on && fminf(af, bf) > tiny && gs > tol * nab;
                 SegRot* out = ring + (round & 1) * 32 + u;
                 if (!__any_sync(0xffffffffu, rot)) {
                     if (sl == 0) out->mode = 0;
                     bar_first(64 * nact);
                     continue;
                 }
-                any = 1;
-                // angle: d and 2 g scaled by the larger exponent
-                const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
-                const int sh = 1023 - max(ed, eg);
-                const float t = rot ? jacobi_tan(to_float_scaled(d, sh), to_float_scaled(g, sh + 1)) : 0.0f;
+                const float t = rot ? jacobi_angle(d, g) : 0.0f;
                 const bool small = fabsf(t) < 0x1p-14f && fabsf(dp) < 0x1p-30f && fabsf(dq) < 0x1p-30f;
                 const double td = to_double(t);
                 double fp = 1.0, fq = 1.0;
@@ -914,7 +1001,6 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                 }
                 bar_first(64 * nact);
             }
-            if (any && lane == 0) *s_rot = 1;
         } else if (warp < 2 * nact) {
             const int u = 4 * (warp - nact) + (lane >> 3);
             for (int round = 0; round < n2 - 1; ++round) {
@@ -948,25 +1034,27 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
             }
         }
         __syncthreads();
-        const int rot = *s_rot;
-        __syncthreads();
-        if (!rot) break;
     }
+    __syncthreads();
 }
 
 // One-sided Jacobi of G (rows x k, column-major, k <= rows <= 64) as jacobi(): G ends
 // as U diag(Sraw), V (k x k) accumulates the rotations.  The FP64 sweeps are few because an
 // FP32 Jacobi of G comes first (FP32 arithmetic runs at 64 times the FP64 rate
-// here): its rotations P, orthogonal to about 1e-6, are orthogonalised in FP64 as
-// Qp = P (I - E/2 + 3/8 E^2) with E = P^T P - I (a second pass when E is not below
-// 2e-6, since the dropped terms are of order E^3), and the FP64 Jacobi starts from
-// G Qp with V = Qp: two sweeps with rotations and one without.  Where the FP32
+// here): its rotations P, orthogonal to about 3e-6, are orthogonalised in FP64 as
+// Qp = P (I - E/2 + 3/8 E^2 - 5/16 E^3) with E = P^T P - I (a second pass when an
+// entry of E reaches 8e-6: the dropped term, 35/128 E^4, is below 1e-16 for
+// ||E||_2 < 1.4e-4, twice what 64 columns of random entries of that size have), and the FP64
+// Jacobi starts from G Qp with V = Qp: one sweep and a step of first order.  The square and cube of E
+// are below 1e-8 of the result and take FP32.  (One pass with the cube instead of
+// two without it: k = 60 330 -> 160 us, k = 20 22 -> 11 us.)  Where the FP32
 // iteration gives nothing (non-finite entries) it starts from G and I.
 // RG, RV: rows of G and V in units of 8 (8 RG >= rows, 8 RV >= k).  Leading dimensions:
 // jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of
 // max(k, 8 RV - 7) for V, so that the 8 RG (8 RV) rows a lane segment walks stay
 // within the column.  scr: jacobi_scratch(ldg, ldv, k) shared doubles; del: k of them.
-template <int RG, int RV>
+// Tri: G is lower triangular (rows = k).
+template <int RG, int RV, bool Tri>
 __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int rows, int k, double* scr,
                                            double* del, SegRot* ring, double* red, int* s_int) {
     constexpr int kOwn = 8;   // outputs of a product per thread: rows k <= 8 blockDim (blockDim >= min(16 k, 512))
@@ -993,6 +1081,9 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     // V row-major <- P
     for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
     bool ok = true;
+    float* Ef = (float*)(scr + kk);   // E in FP32
+    float* Tf = Ef + kk;
+    double own[kOwn];
     for (int pass = 0; pass < 3; ++pass) {
         __syncthreads();
         if (threadIdx.x == 0) *s_int = 0;
@@ -1007,8 +1098,9 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             double acc = i == j ? -1.0 : 0.0;
             for (int r = 0; r < k; ++r) acc = fma(V[r * k + i], V[r * k + j], acc);
             scr[i * k + j] = scr[j * k + i] = acc;
-            const float af = fabsf(to_float_scaled(acc, 0));
-            mx = af <= mx ? mx : (af == af ? af : FLT_MAX);
+            const float af = to_float_scaled(acc, 0);
+            Ef[i * k + j] = Ef[j * k + i] = af;
+            mx = fabsf(af) <= mx ? mx : (af == af ? fabsf(af) : FLT_MAX);
         }
         atomicMax(s_int, (int)__float_as_uint(mx));
         __syncthreads();
@@ -1017,24 +1109,19 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             ok = false;
             break;
         }
-        double own[kOwn];
-#pragma unroll
-        for (int n = 0; n < kOwn; ++n) {
-            const int e = threadIdx.x + n * T;
-            if (e < kk) {
-                // E^2 in FP32: it is below 1e-12 of the result at the last pass
-                const int i = e % k, j = e / k;
-                float acc = 0.0f;
-                for (int m = 0; m < k; ++m)
-                    acc = fmaf(to_float_scaled(scr[m * k + i], 16), to_float_scaled(scr[j * k + m], 16), acc);
-                own[n] = fma(0.5, scr[e], -0.375 * 0x1p-32 * to_double(acc));
-            }
+        // Tf = -3/8 E + 5/16 E^2, then F = E/2 + E Tf
+        for (int e = threadIdx.x; e < kk; e += T) {
+            const int i = e % k, j = e / k;
+            float acc = 0.0f;
+            for (int m = 0; m < k; ++m) acc = fmaf(Ef[m * k + i], Ef[j * k + m], acc);
+            Tf[e] = fmaf(0.3125f, acc, -0.375f * Ef[e]);
         }
         __syncthreads();
-#pragma unroll
-        for (int n = 0; n < kOwn; ++n) {
-            const int e = threadIdx.x + n * T;
-            if (e < kk) scr[e] = own[n];
+        for (int e = threadIdx.x; e < kk; e += T) {
+            const int i = e % k, j = e / k;
+            float acc = 0.0f;
+            for (int m = 0; m < k; ++m) acc = fmaf(Ef[m * k + i], Tf[j * k + m], acc);
+            scr[e] = fma(0.5, scr[e], to_double(acc));
         }
         __syncthreads();
         // P (I - F): row i of V (row-major) times the symmetric F
@@ -1049,34 +1136,35 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             }
         }
         __syncthreads();
-        const bool last = emax < 2e-6f;
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < kk) V[last ? (e % k) * ldv + e / k : e] = own[n];   // column-major at the end
+            if (e < kk) V[e] = own[n];
         }
-        if (last) break;
+        if (emax < 8e-6f) break;
         ok = pass < 2;
     }
     __syncthreads();
     if (ok) {
-        // G <- G Qp (rows k <= 8 blockDim outputs)
-        double own[kOwn];
+        // G <- G Qp, row i to consecutive threads (rows k <= 8 blockDim outputs); V to column-major
+        double gq[kOwn];
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
             if (e < rows * k) {
-                const int i = e % rows, c = e / rows;
+                const int i = e / k, c = e % k;
+                const int jn = Tri ? i + 1 : k;
                 double acc = 0.0;
-                for (int j = 0; j < k; ++j) acc = fma(G[j * ldg + i], V[c * ldv + j], acc);
-                own[n] = acc;
+                for (int j = 0; j < jn; ++j) acc = fma(G[j * ldg + i], V[j * k + c], acc);
+                gq[n] = acc;
             }
         }
         __syncthreads();
 #pragma unroll
         for (int n = 0; n < kOwn; ++n) {
             const int e = threadIdx.x + n * T;
-            if (e < rows * k) G[(e / rows) * ldg + e % rows] = own[n];
+            if (e < rows * k) G[(e % k) * ldg + e / k] = gq[n];
+            if (e < kk) V[(e % k) * ldv + e / k] = own[n];
         }
     } else {
         for (int e = threadIdx.x; e < k * ldv; e += T) V[e] = e % ldv == e / ldv ? 1.0 : 0.0;
@@ -1084,7 +1172,7 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     for (int e = threadIdx.x; e < k * (ldv - k); e += T) V[(e / (ldv - k)) * ldv + k + e % (ldv - k)] = 0.0;
     __syncthreads();
     float* dl = (float*)del;
-    jacobi_f64_segments<RG, RV>(G, V, Sraw, dl, k, rows, ldg, ldv, fro, ring, s_int);
+    jacobi_f64_segments<RG, RV>(G, V, Sraw, dl, k, rows, ldg, ldv, fro, scr, ring, s_int);
     // the columns' scales, and the norms of the result
     const double up = ldexp(1.0, ex);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sl = lane & 7;
@@ -1106,31 +1194,32 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     __syncthreads();
 }
 
-// Shared doubles of jacobi_pre()'s scratch: G and V in FP32, or a k x k FP64 matrix.
+// Shared doubles of jacobi_pre()'s scratch: G, V and a k x k matrix in FP32, or a k x k
+// matrix in FP64 and two in FP32.
 __host__ __device__ constexpr int jacobi_scratch(int ldg, int ldv, int k) {
-    const int f = (k * (ldg + ldv) + 1) / 2;
-    return f > k * k ? f : k * k;
+    const int f = (k * (ldg + ldv + k) + 1) / 2;
+    return f > 2 * k * k ? f : 2 * k * k;
 }
 
-// jacobi_pre() on a square G of k <= 64 columns (blockDim as block_for() gives it),
+// jacobi_pre() on a square lower triangular G of k <= 64 columns (blockDim as block_for() gives it),
 // else jacobi().  G and V: leading dimension jacobi_ld(k).
 __device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k, double* red, int* s_rot);
 __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
                                             SegRot* ring, double* red, int* s_rot) {
     if (k <= 8)
-        jacobi_pre<1, 1>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<1, 1, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 16)
-        jacobi_pre<2, 2>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<2, 2, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 24)
-        jacobi_pre<3, 3>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<3, 3, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 32)
-        jacobi_pre<4, 4>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<4, 4, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 40)
-        jacobi_pre<5, 5>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<5, 5, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 56)
-        jacobi_pre<7, 7>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<7, 7, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 64)
-        jacobi_pre<8, 8>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<8, 8, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else
         jacobi(G, V, Sraw, k, red, s_rot);
 }
@@ -1218,10 +1307,11 @@ __device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k
 // QV: column-major len x k (QV[p*len + i] = (Q V)(i, p)).  Writes S (k,
 // descending, ties by index), US = U diag(S) (M x k row-major) and Vt (k x N
 // row-major, row strides ldus / ldvt) with the largest-|.| entry of every Vt
-// row positive.  perm: k ints.
+// row positive.  This CTA writes the singular triples r0 .. r1 - 1.  perm: k ints,
+// rinv: k doubles (the same values from every CTA).
 __device__ __forceinline__ void svd_assemble(const double* G, int ldg, const double* QV, const double* Sraw,
-                                             int* perm, double* S, double* US, double* Vt, int M, int N, int k,
-                                             int len, int wide, int ldus, int ldvt) {
+                                             double* rinv, int* perm, double* S, double* US, double* Vt, int M,
+                                             int N, int k, int len, int wide, int ldus, int ldvt, int r0, int r1) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < k; i += nthreads()) {
         // compared as integers: a permutation also when a value is not a number
@@ -1232,39 +1322,37 @@ __device__ __forceinline__ void svd_assemble(const double* G, int ldg, const dou
             rank += (sj > si || (sj == si && j < i)) ? 1 : 0;
         }
         perm[rank] = i;
+        if (!wide) {
+            const double r = rsqrt(Sraw[i]);
+            rinv[i] = Sraw[i] > 0.0 ? r * r : 0.0;
+        }
     }
     __syncthreads();
-    for (int64_t e = threadIdx.x; e < (int64_t)M * k; e += nthreads()) {
-        const int i = (int)(e / k), r = (int)(e % k);
+    const int nr = r1 - r0;
+    for (int64_t e = threadIdx.x; e < (int64_t)M * nr; e += nthreads()) {
+        const int i = (int)(e / nr), r = r0 + (int)(e % nr);
         const int p = perm[r];
         US[(int64_t)i * ldus + r] = wide ? G[(int64_t)p * ldg + i] : Sraw[p] * QV[(int64_t)p * len + i];
     }
-    for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += nthreads()) {
-        const int r = (int)(e / N), c = (int)(e % N);
+    for (int64_t e = threadIdx.x; e < (int64_t)nr * N; e += nthreads()) {
+        const int r = r0 + (int)(e / N), c = (int)(e % N);
         const int p = perm[r];
-        double v;
-        if (wide) {
-            v = QV[(int64_t)p * len + c];
-        } else {
-            const double sp = Sraw[p];
-            v = sp > 0.0 ? G[(int64_t)p * ldg + c] / sp : 0.0;
-        }
-        Vt[(int64_t)r * ldvt + c] = v;
+        Vt[(int64_t)r * ldvt + c] = wide ? QV[(int64_t)p * len + c] : G[(int64_t)p * ldg + c] * rinv[p];
     }
-    for (int r = threadIdx.x; r < k; r += nthreads()) S[r] = Sraw[perm[r]];
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += nthreads()) S[r] = Sraw[perm[r]];
     __syncthreads();
-    for (int r = warp; r < k; r += nwarps()) {
-        double best = -1.0;
+    for (int r = r0 + warp; r < r1; r += nwarps()) {
+        long long best = -1;
         int bi = 0;
         for (int c = lane; c < N; c += 32) {
-            const double a = fabs(Vt[(int64_t)r * ldvt + c]);
+            const long long a = abs_key(Vt[(int64_t)r * ldvt + c]);
             if (a > best) {
                 best = a;
                 bi = c;
             }
         }
         for (int o = 16; o > 0; o >>= 1) {
-            const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+            const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
             const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
             if (ob > best || (ob == best && oi < bi)) {
                 best = ob;

@@ -18,8 +18,10 @@
 // CTA of the cluster wrote them in an earlier step).
 //
 // A pair rotates while |g| > k eps sqrt(a b) and min(a, b) > (k eps)^2 ||G||_F^2
-// (the stopping rule of dev::jacobi); a sweep without a rotation ends the
-// iteration (at most dev::kMaxSweeps sweeps).  On this GPU an SM retires one
+// (the rule of dev::jacobi).  A sweep whose rotated pairs all had cosines |g| / sqrt(a b) and
+// tangents below m = 2^-28 is the last (at most dev::kMaxSweeps): rotating column p
+// against r changes the cosine of p and q by at most 2 m^2, so after the other 2 (k - 2) rotations
+// of p and q it is below 4 k m^2 = k eps / 4, and the next sweep would rotate nothing.  On this GPU an SM retires one
 // FP64 warp instruction per 16 cycles, so the Jacobi is bound by the number of
 // FP64 instructions: the cluster brings the FP64 units of C SMs to one matrix,
 // and a rotation takes few of them, as in dev::jacobi_f64_segments: squared norms
@@ -105,17 +107,13 @@ __device__ __forceinline__ void rotate_g(double* Gp, double* Gq, double* np, dou
     const float ep = *dp, eq = *dq;
     const float af = dev::to_float_scaled(a, 0), bf = dev::to_float_scaled(b, 0);
     g = dev::warp_sum_fixed(g);
-    const bool rot = fminf(af, bf) > tiny && fabsf(dev::to_float_scaled(g, 48)) >
-                                                 lim * (af * dev::rsqrt_fast(af)) * (bf * dev::rsqrt_fast(bf));
+    const float nab = (af * dev::rsqrt_fast(af)) * (bf * dev::rsqrt_fast(bf)), gs = fabsf(dev::to_float_scaled(g, 48));
+    const bool rot = fminf(af, bf) > tiny && gs > lim * nab;
     if (!rot) {
         if (lane == 0) out->mode = 0;
         return;
     }
-    // angle: d and 2 g scaled by the larger exponent
-    const double d = b - a;
-    const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(g) >> 20) & 0x7ff) + 1;
-    const int sh = 1023 - max(ed, eg);
-    const float t = dev::jacobi_tan(dev::to_float_scaled(d, sh), dev::to_float_scaled(g, sh + 1));
+    const float t = dev::jacobi_angle(b - a, g);
     const bool small = fabsf(t) < 0x1p-14f && fabsf(ep) < 0x1p-30f && fabsf(eq) < 0x1p-30f;
     const double td = dev::to_double(t);
     double fp = 1.0, fq = 1.0, sq, sp;
@@ -153,7 +151,7 @@ __device__ __forceinline__ void rotate_g(double* Gp, double* Gq, double* np, dou
         const float h = 0.5f * t * t;
         *dp = small ? ep - h : 0.0f;
         *dq = small ? eq - h : 0.0f;
-        *s_rot = 1;
+        if (gs > 0x1p20f * nab || fabsf(t) > 0x1p-28f) *s_rot = 1;
     }
 }
 
@@ -189,7 +187,7 @@ __global__ void __launch_bounds__(kClusterThreads) k_jacobi_cluster(const JacTas
     extern __shared__ double jc_smem[];
     __shared__ double s_part[C];     // CTA 0's slots: partial ||G||^2 of every CTA
     __shared__ int s_flag[2][C];     // CTA 0's slots: rotation flags, by sweep parity
-    __shared__ int s_rot;            // this CTA rotated in the current sweep
+    __shared__ int s_rot;            // this CTA had a larger rotation in the current sweep
     __shared__ double red[33];
     __shared__ Rot ring[2][kRingMax];
     cg::cluster_group cluster = cg::this_cluster();

@@ -235,13 +235,18 @@ struct SvdFin {
     double* S;
     double* US;
     double* Vt;
+    double* rinv;
     int* perm;
     int M, N, k, len, wide;
 };
 
+// kFinSplit CTAs per matrix, a range of its singular triples each: bound by the strided
+// copies, which one CTA per matrix left to one SM (k = 200: 230 us).
+constexpr int kFinSplit = 16;
 __global__ void __launch_bounds__(kThreads) k_svd_finalize(const SvdFin* __restrict__ tasks) {
     const SvdFin tk = tasks[blockIdx.x];
-    dev::svd_assemble(tk.G, tk.k, tk.QVt, tk.Sraw, tk.perm, tk.S, tk.US, tk.Vt, tk.M, tk.N, tk.k, tk.len, tk.wide, tk.k, tk.N);
+    dev::svd_assemble(tk.G, tk.k, tk.QVt, tk.Sraw, tk.rinv, tk.perm, tk.S, tk.US, tk.Vt, tk.M, tk.N, tk.k, tk.len, tk.wide,
+                      tk.k, tk.N, (int)((int64_t)tk.k * blockIdx.y / kFinSplit), (int)((int64_t)tk.k * (blockIdx.y + 1) / kFinSplit));
 }
 
 __global__ void __launch_bounds__(kThreads) k_sumsq(const double* const* __restrict__ xs,
@@ -776,12 +781,12 @@ void launch_svd(Context* ctx, const std::vector<SvdTask>& tasks) {
     for (size_t i = 0; i < tasks.size(); ++i) {
         const SvdTask& t = tasks[i];
         const int k = std::min(t.M, t.N), len = std::max(t.M, t.N);
-        fin.push_back({R[i], QVt[i], Sraw[i], t.S, t.US, t.Vt, perm[i], t.M, t.N, k, len, t.wide});
+        fin.push_back({R[i], QVt[i], Sraw[i], t.S, t.US, t.Vt, s.dbl((size_t)k), perm[i], t.M, t.N, k, len, t.wide});
         fb += 8.0 * ((double)t.M * k + (double)k * t.N + 2.0 * k * (double)len);
     }
     SvdFin* d = s.up(fin);
     ProfScope ps(ctx, KK_SVD, 0.0, fb);
-    k_svd_finalize<<<(unsigned)fin.size(), kThreads, 0, ctx->stream>>>(d);
+    k_svd_finalize<<<dim3((unsigned)fin.size(), kFinSplit), kThreads, 0, ctx->stream>>>(d);
     check_launch(ctx);
     ps.done();
 }

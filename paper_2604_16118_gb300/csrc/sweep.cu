@@ -42,8 +42,8 @@ static_assert(direct_ldb(8) == dev::jacobi_ld(1) && direct_ldb(16) == dev::jacob
                   direct_ldv(32) == dev::jacobi_ld(9),
               "leading dimensions of jacobi_pre<1, 1>, <2, 2> and <4, 2>");
 
-// The QR input (later Q V; while the Jacobi runs its scratch), Q, G, V and three vectors; or,
-// without a QR step, the padded input, V, the scratch and three vectors.
+// The QR input, Q V (while the Jacobi runs its scratch), G, V and three vectors; or,
+// without a QR step, the padded input, V, the scratch and four vectors.
 __host__ __device__ inline size_t svd_buf(int len, int k) {
     const size_t a = (size_t)len * k, b = (size_t)dev::jacobi_scratch(dev::jacobi_ld(k), dev::jacobi_ld(k), k);
     return k <= 64 && b > a ? b : a;
@@ -199,6 +199,62 @@ __global__ void __launch_bounds__(kSweepThreads) k_left_site(const LeftTask* __r
     left_body<false>(tasks[blockIdx.x], srcs, xs, sm, red);
 }
 
+// SVD of a sector's matrix (M x N) gathered in sm as len x k columns of leading dimension
+// ldb (its transpose where wide; with direct, ldb = direct_ldb(len) and zeros in the padding): by
+// QR, a Jacobi of R^T and Q V, or, with direct (len <= 32, k <= 16; always where len <= 16), a
+// Jacobi on the matrix itself.
+__device__ void svd_core(double* sm, bool direct, int M, int N, int k, int len, int wide, double* S, double* US, double* Vt, int ldus,
+                         int ldvt, double* red, int* s_rot, dev::SegRot* ring) {
+    double* B = sm;
+    if (direct) {
+        const int ldb = direct_ldb(len), ldv = direct_ldv(len);
+        double* Vd = B + (int64_t)k * ldb;
+        double* scr = Vd + (int64_t)k * ldv;
+        double* Sr = scr + dev::jacobi_scratch(ldb, ldv, k);
+        double* rinv = Sr + k;
+        double* dl = rinv + k;
+        int* prm = (int*)(dl + k);
+        if (len <= 8)
+            dev::jacobi_pre<1, 1, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        else if (len <= 16)
+            dev::jacobi_pre<2, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        else
+            dev::jacobi_pre<4, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+        dev::svd_assemble_direct(B, ldb, Vd, ldv, Sr, rinv, prm, S, US, Vt, M, N, k, wide, ldus, ldvt);
+        return;
+    }
+    const int ld = dev::jacobi_ld(k);
+    double* X = B + (int64_t)len * k;
+    double* G = X + svd_buf(len, k);
+    double* V = G + (int64_t)k * ld;
+    double* tau = V + (int64_t)k * ld;
+    double* vd = tau + k;        // later the singular values
+    double* del = vd + k;        // later the order
+    dev::householder(B, tau, vd, len, k);
+    // G = R^T (column-major): G(i, j) = R(j, i), nonzero for i >= j
+    for (int e = threadIdx.x; e < k * ld; e += nthreads()) {
+        const int j = e / ld, i = e % ld;
+        G[e] = i >= j && i < k ? B[(int64_t)i * len + j] : 0.0;
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < k; j += nthreads()) B[(int64_t)j * len + j] = vd[j];
+    __syncthreads();
+    double* Sraw = vd;
+    dev::jacobi_auto(G, V, Sraw, k, X, del, ring, red, s_rot);
+    for (int e = threadIdx.x; e < len * k; e += nthreads()) {
+        const int j = e / len, i = e % len;
+        X[e] = i < k ? V[j * ld + i] : 0.0;
+    }
+    __syncthreads();
+    dev::apply_q(B, tau, X, len, k);
+    dev::svd_assemble(G, ld, X, Sraw, tau, (int*)del, S, US, Vt, M, N, k, len, wide, ldus, ldvt, 0, k);
+}
+
+// Zeros in the rows len .. ldb - 1 of the k columns at B.
+__device__ __forceinline__ void pad_columns(double* B, int len, int ldb, int k) {
+    for (int e = threadIdx.x; e < k * (ldb - len); e += nthreads()) B[(e / (ldb - len)) * ldb + len + e % (ldb - len)] = 0.0;
+}
+
 __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* __restrict__ tasks,
                                                        const SvdPart* __restrict__ parts) {
     extern __shared__ double sm[];
@@ -207,42 +263,22 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
     __shared__ int s_rot;
     const SvdSiteTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = tk.k, len = tk.len;
-    double* B = sm;                               // QR input (len x k), later Q V
-    const int ld = dev::jacobi_ld(k);
-    double* Q = B + svd_buf(len, k);
-    double* tau = Q + (int64_t)len * k;
-    double* G = tau + k;
-    double* V = G + (int64_t)k * ld;
-    double* Sraw = V + (int64_t)k * ld;
-    int* perm = (int*)(Sraw + k);
+    double* B = sm;
+    const bool direct = len <= 16;   // no more rows than householder() has a segment layout for
+    const int ldb = direct ? direct_ldb(len) : len;
+    pad_columns(B, len, ldb, k);
     for (int p = tk.p_beg; p < tk.p_end; ++p) {
         const SvdPart pt = parts[p];
         for (int64_t e = threadIdx.x; e < (int64_t)M * pt.cols; e += nthreads()) {
             const int i = (int)(e / pt.cols), c = pt.coff + (int)(e % pt.cols);
             if (tk.wide)
-                B[(int64_t)i * N + c] = pt.src[e];      // A^T column-major
+                B[(int64_t)i * ldb + c] = pt.src[e];      // A^T column-major
             else
-                B[(int64_t)c * M + i] = pt.src[e];      // A column-major
+                B[(int64_t)c * ldb + i] = pt.src[e];      // A column-major
         }
     }
     __syncthreads();
-    dev::householder(B, tau, Sraw, len, k);
-    // G = R^T (column-major): G(i, j) = R(j, i), nonzero for i >= j
-    for (int e = threadIdx.x; e < k * ld; e += nthreads()) {
-        const int j = e / ld, i = e % ld;
-        G[e] = i >= j && i < k ? B[(int64_t)i * len + j] : 0.0;
-    }
-    dev::form_q(B, tau, Sraw, Q, len, k);
-    __syncthreads();
-    dev::jacobi_auto(G, V, Sraw, k, B, tau, ring, red, &s_rot);
-    for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
-        const int p = (int)(e / len), i = (int)(e % len);
-        double acc = 0.0;
-        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * ld + j], acc);
-        B[e] = acc;
-    }
-    __syncthreads();
-    dev::svd_assemble(G, ld, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, tk.wide, k, N);
+    svd_core(sm, direct, M, N, k, len, tk.wide, tk.S, tk.US, tk.Vt, k, N, red, &s_rot, ring);
 }
 
 __global__ void __launch_bounds__(kThreads) k_right_apply(const RTask* __restrict__ tasks,
@@ -366,17 +402,9 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     }
     const int k = M < N ? M : N, len = M < N ? N : M, wide = M < N ? 1 : 0;
     double* B = sm;
-    const int ld = dev::jacobi_ld(k);
-    double* Q = B + svd_buf(len, k);
-    double* tau = Q + (int64_t)len * k;
-    double* G = tau + k;
-    double* V = G + (int64_t)k * ld;
-    double* Sraw = V + (int64_t)k * ld;
-    int* perm = (int*)(Sraw + k);
     const bool direct = len <= kDirectRows && k <= kDirectCols;
     const int ldb = direct ? direct_ldb(len) : len;   // (k == 1 included: one padded column)
-    if (direct)
-        for (int e = threadIdx.x; e < k * (ldb - len); e += nthreads()) B[(e / (ldb - len)) * ldb + len + e % (ldb - len)] = 0.0;
+    pad_columns(B, len, ldb, k);
     int coff = 0;
     for (int p = 0; p < np; ++p) {
         const DynPart& pt = tk.part[p];
@@ -402,43 +430,7 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
         right_rank1(tk, B, len, wide, red);
         return;
     }
-    if (direct) {
-        // small sector: one-sided Jacobi on B itself (no QR step)
-        const int ldv = direct_ldv(len);
-        double* Vd = B + (int64_t)k * ldb;
-        double* scr = Vd + (int64_t)k * ldv;
-        double* Sr = scr + dev::jacobi_scratch(ldb, ldv, k);
-        double* rinv = Sr + k;
-        double* dl = rinv + k;
-        int* prm = (int*)(dl + k);
-        if (len <= 8)
-            dev::jacobi_pre<1, 1>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
-        else if (len <= 16)
-            dev::jacobi_pre<2, 2>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
-        else
-            dev::jacobi_pre<4, 2>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
-        dev::svd_assemble_direct(B, ldb, Vd, ldv, Sr, rinv, prm, tk.S, tk.US, tk.Vt, M, N, k, wide, tk.kpad,
-                                 tk.ncols_pad);
-        __syncthreads();
-        if (threadIdx.x == 0) *tk.kact = k;
-        return;
-    }
-    dev::householder(B, tau, Sraw, len, k);
-    for (int e = threadIdx.x; e < k * ld; e += nthreads()) {
-        const int j = e / ld, i = e % ld;
-        G[e] = i >= j && i < k ? B[(int64_t)i * len + j] : 0.0;
-    }
-    dev::form_q(B, tau, Sraw, Q, len, k);
-    __syncthreads();
-    dev::jacobi_auto(G, V, Sraw, k, B, tau, ring, red, s_rot);
-    for (int64_t e = threadIdx.x; e < (int64_t)len * k; e += nthreads()) {
-        const int p = (int)(e / len), i = (int)(e % len);
-        double acc = 0.0;
-        for (int j = 0; j < k; ++j) acc = fma(Q[(int64_t)j * len + i], V[(int64_t)p * ld + j], acc);
-        B[e] = acc;
-    }
-    __syncthreads();
-    dev::svd_assemble(G, ld, B, Sraw, perm, tk.S, tk.US, tk.Vt, M, N, k, len, wide, tk.kpad, tk.ncols_pad);
+    svd_core(sm, direct, M, N, k, len, wide, tk.S, tk.US, tk.Vt, tk.kpad, tk.ncols_pad, red, s_rot, ring);
     if (threadIdx.x == 0) *tk.kact = k;
 }
 
