@@ -102,3 +102,42 @@ def test_zero_iterate(nat, ctx):
     z = nat.mps_create(ctx, wl.n_orb, 0, wl.n_up, 0, 110, np.zeros(n_random(wl, 110)))
     y, dt, _ = nat.truncate(ctx, z, 0.0)
     assert dt == 0.0 and np.all(np.isfinite(y.export()))
+
+
+def with_spectrum(x, t, s_of):
+    """x with the singular values of bond t replaced: sector q of width d takes s_of(d)."""
+    rc, _, _ = OB.truncate(x, 0.0)                 # right-orthogonal
+    lc = OB.left_orthogonalize(rc)
+    assert lc.bonds == rc.bonds == x.bonds
+    rng = np.random.default_rng(7)
+    cores = [dict(c) for c in lc.cores[:t]] + [dict(c) for c in rc.cores[t:]]
+    for q, d in x.bonds[t].items():
+        u, _ = np.linalg.qr(rng.standard_normal((d, d)))
+        v, _ = np.linalg.qr(rng.standard_normal((d, d)))
+        C = (u * s_of(d)) @ v.T
+        for key in cores[t]:
+            if key[0] == q:
+                cores[t][key] = C @ cores[t][key]
+    return OB.BSMPS(x.species, x.target, x.bonds, cores)
+
+
+@pytest.mark.parametrize("K,N", [(8, 4), (12, 6), (14, 7)])
+@pytest.mark.parametrize("gap", [0.0, 1e-13, 1e-9, 1e-5])
+def test_nearly_equal_singular_values(nat, ctx, K, N, gap):
+    """Pairs of values a relative gap apart: rotations by large angles in the last sweeps, which a
+    step of first order must not stand in for.  Nothing is cut: the tensor stays, and every core
+    right of the first has orthonormal rows to k^2 eps (cosines up to k eps, k < 64)."""
+    wl = spinless_random_chain(K=K, N=N, seed=2)
+    r = 4096
+    vals = random_block_values(n_random(wl, r), 9)
+    ox = with_spectrum(oracle_random(wl, r, vals), K // 2,
+                       lambda d: 10.0 ** (-0.3 * (np.arange(d) // 2)) * (1.0 + gap * (np.arange(d) % 2)))
+    x = nat.mps_create(ctx, wl.n_orb, wl.spin, wl.n_up, wl.n_dn, r, ox.to_flat())
+    y, dt, _ = nat.truncate(ctx, x, 0.0)
+    oy = to_oracle(wl, y)
+    assert dt == 0.0 and oy.bonds == ox.bonds
+    assert rel_distance(oy, ox) <= 1e-12
+    for t in range(1, K):
+        for q, d in oy.bonds[t].items():
+            rows = np.hstack([B for key, B in oy.cores[t].items() if key[0] == q])
+            assert np.linalg.norm(rows @ rows.T - np.eye(d)) <= 1e-12
