@@ -478,7 +478,7 @@ BSMPS_API bsmps_status bsmps_eigensolve_step(bsmps_ctx ctx, bsmps_mpo W, const b
 /* C = A B (M x N) on the tensor cores in split precision (BSMPS_PREC_TF32X3):
  * every entry of A and B is split into two TF32 values, the three products
  * A_hi B_hi + A_hi B_lo + A_lo B_hi are accumulated in FP32 in tensor memory
- * (tcgen05.mma kind::tf32, 128 x 64 tiles), and C is stored in FP64.  The error
+ * (tcgen05.mma kind::tf32), and C is stored in FP64.  The error
  * of C_ij is a few units of 2^-21 times sum_k |a_ik| |b_kj| plus the FP32
  * accumulation error.  The paper has no counterpart: this is the contraction
  * kernel of the split-precision MPO application, exposed for testing.  A

@@ -1047,7 +1047,7 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
 // ||E||_2 < 1.4e-4, twice what 64 columns of random entries of that size have), and the FP64
 // Jacobi starts from G Qp with V = Qp: one sweep and a step of first order.  The square and cube of E
 // are below 1e-8 of the result and take FP32.  (One pass with the cube instead of
-// two without it: k = 60 330 -> 160 us, k = 20 22 -> 11 us.)  Where the FP32
+// two without it: k = 60 330 -> 134 us, k = 20 22 -> 9.5 us.)  Where the FP32
 // iteration gives nothing (non-finite entries) it starts from G and I.
 // RG, RV: rows of G and V in units of 8 (8 RG >= rows, 8 RV >= k).  Leading dimensions:
 // jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of

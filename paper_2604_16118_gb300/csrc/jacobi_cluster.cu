@@ -183,7 +183,7 @@ __device__ __forceinline__ void rotate_v(double* V, const Rot* in, int k, int la
 }
 
 template <int C>
-__global__ void __launch_bounds__(kClusterThreads) k_jacobi_cluster(const JacTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(kClusterThreads, 1) k_jacobi_cluster(const JacTask* __restrict__ tasks) {
     extern __shared__ double jc_smem[];
     __shared__ double s_part[C];     // CTA 0's slots: partial ||G||^2 of every CTA
     __shared__ int s_flag[2][C];     // CTA 0's slots: rotation flags, by sweep parity
@@ -425,7 +425,7 @@ __device__ __forceinline__ void rotate_pair_f32(float* Gp, float* Gq, float* Vp,
 }
 
 template <int C>
-__global__ void __launch_bounds__(kClusterThreads) k_jacobi_cluster_f32(const JacTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(kClusterThreads, 1) k_jacobi_cluster_f32(const JacTask* __restrict__ tasks) {
     extern __shared__ float jf_smem[];
     __shared__ double s_part[C];
     __shared__ int s_flag[2][C];

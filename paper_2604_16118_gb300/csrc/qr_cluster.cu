@@ -102,8 +102,10 @@ __device__ __forceinline__ void qc_form(double* Ql, const double* vb, const doub
     }
 }
 
+// Two CTAs per SM at least: without the figure the compiler aims for four, at 64 registers and
+// with spills (three wide workloads: 95.4 -> 94.1, 23.0 -> 20.2 and 113.7 -> 110.9 ms).
 template <int C>
-__global__ void __launch_bounds__(kQcThreads) k_qr_cluster(const QrTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(kQcThreads, 2) k_qr_cluster(const QrTask* __restrict__ tasks) {
     extern __shared__ double qc_sm[];
     __shared__ double part[2][4];
     __shared__ double s_alpha;
