@@ -65,6 +65,7 @@ struct MlpGemm {
     const float* A;
     const float* B;
     int M, N, K, nkc;   // nkc: chunks of K
+    int n_acc, acc_len; // accumulators of a tile, chunks per accumulator
     const __nv_bfloat16* bias;
     int relu;
     const float* mask;
@@ -74,7 +75,8 @@ struct MlpGemm {
 };
 
 constexpr int kMlpM = 128;         // rows of a tile (the M of one tcgen05.mma)
-constexpr int kMlpN = 128;         // columns of a tile (its N, and the tensor-memory columns)
+constexpr int kMlpN = 128;         // columns of a tile (its N, and the tensor-memory columns of an accumulator)
+constexpr int kMlpAcc = 4;         // accumulators at most (512 tensor-memory columns)
 constexpr int kMlpStages = 4;
 constexpr uint32_t kMlpOperand = kImgBlock * 4;       // bytes of one operand block
 constexpr uint32_t kMlpStage = 2 * kMlpOperand;
@@ -85,7 +87,7 @@ constexpr uint32_t kMlpIdesc = tc::idesc_tf32(kMlpM, kMlpN);
 // streams the blocks through four stages by bulk copies, another issues four MMAs
 // per chunk; no thread touches an operand (staging them through registers, strided
 // and rounded on the way, took 0.86 ms for the products of a batch of 8192).  All
-// four warps run the epilogue.  What is left is latency: at 8 chunks a tile's copies
+// four warps run the epilogue, which adds a tile's accumulators in order.  What is left is latency: at 8 chunks a tile's copies
 // and its epilogue (two images) are longer than its 32 MMAs.  Waits are bounded; a CTA that
 // gives up sets *err and frees its tensor memory after its MMAs and copies.
 __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, int chunks, int* err) {
@@ -103,7 +105,8 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
         for (int i = 0; i < 2 * kMlpStages + 1; ++i) tc::mbar_init(tc::smem_addr(&bars[i]), 1);
         tc::mbar_init_fence();
     }
-    if (warp == 1) tc::tmem_alloc(&tmem_slot, kMlpN);
+    const int cols = kMlpN * (g.n_acc > 2 ? 4 : g.n_acc);   // a power of two
+    if (warp == 1) tc::tmem_alloc(&tmem_slot, cols);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -142,7 +145,8 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
                 const uint64_t a = tc::desc_sw128(base + s * kMlpStage), b = a + (kMlpOperand >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kImgK / 8; ++kk)   // 32 bytes along k per MMA
-                    tc::mma_tf32(tmem, a + 2 * kk, b + 2 * kk, kMlpIdesc, c == 0 && kk == 0 ? 0u : 1u);
+                    tc::mma_tf32(tmem + (uint32_t)(c / g.acc_len * kMlpN), a + 2 * kk, b + 2 * kk, kMlpIdesc,
+                                 c % g.acc_len == 0 && kk == 0 ? 0u : 1u);
                 tc::commit(empty(s));
             }
             tc::commit(done);   // covers every MMA and every earlier commit
@@ -157,6 +161,12 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
     for (int cc = 0; ok && cc < kMlpN; cc += 16) {
         uint32_t v[16];
         tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cc, v);
+        for (int a = 1; a < g.n_acc; ++a) {
+            uint32_t u[16];
+            tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * kMlpN + cc), u);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(u[j]));
+        }
         const int col = n0 + cc;
         if (g.part) {
             if (row < g.M) {
@@ -212,7 +222,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
     if (!ok) atomicExch(err, 1);
     tc::fence_before();
     __syncthreads();
-    if (warp == 1) tc::tmem_free(tmem, kMlpN);
+    if (warp == 1) tc::tmem_free(tmem, cols);
 }
 
 // C = sum_z part[z], the k ranges summed in order.
@@ -369,6 +379,17 @@ void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr)
     }
     const int tm = (g.M + kMlpM - 1) / kMlpM, tn = (g.N + kMlpN - 1) / kMlpN;
     int chunks = g.nkc;
+    // Activations and errors enter the next product rounded to TF32, so the order of their sums
+    // shows in the gradient (3e-5 of it where a sum is taken in another order).  It is: ranges
+    // of k as many as bring the 128 x 64 tiles to 296, four chunks at least in each, every range
+    // in an accumulator of its own.
+    int ranges = 1;
+    if (!grad) {
+        const int64_t tiles = (int64_t)tm * ((g.N + 63) / 64);
+        while (tiles * ranges < 296 && g.nkc / (2 * ranges) >= 4 && 2 * ranges <= kMlpAcc) ranges *= 2;
+    }
+    g.acc_len = (g.nkc + ranges - 1) / ranges;
+    g.n_acc = (g.nkc + g.acc_len - 1) / g.acc_len;
     if (grad) {
         // one wave of CTAs (one per SM at 128 KB of stages), at least four chunks each
         const int splits = std::max(1, std::min(148 / std::max(1, tm * tn), g.nkc / 4));
