@@ -197,6 +197,12 @@ BSMPS_API bsmps_status bsmps_ctx_kernel_stats(bsmps_ctx ctx, int kind, int reset
  * 1), CUDA. */
 BSMPS_API bsmps_status bsmps_check_grid_wait(bsmps_ctx ctx, int skip_cta, int* timed_out);
 
+/* Check of the step that turns the FP32 rotations of a sector SVD into an FP64
+ * orthogonal matrix (no counterpart in the paper).  P, Q: k x k, row-major, host,
+ * 1 <= k <= 64; Q is orthogonal to within k eps and next to P, *ok = 0 (Q undefined)
+ * when ||P^T P - I||_F is not below 1/4.  Errors: INVALID_ARG, OOM, CUDA. */
+BSMPS_API bsmps_status bsmps_check_orthogonalise(bsmps_ctx ctx, int k, const double* P, double* Q, int* ok);
+
 /* ---- problem set-up (host only, no device needed) ----------------------- */
 
 /* theta[i] = gamma/N + t_ii + sum_{j=k_i+1}^{k_i+N} (v_ijji - v_ijij),

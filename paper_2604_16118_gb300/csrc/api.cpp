@@ -294,6 +294,13 @@ bsmps_status bsmps_check_grid_wait(bsmps_ctx ctx, int skip_cta, int* timed_out) 
     });
 }
 
+bsmps_status bsmps_check_orthogonalise(bsmps_ctx ctx, int k, const double* P, double* Q, int* ok) {
+    return guarded(ctx, [&] {
+        BSM_REQUIRE(k >= 1 && k <= 64 && P && Q && ok, BSMPS_ERR_INVALID_ARG, "1 <= k <= 64 and arrays required");
+        *ok = bsm::check_orthogonalise(C(ctx), k, P, Q) ? 1 : 0;
+    });
+}
+
 bsmps_status bsmps_ctx_sync(bsmps_ctx ctx) {
     return guarded(ctx, [&] { C(ctx)->sync(); });
 }

@@ -1038,57 +1038,26 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
     __syncthreads();
 }
 
-// One-sided Jacobi of G (rows x k, column-major, k <= rows <= 64) as jacobi(): G ends
-// as U diag(Sraw), V (k x k) accumulates the rotations.  The FP64 sweeps are few because an
-// FP32 Jacobi of G comes first (FP32 arithmetic runs at 64 times the FP64 rate
-// here): its rotations P, orthogonal to about 3e-6, are orthogonalised in FP64 as
-// Qp = P (I - E/2 + 3/8 E^2 - 5/16 E^3) with E = P^T P - I (a second pass when an
-// entry of E reaches 8e-6: the dropped term, 35/128 E^4, is below 1e-16 for
-// ||E||_2 < 1.4e-4, twice what 64 columns of random entries of that size have), and the FP64
-// Jacobi starts from G Qp with V = Qp: one sweep and a step of first order.  The square and cube of E
-// are below 1e-8 of the result and take FP32.  (One pass with the cube instead of
-// two without it: k = 60 330 -> 134 us, k = 20 22 -> 9.5 us.)  Where the FP32
-// iteration gives nothing (non-finite entries) it starts from G and I.
-// RG, RV: rows of G and V in units of 8 (8 RG >= rows, 8 RV >= k).  Leading dimensions:
-// jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of
-// max(k, 8 RV - 7) for V, so that the 8 RG (8 RV) rows a lane segment walks stay
-// within the column.  scr: jacobi_scratch(ldg, ldv, k) shared doubles; del: k of them.
-// Tri: G is lower triangular (rows = k).
-template <int RG, int RV, bool Tri>
-__device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int rows, int k, double* scr,
-                                           double* del, SegRot* ring, double* red, int* s_int) {
-    constexpr int kOwn = 8;   // outputs of a product per thread: rows k <= 8 blockDim (blockDim >= min(16 k, 512))
-    const int T = nthreads(), kk = k * k;
-    const int ldg = jacobi_ld(max(rows, 8 * RG - 7)), ldv = jacobi_ld(max(k, 8 * RV - 7));   // >= 8 RG, 8 RV
-    double f = 0.0;
-    for (int e = threadIdx.x; e < k * ldg; e += T) f = fma(G[e], G[e], f);
-    f = block_sum(f, red);
-    // exact scaling to ||G||_F in [1/2, 1)
-    int ex = 0;
-    if (f > 0.0 && f < DBL_MAX) frexp(sqrt(f), &ex);
-    const double sc = ldexp(1.0, -ex);
-    const double fro = f * sc * sc;
-    float* Gf = (float*)scr;
-    float* Vf = Gf + k * ldg;
-    for (int e = threadIdx.x; e < k * ldg; e += T) {
-        const double x = G[e] * sc;
-        G[e] = x;
-        Gf[e] = (float)x;
-    }
-    for (int e = threadIdx.x; e < k * ldv; e += T) Vf[e] = e % ldv == e / ldv ? 1.0f : 0.0f;
-    __syncthreads();
-    jacobi_f32_segments<RG, RV>(Gf, Vf, k, ldg, ldv, s_int);
-    // V row-major <- P
-    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
-    bool ok = true;
+// V (k x k row-major, k <= 64) <- an orthogonal matrix Qp = P (I - E/2 + 3/8 E^2 - 5/16 E^3) next
+// to P = V, E = P^T P - I, with the square and cube of E in FP32 (they take a third of the FP64
+// instructions otherwise).  What one pass leaves of Qp^T Qp - I is bounded through ||E||_F, which
+// bounds ||E||_2 whatever the signs of the entries: the dropped term, 35/64 ||E||^4, and the FP32
+// rounding of 3/4 E^2, at most (4 + k) 2^-24 of it (sums of k terms; sqrt(k) in place of k where
+// roundings are random).  ||E||_F^2 < 6e-11 k keeps the first below 2e-21 k^2 and the second
+// below k eps (k eps / 6 at random roundings), the limit to which the Jacobi itself takes cosines;
+// otherwise another pass follows.  false: E is not small (non-finite entries, no rotations to speak of).
+// scr: 2 k^2 doubles; own: this thread's entries threadIdx.x + n blockDim of the result; red: 33 doubles.
+// (One pass with the cube instead of two without it: k = 60 330 -> 134 us, k = 20 22 -> 9.5 us.)
+constexpr float kOrthOnePass = 6e-11f;
+constexpr int kOwn = 8;   // outputs of a product per thread: rows k <= 8 blockDim (blockDim >= min(16 k, 512))
+__device__ __forceinline__ bool orthogonalise(double* V, int k, double* scr, double (&own)[kOwn], double* red) {
+    const int T = nthreads(), kk = k * k, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float* Ef = (float*)(scr + kk);   // E in FP32
     float* Tf = Ef + kk;
-    double own[kOwn];
+    float* part = (float*)red;
     for (int pass = 0; pass < 3; ++pass) {
         __syncthreads();
-        if (threadIdx.x == 0) *s_int = 0;
-        float mx = 0.0f;
-        __syncthreads();
+        float f2 = 0.0f;
         for (int e = threadIdx.x; e < k * (k + 1) / 2; e += T) {
             // row i, column j <= i of the symmetric E
             int i = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
@@ -1100,15 +1069,14 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             scr[i * k + j] = scr[j * k + i] = acc;
             const float af = to_float_scaled(acc, 0);
             Ef[i * k + j] = Ef[j * k + i] = af;
-            mx = fabsf(af) <= mx ? mx : (af == af ? fabsf(af) : FLT_MAX);
+            f2 = fmaf(i == j ? af : 2.0f * af, af, f2);
         }
-        atomicMax(s_int, (int)__float_as_uint(mx));
+        for (int o = 16; o > 0; o >>= 1) f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+        if (lane == 0) part[warp] = f2;
         __syncthreads();
-        const float emax = __uint_as_float((unsigned)*s_int);
-        if (!(emax < 1e-2f)) {
-            ok = false;
-            break;
-        }
+        f2 = 0.0f;
+        for (int w = 0; w < nwarps(); ++w) f2 += part[w];
+        if (!(f2 < 0.0625f)) return false;
         // Tf = -3/8 E + 5/16 E^2, then F = E/2 + E Tf
         for (int e = threadIdx.x; e < kk; e += T) {
             const int i = e % k, j = e / k;
@@ -1141,9 +1109,50 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
             const int e = threadIdx.x + n * T;
             if (e < kk) V[e] = own[n];
         }
-        if (emax < 8e-6f) break;
-        ok = pass < 2;
+        if (f2 < kOrthOnePass * (float)k) return true;
     }
+    return false;
+}
+
+// One-sided Jacobi of G (rows x k, column-major, k <= rows <= 64) as jacobi(): G ends
+// as U diag(Sraw), V (k x k) accumulates the rotations.  The FP64 sweeps are few because an
+// FP32 Jacobi of G comes first (FP32 arithmetic runs at 64 times the FP64 rate
+// here): its rotations P, orthogonal to about 3e-6, are orthogonalised in FP64
+// (orthogonalise()), and the FP64 Jacobi starts from G Qp with V = Qp: one sweep and a
+// step of first order.  Where the FP32
+// iteration gives nothing (non-finite entries) it starts from G and I.
+// RG, RV: rows of G and V in units of 8 (8 RG >= rows, 8 RV >= k).  Leading dimensions:
+// jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of
+// max(k, 8 RV - 7) for V, so that the 8 RG (8 RV) rows a lane segment walks stay
+// within the column.  scr: jacobi_scratch(ldg, ldv, k) shared doubles; del: k of them.
+// Tri: G is lower triangular (rows = k).
+template <int RG, int RV, bool Tri>
+__device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int rows, int k, double* scr,
+                                           double* del, SegRot* ring, double* red, int* s_int) {
+    const int T = nthreads(), kk = k * k;
+    const int ldg = jacobi_ld(max(rows, 8 * RG - 7)), ldv = jacobi_ld(max(k, 8 * RV - 7));   // >= 8 RG, 8 RV
+    double f = 0.0;
+    for (int e = threadIdx.x; e < k * ldg; e += T) f = fma(G[e], G[e], f);
+    f = block_sum(f, red);
+    // exact scaling to ||G||_F in [1/2, 1)
+    int ex = 0;
+    if (f > 0.0 && f < DBL_MAX) frexp(sqrt(f), &ex);
+    const double sc = ldexp(1.0, -ex);
+    const double fro = f * sc * sc;
+    float* Gf = (float*)scr;
+    float* Vf = Gf + k * ldg;
+    for (int e = threadIdx.x; e < k * ldg; e += T) {
+        const double x = G[e] * sc;
+        G[e] = x;
+        Gf[e] = (float)x;
+    }
+    for (int e = threadIdx.x; e < k * ldv; e += T) Vf[e] = e % ldv == e / ldv ? 1.0f : 0.0f;
+    __syncthreads();
+    jacobi_f32_segments<RG, RV>(Gf, Vf, k, ldg, ldv, s_int);
+    // V row-major <- P
+    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
+    double own[kOwn];
+    const bool ok = orthogonalise(V, k, scr, own, red);
     __syncthreads();
     if (ok) {
         // G <- G Qp, row i to consecutive threads (rows k <= 8 blockDim outputs); V to column-major

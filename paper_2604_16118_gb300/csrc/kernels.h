@@ -306,6 +306,8 @@ bool launch_right_sweep(Context* ctx, const std::vector<DynTask>& tasks, const s
 // Two-CTA cooperative kernel meeting at one phase boundary; CTA skip_cta (if
 // >= 0) never arrives.  Returns the error word of the wait (1: a wait gave up).
 int check_grid_wait(Context* ctx, int skip_cta);
+// Q = the orthogonalised P (k x k, row-major, k <= 64, host arrays); false: P is not near an orthogonal matrix.
+bool check_orthogonalise(Context* ctx, int k, const double* P, double* Q);
 
 // ---- environment sweep with structures shared by groups of problems ----
 //

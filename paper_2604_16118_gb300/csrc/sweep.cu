@@ -770,6 +770,19 @@ __global__ void k_grid_wait_check(int skip_cta, GridSync* gs) {
     phase_end(gs, 0u, &s_flag);
 }
 
+// orthogonalise() of one k x k matrix (row-major), as the one-CTA SVD runs it on its FP32 rotations.
+__global__ void __launch_bounds__(kSweepThreads) k_orthogonalise_check(const double* __restrict__ P, int k,
+                                                                       double* __restrict__ Q, int* __restrict__ ok) {
+    extern __shared__ double sm[];
+    __shared__ double red[33];
+    double own[dev::kOwn];
+    for (int e = threadIdx.x; e < k * k; e += nthreads()) sm[e] = P[e];
+    const bool good = dev::orthogonalise(sm, k, sm + k * k, own, red);
+    __syncthreads();
+    for (int e = threadIdx.x; e < k * k; e += nthreads()) Q[e] = sm[e];
+    if (threadIdx.x == 0) *ok = good ? 1 : 0;
+}
+
 // Environment sweep: every phase is a set of independent 32 x 32 output tiles whose
 // inputs may have been written in earlier phases (loads go through L2).  A CTA
 // stages 32 values of k of both factors in shared memory; the right factor of an
@@ -1283,6 +1296,21 @@ int check_grid_wait(Context* ctx, int skip_cta) {
     BSM_CUDA(cudaMemcpyAsync(&h, gs, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     ctx->sync();
     return h.err;
+}
+
+bool check_orthogonalise(Context* ctx, int k, const double* P, double* Q) {
+    Scratch s(ctx);
+    const size_t n = (size_t)k * k;
+    double* d = s.dbl(2 * n + 1);
+    BSM_CUDA(cudaMemcpyAsync(d, P, sizeof(double) * n, cudaMemcpyHostToDevice, ctx->stream));
+    allow_smem(k_orthogonalise_check);
+    k_orthogonalise_check<<<1, svd_block_for(k), sizeof(double) * 3 * n, ctx->stream>>>(d, k, d + n, (int*)(d + 2 * n));
+    count_launch(ctx);
+    int ok = 0;
+    BSM_CUDA(cudaMemcpyAsync(Q, d + n, sizeof(double) * n, cudaMemcpyDeviceToHost, ctx->stream));
+    BSM_CUDA(cudaMemcpyAsync(&ok, d + 2 * n, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    ctx->sync();
+    return ok != 0;
 }
 
 bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,

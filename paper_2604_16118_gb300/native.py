@@ -140,6 +140,7 @@ _SIGS = {
     "bsmps_dot": (_i, [_vp, _vp, _vp, _vp, _d, _pd]),
     "bsmps_dot_noalloc": (_i, [_vp, _vp, _vp, _vp, _d, _pd]),
     "bsmps_check_grid_wait": (_i, [_vp, _i, C.POINTER(C.c_int)]),
+    "bsmps_check_orthogonalise": (_i, [_vp, _i, _pd, _pd, C.POINTER(C.c_int)]),
     "bsmps_eigensolve_outer": (_i, [_vp, _vp, _vp, _vp, _d, _d, _i, _i, C.POINTER(_vp), _vp,
                                     C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     "bsmps_mlp_create": (_i, [_vp, _i, _pi, C.POINTER(C.c_float), _i64, C.POINTER(_vp)]),
@@ -575,6 +576,15 @@ def check_grid_wait(ctx, skip_cta=-1):
     out = C.c_int()
     _check(ctx, lib().bsmps_check_grid_wait(ctx.h, skip_cta, C.byref(out)))
     return bool(out.value)
+
+
+def check_orthogonalise(ctx, P):
+    """The orthogonal matrix next to P as the sector SVD forms it, None where P is not close to one."""
+    P = np.ascontiguousarray(P, dtype=np.float64)
+    Q, ok = np.empty_like(P), C.c_int()
+    _check(ctx, lib().bsmps_check_orthogonalise(ctx.h, P.shape[0], P.ctypes.data_as(_pd), Q.ctypes.data_as(_pd),
+                                                C.byref(ok)))
+    return Q if ok.value else None
 
 
 def solver_params(c, delta, eps_num=None, t_eig=0.5, tau=1e-8, r_max=0, u_rel=1e-13):
