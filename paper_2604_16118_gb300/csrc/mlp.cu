@@ -55,7 +55,7 @@ __device__ __forceinline__ float tf32_round(float f) { return __uint_as_float(tc
 
 // One product of the network on the tensor cores, C(m, n) = epi( sum_k a(m, k) b(n, k) ),
 // both factors given as operand images over nkc chunks of 32 values of k.  Outputs:
-//  - part: raw sums of a k range to part[z] (row-major), summed by k_mlp_reduce;
+//  - part: raw sums of a k range to part[z] (row-major), summed by k_mlp_reduce or k_mlp_finish;
 //  - y: row-major FP32 (the network's output);
 //  - i1, i2: the operand images of the result (rows = m; rows = n), rounded to TF32
 //    as the next products read them.
@@ -235,6 +235,38 @@ __global__ void k_mlp_reduce(const float* __restrict__ part, float* __restrict__
     C[e] = acc;
 }
 
+// The result of a product whose k ranges were summed by different CTAs: the ranges in order, then
+// what the epilogue of k_mlp_gemm_tc does (bias, ReLU or mask; y, or the images i1 and i2).
+// 32 x 32 tiles through shared memory, so that both images are written along their rows.
+__global__ void __launch_bounds__(256) k_mlp_finish(const MlpGemm g, int n_parts) {
+    __shared__ float t[32][33];
+    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32, x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int nk1 = img_chunks(g.N), nk2 = img_chunks(g.M);
+    for (int i = y; i < 32; i += 8) {
+        const int r = r0 + i, c = c0 + x;
+        const bool in = r < g.M && c < g.N;
+        float v = 0.0f;
+        if (in) {
+#pragma unroll 8
+            for (int z = 0; z < n_parts; ++z) v += g.part[((int64_t)z * g.M + r) * g.N + c];
+            if (g.bias) v += __bfloat162float(g.bias[c]);
+            if (g.relu) v = fmaxf(v, 0.0f);
+            if (g.mask && !(g.mask[img_at(r, c, nk1)] > 0.0f)) v = 0.0f;
+        }
+        if (g.y) {
+            if (in) g.y[(int64_t)r * g.N + c] = v;
+            continue;
+        }
+        v = tf32_round(v);
+        t[i][x] = v;
+        if (r < g.M) g.i1[img_at(r, c, nk1)] = v;
+    }
+    if (g.y || !g.i2) return;
+    __syncthreads();
+    for (int i = y; i < 32; i += 8)
+        if (c0 + i < g.N) g.i2[img_at(c0 + i, r0 + x, nk2)] = t[x][i];
+}
+
 // The operand images of a row-major matrix X (n x K): rows of X, and (i2 not
 // null) rows of X^T over n.  32 x 32 tiles through shared memory.
 __global__ void __launch_bounds__(256) k_mlp_pack(const float* __restrict__ X, int n, int K, float* __restrict__ i1,
@@ -368,8 +400,19 @@ MlpLayers layers_of(const bsmps_mlp_s* net) {
 
 float* floats(Scratch& s, int64_t n) { return (float*)s.dbl((size_t)(n + 1) / 2); }
 
-// One product.  grad != null: the k range is split over gridDim.z CTAs per tile
-// (partials reduced in order into grad) as far as the tiles alone leave SMs idle.
+// A product's sum over k is taken in ranges, each from zero in an FP32 accumulator of its own
+// (the tensor cores truncate every addition to an accumulator: a sum of positive terms over
+// 4096 values of k loses 68 units of 2^-24 in 4 ranges and 3.6 in 32).  As many ranges as bring
+// the 128 x 64 tiles to kMlpRangeTiles, four chunks at least in each.  The rule is part of the
+// result: activations and errors enter the next product rounded to TF32, so the order of their
+// sums shows in the gradient (3e-5 of it).
+constexpr int kMlpRangeTiles = 296;
+
+// One product.  Up to four ranges are the accumulators of one CTA; more go to a CTA each
+// (there are few tiles then; 4096 x 4096 at a batch of 16: 57 -> 30 us), summed in order by
+// k_mlp_finish.  grad != null: the k range is
+// split over gridDim.z CTAs per tile (partials reduced in order into grad) as far as the
+// tiles alone leave SMs idle.
 void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr) {
     const int smem = kMlpStages * (int)kMlpStage + 1024;
     static bool attr = false;
@@ -379,31 +422,35 @@ void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr)
     }
     const int tm = (g.M + kMlpM - 1) / kMlpM, tn = (g.N + kMlpN - 1) / kMlpN;
     int chunks = g.nkc;
-    // Activations and errors enter the next product rounded to TF32, so the order of their sums
-    // shows in the gradient (3e-5 of it where a sum is taken in another order).  It is: ranges
-    // of k as many as bring the 128 x 64 tiles to 296, four chunks at least in each, every range
-    // in an accumulator of its own.
     int ranges = 1;
     if (!grad) {
         const int64_t tiles = (int64_t)tm * ((g.N + 63) / 64);
-        while (tiles * ranges < 296 && g.nkc / (2 * ranges) >= 4 && 2 * ranges <= kMlpAcc) ranges *= 2;
+        while (tiles * ranges < kMlpRangeTiles && g.nkc / (2 * ranges) >= 4) ranges *= 2;
     }
     g.acc_len = (g.nkc + ranges - 1) / ranges;
     g.n_acc = (g.nkc + g.acc_len - 1) / g.acc_len;
+    if (g.n_acc > kMlpAcc) {
+        chunks = g.acc_len;
+        g.n_acc = 1;
+    }
     if (grad) {
         // one wave of CTAs (one per SM at 128 KB of stages), at least four chunks each
         const int splits = std::max(1, std::min(148 / std::max(1, tm * tn), g.nkc / 4));
         chunks = (g.nkc + splits - 1) / splits;
     }
     const int parts = (g.nkc + chunks - 1) / chunks;
-    if (grad) g.part = parts > 1 ? floats(s, (int64_t)parts * g.M * g.N) : grad;
+    if (parts > 1) g.part = floats(s, (int64_t)parts * g.M * g.N);
+    else if (grad) g.part = grad;
     const double fl = 2.0 * g.M * (double)g.N * g.K;
     const double by = 4.0 * ((double)(g.M + g.N) * g.K + (double)g.M * g.N);
     ProfScope ps(ctx, KK_MLP, fl, by);
     k_mlp_gemm_tc<<<dim3((unsigned)tm, (unsigned)tn, (unsigned)parts), kMlpThreads, smem, ctx->stream>>>(
         g, chunks, ctx->err_word());
     done(ctx);
-    if (parts > 1) {
+    if (parts > 1 && !grad) {
+        k_mlp_finish<<<dim3((unsigned)img_chunks(g.M), (unsigned)img_chunks(g.N)), 256, 0, ctx->stream>>>(g, parts);
+        done(ctx);
+    } else if (parts > 1) {
         const int64_t n = (int64_t)g.M * g.N;
         k_mlp_reduce<<<grid(n), kT, 0, ctx->stream>>>(g.part, grad, n, parts);
         done(ctx);
