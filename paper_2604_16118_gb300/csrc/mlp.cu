@@ -65,7 +65,7 @@ struct MlpGemm {
     const float* A;
     const float* B;
     int M, N, K, nkc;   // nkc: chunks of K
-    int n_acc, acc_len; // accumulators of a tile, chunks per accumulator
+    int n_acc, acc_len; // accumulators of a CTA (at most), chunks per accumulator
     const __nv_bfloat16* bias;
     int relu;
     const float* mask;
@@ -157,11 +157,12 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
     ok = __all_sync(0xffffffffu, tc::mbar_wait(done, 0) && ok);
     tc::fence_after();
     const int row = m0 + warp * 32 + lane;
+    const int n_acc = (nc + g.acc_len - 1) / g.acc_len;   // (the last range of k may be shorter)
     const int nk1 = img_chunks(g.N), nk2 = img_chunks(g.M);   // chunks of the result's images
     for (int cc = 0; ok && cc < kMlpN; cc += 16) {
         uint32_t v[16];
         tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cc, v);
-        for (int a = 1; a < g.n_acc; ++a) {
+        for (int a = 1; a < n_acc; ++a) {
             uint32_t u[16];
             tc::ld_32x32b_x16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(a * kMlpN + cc), u);
 #pragma unroll
@@ -410,9 +411,8 @@ constexpr int kMlpRangeTiles = 296;
 
 // One product.  Up to four ranges are the accumulators of one CTA; more go to a CTA each
 // (there are few tiles then; 4096 x 4096 at a batch of 16: 57 -> 30 us), summed in order by
-// k_mlp_finish.  grad != null: the k range is
-// split over gridDim.z CTAs per tile (partials reduced in order into grad) as far as the
-// tiles alone leave SMs idle.
+// k_mlp_finish.  grad != null: one wave of CTAs over tiles and k, each with accumulators no
+// longer than a range, the CTAs' sums added in order into grad.
 void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr) {
     const int smem = kMlpStages * (int)kMlpStage + 1024;
     static bool attr = false;
@@ -421,22 +421,24 @@ void launch_mlp_gemm(Context* ctx, MlpGemm g, Scratch& s, float* grad = nullptr)
         attr = true;
     }
     const int tm = (g.M + kMlpM - 1) / kMlpM, tn = (g.N + kMlpN - 1) / kMlpN;
-    int chunks = g.nkc;
+    const int64_t tiles = (int64_t)tm * ((g.N + 63) / 64);
     int ranges = 1;
-    if (!grad) {
-        const int64_t tiles = (int64_t)tm * ((g.N + 63) / 64);
-        while (tiles * ranges < kMlpRangeTiles && g.nkc / (2 * ranges) >= 4) ranges *= 2;
-    }
-    g.acc_len = (g.nkc + ranges - 1) / ranges;
-    g.n_acc = (g.nkc + g.acc_len - 1) / g.acc_len;
-    if (g.n_acc > kMlpAcc) {
-        chunks = g.acc_len;
-        g.n_acc = 1;
-    }
+    while (tiles * ranges < kMlpRangeTiles && g.nkc / (2 * ranges) >= 4) ranges *= 2;
+    const int len = (g.nkc + ranges - 1) / ranges;
+    int chunks = g.nkc;   // of one CTA
+    g.acc_len = len;
+    g.n_acc = (g.nkc + len - 1) / len;
     if (grad) {
-        // one wave of CTAs (one per SM at 128 KB of stages), at least four chunks each
-        const int splits = std::max(1, std::min(148 / std::max(1, tm * tn), g.nkc / 4));
+        // one CTA per SM (128 KB of stages), at least four chunks each
+        int nsm = 0;
+        BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+        const int splits = std::max(1, std::min(nsm / std::max(1, tm * tn), g.nkc / 4));
         chunks = (g.nkc + splits - 1) / splits;
+        g.n_acc = std::min(kMlpAcc, (chunks + len - 1) / len);   // (at most four by the rule of the ranges)
+        g.acc_len = (chunks + g.n_acc - 1) / g.n_acc;
+    } else if (g.n_acc > kMlpAcc) {
+        chunks = len;
+        g.n_acc = 1;
     }
     const int parts = (g.nkc + chunks - 1) / chunks;
     if (parts > 1) g.part = floats(s, (int64_t)parts * g.M * g.N);

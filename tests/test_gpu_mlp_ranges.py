@@ -25,12 +25,16 @@ def ctx(nat):
     return nat.Context(0)
 
 
-def loss_of_sums(M, N, K):
+def range_chunks(M, N, K):
     chunks, ranges = -(-K // 32), 1
     tiles = -(-M // 128) * -(-N // 64)
     while tiles * ranges < 296 and chunks // (2 * ranges) >= 4:
         ranges *= 2
-    length = -(-chunks // ranges)
+    return chunks, -(-chunks // ranges)
+
+
+def loss_of_sums(M, N, K):
+    chunks, length = range_chunks(M, N, K)
     return (2 * length + 1) * 2.0 ** -23 + (-(-chunks // length) / 2 + 1) * 2.0 ** -24
 
 
@@ -52,6 +56,23 @@ def test_forward_sums(nat, ctx, K, N, B):
     y = nat.MLP(ctx, [K, N], np.concatenate([w.ravel(), np.zeros(N, np.float32)])).forward(x)
     exact = x.astype(np.float64) @ w.astype(np.float64).T
     assert np.abs(y / exact - 1.0).max() <= loss_of_sums(B, N, K)
+
+
+@pytest.mark.parametrize("K,N,B", [(256, 256, 8192), (128, 256, 8192), (300, 70, 5000), (40, 3, 8192),
+                                   (1024, 512, 2048)])
+def test_weight_gradient_sums(nat, ctx, K, N, B):
+    """The mean error shows how long the sums are (roundings to nearest average out): after i of 4 c
+    additions the sum is i / (4 c) of the total, an addition of eight products to an accumulator truncates twice at most, by 2^-24
+    of the sum on average: (4 c + 1) 2^-24."""
+    w, x = positive(K, N, B)
+    net = nat.MLP(ctx, [K, N], np.concatenate([w.ravel(), np.zeros(N, np.float32)]))
+    _, g = net.loss_grad(x, np.zeros((B, N), np.float32))
+    y = net.forward(x)
+    dy = tf32(np.float32(2.0) * (np.float32(1.0) / np.float32(B * N)) * y)
+    exact = dy.astype(np.float64).T @ x.astype(np.float64)
+    err = g[:N * K].reshape(N, K) / exact - 1.0
+    assert abs(err.mean()) <= (4 * range_chunks(N, K, B)[1] + 1) * 2.0 ** -24
+    assert np.abs(err).max() <= loss_of_sums(N, K, B) + 2.0 ** -22
 
 
 @pytest.mark.parametrize("widths,batch", [([1030, 1100, 1025, 3], 33), ([2048, 992, 1056], 5), ([37, 4096, 1], 130)])
