@@ -40,16 +40,24 @@ constexpr int kT = 256;
 
 // Operand image of a matrix of n rows x K values (FP32, already rounded to TF32):
 // blocks of 128 rows x 32 values (16 KB, K-major with 128-byte swizzle), the blocks
-// of a row range contiguous along K, so that a chunk of a tile is one bulk copy.
-// Values of k >= K are zero (the products run over whole chunks); rows >= n hold
-// anything (they reach only entries that are not stored).
+// of a row range contiguous along K, so that a chunk of a tile is one bulk copy.  The
+// blocks of the last row range end with row n - 1: a layer of 2 outputs and a batch of
+// 10^6 takes 8 MB and not 512.  Values of k >= K are zero (the products run over whole
+// chunks); the rows that a block lacks are whatever stands in shared memory behind its
+// copy (they reach only entries that are not stored).
 constexpr int kImgRows = 128, kImgK = 32;
 constexpr int64_t kImgBlock = kImgRows * kImgK;   // floats
 __host__ __device__ __forceinline__ int img_chunks(int K) { return (K + kImgK - 1) / kImgK; }
-inline int64_t img_size(int n, int K) { return (int64_t)((n + kImgRows - 1) / kImgRows) * img_chunks(K) * kImgBlock; }
-__device__ __forceinline__ int64_t img_at(int r, int k, int nkc) {
-    return ((int64_t)(r / kImgRows) * nkc + k / kImgK) * kImgBlock + (r % kImgRows) * kImgK +
-           ((((k >> 2) & 7) ^ (r & 7)) << 2) + (k & 3);
+inline int64_t img_size(int n, int K) { return (int64_t)n * img_chunks(K) * kImgK; }
+// Rows of the block that holds row r of n.
+__host__ __device__ __forceinline__ int img_rows(int r, int n) {
+    const int left = n - r / kImgRows * kImgRows;
+    return left < kImgRows ? left : kImgRows;
+}
+// Row r < n, value k, over nkc chunks.
+__host__ __device__ __forceinline__ int64_t img_at(int r, int k, int n, int nkc) {
+    return (int64_t)(r / kImgRows) * nkc * kImgBlock + (int64_t)(k / kImgK) * img_rows(r, n) * kImgK +
+           (r % kImgRows) * kImgK + ((((k >> 2) & 7) ^ (r & 7)) << 2) + (k & 3);
 }
 __device__ __forceinline__ float tf32_round(float f) { return __uint_as_float(tc::tf32_bits(f)); }
 
@@ -98,6 +106,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * kMlpM, n0 = blockIdx.y * kMlpN;
     const int c0 = blockIdx.z * chunks, nc = min(chunks, g.nkc - c0);   // >= 1
+    const int rows_a = img_rows(m0, g.M), rows_b = img_rows(n0, g.N);
     auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
     auto empty = [&](int s) { return tc::smem_addr(&bars[kMlpStages + s]); };
     const uint32_t done = tc::smem_addr(&bars[2 * kMlpStages]);
@@ -114,8 +123,9 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
     bool ok = true;
     if (warp == 0) {
         if (lane == 0) {
-            const float* a = g.A + ((int64_t)blockIdx.x * g.nkc + c0) * kImgBlock;
-            const float* b = g.B + ((int64_t)blockIdx.y * g.nkc + c0) * kImgBlock;
+            const int64_t step_a = rows_a * kImgK, step_b = rows_b * kImgK;   // floats of a chunk
+            const float* a = g.A + (int64_t)blockIdx.x * g.nkc * kImgBlock + c0 * step_a;
+            const float* b = g.B + (int64_t)blockIdx.y * g.nkc * kImgBlock + c0 * step_b;
             int c = 0;
             for (; c < nc; ++c) {
                 const int s = c % kMlpStages;
@@ -124,9 +134,9 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
                     break;
                 }
                 const uint32_t dst = base + s * kMlpStage;
-                tc::mbar_expect(full(s), kMlpStage);
-                tc::bulk_load(dst, a + c * kImgBlock, kMlpOperand, full(s));
-                tc::bulk_load(dst + kMlpOperand, b + c * kImgBlock, kMlpOperand, full(s));
+                tc::mbar_expect(full(s), (uint32_t)(step_a + step_b) * 4);
+                tc::bulk_load(dst, a + c * step_a, (uint32_t)step_a * 4, full(s));
+                tc::bulk_load(dst + kMlpOperand, b + c * step_b, (uint32_t)step_b * 4, full(s));
             }
             // copies in flight land before the CTA may end
             for (int i = c > kMlpStages ? c - kMlpStages : 0; i < c; ++i)
@@ -192,10 +202,10 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
             if (g.relu) acc = fmaxf(acc, 0.0f);
             w[j] = acc;
         }
-        if (g.mask && col < nk1 * kImgK) {
+        if (g.mask && row < g.M && col < nk1 * kImgK) {
 #pragma unroll
             for (int j = 0; j < 16; j += 4) {
-                const float4 h = *(const float4*)(g.mask + img_at(row, col + j, nk1));
+                const float4 h = *(const float4*)(g.mask + img_at(row, col + j, g.M, nk1));
                 if (!(h.x > 0.0f)) w[j] = 0.0f;
                 if (!(h.y > 0.0f)) w[j + 1] = 0.0f;
                 if (!(h.z > 0.0f)) w[j + 2] = 0.0f;
@@ -211,14 +221,14 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_gemm_tc(const MlpGemm g, in
         }
 #pragma unroll
         for (int j = 0; j < 16; ++j) w[j] = row < g.M && col + j < g.N ? tf32_round(w[j]) : 0.0f;
-        if (col < nk1 * kImgK)
+        if (row < g.M && col < nk1 * kImgK)
 #pragma unroll
             for (int j = 0; j < 16; j += 4)
-                *(float4*)(g.i1 + img_at(row, col + j, nk1)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+                *(float4*)(g.i1 + img_at(row, col + j, g.M, nk1)) = make_float4(w[j], w[j + 1], w[j + 2], w[j + 3]);
         if (g.i2 && row < nk2 * kImgK)
 #pragma unroll
             for (int j = 0; j < 16; ++j)
-                if (col + j < g.N) g.i2[img_at(col + j, row, nk2)] = w[j];
+                if (col + j < g.N) g.i2[img_at(col + j, row, g.N, nk2)] = w[j];
     }
     if (!ok) atomicExch(err, 1);
     tc::fence_before();
@@ -252,7 +262,7 @@ __global__ void __launch_bounds__(256) k_mlp_finish(const MlpGemm g, int n_parts
             for (int z = 0; z < n_parts; ++z) v += g.part[((int64_t)z * g.M + r) * g.N + c];
             if (g.bias) v += __bfloat162float(g.bias[c]);
             if (g.relu) v = fmaxf(v, 0.0f);
-            if (g.mask && !(g.mask[img_at(r, c, nk1)] > 0.0f)) v = 0.0f;
+            if (g.mask && !(g.mask[img_at(r, c, g.M, nk1)] > 0.0f)) v = 0.0f;
         }
         if (g.y) {
             if (in) g.y[(int64_t)r * g.N + c] = v;
@@ -260,12 +270,12 @@ __global__ void __launch_bounds__(256) k_mlp_finish(const MlpGemm g, int n_parts
         }
         v = tf32_round(v);
         t[i][x] = v;
-        if (r < g.M) g.i1[img_at(r, c, nk1)] = v;
+        if (r < g.M) g.i1[img_at(r, c, g.M, nk1)] = v;
     }
     if (g.y || !g.i2) return;
     __syncthreads();
     for (int i = y; i < 32; i += 8)
-        if (c0 + i < g.N) g.i2[img_at(c0 + i, r0 + x, nk2)] = t[x][i];
+        if (c0 + i < g.N) g.i2[img_at(c0 + i, r0 + x, g.N, nk2)] = t[x][i];
 }
 
 // The operand images of a row-major matrix X (n x K): rows of X, and (i2 not
@@ -279,12 +289,12 @@ __global__ void __launch_bounds__(256) k_mlp_pack(const float* __restrict__ X, i
         const int r = r0 + i, k = k0 + x;
         const float v = r < n && k < K ? tf32_round(X[(int64_t)r * K + k]) : 0.0f;
         t[i][x] = v;
-        if (r < n) i1[img_at(r, k, nk1)] = v;
+        if (r < n) i1[img_at(r, k, n, nk1)] = v;
     }
     if (!i2) return;
     __syncthreads();
     for (int i = y; i < 32; i += 8)
-        if (k0 + i < K) i2[img_at(k0 + i, r0 + x, nk2)] = t[x][i];
+        if (k0 + i < K) i2[img_at(k0 + i, r0 + x, K, nk2)] = t[x][i];
 }
 
 // dY of the loss 1/(B out) sum (Y - T)^2 as operand images (rows = batch, rows =
@@ -301,23 +311,28 @@ __global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, 
         v = tf32_round(2.0f * scale * d);
         sq[(int64_t)b * out + o] = d * d;
     }
-    if (b < B) d1[img_at(b, o, nk1)] = v;
-    if (o < out) d2[img_at(o, b, nk2)] = v;
+    if (b < B) d1[img_at(b, o, B, nk1)] = v;
+    if (o < out) d2[img_at(o, b, out, nk2)] = v;
 }
 
 // db[o] = sum_b dY[b, o] (rounded as the weight-gradient product reads it), eight o
 // per CTA: their rows are a contiguous 1 KB of every block of the image (rows = o, k
-// = b, zeros beyond B), a warp's eight lanes per row, the blocks dealt to the warps.
+// = b, zeros beyond B; fewer in the last CTA), a warp's eight lanes per row, the blocks
+// dealt to the warps.
 constexpr int kBiasThreads = 512;
 __global__ void __launch_bounds__(kBiasThreads) k_mlp_bgrad(const float* __restrict__ d2, float* __restrict__ db, int B,
                                                             int out) {
     __shared__ float red[kBiasThreads / 32][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o0 = 8 * blockIdx.x, nk2 = img_chunks(B);
-    const float4* src = (const float4*)(d2 + (int64_t)(o0 / kImgRows) * nk2 * kImgBlock + (o0 % kImgRows) * kImgK);
-    float s0 = 0.0f, s1 = 0.0f;   // rows lane / 8 and 4 + lane / 8
+    const int64_t step = (int64_t)(kBiasThreads / 32) * img_rows(o0, out) * (kImgK / 4);   // float4
+    const float4* p = (const float4*)(d2 + img_at(o0, 0, out, nk2)) + (int64_t)warp * img_rows(o0, out) * (kImgK / 4);
+    // rows lane / 8 and 4 + lane / 8; lanes of rows that the image lacks read its last one
+    const float4* p0 = p + min(lane >> 3, out - 1 - o0) * 8 + (lane & 7);
+    const float4* p1 = p + min(4 + (lane >> 3), out - 1 - o0) * 8 + (lane & 7);
+    float s0 = 0.0f, s1 = 0.0f;
 #pragma unroll 4
-    for (int c = warp; c < nk2; c += kBiasThreads / 32) {
-        const float4 x = src[(int64_t)c * (kImgBlock / 4) + lane], y = src[(int64_t)c * (kImgBlock / 4) + 32 + lane];
+    for (int c = warp; c < nk2; c += kBiasThreads / 32, p0 += step, p1 += step) {
+        const float4 x = *p0, y = *p1;
         s0 += (x.x + x.y) + (x.z + x.w);
         s1 += (y.x + y.y) + (y.z + y.w);
     }
@@ -352,8 +367,8 @@ __device__ __forceinline__ void store_bf16(const MlpLayers& L, float* img, __nv_
         if (d < 0 || d >= (int64_t)L.in[l] * L.out[l]) continue;
         const int o = (int)(d / L.in[l]), i = (int)(d % L.in[l]);
         const float w = __bfloat162float(h);
-        img[L.w1[l] + img_at(o, i, img_chunks(L.in[l]))] = w;
-        img[L.w2[l] + img_at(i, o, img_chunks(L.out[l]))] = w;
+        img[L.w1[l] + img_at(o, i, L.out[l], img_chunks(L.in[l]))] = w;
+        img[L.w2[l] + img_at(i, o, L.in[l], img_chunks(L.out[l]))] = w;
     }
 }
 
