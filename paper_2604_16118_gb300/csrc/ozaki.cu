@@ -47,7 +47,9 @@ constexpr uint32_t kOzIdesc = tc::idesc_bf16(kOzM, kOzN);
 // blocks of `blk` rows x 32 k values, all S slices of a block one after the
 // other, each in the K-major operand layout with 64-byte swizzle (rows of 32
 // values, 8-row groups kOzSbo apart), so that a chunk of a tile is one contiguous
-// copy.
+// copy.  The slices of the last row range end with its last row (padded to 128 rows, one
+// row over 2^22 values of k took 7.5 GB); they are copied one by one.
+constexpr int kOzRow = kOzKStep * 2;   // bytes of a row of a slice
 struct OzSide : ScanSide {
     int nkc, blk;
     int64_t dst;         // bytes from the slice buffer to block (0, 0)
@@ -108,10 +110,11 @@ __global__ void __launch_bounds__(256) k_oz_slice(const OzSide* __restrict__ sid
             X[t] = (b >> 63) ? -(long long)f : (long long)f;
         }
     }
-    const int row = 8 * rg, blk = row / sd.blk;
-    const int64_t slice = (int64_t)sd.blk * kOzKStep * 2;
-    unsigned char* dst = buf + sd.dst + ((int64_t)blk * sd.nkc + kc) * S * slice + (row % sd.blk) / 8 * kOzSbo +
-                         (lane & 7) * 64 + (kg ^ ((lane >> 1) & 3)) * 16;
+    if (!on) return;
+    const int row0 = r / sd.blk * sd.blk;   // of the block
+    const int64_t slice = (int64_t)min(sd.blk, sd.n - row0) * kOzRow;
+    unsigned char* dst = buf + sd.dst + (int64_t)row0 * sd.nkc * S * kOzRow + (int64_t)kc * S * slice +
+                         (r - row0) * kOzRow + (kg ^ ((lane >> 1) & 3)) * 16;
     for (int p = S - 1; p >= 0; --p) {
         uint32_t w[4];
 #pragma unroll
@@ -209,6 +212,17 @@ __device__ __forceinline__ int oz_int(float v) {
     return ((int)__float_as_uint(h) - 0x4B400000) * 4 + ((int)__float_as_uint(l) - 0x4B400000);
 }
 
+// The S slices of a chunk, `bytes` each, to `stride` bytes apart in shared memory.
+template <int S>
+__device__ __forceinline__ void load_slices(uint32_t dst, const unsigned char* src, uint32_t bytes, uint32_t stride,
+                                            uint32_t bar) {
+    if (bytes == stride) {
+        tc::bulk_load(dst, src, S * stride, bar);
+        return;
+    }
+    for (int p = 0; p < S; ++p) tc::bulk_load(dst + p * stride, src + (int64_t)p * bytes, bytes, bar);
+}
+
 template <int S, int B>
 __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restrict__ prods,
                                                            const OzTile* __restrict__ tiles, int n_tiles,
@@ -248,8 +262,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                 const OzTile tl = tiles[t];
                 const OzProd& pd = prods[tl.prod];
                 const int nkc = pd.nkc;
-                const unsigned char* a = slices + pd.a_off + (int64_t)(tl.m0 / kOzM) * nkc * kBytesA;
-                const unsigned char* b = slices + pd.b_off + (int64_t)(tl.n0 / kOzN) * nkc * kBytesB;
+                const unsigned char* a = slices + pd.a_off + (int64_t)tl.m0 * nkc * (S * kOzRow);
+                const unsigned char* b = slices + pd.b_off + (int64_t)tl.n0 * nkc * (S * kOzRow);
+                // bytes of a slice; the rows that the last blocks lack are whatever stands in shared
+                // memory there (they reach only entries that are not stored)
+                const uint32_t sa = (uint32_t)min(kOzM, pd.M - tl.m0) * kOzRow;
+                const uint32_t sb = (uint32_t)min(kOzN, pd.N - tl.n0) * kOzRow;
                 for (int c = 0; c < nkc; ++c, ++it) {
                     const int s = it % kStages;
                     if (it >= kStages && !tc::mbar_wait(empty(s), (it / kStages - 1) & 1)) {
@@ -257,9 +275,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                         break;
                     }
                     const uint32_t dst = base + s * kStage;
-                    tc::mbar_expect(full(s), kStage);
-                    tc::bulk_load(dst, a + (int64_t)c * kBytesA, kBytesA, full(s));
-                    tc::bulk_load(dst + kBytesA, b + (int64_t)c * kBytesB, kBytesB, full(s));
+                    tc::mbar_expect(full(s), S * (sa + sb));
+                    load_slices<S>(dst, a + (int64_t)c * (S * sa), sa, kOzSliceA, full(s));
+                    load_slices<S>(dst + kBytesA, b + (int64_t)c * (S * sb), sb, kOzSliceB, full(s));
                 }
             }
             // copies in flight land before the CTA may end
@@ -412,7 +430,7 @@ void launch_gemm_ozaki_group(Context* ctx, const std::vector<OzGemm>& gs, int sl
     double fl = 0.0;
     auto side = [&](const double* src, int64_t rs, int64_t ks, int n, int K, int nkc, int blk) {
         const OzSide sd{{src, rs, ks, n, K, rows, max_ctas}, nkc, blk, bytes, cut_ctas};
-        bytes += (int64_t)((n + blk - 1) / blk) * nkc * S * blk * kOzKStep * 2;
+        bytes += (int64_t)n * nkc * S * kOzRow;
         rows += n;
         const int groups = (n + 7) / 8;
         max_ctas += scan_ctas(ks, n, K);

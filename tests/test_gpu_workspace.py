@@ -37,3 +37,9 @@ def test_narrow_network_on_a_large_batch():
     call = "net.loss_grad(x, x)"
     setup = "x = np.ones((1 << 21, 2), np.float32); net = nat.MLP(ctx, [2, 2], np.ones(6, np.float32))"
     assert taken(setup, call) <= 2 * 256 * MB + 8 * 64 * MB
+
+
+def test_thin_emulated_product():
+    """One row times one column over 2^22 values of k: 16 bytes of slices a value (two factors), 64 MB aside."""
+    setup = "A = torch.ones(1, 1 << 22, dtype=torch.float64, device='cuda'); B = A.T.contiguous(); C = A[:, :1].clone()"
+    assert taken(setup, "nat.gemm_ozaki(ctx, A, B, C)") <= 2 * 16 * (4 * MB) + 64 * MB
