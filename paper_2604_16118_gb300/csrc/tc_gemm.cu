@@ -286,9 +286,11 @@ finish:
 // A once per 64 columns of C) and scans them for the scales first; for one product
 // of 3000 x 1100 x 700 that took 800 us.  Here k_row_max finds the scales, k_tc_split
 // writes the TF32 parts once, in operand layout (128 rows x 32 k values per block,
-// 128-byte swizzle: the high parts, then the low parts), and k_gemm_split streams
-// blocks by bulk copies through a ring of stages: the same products in the same
-// order per entry.
+// 128-byte swizzle: the high parts, then the low parts; the blocks of the last row range
+// end with its last row), and k_gemm_split streams blocks by bulk copies through a ring of
+// stages: the same products in the same order per entry.  Workspace: 8 bytes per value of
+// the factors, K rounded up to 32; where the device has no room for it the grouped
+// kernel, which needs none, takes the product.
 
 // One factor with its split blocks and power-of-two exponents (alpha folded into A).
 struct SplitSide : ScanSide {
@@ -300,7 +302,8 @@ struct SplitSide : ScanSide {
 };
 
 constexpr int kSpTile = 128;                          // rows and columns of a tile
-constexpr uint32_t kSpPart = kSpTile * kTcK * 4;      // bytes of the high (or low) parts of a block
+constexpr int kSpRow = kTcK * 4;                      // bytes of a row of a part
+constexpr uint32_t kSpPart = kSpTile * kSpRow;        // bytes of the high (or low) parts of a full block
 constexpr uint32_t kSpStage = 4 * kSpPart;            // A and B blocks of one chunk
 constexpr int kSpStages = 3;
 constexpr int kSpThreads = 192;                       // producer warp, MMA warp, four epilogue warps
@@ -323,8 +326,10 @@ __global__ void __launch_bounds__(256) k_tc_split(const SplitSide* __restrict__ 
         kc = u / ng;
     }
     if (kc >= sd.nkc || 8 * rg >= sd.n) return;
-    unsigned char* dst = buf + sd.dst + ((int64_t)(8 * rg / kSpTile) * sd.nkc + kc) * (2 * kSpPart) +
-                         (8 * rg % kSpTile) / 8 * 1024;
+    const int row0 = 8 * rg / kSpTile * kSpTile;   // of the block
+    const int64_t part = (int64_t)min(kSpTile, sd.n - row0) * kSpRow;
+    unsigned char* dst =
+        buf + sd.dst + (int64_t)row0 * sd.nkc * (2 * kSpRow) + kc * 2 * part + (8 * rg - row0) * kSpRow;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         // rows contiguous in k: eight lanes along k; rows contiguous across: eight lanes along the rows
@@ -337,20 +342,32 @@ __global__ void __launch_bounds__(256) k_tc_split(const SplitSide* __restrict__ 
         const int sc = sd.is_b ? pow2_exponent(top)
                                              : mxa > 0.0 ? pow2_exponent((unsigned long long)__double_as_longlong(mxa)) : 0;
         if (r < sd.n && kc == 0 && kg == 0) exps[sd.row0 + r] = sc;
+        if (r >= sd.n) continue;
         uint32_t hi[4], lo[4];
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             const int k = kTcK * kc + 4 * kg + t;
             hi[t] = lo[t] = 0u;
-            if (r < sd.n && k < sd.K)
+            if (k < sd.K)
                 split_scaled(
                     (unsigned long long)__double_as_longlong(sd.alpha * sd.src[(int64_t)r * sd.rs + k * sd.ks]), sc,
                     &hi[t], &lo[t]);
         }
-        unsigned char* o = dst + rr * 128 + (kg ^ rr) * 16;
+        unsigned char* o = dst + rr * kSpRow + (kg ^ rr) * 16;
         *(uint4*)o = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *(uint4*)(o + kSpPart) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        *(uint4*)(o + part) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
+}
+
+// High and low parts of one block (`part` bytes each) to kSpPart apart in shared memory; the
+// rows that a last block lacks are whatever stands there (they reach only entries that are not stored).
+__device__ __forceinline__ void load_parts(uint32_t dst, const unsigned char* src, uint32_t part, uint32_t bar) {
+    if (part == kSpPart) {
+        tc::bulk_load(dst, src, 2 * kSpPart, bar);
+        return;
+    }
+    tc::bulk_load(dst, src, part, bar);
+    tc::bulk_load(dst + kSpPart, src + part, part, bar);
 }
 
 // C tile (128 x 128 per CTA): one thread streams the chunks (64 KB each) into three
@@ -381,8 +398,9 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, i
     bool ok = true;
     if (warp == 0) {
         if (lane == 0) {
-            const unsigned char* a = A + (int64_t)blockIdx.x * nkc * (2 * kSpPart);
-            const unsigned char* b = B + (int64_t)blockIdx.y * nkc * (2 * kSpPart);
+            const unsigned char* a = A + (int64_t)m0 * nkc * (2 * kSpRow);
+            const unsigned char* b = B + (int64_t)n0 * nkc * (2 * kSpRow);
+            const uint32_t pa = min(kSpTile, o.M - m0) * kSpRow, pb = min(kSpTile, o.N - n0) * kSpRow;
             int c = 0;
             for (; c < nkc; ++c) {
                 const int s = c % kSpStages;
@@ -391,9 +409,9 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, i
                     break;
                 }
                 const uint32_t dst = base + s * kSpStage;
-                tc::mbar_expect(full(s), kSpStage);
-                tc::bulk_load(dst, a + (int64_t)c * (2 * kSpPart), 2 * kSpPart, full(s));
-                tc::bulk_load(dst + 2 * kSpPart, b + (int64_t)c * (2 * kSpPart), 2 * kSpPart, full(s));
+                tc::mbar_expect(full(s), 2 * (pa + pb));
+                load_parts(dst, a + (int64_t)c * (2 * pa), pa, full(s));
+                load_parts(dst + 2 * kSpPart, b + (int64_t)c * (2 * pb), pb, full(s));
             }
             // copies in flight land before the CTA may end
             for (int i = c > kSpStages ? c - kSpStages : 0; i < c; ++i)
@@ -451,14 +469,15 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, i
     if (warp == 1) tc::tmem_free(tmem, kSpTile);
 }
 
-void launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kind) {
+// false, with nothing launched: no room for the parts on the device.
+bool launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kind) {
     const int nkc = (in.K + kTcK - 1) / kTcK;
     std::vector<SplitSide> sides;
     int64_t bytes = 0;
     int rows = 0, max_ctas = 0, cut_ctas = 0;
     auto side = [&](const double* src, int64_t rs, int64_t ks, int n, double alpha, int is_b) {
         sides.push_back({{src, rs, ks, n, in.K, rows, max_ctas}, nkc, alpha, is_b, bytes, cut_ctas});
-        bytes += (int64_t)((n + kSpTile - 1) / kSpTile) * nkc * (2 * kSpPart);
+        bytes += (int64_t)n * nkc * (2 * kSpRow);
         rows += n;
         const int groups = (n + 7) / 8;
         max_ctas += scan_ctas(ks, n, in.K);
@@ -466,12 +485,19 @@ void launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kin
     };
     side(in.A, in.lda, 1, o.M, in.alpha, 0);
     side(in.B, 1, in.ldb, o.N, 1.0, 1);
+    Scratch s(ctx);
+    unsigned char* buf = nullptr;
+    try {
+        buf = (unsigned char*)ctx->alloc((size_t)bytes);
+    } catch (const Error& e) {
+        if (e.code != BSMPS_ERR_OOM) throw;
+        (void)cudaGetLastError();
+        return false;
+    }
+    s.ptrs.push_back(buf);
     const double fl = 2.0 * o.M * (double)o.N * in.K;
     const double by = 8.0 * ((double)o.M * in.K + (double)in.K * o.N + o.M * (double)o.N * (o.beta == 0.0 ? 1.0 : 2.0));
     ctx->flops += fl;
-    Scratch s(ctx);
-    unsigned char* buf = (unsigned char*)ctx->alloc((size_t)bytes);
-    s.ptrs.push_back(buf);
     unsigned long long* mx = (unsigned long long*)ctx->alloc(sizeof(unsigned long long) * (size_t)rows);
     s.ptrs.push_back(mx);
     int* exps = (int*)ctx->alloc(sizeof(int) * (size_t)rows);
@@ -494,6 +520,7 @@ void launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kin
                                                           buf + sides[1].dst, exps, ctx->err_word());
     check_launch(ctx);
     ps.done();
+    return true;
 }
 
 }  // namespace
@@ -513,10 +540,9 @@ void launch_gemm_tf32x3(Context* ctx, const std::vector<GemmOut>& outs, const st
     // several contributions).
     if (outs.size() == 1 && outs[0].end == outs[0].beg + 1 && !ins[outs[0].beg].transA && outs[0].M > 0 &&
         outs[0].N > 0 && ins[outs[0].beg].K > 0 &&
-        (double)outs[0].M * outs[0].N * ins[outs[0].beg].K >= (double)(1 << 17)) {
-        launch_gemm_split(ctx, outs[0], ins[outs[0].beg], kind);
+        (double)outs[0].M * outs[0].N * ins[outs[0].beg].K >= (double)(1 << 17) &&
+        launch_gemm_split(ctx, outs[0], ins[outs[0].beg], kind))
         return;
-    }
     std::vector<TcTile> tiles;
     double fl = 0.0, by = 0.0;
     for (int o = 0; o < (int)outs.size(); ++o) {

@@ -43,3 +43,30 @@ def test_thin_emulated_product():
     """One row times one column over 2^22 values of k: 16 bytes of slices a value (two factors), 64 MB aside."""
     setup = "A = torch.ones(1, 1 << 22, dtype=torch.float64, device='cuda'); B = A.T.contiguous(); C = A[:, :1].clone()"
     assert taken(setup, "nat.gemm_ozaki(ctx, A, B, C)") <= 2 * 16 * (4 * MB) + 64 * MB
+
+
+def test_thin_split_product():
+    """Two rows times two columns over 2^20 values of k: 8 bytes of parts a value, 64 MB aside."""
+    setup = "A = torch.ones(2, 1 << 20, dtype=torch.float64, device='cuda'); B = A.T.contiguous(); C = A[:, :2].clone()"
+    assert taken(setup, "nat.gemm_tf32x3(ctx, A, B, C)") <= 4 * 8 * MB + 64 * MB
+
+
+def test_split_product_without_room_for_its_parts():
+    """The device full up to half of the workspace of the product: it runs on the kernel that needs none."""
+    setup = """
+n, k = 2048, 65536
+g = torch.Generator(device="cuda").manual_seed(1)
+A = torch.randn(n, k, dtype=torch.float64, device="cuda", generator=g)
+B = torch.randn(k, n, dtype=torch.float64, device="cuda", generator=g)
+C = torch.empty(n, n, dtype=torch.float64, device="cuda")
+nat.gemm_tf32x3(ctx, A[:64, :64], B[:64, :64], C[:64, :64])
+full = torch.empty(torch.cuda.mem_get_info()[0] - 8 * n * k, dtype=torch.uint8, device="cuda")
+"""
+    check = """
+ctx.sync()
+del full
+torch.cuda.empty_cache()
+R, S = A[:100] @ B, A[:100].abs() @ B.abs()
+assert ((C[:100] - R).abs() <= 2.0 ** -21 * (4 + k ** 0.5) * S).all()
+"""
+    taken(setup, "nat.gemm_tf32x3(ctx, A, B, C)" + check)
