@@ -372,7 +372,9 @@ __device__ __forceinline__ void load_parts(uint32_t dst, const unsigned char* sr
 
 // C tile (128 x 128 per CTA): one thread streams the chunks (64 KB each) into three
 // stages, one issues 12 MMAs per chunk (A_lo B_hi, A_hi B_lo, A_hi B_hi per 8 values of k),
-// four warps read the accumulators and store FP64.  Waits bounded as above.
+// four warps read the accumulators and store FP64.  Waits bounded as above; the wait for the
+// last product covers all of K (0.4 us a chunk) and has another second for every 65536 chunks.
+// Tiles in one grid dimension, rows first (the others end at 65535).
 __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, int nkc, int e_a, int e_b,
                                                               const unsigned char* __restrict__ A,
                                                               const unsigned char* __restrict__ B,
@@ -382,7 +384,8 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, i
     __shared__ uint32_t tmem_slot;
     const uint32_t base = (smem_addr(sp_smem) + 1023u) & ~1023u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * kSpTile, n0 = blockIdx.y * kSpTile;
+    const int tm = (o.M + kSpTile - 1) / kSpTile;
+    const int m0 = (int)(blockIdx.x % tm) * kSpTile, n0 = (int)(blockIdx.x / tm) * kSpTile;
     auto full = [&](int s) { return smem_addr(&bars[s]); };
     auto empty = [&](int s) { return smem_addr(&bars[kSpStages + s]); };
     const uint32_t done = smem_addr(&bars[2 * kSpStages]);
@@ -443,7 +446,8 @@ __global__ void __launch_bounds__(kSpThreads, 1) k_gemm_split(const GemmOut o, i
         }
         __syncwarp();
     } else {
-        ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
+        ok = false;
+        for (int i = 0; i <= nkc >> 16 && !ok; ++i) ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
         tc::fence_after();
         const int quad = warp & 3, row = m0 + quad * 32 + lane;
         const int e = row < o.M ? exps[e_a + row] : 0;
@@ -515,8 +519,8 @@ bool launch_gemm_split(Context* ctx, const GemmOut& o, const GemmIn& in, int kin
     check_launch(ctx);
     k_tc_split<<<cut_ctas, 256, 0, ctx->stream>>>(d_sides, mx, exps, buf);
     check_launch(ctx);
-    const dim3 grid((unsigned)((o.M + kSpTile - 1) / kSpTile), (unsigned)((o.N + kSpTile - 1) / kSpTile));
-    k_gemm_split<<<grid, kSpThreads, smem, ctx->stream>>>(o, nkc, sides[0].row0, sides[1].row0, buf + sides[0].dst,
+    const unsigned tiles = (unsigned)((o.M + kSpTile - 1) / kSpTile) * (unsigned)((o.N + kSpTile - 1) / kSpTile);
+    k_gemm_split<<<tiles, kSpThreads, smem, ctx->stream>>>(o, nkc, sides[0].row0, sides[1].row0, buf + sides[0].dst,
                                                           buf + sides[1].dst, exps, ctx->err_word());
     check_launch(ctx);
     ps.done();
