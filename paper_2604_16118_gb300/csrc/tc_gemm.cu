@@ -538,15 +538,22 @@ bool gemm_tf32x3_eligible(const std::vector<GemmOut>& outs, const std::vector<Ge
 
 void launch_gemm_tf32x3(Context* ctx, const std::vector<GemmOut>& outs, const std::vector<GemmIn>& ins, int kind) {
     if (outs.empty()) return;
-    // One product with one contribution (bsmps_gemm_tf32x3, whole iterates): split once.  Below
-    // 2^17 multiplications its three launches cost more than the grouped kernel's repeated splits
-    // save; the grouped launches of the zip-up stay on the grouped kernel (the scales there span
-    // several contributions).
+    // One product with one contribution (bsmps_gemm_tf32x3, a contraction with a single block): split
+    // once.  Below 2^17 multiplications its three launches cost more than the grouped kernel's repeated splits
+    // save, and so they do where few rows meet short sums (the columns are split once either way,
+    // and their parts padded to 32 values of k and written to memory): rows x columns x k, grouped
+    // against split, 1 x 131072 x 1 76 and 146 us, 1 x 20000 x 64 51 and 63, x 128 76 and 65; 16 x 20000 x
+    // 32 44 and 61, x 80 66 and 63; 32 x 20000 x 32 52 and 66, x 64 72 and 71; 64 x 20000 x 32 72 and 71.
+    // The grouped launches of the zip-up stay on the grouped kernel (the scales there span several
+    // contributions).
     if (outs.size() == 1 && outs[0].end == outs[0].beg + 1 && !ins[outs[0].beg].transA && outs[0].M > 0 &&
-        outs[0].N > 0 && ins[outs[0].beg].K > 0 &&
-        (double)outs[0].M * outs[0].N * ins[outs[0].beg].K >= (double)(1 << 17) &&
-        launch_gemm_split(ctx, outs[0], ins[outs[0].beg], kind))
-        return;
+        outs[0].N > 0 && ins[outs[0].beg].K > 0) {
+        const GemmIn& in = ins[outs[0].beg];
+        const int nkc = (in.K + kTcK - 1) / kTcK;
+        if ((double)outs[0].M * outs[0].N * in.K >= (double)(1 << 17) && (nkc >= 4 || outs[0].M >= (128 >> nkc)) &&
+            launch_gemm_split(ctx, outs[0], in, kind))
+            return;
+    }
     std::vector<TcTile> tiles;
     double fl = 0.0, by = 0.0;
     for (int o = 0; o < (int)outs.size(); ++o) {

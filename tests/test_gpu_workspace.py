@@ -70,3 +70,11 @@ R, S = A[:100] @ B, A[:100].abs() @ B.abs()
 assert ((C[:100] - R).abs() <= 2.0 ** -21 * (4 + k ** 0.5) * S).all()
 """
     taken(setup, "nat.gemm_tf32x3(ctx, A, B, C)" + check)
+
+
+def test_few_rows_and_short_sums_take_no_parts():
+    """One row times 2^20 columns, one value of k: the kernel without a workspace (a list of 2^14 tiles)
+    is the faster one there."""
+    setup = "A = torch.ones(1, 1, dtype=torch.float64, device='cuda'); B = torch.ones(1, MB, dtype=torch.float64, " \
+            "device='cuda'); C = B.clone()".replace("MB", str(MB))
+    assert taken(setup, "nat.gemm_tf32x3(ctx, A, B, C)") <= 64 * MB
