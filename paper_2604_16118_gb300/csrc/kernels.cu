@@ -324,8 +324,10 @@ struct FlatCores {
     int n;
 };
 
-__global__ void __launch_bounds__(kThreads) k_flat_cores(const FlatCores fc, double* __restrict__ flat, int to_cores) {
-    for (int64_t e = fc.beg[0] + (int64_t)blockIdx.x * kThreads + threadIdx.x; e < fc.beg[fc.n];
+// Entries lo_e .. hi_e of the concatenated cores, entry e at flat[e - flat0].
+__global__ void __launch_bounds__(kThreads) k_flat_cores(const FlatCores fc, double* __restrict__ flat, int64_t flat0,
+                                                         int64_t lo_e, int64_t hi_e, int to_cores) {
+    for (int64_t e = lo_e + (int64_t)blockIdx.x * kThreads + threadIdx.x; e < hi_e;
          e += (int64_t)gridDim.x * kThreads) {
         int lo = 0, hi = fc.n - 1;
         while (lo < hi) {
@@ -334,13 +336,13 @@ __global__ void __launch_bounds__(kThreads) k_flat_cores(const FlatCores fc, dou
             else hi = mid - 1;
         }
         double* c = fc.core[lo] + (e - fc.beg[lo]);
-        if (to_cores) *c = flat[e];
-        else flat[e] = *c;
+        if (to_cores) *c = flat[e - flat0];
+        else flat[e - flat0] = *c;
     }
 }
 
 void launch_flat_cores(Context* ctx, const std::vector<double*>& core, const std::vector<int64_t>& n, double* flat,
-                       bool to_cores) {
+                       int64_t beg, int64_t end, bool to_cores) {
     configure_carveout();
     int64_t off = 0;
     for (size_t t = 0; t < core.size();) {
@@ -354,10 +356,11 @@ void launch_flat_cores(Context* ctx, const std::vector<double*>& core, const std
         }
         fc.beg[fc.n] = off;
         if (fc.n == 0) continue;
-        const int64_t total = off - fc.beg[0];
+        const int64_t lo = std::max(beg, fc.beg[0]), hi = std::min(end, off), total = hi - lo;
+        if (total <= 0) continue;
         const unsigned ctas = (unsigned)std::min<int64_t>((total + 4 * kThreads - 1) / (4 * kThreads), 1024);
         ProfScope ps(ctx, KK_COPY, 0.0, 16.0 * (double)total);
-        k_flat_cores<<<ctas, kThreads, 0, ctx->stream>>>(fc, flat, to_cores ? 1 : 0);
+        k_flat_cores<<<ctas, kThreads, 0, ctx->stream>>>(fc, flat, beg, lo, hi, to_cores ? 1 : 0);
         check_launch(ctx);
         ps.done();
     }

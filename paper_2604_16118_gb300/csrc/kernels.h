@@ -128,10 +128,10 @@ void launch_copy(Context* ctx, const std::vector<CopyTask>& tasks, int kind = KK
 // Sets n[i] doubles at ptr[i] to zero, all regions in one launch.
 void launch_zero(Context* ctx, const std::vector<double*>& ptr, const std::vector<int64_t>& n,
                  int kind = KK_COPY);
-// Copies between the cores (n[t] doubles at core[t], one buffer each) and their
-// concatenation `flat`: into the cores (to_cores) or out of them.
+// Copies between the cores (n[t] doubles at core[t], one buffer each) and the entries
+// beg .. end of their concatenation, held at `flat`: into the cores (to_cores) or out of them.
 void launch_flat_cores(Context* ctx, const std::vector<double*>& core, const std::vector<int64_t>& n, double* flat,
-                       bool to_cores);
+                       int64_t beg, int64_t end, bool to_cores);
 // Counts a launch and raises the launch error, if any.
 void check_launch(Context* ctx);
 // The same grouped GEMM on the tensor cores in split precision (3xTF32, FP32

@@ -41,14 +41,22 @@ static MpsPtr make_mps(Context* ctx, const Layout& L, bool zero) { return MpsPtr
 
 // The flat layout of an iterate and its cores (one buffer per core) meet in one
 // staging buffer: one host copy and one kernel instead of a copy per core (a
-// small copy from or to pageable memory costs 10 to 20 us).
+// small copy from or to pageable memory costs 10 to 20 us).  Iterates beyond 64 MB pass
+// through it in pieces (a piece's copy takes milliseconds), so that an import or
+// export needs no second buffer of the iterate's size.
+constexpr int64_t kStageDoubles = (int64_t)8 << 20;
+
 void mps_upload(Mps* x, const double* host) {
     const int64_t n = x->lay.total();
     if (n > 0) {
         Scratch s(x->ctx);
-        double* flat = s.dbl((size_t)n);
-        BSM_CUDA(cudaMemcpyAsync(flat, host, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, x->ctx->stream));
-        launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, true);
+        double* flat = s.dbl((size_t)std::min(n, kStageDoubles));
+        for (int64_t b = 0; b < n; b += kStageDoubles) {
+            const int64_t e = std::min(n, b + kStageDoubles);
+            BSM_CUDA(cudaMemcpyAsync(flat, host + b, (size_t)(e - b) * sizeof(double), cudaMemcpyHostToDevice,
+                                     x->ctx->stream));
+            launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, b, e, true);
+        }
     }
     x->ctx->sync();
 }
@@ -57,9 +65,13 @@ void mps_download(const Mps* x, double* host) {
     const int64_t n = x->lay.total();
     if (n > 0) {
         Scratch s(x->ctx);
-        double* flat = s.dbl((size_t)n);
-        launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, false);
-        BSM_CUDA(cudaMemcpyAsync(host, flat, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, x->ctx->stream));
+        double* flat = s.dbl((size_t)std::min(n, kStageDoubles));
+        for (int64_t b = 0; b < n; b += kStageDoubles) {
+            const int64_t e = std::min(n, b + kStageDoubles);
+            launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, b, e, false);
+            BSM_CUDA(cudaMemcpyAsync(host + b, flat, (size_t)(e - b) * sizeof(double), cudaMemcpyDeviceToHost,
+                                     x->ctx->stream));
+        }
         x->ctx->sync();
         return;
     }

@@ -78,3 +78,24 @@ def test_few_rows_and_short_sums_take_no_parts():
     setup = "A = torch.ones(1, 1, dtype=torch.float64, device='cuda'); B = torch.ones(1, MB, dtype=torch.float64, " \
             "device='cuda'); C = B.clone()".replace("MB", str(MB))
     assert taken(setup, "nat.gemm_tf32x3(ctx, A, B, C)") <= 64 * MB
+
+
+def test_import_write_and_export_of_a_large_iterate():
+    """Eight blocks of 3000 x 3000 (576 MB): what the calls need beside the iterate is one piece of 64 MB, and
+    the values come back as they went in, across the edges of cores and pieces."""
+    setup = """
+d = 3000
+bonds = [{(0, 0): 1}, {(0, 0): d, (1, 0): d}, {(0, 0): d, (1, 0): d, (2, 0): d}, {(1, 0): d, (2, 0): d}, {(2, 0): 1}]
+n = 8 * d * d + 4 * d
+v = np.random.default_rng(1).standard_normal(n)
+x = nat.mps_import(ctx, 4, 0, 2, 0, bonds, np.zeros(n))
+del x
+import gc; gc.collect()
+x = nat.mps_import(ctx, 4, 0, 2, 0, bonds, v)
+assert np.array_equal(x.export(), v)
+x.write(v[::-1].copy())
+assert np.array_equal(x.export(), v[::-1])
+"""
+    head = "base = torch.cuda.mem_get_info()[0]\n"
+    check = "assert base - torch.cuda.mem_get_info()[0] <= 8 * n + 8 * 64 * 2 ** 20, base - torch.cuda.mem_get_info()[0]"
+    taken(head + setup, check)
