@@ -367,12 +367,14 @@ __device__ __forceinline__ void reflect_segments(double* A, double tj, double vj
     const double* v = A + (int64_t)j * M;
     for (int cb = c0 + 4 * w; cb < N; cb += 4 * nw) {
         const int c = cb + (lane >> 3);
-        double* a = A + (int64_t)(c < N ? c : cb) * M;
-        const double a_j = a[j];
+        const bool on = c < N;   // (a segment without a column reads none: another one may be writing it)
+        double* a = A + (int64_t)(on ? c : cb) * M;
+        const double a_j = on ? a[j] : 0.0;
         double d = sl == 0 ? vj * a_j : 0.0;
-        for (int i = j + 1 + sl; i < M; i += 8) d = fma(v[i], a[i], d);
+        if (on)
+            for (int i = j + 1 + sl; i < M; i += 8) d = fma(v[i], a[i], d);
         const double tw = tj * seg8_sum(d);
-        if (c < N) {
+        if (on) {
             if (sl == 0) a[j] = fma(-tw, vj, a_j);
             for (int i = j + 1 + sl; i < M; i += 8) a[i] = fma(-tw, v[i], a[i]);
         }
@@ -459,7 +461,8 @@ __device__ __forceinline__ void apply_q(const double* A, const double* tau, doub
             const double* v = A + (int64_t)j * M;
             const int i0 = j + ((sl - j) & 7);
             double d = 0.0;
-            for (int i = i0; i < M; i += 8) d = fma(v[i], x[i], d);
+            if (own)
+                for (int i = i0; i < M; i += 8) d = fma(v[i], x[i], d);
             const double tw = tj * seg8_sum(d);
             if (own)
                 for (int i = i0; i < M; i += 8) x[i] = fma(-tw, v[i], x[i]);
@@ -707,6 +710,7 @@ __device__ __forceinline__ float jacobi_angle(double d, double g) {
 
 // Round-robin over k columns, one pair per 8-lane segment u: the pair of a round
 // follows from the one before (position 0 stands still, the others move on by one).
+// get(): false, and columns that other segments may be writing, for a segment without a pair.
 struct SegPair {
     int a, b, n2, k;
     bool fixed;
@@ -758,8 +762,8 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
 #pragma unroll
                 for (int r = 0; r < RG; ++r) {
                     const int i = sl + 8 * r;
-                    xp[r] = Gp[i];
-                    xq[r] = Gq[i];
+                    xp[r] = on ? Gp[i] : 0.0f;
+                    xq[r] = on ? Gq[i] : 0.0f;
                     a = fmaf(xp[r], xp[r], a);
                     b = fmaf(xq[r], xq[r], b);
                     g = fmaf(xp[r], xq[r], g);
@@ -767,8 +771,8 @@ __device__ __forceinline__ void jacobi_f32_segments(float* G, float* V, int k, i
 #pragma unroll
                 for (int r = 0; r < RV; ++r) {
                     const int i = sl + 8 * r;
-                    vp[r] = Vp[i];
-                    vq[r] = Vq[i];
+                    vp[r] = on ? Vp[i] : 0.0f;
+                    vq[r] = on ? Vq[i] : 0.0f;
                 }
                 a = seg8_sum(a);
                 b = seg8_sum(b);
@@ -892,7 +896,7 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
                     t = jacobi_angle(b - a, g);
                     over |= gs > 0x1p20f * nab || fabsf(t) > 0x1p-28f ? 3 : 1;
                 }
-                if (sl == 0) {
+                if (sl == 0 && eb + (lane >> 3) < np) {
                     Xf[q * k + p] = -t;
                     Xf[p * k + q] = t;
                 }
@@ -934,12 +938,12 @@ __device__ __forceinline__ void jacobi_f64_segments(double* G, double* V, double
 #pragma unroll
                 for (int r = 0; r < RG; ++r) {
                     const int i = sl + 8 * r;
-                    xp[r] = Gp[i];
-                    xq[r] = Gq[i];
+                    xp[r] = on ? Gp[i] : 0.0;
+                    xq[r] = on ? Gq[i] : 0.0;
                     g = fma(xp[r], xq[r], g);
                 }
-                const double a = nrm[p], b = nrm[q];
-                const float dp = del[p], dq = del[q];
+                const double a = on ? nrm[p] : 0.0, b = on ? nrm[q] : 0.0;
+                const float dp = on ? del[p] : 0.0f, dq = on ? del[q] : 0.0f;
                 const float af = to_float_scaled(a, 0), bf = to_float_scaled(b, 0);
                 const float nab = (af * rsqrt_fast(af)) * (bf * rsqrt_fast(bf));
                 const double d = b - a;

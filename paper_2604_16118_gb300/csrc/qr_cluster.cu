@@ -66,8 +66,11 @@ __device__ __forceinline__ void qc_update(double* Al, const double* v, double tj
         const int lp = cb + lane / L;
         const bool on = lp < n && lp != skip;
         double* a = Al + (size_t)(on ? lp : lp0) * M;
-        double d = sl == 0 ? vj * a[j] : 0.0;
-        for (int i = j + 1 + sl; i < M; i += L) d = fma(v[i], a[i], d);
+        double d = 0.0;
+        if (on) {   // (a segment without a column reads none: another one may be writing it)
+            if (sl == 0) d = vj * a[j];
+            for (int i = j + 1 + sl; i < M; i += L) d = fma(v[i], a[i], d);
+        }
         const double tw = tj * seg_sum_of<L>(d);
         if (on) {
             if (sl == 0) a[j] = fma(-tw, vj, a[j]);
