@@ -12,6 +12,8 @@ profiled per kernel kind with CUDA events on the library's stream.
 value: MPO.MPS apply throughput, TFLOP/s: the algorithmic flops of the zip-up
 contraction stage (sum of 2mnk over its grouped-GEMM work list, which includes
 the MPO channel combine) over that stage's device time in the timed steps.
+The kernels sum entries that share a block of the iterate before they multiply;
+fractions of a peak are taken of the flops they run ("flops_run").
 The whole step's algorithmic flops and time are reported beside it ("step").
 --precision tf32x3 runs the contraction on the tensor cores in split precision
 (the solver's policy falls back to FP64 once the split error estimate nears the
@@ -250,6 +252,18 @@ def apply_flops_per_branch(nat, ctx, S):
     return st["apply"][2]
 
 
+def profiled_kinds(ctx):
+    """{kind: (launches, ms, flops, bytes, flops run)} of the profiled launches, cleared after reading.
+    flops: 2 m n k of every term's product (the throughput unit, the same for every arm); flops run: what
+    the kernels do for them, which is what may be set against a peak rate."""
+    run = ctx.kernel_executed()
+    return {k: (*v, run[k]) for k, v in ctx.kernel_stats(reset=True).items()}
+
+
+def kinds_json(kinds):
+    return {k: {"launches": v[0], "ms": v[1], "flops": v[2], "bytes": v[3], "flops_run": v[4]} for k, v in kinds.items()}
+
+
 def run_reference(args):
     """The oracle arm: each step is the oracle's zip-up application of one
     preconditioner branch of the full-rank iterate (a bounded sample of the
@@ -382,9 +396,9 @@ def main_joint(args):
     clocks = sampler.stop()
     ctx.profile(True)
     x, _ = nat.eigensolve_joint_step(ctx, S["W"], S["p"], S["sp"], st, x)
-    stats = ctx.kernel_stats(reset=True)
+    stats = profiled_kinds(ctx)
     ctx.profile(False)
-    name, (nl, kms, kfl, kby) = max(stats.items(), key=lambda kv: kv[1][1])
+    name, (nl, kms, _, kby, kfl) = max(stats.items(), key=lambda kv: kv[1][1])
     # end to end through the C ABI with host buffers, from the post-warm-up iterate
     hx, bonds, st.eta_res, st.n = x_after_warmup
     pinned = torch.empty(len(hx), dtype=torch.float64).pin_memory()
@@ -421,7 +435,7 @@ def main_joint(args):
                      "peak": fp64, "unit": "TFLOP/s", "frac": (kfl / (kms * 1e-3) / 1e12 / fp64) if kms else None,
                      "traffic": None, "peak_source": "cuBLAS FP64 GEMM 4096^3 measured in this run",
                      "launches": nl, "kernel_ms": kms},
-        "kernels": {k: {"launches": v[0], "ms": v[1], "flops": v[2], "bytes": v[3]} for k, v in stats.items()},
+        "kernels": kinds_json(stats),
         "steps_info": [{"lambda": [float(v) for v in i["lambda"]], "rho1": float(i["rho"][0]),
                         "eta_tries": i["eta_tries"], "max_rank": i["max_rank"], "flops": i["flops"]}
                        for i in [info0] + infos],
@@ -632,10 +646,10 @@ def main_e1(args):
     # per-kernel roofline from one profiled step (events around every launch)
     ctx.profile(True)
     x, _ = one_step(x)
-    stats = ctx.kernel_stats(reset=True)
+    stats = profiled_kinds(ctx)
     ctx.profile(False)
     dom = max(stats.items(), key=lambda kv: kv[1][1])
-    name, (nl, kms, kfl, kby) = dom
+    name, (nl, kms, _, kby, kfl) = dom
 
     # end to end through the C ABI with host buffers: the same K steps again from
     # the post-warm-up iterate, uploaded from and read back to pinned host memory
@@ -678,7 +692,7 @@ def main_e1(args):
                      "launches": nl, "kernel_ms": kms, "kernel_bytes": kby,
                      "achieved_gbs": kby / (kms * 1e-3) / 1e9 if kms else None,
                      "hbm_peak_gbs": peaks.get("hbm_gbs"), "hbm_peak_source": src},
-        "kernels": {k: {"launches": v[0], "ms": v[1], "flops": v[2], "bytes": v[3]} for k, v in stats.items()},
+        "kernels": kinds_json(stats),
         "steps_info": [{"lambda": i["lambda"], "rho": i["rho"], "eta_tries": i["eta_tries"],
                         "max_rank": i["max_rank"], "flops": i["flops"]} for i in infos],
         "energy": infos[-1]["lambda"] - S["gamma"] if infos else None,
@@ -773,9 +787,9 @@ def main_full(args):
             fl += info["flops"]
             infos.append(info)
             if profile:
-                for k, v in ctx.kernel_stats(reset=True).items():
-                    a = kinds.setdefault(k, [0, 0.0, 0.0, 0.0])
-                    for i in range(4):
+                for k, v in profiled_kinds(ctx).items():
+                    a = kinds.setdefault(k, [0, 0.0, 0.0, 0.0, 0.0])
+                    for i in range(5):
                         a[i] += v[i]
         if profile:
             ctx.profile(False)
@@ -795,12 +809,13 @@ def main_full(args):
     clocks = sampler.stop()
     # the same steps again, every launch bracketed by events
     prof_ms, _, prof_infos, kinds = timed_steps(True)
-    apply_n, apply_ms, apply_fl, apply_by = kinds.get("apply", [0, 0.0, 0.0, 0.0])
-    aq_n, aq_ms, aq_fl, _ = kinds.get("apply_qr", [0, 0.0, 0.0, 0.0])
+    apply_n, apply_ms, apply_fl, apply_by, apply_run = kinds.get("apply", [0, 0.0, 0.0, 0.0, 0.0])
+    aq_n, aq_ms, aq_fl, _, _ = kinds.get("apply_qr", [0, 0.0, 0.0, 0.0, 0.0])
     # the apply: contraction + the zip-up's own factorisation launches; its
     # algorithmic work is the contraction's (Sec. 2.4 work list)
     value = apply_fl / ((apply_ms + aq_ms) * 1e-3) / 1e12 if apply_ms else None
     contraction = apply_fl / (apply_ms * 1e-3) / 1e12 if apply_ms else None
+    contraction_run = apply_run / (apply_ms * 1e-3) / 1e12 if apply_ms else None
     # end to end through the C ABI with host buffers: upload from pinned memory,
     # the step, the iterate read back
     pinned = torch.empty(len(hx), dtype=torch.float64).pin_memory()
@@ -820,7 +835,7 @@ def main_full(args):
     peaks, src = measured_peaks()
     fp64 = fp64_gemm_peak(torch, dev)
     dom = max(kinds.items(), key=lambda kv: kv[1][1])
-    dname, (dn, dms, dfl, dby) = dom
+    dname, (dn, dms, _, dby, dfl) = dom
     dpeak, dbound, dsrc = kind_peak(dname, args.precision, fp64, peaks, src)
     apeak, abound, asrc = kind_peak("apply", args.precision, fp64, peaks, src)
     ach = dfl / (dms * 1e-3) / 1e12 if dms else None
@@ -833,7 +848,9 @@ def main_full(args):
                    "precision": args.precision, "jacobi_precond": args.jacobi_precond,
                    "l2": "flushed between steps (256 MB write)",
                    "parallelism": "replicas" if world > 1 else "single",
-                   "value": "zip-up MPO application (all preconditioner branches): contraction flops / device "
+                   "value": "zip-up MPO application (all preconditioner branches): contraction flops (2 m n k of "
+                            "every operator entry's product, nominal: entries that share a block of the "
+                            "iterate are summed before they are multiplied, see apply.contraction.flops_run) / device "
                             "time of the contraction and the zip-up's factorisation launches, from the timed steps "
                             "rerun with per-launch events"},
         "gpu_launches": launches,
@@ -848,15 +865,16 @@ def main_full(args):
         "apply": {"tflops": value, "ms": apply_ms + aq_ms, "flops": apply_fl,
                   "contraction": {"kernel": "k_gemm_tf32x3" if args.precision == "tf32x3" else "k_gemm/k_gemm_small",
                                   "launches": apply_n, "ms": apply_ms, "bytes": apply_by, "tflops": contraction,
+                                  "flops_run": apply_run, "tflops_run": contraction_run,
                                   "peak": apeak, "bound": abound,
-                                  "frac": contraction / apeak if (contraction and apeak) else None,
+                                  "frac": contraction_run / apeak if (contraction_run and apeak) else None,
                                   "peak_source": asrc,
                                   "achieved_gbs": apply_by / (apply_ms * 1e-3) / 1e9 if apply_ms else None,
                                   "hbm_peak_gbs": peaks.get("hbm_gbs")},
                   "factorisation": {"launches": aq_n, "ms": aq_ms, "flops": aq_fl}},
         "step": {"ms": total_ms / args.steps, "tflops": total_flops / (total_ms * 1e-3) / 1e12,
                  "profiled_ms": prof_ms / args.steps},
-        "kernels": {k: {"launches": v[0], "ms": v[1], "flops": v[2], "bytes": v[3]} for k, v in kinds.items()},
+        "kernels": kinds_json(kinds),
         "steps_info": [{"lambda": i["lambda"], "rho": i["rho"], "eta_tries": i["eta_tries"], "max_rank": i["max_rank"],
                         "flops": i["flops"], "precision": i["precision"]} for i in infos],
         "energy": infos[-1]["lambda"] - S["gamma"] if infos else None,

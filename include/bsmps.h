@@ -182,11 +182,18 @@ BSMPS_API int64_t bsmps_ctx_alloc_count(bsmps_ctx ctx);
  * factorisation launches: zeroing, gathers, QR; 7 the tensor-core products
  * of the learned controller's network, FP32 flops), the number
  * of recorded launches, their summed device time in ms and summed
- * algorithmic FP64 flops and bytes; `reset` != 0 clears the records after
- * reading.  Errors: INVALID_ARG (kind out of range), CUDA. */
+ * algorithmic FP64 flops and bytes (products: 2 m n k for every term of the
+ * method; factorisations: their nominal counts); `reset` != 0 clears the records
+ * after reading.  Errors: INVALID_ARG (kind out of range), CUDA. */
 BSMPS_API bsmps_status bsmps_ctx_profile(bsmps_ctx ctx, int enable);
 BSMPS_API bsmps_status bsmps_ctx_kernel_stats(bsmps_ctx ctx, int kind, int reset, int64_t* launches,
                                               double* ms, double* flops, double* bytes);
+/* Flops the recorded launches of a kind ran for those terms, to be set against a
+ * peak rate: contributions of a grouped product or an environment that share a
+ * factor are summed before they are multiplied, which takes fewer operations than
+ * a product each.  The other kinds as in bsmps_ctx_kernel_stats.  To be read
+ * before the records are cleared.  Errors: INVALID_ARG. */
+BSMPS_API bsmps_status bsmps_ctx_kernel_executed(bsmps_ctx ctx, int kind, double* flops);
 
 /* Diagnostic of the bounded grid-wide waits used by the persistent sweep
  * kernels (no counterpart in the paper).  Launches a two-CTA cooperative

@@ -318,6 +318,16 @@ bsmps_status bsmps_ctx_profile(bsmps_ctx ctx, int enable) {
     });
 }
 
+bsmps_status bsmps_ctx_kernel_executed(bsmps_ctx ctx, int kind, double* flops) {
+    return guarded(ctx, [&] {
+        bsm::Context* c = C(ctx);
+        BSM_REQUIRE(kind >= 0 && kind < bsm::KK_COUNT && flops, BSMPS_ERR_INVALID_ARG, "kernel kind out of range or null out");
+        *flops = 0.0;
+        for (const auto& r : c->prof)
+            if (r.kind == kind) *flops += r.executed;
+    });
+}
+
 bsmps_status bsmps_ctx_kernel_stats(bsmps_ctx ctx, int kind, int reset, int64_t* launches, double* ms,
                                     double* flops, double* bytes) {
     return guarded(ctx, [&] {

@@ -134,7 +134,8 @@ struct PlanArena {
 // Per-launch record of the optional profiler (events resolved on query).
 struct ProfRec {
     int kind;
-    double flops, bytes;
+    double flops, bytes;   // of the method's terms
+    double executed;       // flops the kernel ran for them
     cudaEvent_t e0, e1;
 };
 
@@ -175,7 +176,7 @@ struct Context {
         BSM_CUDA(cudaStreamWaitEvent(stream, join_ev, 0));
         side_open = false;
     }
-    double flops = 0.0;              // algorithmic FP64 flops issued (running total)
+    double flops = 0.0;              // algorithmic FP64 flops issued (running total; 2 m n k of every term's product)
     bool profiling = false;
     int gemm_emulation_log2 = 0;     // block products >= 2^this flops on the tensor cores (0: never)
     int apply_precision = BSMPS_PREC_FP64;   // arithmetic of the zip-up contraction stage
@@ -186,7 +187,7 @@ struct Context {
     std::vector<cudaEvent_t> event_pool;
     cudaEvent_t take_event();
     void prof_begin(cudaEvent_t* e0);
-    void prof_end(int kind, double flops, double bytes, cudaEvent_t e0);
+    void prof_end(int kind, double flops, double bytes, cudaEvent_t e0, double executed = -1.0);   // < 0: as flops
     // pinned staging ring for task uploads (a copy from pageable memory can
     // make the host wait for the stream): two halves, filled in turn; an event
     // recorded when a half is left gates its reuse
@@ -266,12 +267,13 @@ struct ProfScope {
     Context* ctx;
     int kind;
     double flops, bytes;
+    double executed = -1.0;
     cudaEvent_t e0 = nullptr;
     ProfScope(Context* c, int k, double f, double b) : ctx(c), kind(k), flops(f), bytes(b) {
         if (ctx->profiling) ctx->prof_begin(&e0);
     }
     void done() {
-        if (ctx->profiling) ctx->prof_end(kind, flops, bytes, e0);
+        if (ctx->profiling) ctx->prof_end(kind, flops, bytes, e0, executed);
     }
 };
 

@@ -50,7 +50,7 @@ constexpr int kSmallGemmThreads = 128;
 // sum_c alpha_c A_c B = (sum_c alpha_c A_c) B.  In the zip-up contraction every output has at
 // most two B blocks (one per occupation of the site) and as many contributions as operator
 // entries, so the products shrink from one per entry to two.
-__device__ __forceinline__ bool same_b(const GemmIn& x, const GemmIn& y) {
+__host__ __device__ __forceinline__ bool same_b(const GemmIn& x, const GemmIn& y) {
     return x.B == y.B && x.K == y.K && x.ldb == y.ldb && !x.transA && !y.transA;
 }
 
@@ -300,10 +300,10 @@ void Context::prof_begin(cudaEvent_t* e0) {
     BSM_CUDA(cudaEventRecord(*e0, stream));
 }
 
-void Context::prof_end(int kind, double fl, double by, cudaEvent_t e0) {
+void Context::prof_end(int kind, double fl, double by, cudaEvent_t e0, double executed) {
     cudaEvent_t e1 = take_event();
     BSM_CUDA(cudaEventRecord(e1, stream));
-    prof.push_back({kind, fl, by, e0, e1});
+    prof.push_back({kind, fl, by, executed < 0.0 ? fl : executed, e0, e1});
 }
 
 struct ZeroChunk {
@@ -414,7 +414,9 @@ void launch_gemm_fp64(Context* ctx, const std::vector<GemmOut>& outs, const std:
     configure_carveout();
     std::vector<GemmTile> tiles;
     std::vector<int> small, emulated;
-    double fl = 0.0, by = 0.0;
+    // fl: of the terms, a product each; ex: what the kernels run for them (k_gemm sums the left factors of a
+    // run before it multiplies, once per tile column, and reads the right factor once)
+    double fl = 0.0, ex = 0.0, by = 0.0;
     for (int o = 0; o < (int)outs.size(); ++o) {
         const GemmOut& g = outs[o];
         // outputs of at least 2^gemm_emulation_log2 flops with one untransposed
@@ -432,9 +434,17 @@ void launch_gemm_fp64(Context* ctx, const std::vector<GemmOut>& outs, const std:
             for (int m0 = 0; m0 < g.M; m0 += kTile)
                 for (int n0 = 0; n0 < g.N; n0 += kTile) tiles.push_back({o, m0, n0});
         }
-        for (int c = g.beg; c < g.end; ++c) {
-            fl += 2.0 * g.M * g.N * (double)ins[c].K;
-            by += 8.0 * ((double)g.M * ins[c].K + (double)ins[c].K * g.N);
+        const bool one_by_one = std::max(g.M, g.N) <= small_max;
+        for (int c = g.beg; c < g.end && !ctx->profiling; ++c) fl += 2.0 * g.M * g.N * (double)ins[c].K;
+        for (int c = g.beg; c < g.end && ctx->profiling;) {
+            const int end = std::min(g.end, c + kGemmIns - (c - g.beg) % kGemmIns);   // descriptors staged together
+            int v = c + 1;
+            while (!one_by_one && v < end && same_b(ins[v], ins[c])) ++v;
+            const double n = v - c, mk = (double)g.M * ins[c].K;
+            fl += 2.0 * mk * g.N * n;
+            ex += 2.0 * mk * g.N + (n > 1 ? 2.0 * mk * n * ((g.N + kTile - 1) / kTile) : 0.0);
+            by += 8.0 * (mk * n + (double)ins[c].K * g.N);
+            c = v;
         }
         by += 8.0 * g.M * (double)g.N * (g.beta == 0.0 ? 1.0 : 2.0);
     }
@@ -470,6 +480,7 @@ void launch_gemm_fp64(Context* ctx, const std::vector<GemmOut>& outs, const std:
     const GemmOut* d_o = (const GemmOut*)(d + oo);
     const GemmIn* d_i = (const GemmIn*)(d + oi);
     ProfScope ps(ctx, kind, fl, by);
+    ps.executed = ex;
     if (!small.empty()) {
         k_gemm_small<<<(unsigned)small.size(), kSmallGemmThreads, 0, ctx->stream>>>(d_o, d_i, (const int*)(d + os));
         check_launch(ctx);

@@ -1135,8 +1135,8 @@ bool right_sweep_batch(Context* ctx, const std::vector<TruncJob*>& jobs, GridSyn
     }
     ctx->flops += fl;
     if (!prof_idx.empty() && prof_idx[0] >= 0) {
-        for (int idx : prof_idx) ctx->prof[idx].flops = 0.0;
-        ctx->prof[prof_idx[0]].flops = fl;   // attributed to the sweep's first SVD launch record
+        for (int idx : prof_idx) ctx->prof[idx].flops = ctx->prof[idx].executed = 0.0;
+        ctx->prof[prof_idx[0]].flops = ctx->prof[prof_idx[0]].executed = fl;   // attributed to the sweep's first SVD launch record
     }
     launch_copy(ctx, cp);
     launch_gemm(ctx, go, gi);

@@ -753,12 +753,13 @@ struct Prof {
     Context* ctx;
     int kind;
     double fl, by;
+    double executed = -1.0;
     cudaEvent_t e0 = nullptr;
     Prof(Context* c, int k, double f, double b) : ctx(c), kind(k), fl(f), by(b) {
         if (ctx->profiling) ctx->prof_begin(&e0);
     }
     void done() {
-        if (ctx->profiling) ctx->prof_end(kind, fl, by, e0);
+        if (ctx->profiling) ctx->prof_end(kind, fl, by, e0, executed);
     }
 };
 
@@ -1328,11 +1329,17 @@ bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const st
     std::vector<int> tiles_of(outs.size(), 0);   // flops per output template times its members
     for (const EnvTileT& t : tiles)
         if (t.m0 == 0 && t.n0 == 0) tiles_of[t.out] += 1;
-    // flops of the operator's terms (one product per contribution), as the contraction counts them
+    // fl: of the operator's terms (one product per contribution), as the contraction counts them; ex: what the
+    // kernel runs (the right factors of an update summed once per tile row, kEnvCons at a time, then one product)
+    double ex = 0.0;
     for (size_t o = 0; o < outs.size(); ++o)
         for (int r = outs[o].beg; r < outs[o].end; ++r) {
             const double n = runs[r].cend - runs[r].cbeg, kk = runs[r].K;
-            fl += 2.0 * outs[o].M * outs[o].N * kk * n * tiles_of[o];
+            const double one = 2.0 * outs[o].M * outs[o].N * kk * tiles_of[o];
+            fl += one * n;
+            if (!ctx->profiling) continue;
+            ex += one * ((runs[r].cend - runs[r].cbeg + kEnvCons - 1) / kEnvCons);
+            if (runs[r].abuf < 0) ex += 2.0 * kk * outs[o].N * n * ((outs[o].M + 31) / 32) * tiles_of[o];
             by += 8.0 * ((double)outs[o].M * kk + n * kk * outs[o].N) * tiles_of[o];
         }
     int nsm = 0;
@@ -1367,6 +1374,7 @@ bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const st
     GridSync* a17 = gs;
     void* args[] = {&a0, &a1, &a1c, &a2, &a3, &a4, &a5, &a6, &a7, &a8, &a9, &a10, &a11, &a12, &a13, &a14, &a15, &a16, &a17};
     Prof pr(ctx, KK_GEMM, fl, by);
+    pr.executed = ex;
     BSM_CUDA(cudaLaunchCooperativeKernel((const void*)k_env_sweep_t, dim3(grid), dim3(kEnvThreads), args, 0,
                                          ctx->stream));
     count_launch(ctx);

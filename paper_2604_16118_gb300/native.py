@@ -102,6 +102,7 @@ _SIGS = {
     "bsmps_ctx_launch_count": (_i64, [_vp]),
     "bsmps_ctx_alloc_count": (_i64, [_vp]),
     "bsmps_ctx_profile": (_i, [_vp, _i]),
+    "bsmps_ctx_kernel_executed": (_i, [_vp, _i, _pd]),
     "bsmps_ctx_kernel_stats": (_i, [_vp, _i, _i, _pi64, _pd, _pd, _pd]),
     "bsmps_precond_theta": (_i, [_i, _pd, _pd, _i, _i, _d, _pd]),
     "bsmps_precond_interval": (_i, [_i, _i, _pd, _pd, _i, _i, _pd, _pd]),
@@ -244,6 +245,15 @@ class Context:
 
     def profile(self, enable=True):
         _check(self, lib().bsmps_ctx_profile(self.h, 1 if enable else 0))
+
+    def kernel_executed(self):
+        """{kind: flops run} of the profiled launches (bsmps_ctx_kernel_executed); before kernel_stats(reset)."""
+        out = {}
+        for k, name in enumerate(self.KERNELS):
+            fl = C.c_double()
+            _check(self, lib().bsmps_ctx_kernel_executed(self.h, k, C.byref(fl)))
+            out[name] = fl.value
+        return out
 
     def kernel_stats(self, reset=True):
         """{kind: (launches, ms, flops, bytes)} of the profiled launches."""
