@@ -446,6 +446,69 @@ __device__ __forceinline__ void form_q(const double* A, const double* tau, const
     __syncthreads();
 }
 
+// householder() and form_q() for a matrix in global memory (one that neither a CTA's nor a cluster's
+// shared memory holds): every column is read by a whole warp (256 contiguous bytes a load) and the
+// reflector's column by the whole CTA, since the loads from L2 bound it; the 8-lane segments and the one-warp
+// chain of householder() lose there (truncation at rank 2000 over one charge 2.05 -> 1.64 s, zip-up of a
+// chain of 16 at rank 100 184 -> 150 ms).
+// v_j = 1 is implicit, v below the diagonal scaled to it.  red: 33 shared doubles.
+__device__ __forceinline__ void householder_global(double* A, double* tau, int M, int N, double* red) {
+    const int k = M < N ? M : N;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j = 0; j < k; ++j) {
+        double* x = A + (int64_t)j * M;
+        double s = 0.0;
+        for (int i = j + 1 + threadIdx.x; i < M; i += nthreads()) s = fma(x[i], x[i], s);
+        s = block_sum(s, red);
+        const double alpha = x[j];
+        double tj = 0.0, scale = 0.0, beta = alpha;
+        if (s != 0.0) {
+            beta = alpha >= 0.0 ? -sqrt(fma(alpha, alpha, s)) : sqrt(fma(alpha, alpha, s));
+            tj = (beta - alpha) / beta;
+            scale = 1.0 / (alpha - beta);
+        }
+        __syncthreads();   // every thread has read alpha
+        if (threadIdx.x == 0) {
+            x[j] = beta;
+            tau[j] = tj;
+        }
+        if (tj != 0.0) {
+            for (int i = j + 1 + threadIdx.x; i < M; i += nthreads()) x[i] *= scale;
+            __syncthreads();
+            for (int c = j + 1 + warp; c < N; c += nwarps()) {
+                double* a = A + (int64_t)c * M;
+                const double a_j = a[j];
+                double w = 0.0;
+                for (int i = j + 1 + lane; i < M; i += 32) w = fma(x[i], a[i], w);
+                const double tw = tj * (warp_sum(w) + a_j);
+                if (lane == 0) a[j] = a_j - tw;
+                for (int i = j + 1 + lane; i < M; i += 32) a[i] = fma(-tw, x[i], a[i]);
+            }
+        }
+        __syncthreads();
+    }
+}
+__device__ __forceinline__ void form_q_global(const double* A, const double* tau, double* Q, int M, int k) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // column c needs H_c ... H_0 only: one warp takes it through all of them, longest columns first
+    for (int cb = warp; cb < k; cb += nwarps()) {
+        const int c = k - 1 - cb;
+        double* q = Q + (int64_t)c * M;
+        for (int i = lane; i < M; i += 32) q[i] = i == c ? 1.0 : 0.0;
+        for (int j = c; j >= 0; --j) {
+            const double tj = tau[j];
+            if (tj == 0.0) continue;
+            const double* v = A + (int64_t)j * M;
+            const int i0 = j + ((lane - j) & 31);   // every lane keeps to the rows i = lane mod 32
+            double w = 0.0;
+            for (int i = i0; i < M; i += 32) w = fma(i == j ? 1.0 : v[i], q[i], w);
+            const double tw = tj * warp_sum(w);
+            for (int i = i0; i < M; i += 32) q[i] = fma(-tw, i == j ? 1.0 : v[i], q[i]);
+        }
+    }
+    __syncthreads();
+}
+
 // X (M x k, column-major) <- H_0 ... H_{k-1} X with householder()'s reflectors (M > 16),
 // whose diagonal entries stand in A: every 8-lane segment takes a column through
 // all of them without a barrier, as in form_q().  Q V this way takes 2 k (M k - k^2 / 2)

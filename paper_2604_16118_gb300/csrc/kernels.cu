@@ -163,19 +163,23 @@ __global__ void __launch_bounds__(kSmallGemmThreads) k_gemm_small(const GemmOut*
 // tau = (beta - alpha)/beta, v = x/(alpha - beta).
 __global__ void __launch_bounds__(kThreads) k_qr(const QrTask* __restrict__ tasks) {
     extern __shared__ double sm[];
+    __shared__ double red[33];
     const QrTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = M < N ? M : N;
     double* A = tk.smem ? sm : tk.A;
     double* Q = tk.smem ? sm + (int64_t)M * N : tk.Q;
     double* tau = tk.smem ? sm + (int64_t)M * N + (int64_t)M * k : tk.tau;
-    double* vd = tk.smem ? tau + k : tk.R;   // the reflectors' diagonals, until Q is formed
+    double* vd = tau + k;   // the reflectors' diagonals, until Q is formed (in shared memory only)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (tk.smem) {
         for (int64_t e = threadIdx.x; e < (int64_t)M * N; e += kThreads) A[e] = tk.A[e];
         __syncthreads();
+        dev::householder(A, tau, vd, M, N);
+        dev::form_q(A, tau, vd, Q, M, k);
+    } else {
+        dev::householder_global(A, tau, M, N, red);
+        dev::form_q_global(A, tau, Q, M, k);
     }
-    dev::householder(A, tau, vd, M, N);
-    dev::form_q(A, tau, vd, Q, M, k);
     __syncthreads();
     // R (k x N row-major) from the upper trapezoid
     for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += kThreads) {

@@ -61,3 +61,26 @@ def test_truncation_with_a_tall_stack(nat, ctx, rows, cols):
         assert y.bonds() == oy.bonds
         assert abs(dt - odt) <= 1e-12 * nrm
         assert rel_distance(OB.BSMPS.from_flat([0] * K, (N, 0), y.bonds(), y.export()), oy) <= 1e-12
+
+
+@pytest.mark.parametrize("cols", [300, 331])
+def test_stack_beyond_a_cluster(nat, ctx, cols):
+    """924 rows: neither one CTA nor a cluster of 16 holds the stack, which is factorised in global memory."""
+    K, N = 22, 11
+    bonds = [{(q, 0): min(math.comb(b, q), 6 if b > 12 else math.comb(K - b, N - q))
+              for q in range(max(0, N - (K - b)), min(b, N) + 1)} for b in range(K + 1)]
+    bonds[11] = {(q, 0): 462 if q in (5, 6) else 6 for q in range(12)}
+    bonds[12] = {(q, 0): cols if q == 6 else 6 for q in range(1, 12)}
+    bonds[13][(6, 0)] = bonds[13][(7, 0)] = cols
+    ox = OB.BSMPS([0] * K, (N, 0), bonds, [dict() for _ in range(K)])
+    n = ox.layout()[1]
+    ox = OB.BSMPS.from_flat([0] * K, (N, 0), bonds, np.random.default_rng(cols).standard_normal(n) / 16.0)
+    lo = OB.left_orthogonalize(ox)
+    assert lo.bonds[11][(5, 0)] + lo.bonds[11][(6, 0)] == 924 and lo.bonds[12][(6, 0)] == cols
+    x = nat.mps_import(ctx, K, 0, N, 0, ox.bonds, ox.to_flat())
+    nrm = float(np.sqrt(OB.dot(ox, ox)))
+    y, dt, _ = nat.truncate(ctx, x, 1e-2 * nrm)
+    oy, odt, _ = OB.truncate(ox, 1e-2 * nrm)
+    assert y.bonds() == oy.bonds
+    assert abs(dt - odt) <= 1e-12 * nrm
+    assert rel_distance(OB.BSMPS.from_flat([0] * K, (N, 0), y.bonds(), y.export()), oy) <= 1e-12
