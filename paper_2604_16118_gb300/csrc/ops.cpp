@@ -39,43 +39,77 @@ Mps* new_mps(Context* ctx, const Layout& L, bool zero) {
 
 static MpsPtr make_mps(Context* ctx, const Layout& L, bool zero) { return MpsPtr(new_mps(ctx, L, zero)); }
 
-// The flat layout of an iterate and its cores (one buffer per core) meet in one
+// The flat layout of an iterate and its cores (one buffer per core) meet in a
 // staging buffer: one host copy and one kernel instead of a copy per core (a
-// small copy from or to pageable memory costs 10 to 20 us).  Iterates beyond 64 MB pass
-// through it in pieces (a piece's copy takes milliseconds), so that an import or
-// export needs no second buffer of the iterate's size.
-constexpr int64_t kStageDoubles = (int64_t)8 << 20;
+// small copy from or to pageable memory costs 10 to 20 us).
+//  - Upload: the buffer takes up to 64 MB at a time; cores of 16 MB and more are copied by themselves
+//    (549 MB of eight blocks: 2.85 ms, 3.3 through one buffer of that size).
+//  - Download: one copy of everything (549 MB: 21.5 ms; core by core, and in pieces, 24 ms and
+//    at times ten times that, the host's pages being touched for the first time by several copies).
+//    Where the device has no room for a buffer of the iterate's size, core by core.
+namespace {
+constexpr int64_t kStageDoubles = (int64_t)8 << 20, kDirectDoubles = (int64_t)2 << 20;
+
+// core(t, off, n): core t, n doubles at flat offset off, is copied by itself; stage(beg, end): the
+// flat range, whole cores below kDirectDoubles, goes through the buffer.
+template <class Core, class Stage>
+void for_pieces(const Layout& L, const Core& core, const Stage& stage) {
+    int64_t off = 0, beg = 0;
+    for (int t = 0; t < L.K; ++t) {
+        const int64_t n = L.core_size[t];
+        const bool direct = n >= kDirectDoubles;
+        if (off > beg && (direct || off + n - beg > kStageDoubles)) stage(beg, off);
+        if (direct || off + n - beg > kStageDoubles) beg = off;
+        if (direct) {
+            core(t, off, n);
+            beg = off + n;
+        }
+        off += n;
+    }
+    if (off > beg) stage(beg, off);
+}
+}  // namespace
 
 void mps_upload(Mps* x, const double* host) {
-    const int64_t n = x->lay.total();
-    if (n > 0) {
-        Scratch s(x->ctx);
-        double* flat = s.dbl((size_t)std::min(n, kStageDoubles));
-        for (int64_t b = 0; b < n; b += kStageDoubles) {
-            const int64_t e = std::min(n, b + kStageDoubles);
-            BSM_CUDA(cudaMemcpyAsync(flat, host + b, (size_t)(e - b) * sizeof(double), cudaMemcpyHostToDevice,
-                                     x->ctx->stream));
-            launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, b, e, true);
-        }
-    }
-    x->ctx->sync();
+    Context* ctx = x->ctx;
+    Scratch s(ctx);
+    int64_t most = 0;
+    for_pieces(x->lay, [](int, int64_t, int64_t) {}, [&](int64_t b, int64_t e) { most = std::max(most, e - b); });
+    double* flat = s.dbl((size_t)most);
+    auto up = [&](double* dst, const double* src, int64_t n) {
+        BSM_CUDA(cudaMemcpyAsync(dst, src, (size_t)n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+    };
+    for_pieces(
+        x->lay, [&](int t, int64_t off, int64_t n) { up(x->core[t], host + off, n); },
+        [&](int64_t b, int64_t e) {
+            up(flat, host + b, e - b);
+            launch_flat_cores(ctx, x->core, x->lay.core_size, flat, b, e, true);
+        });
+    ctx->sync();
 }
 
 void mps_download(const Mps* x, double* host) {
+    Context* ctx = x->ctx;
     const int64_t n = x->lay.total();
-    if (n > 0) {
-        Scratch s(x->ctx);
-        double* flat = s.dbl((size_t)std::min(n, kStageDoubles));
-        for (int64_t b = 0; b < n; b += kStageDoubles) {
-            const int64_t e = std::min(n, b + kStageDoubles);
-            launch_flat_cores(x->ctx, x->core, x->lay.core_size, flat, b, e, false);
-            BSM_CUDA(cudaMemcpyAsync(host + b, flat, (size_t)(e - b) * sizeof(double), cudaMemcpyDeviceToHost,
-                                     x->ctx->stream));
-        }
-        x->ctx->sync();
-        return;
+    auto down = [&](double* dst, const double* src, int64_t m) {
+        BSM_CUDA(cudaMemcpyAsync(dst, src, (size_t)m * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    };
+    Scratch s(ctx);
+    double* flat = nullptr;
+    try {
+        flat = s.dbl((size_t)n);
+    } catch (const Error& e) {
+        if (e.code != BSMPS_ERR_OOM) throw;
+        (void)cudaGetLastError();
+        int64_t off = 0;
+        for (int t = 0; t < x->lay.K; off += x->lay.core_size[t++])
+            if (x->lay.core_size[t] > 0) down(host + off, x->core[t], x->lay.core_size[t]);
     }
-    x->ctx->sync();
+    if (flat) {
+        launch_flat_cores(ctx, x->core, x->lay.core_size, flat, 0, n, false);
+        down(host, flat, n);
+    }
+    ctx->sync();
 }
 
 bool same_space(const Layout& a, const Layout& b) {
