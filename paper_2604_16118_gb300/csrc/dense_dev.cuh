@@ -675,6 +675,86 @@ __device__ __forceinline__ void jacobi_small(double* G, double* V, double* Sraw,
     __syncthreads();
 }
 
+// FP64 one-sided Jacobi of B (rows x k, column-major, rows <= 32) with the rotations accumulated in V:
+// one pair per warp, its inner products in aligned segments of S = pow2_at_least(rows)
+// lanes.  For the smallest sectors, where a handful of rotations is all there is to do and the stages
+// of jacobi_pre() (an FP32 iteration, the orthogonalisation of its rotations, a Gram test) cost more than
+// they save.  Threshold |g| > rows eps sqrt(a b), columns below the numerical-zero level
+// (rows eps)^2 ||B||_F^2 are left alone.  Sraw: column norms of the result.
+__device__ __forceinline__ void jacobi_tiny(double* B, double* V, double* Sraw, int rows, int k, int ldb, int ldv,
+                                            double* red, int* s_rot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double f = 0.0;
+    for (int e = threadIdx.x; e < k * ldb; e += nthreads()) f = fma(B[e], B[e], f);   // (padding zero)
+    for (int e = threadIdx.x; e < k * ldv; e += nthreads()) V[e] = e % ldv == e / ldv ? 1.0 : 0.0;
+    f = block_sum(f, red);
+    const double tol = (double)rows * DBL_EPSILON;
+    const double tol2 = tol * tol, tiny2 = tol2 * f;
+    const int n2 = k + (k & 1);
+    const int S = pow2_at_least(rows);
+    const int i = lane % S, sg = lane / S;
+    for (int sweep = 0; sweep < kMaxSweeps && k > 1; ++sweep) {
+        if (threadIdx.x == 0) *s_rot = 0;
+        __syncthreads();
+        for (int round = 0; round < n2 - 1; ++round) {
+            for (int pi = warp; pi < n2 / 2; pi += nwarps()) {
+                const int u = rr_player(pi, round, n2), v = rr_player(n2 - 1 - pi, round, n2);
+                if (u >= k || v >= k) continue;
+                double* Bp = B + min(u, v) * ldb;
+                double* Bq = B + max(u, v) * ldb;
+                const double xp = i < rows ? Bp[i] : 0.0, xq = i < rows ? Bq[i] : 0.0;
+                double a, b, g;
+                if (S <= 8) {   // segment 0: xp xp, 1: xq xq, 2: xp xq
+                    const double prod =
+                        seg_sum(sg < 3 ? (sg == 1 ? xq : xp) * (sg == 0 ? xp : xq) : 0.0, S);
+                    a = __shfl_sync(0xffffffffu, prod, 0);
+                    b = __shfl_sync(0xffffffffu, prod, S);
+                    g = __shfl_sync(0xffffffffu, prod, 2 * S);
+                } else if (S == 16) {
+                    const double x = sg == 0 ? xp : xq;
+                    const double ab = seg_sum(x * x, 16);
+                    g = seg_sum(xp * xq, 16);
+                    a = __shfl_sync(0xffffffffu, ab, 0);
+                    b = __shfl_sync(0xffffffffu, ab, 16);
+                } else {
+                    a = warp_sum(xp * xp);
+                    b = warp_sum(xq * xq);
+                    g = warp_sum(xp * xq);
+                }
+                if (g * g > tol2 * (a * b) && nonneg_key(a) > nonneg_key(tiny2) && nonneg_key(b) > nonneg_key(tiny2)) {
+                    double c, s;
+                    jacobi_rotation_fast(a, b, g, &c, &s);
+                    double* Vp = V + min(u, v) * ldv;
+                    double* Vq = V + max(u, v) * ldv;
+                    if (lane < S && i < rows) {
+                        Bp[i] = c * xp - s * xq;
+                        Bq[i] = s * xp + c * xq;
+                    }
+                    // V on the second segment, or after B where the rows take the warp
+                    if ((S <= 16 ? sg == 1 : true) && i < k) {
+                        const double vp = Vp[i], vq = Vq[i];
+                        Vp[i] = c * vp - s * vq;
+                        Vq[i] = s * vp + c * vq;
+                    }
+                    if (lane == 0) *s_rot = 1;
+                }
+            }
+            __syncthreads();
+        }
+        const int rot = *s_rot;
+        __syncthreads();
+        if (!rot) break;
+    }
+    const int Gc = 32 / S;   // columns per warp instruction
+    for (int j0 = warp * Gc; j0 < k; j0 += nwarps() * Gc) {
+        const int j = j0 + sg;
+        const double x = (j < k && i < rows) ? B[j * ldb + i] : 0.0;
+        const double a = seg_sum(x * x, S);
+        if (j < k && i == 0) Sraw[j] = sqrt_via_rsqrt(a);
+    }
+    __syncthreads();
+}
+
 // SVD factors from a Jacobi on B itself (B V = U diag(Sraw), B = M for a tall M, B =
 // M^T for a wide M): tall: US = columns of B, Vt = rows V^T; wide: US = V
 // diag(S), Vt = (B diag(1/S))^T.  Order, tie rule and sign rule as in

@@ -34,6 +34,10 @@ size_t cut_smem(const CutTask& c) {
 
 // Sectors of at most this many rows and kept columns go to Jacobi without a QR step.
 constexpr int kDirectRows = 32, kDirectCols = 16;
+// Of those, the ones of at most this many columns are rotated in FP64 from the start (truncations of six sites at
+// rank 4 183 -> 157 us, of 64 sites at rank 4 1030 -> 957 us; 4 instead of 2 columns level, 6 and 8 slower:
+// 20 sites at rank 20 1028 -> 1213 and 1373 us).
+constexpr int kTinyCols = 2;
 // Their leading dimensions by the three instances of jacobi_pre() (8, 16 or 32 rows).
 __host__ __device__ constexpr int direct_ldb(int len) { return len <= 8 ? 8 : len <= 16 ? 24 : 40; }
 __host__ __device__ constexpr int direct_ldv(int len) { return len <= 8 ? 8 : 24; }
@@ -216,7 +220,9 @@ __device__ void svd_core(double* sm, bool direct, int M, int N, int k, int len, 
         double* rinv = Sr + k;
         double* dl = rinv + k;
         int* prm = (int*)(dl + k);
-        if (len <= 8)
+        if (k <= kTinyCols)
+            dev::jacobi_tiny(B, Vd, Sr, len, k, ldb, ldv, red, s_rot);
+        else if (len <= 8)
             dev::jacobi_pre<1, 1, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
         else if (len <= 16)
             dev::jacobi_pre<2, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
@@ -709,8 +715,9 @@ unsigned char* upload_pack(Scratch& s, const Pack& p) {
 // lengthen the barriers between reflectors.
 int block_for(int kmax, int max_warps = 8) { return 32 * std::max(1, std::min(max_warps, (kmax + 1) / 2)); }
 constexpr int kSvdWarps = kSweepThreads / 32;
-// The SVD kernels: at least two warps (the Jacobi's G and V warps), and enough for 8 blockDim >= k^2.
-int svd_block_for(int kmax) { return std::max(64, block_for(kmax, kSvdWarps)); }
+// The SVD kernels: a warp per pair where jacobi_tiny() takes every sector, else at least two warps (the
+// Jacobi's G and V warps), and enough for 8 blockDim >= k^2.
+int svd_block_for(int kmax) { return std::max(kmax <= kTinyCols ? 32 : 64, block_for(kmax, kSvdWarps)); }
 
 // The attributes are per function and per process: set them once per kernel.
 template <class F>
