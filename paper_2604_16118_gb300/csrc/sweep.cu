@@ -162,14 +162,22 @@ __device__ void left_body(const LeftTask& tk, const LeftSrc* __restrict__ srcs, 
         left_rank1<CG>(tk, srcs, xs, A, red);
         return;
     }
-    dev::householder(A, tau, R, M, N);   // R's first k entries hold the reflectors' diagonals until Q is formed
+    // R's first k entries hold the reflectors' diagonals until Q is formed (none up to 16 rows: R is
+    // written beside Q there)
+    auto write_r = [&]() {
+        for (int e = threadIdx.x; e < k * N; e += nthreads()) {
+            const int r = e / N, c = e % N;
+            R[e] = c >= r ? A[(int64_t)c * M + r] : 0.0;
+        }
+    };
+    dev::householder(A, tau, R, M, N);
+    if (M <= 16) write_r();
     dev::form_q(A, tau, R, Q, M, k);
     __syncthreads();
-    for (int64_t e = threadIdx.x; e < (int64_t)k * N; e += nthreads()) {
-        const int r = (int)(e / N), c = (int)(e % N);
-        R[e] = c >= r ? A[(int64_t)c * M + r] : 0.0;
+    if (M > 16) {
+        write_r();
+        __syncthreads();
     }
-    __syncthreads();
     for (int j = warp; j < k; j += nwarps()) {
         if (A[(int64_t)j * M + j] < 0.0) {
             for (int c = lane; c < N; c += 32) R[(int64_t)j * N + c] = -R[(int64_t)j * N + c];
