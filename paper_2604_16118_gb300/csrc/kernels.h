@@ -323,7 +323,7 @@ struct EnvGroupPhase {
 // Output C (M x N, row-major) = sum over runs beg .. end.
 struct EnvOutT {
     int M, N, beg, end;
-    int gp;    // its group-phase entry
+    int gp;    // its group-phase entry; complemented by launch_env_sweep_t for outputs summed without staging
     int cbuf;
     int64_t coff;
 };
@@ -352,7 +352,7 @@ struct EnvTileT {
 struct EnvMemberFac {
     int row[4];
 };
-bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
+bool launch_env_sweep_t(Context* ctx, std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
                         const std::vector<EnvConT>& cons, const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
                         const std::vector<EnvGroupPhase>& gph, const std::vector<EnvMemberFac>& mfac,
                         const std::vector<double>& ftab, int K, double* const base[4],

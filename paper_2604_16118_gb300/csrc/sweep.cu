@@ -810,6 +810,20 @@ __global__ void __launch_bounds__(kSweepThreads) k_orthogonalise_check(const dou
 constexpr int kEnvThreads = 128;
 constexpr int kEnvCons = 64;    // contributions resolved at a time
 constexpr int kEnvPerSm = 8;
+// Outputs of at most one entry per thread whose sums have at most this many terms skip the staging: a thread
+// sums its entry from L2 without a barrier (inner products of 64 sites at rank 4 727 -> 598 us, 6 sites
+// 94 -> 81, 20 sites at rank 32 295 -> 258; limit 16: 271, 64: 259).
+constexpr int kEnvDirect = 32;
+
+// Weight of a contribution for one member: the operator's entry (and shift) times its occupations' factors.
+__device__ __forceinline__ double env_weight(const EnvConT& c, double shift, const EnvMemberFac& mf,
+                                             const double* __restrict__ ftab, int K, int site) {
+    double w = c.w + ((c.fac & 4) ? shift : 0.0);
+    const int ra = mf.row[c.fac & 1], rb = mf.row[2 + ((c.fac >> 1) & 1)];
+    if (ra >= 0) w *= ftab[(int64_t)ra * K + site];
+    if (rb >= 0) w *= ftab[(int64_t)rb * K + site];
+    return w;
+}
 
 __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __restrict__ outs,
                                                              const EnvRunT* __restrict__ runs,
@@ -836,9 +850,32 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __re
         for (int ti = phase_beg[p] + (int)blockIdx.x; ti < phase_beg[p + 1]; ti += (int)gridDim.x) {
             const EnvTileT tl = tiles[ti];
             const EnvOutT o = outs[tl.out];
-            const EnvGroupPhase g = gph[o.gp];
+            const bool direct = o.gp < 0;
+            const EnvGroupPhase g = gph[direct ? ~o.gp : o.gp];
             const EnvMemberFac mf = mfac[g.mem_beg + tl.member];
             const int64_t mem = tl.member;
+            if (direct) {
+                if ((int)threadIdx.x < o.M * o.N) {
+                    const int m = threadIdx.x / o.N, n = threadIdx.x - m * o.N;
+                    const double* T = bases[0] + g.base[0] + mem * g.stride[0];
+                    double acc = 0.0;
+                    for (int r = o.beg; r < o.end; ++r) {
+                        const EnvRunT run = runs[r];
+                        if (!upd) {
+                            const double* E = bases[run.abuf] + g.base[run.abuf] + mem * g.stride[run.abuf] + run.off;
+                            acc = dev::dot_global<true, true>(E + (int64_t)m * run.K, 1, run.ptr + n, o.N, run.K, acc);
+                            continue;
+                        }
+                        for (int c = run.cbeg; c < run.cend; ++c) {
+                            const EnvConT con = cons[c];
+                            acc = fma(env_weight(con, g.shift, mf, ftab, K, run.site),
+                                      dev::dot_global<true, true>(run.ptr + m, o.M, T + con.off + n, o.N, run.K, 0.0), acc);
+                        }
+                    }
+                    const_cast<double*>(bases[o.cbuf])[g.base[o.cbuf] + mem * g.stride[o.cbuf] + o.coff + threadIdx.x] = acc;
+                }
+                continue;
+            }
             // the tile's entries, flat over its valid rows and columns (small blocks fill few lanes otherwise)
             const int tm = min(32, o.M - tl.m0), tn = min(32, o.N - tl.n0), n_el = tm * tn;
             int em[kPer], en[kPer];
@@ -859,12 +896,8 @@ __global__ void __launch_bounds__(kEnvThreads) k_env_sweep_t(const EnvOutT* __re
                     if (upd) {
                         if ((int)threadIdx.x < nc) {
                             const EnvConT c = cons[cb + threadIdx.x];
-                            double w = c.w + ((c.fac & 4) ? g.shift : 0.0);
-                            const int ra = mf.row[c.fac & 1], rb = mf.row[2 + ((c.fac >> 1) & 1)];
-                            if (ra >= 0) w *= ftab[(int64_t)ra * K + run.site];
-                            if (rb >= 0) w *= ftab[(int64_t)rb * K + run.site];
                             s_ptr[threadIdx.x] = T + c.off;
-                            s_w[threadIdx.x] = w;
+                            s_w[threadIdx.x] = env_weight(c, g.shift, mf, ftab, K, run.site);
                         }
                         __syncthreads();
                     }
@@ -1329,7 +1362,7 @@ bool check_orthogonalise(Context* ctx, int k, const double* P, double* Q) {
     return ok != 0;
 }
 
-bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
+bool launch_env_sweep_t(Context* ctx, std::vector<EnvOutT>& outs, const std::vector<EnvRunT>& runs,
                         const std::vector<EnvConT>& cons, const std::vector<EnvTileT>& tiles, const std::vector<int>& phase_beg,
                         const std::vector<EnvGroupPhase>& gph, const std::vector<EnvMemberFac>& mfac,
                         const std::vector<double>& ftab, int K, double* const base[4],
@@ -1347,16 +1380,21 @@ bool launch_env_sweep_t(Context* ctx, const std::vector<EnvOutT>& outs, const st
     // fl: of the operator's terms (one product per contribution), as the contraction counts them; ex: what the
     // kernel runs (the right factors of an update summed once per tile row, kEnvCons at a time, then one product)
     double ex = 0.0;
-    for (size_t o = 0; o < outs.size(); ++o)
-        for (int r = outs[o].beg; r < outs[o].end; ++r) {
+    for (size_t o = 0; o < outs.size(); ++o) {
+        int64_t terms = 0;
+        for (int r = outs[o].beg; r < outs[o].end; ++r) terms += (int64_t)(runs[r].cend - runs[r].cbeg) * runs[r].K;
+        const int M = outs[o].M, N = outs[o].N;
+        const bool direct = terms <= kEnvDirect && M <= 32 && N <= 32 && M * N <= kEnvThreads;
+        if (direct) outs[o].gp = ~outs[o].gp;
+        const double mn = 2.0 * M * N * tiles_of[o];
+        fl += mn * terms;
+        for (int r = outs[o].beg; r < outs[o].end && ctx->profiling; ++r) {
             const double n = runs[r].cend - runs[r].cbeg, kk = runs[r].K;
-            const double one = 2.0 * outs[o].M * outs[o].N * kk * tiles_of[o];
-            fl += one * n;
-            if (!ctx->profiling) continue;
-            ex += one * ((runs[r].cend - runs[r].cbeg + kEnvCons - 1) / kEnvCons);
-            if (runs[r].abuf < 0) ex += 2.0 * kk * outs[o].N * n * ((outs[o].M + 31) / 32) * tiles_of[o];
-            by += 8.0 * ((double)outs[o].M * kk + n * kk * outs[o].N) * tiles_of[o];
+            ex += mn * kk * (direct ? n : (runs[r].cend - runs[r].cbeg + kEnvCons - 1) / kEnvCons);
+            if (runs[r].abuf < 0 && !direct) ex += 2.0 * kk * N * n * ((M + 31) / 32) * tiles_of[o];
+            by += 8.0 * (M * kk + n * kk * N) * tiles_of[o];
         }
+    }
     int nsm = 0;
     BSM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     const int cap = coresident_ctas(k_env_sweep_t, kEnvThreads, 0);
