@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_left_site(const LeftTask* __r
 // Jacobi on the matrix itself.  Bound by the FP64 warp instructions of the one SM and, below
 // 32 columns, by the latency of the chains.  120 x 60: 947 us (QR 185, FP32 Jacobi 104,
 // orthogonalisation 134, FP64 264, Q V 222, assembly 20), 32 x 20: 126 us.
-__device__ void svd_core(double* sm, bool direct, int M, int N, int k, int len, int wide, double* S, double* US, double* Vt, int ldus,
+__device__ void svd_core(double* sm, int direct, int M, int N, int k, int len, int wide, double* S, double* US, double* Vt, int ldus,
                          int ldvt, double* red, int* s_rot, dev::SegRot* ring) {
     double* B = sm;
     if (direct) {
@@ -228,7 +228,7 @@ __device__ void svd_core(double* sm, bool direct, int M, int N, int k, int len, 
         double* rinv = Sr + k;
         double* dl = rinv + k;
         int* prm = (int*)(dl + k);
-        if (k <= kTinyCols)
+        if (direct == 2)
             dev::jacobi_tiny(B, Vd, Sr, len, k, ldb, ldv, red, s_rot);
         else if (len <= 8)
             dev::jacobi_pre<1, 1, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
@@ -418,7 +418,7 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
     }
     const int k = M < N ? M : N, len = M < N ? N : M, wide = M < N ? 1 : 0;
     double* B = sm;
-    const bool direct = len <= kDirectRows && k <= kDirectCols;
+    const int direct = len > kDirectRows || k > kDirectCols ? 0 : k > kTinyCols ? 1 : 2;
     const int ldb = direct ? direct_ldb(len) : len;   // (k == 1 included: one padded column)
     pad_columns(B, len, ldb, k);
     int coff = 0;
@@ -723,9 +723,10 @@ unsigned char* upload_pack(Scratch& s, const Pack& p) {
 // lengthen the barriers between reflectors.
 int block_for(int kmax, int max_warps = 8) { return 32 * std::max(1, std::min(max_warps, (kmax + 1) / 2)); }
 constexpr int kSvdWarps = kSweepThreads / 32;
-// The SVD kernels: a warp per pair where jacobi_tiny() takes every sector, else at least two warps (the
-// Jacobi's G and V warps), and enough for 8 blockDim >= k^2.
-int svd_block_for(int kmax) { return std::max(kmax <= kTinyCols ? 32 : 64, block_for(kmax, kSvdWarps)); }
+// The SVD kernels: at least two warps (the Jacobi's G and V warps), and enough for 8 blockDim >= k^2; a warp
+// per pair where jacobi_tiny() takes every sector.
+int svd_block_for(int kmax, bool tiny = false) { return std::max(tiny ? 32 : 64, block_for(kmax, kSvdWarps)); }
+bool is_tiny(const DynTask& t) { return t.kpad <= kTinyCols && std::max(t.M, t.ncols_pad) <= kDirectRows; }
 
 // The attributes are per function and per process: set them once per kernel.
 template <class F>
@@ -1221,7 +1222,8 @@ int launch_right_dyn(Context* ctx, const std::vector<DynTask>& tasks_in, const s
     unsigned char* d = upload_pack(s, pk);
     Prof pr(ctx, KK_SVD, fl, by);
     allow_smem(k_right_dyn);
-    k_right_dyn<<<(unsigned)tasks.size(), svd_block_for(kmax), smem, ctx->stream>>>((const DynTask*)(d + ot));
+    const bool tiny = std::all_of(tasks.begin(), tasks.end(), is_tiny);
+    k_right_dyn<<<(unsigned)tasks.size(), svd_block_for(kmax, tiny), smem, ctx->stream>>>((const DynTask*)(d + ot));
     count_launch(ctx);
     pr.done();
     return ctx->profiling ? (int)ctx->prof.size() - 1 : -1;
@@ -1305,7 +1307,7 @@ bool launch_right_sweep(Context* ctx, const std::vector<DynTask>& tasks_in, cons
     const size_t pb_off = (smem + 15) & ~size_t(15);   // phase_beg staged behind the working set
     smem = pb_off + sizeof(int) * (size_t)(n_phase + 1);
     if (smem > kSweepSmem) return false;
-    const int threads = svd_block_for(kmax);
+    const int threads = svd_block_for(kmax, std::all_of(tasks.begin(), tasks.end(), is_tiny));
     allow_smem(k_right_sweep);
     const int cap = coresident_ctas(k_right_sweep, threads, smem);
     if (cap <= 0) return false;

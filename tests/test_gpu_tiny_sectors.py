@@ -60,3 +60,22 @@ def test_truncation(nat, ctx, rows, kind):
         assert y.bonds() == oy.bonds
         assert abs(dt - odt) <= 1e-12 * nrm
         assert rel_distance(OB.BSMPS.from_flat([0] * K, (N, 0), y.bonds(), y.export()), oy) <= 1e-12
+
+
+@pytest.mark.parametrize("sites,r,D", [(4, 4, 3), (8, 4, 17), (12, 4, 33), (12, 6, 40), (12, 4, 70)])
+def test_joint_iterates_of_few_rows_and_many_vectors(nat, ctx, sites, r, D):
+    """Two rows over as many columns as vectors: sectors of two kept columns that are too long for the plain Jacobi,
+    in launches that hold no wider ones."""
+    wl_species, target = [0] * sites, (sites // 2, 0)
+    n = nat.mps_joint_random_size(sites, 0, sites // 2, 0, r, D)
+    vals = np.random.default_rng(D).standard_normal(n)
+    x = nat.mps_create_joint(ctx, sites, 0, sites // 2, 0, D, r_max=r, values=vals)
+    ox = OB.BSMPS.from_flat(wl_species, target, OB.default_dims(wl_species, target, r, D), vals)
+    assert x.bonds() == ox.bonds
+    nrm = float(np.sqrt(sum(np.sum(B * B) for B in OB.left_orthogonalize(ox).cores[-1].values())))
+    for rel in (1e-11, 1e-1):
+        y, dt, _ = nat.truncate(ctx, x, rel * nrm)
+        oy, odt, _ = OB.truncate(ox, rel * nrm)
+        assert y.bonds() == oy.bonds
+        assert abs(dt - odt) <= 1e-12 * nrm
+        assert rel_distance(OB.BSMPS.from_flat(wl_species, target, y.bonds(), y.export()), oy) <= 1e-12
