@@ -679,7 +679,8 @@ __device__ __forceinline__ void jacobi_small(double* G, double* V, double* Sraw,
 // one pair per warp, its inner products in aligned segments of S = pow2_at_least(rows)
 // lanes.  For the smallest sectors, where a handful of rotations is all there is to do and the stages
 // of jacobi_pre() (an FP32 iteration, the orthogonalisation of its rotations, a Gram test) cost more than
-// they save.  Threshold |g| > rows eps sqrt(a b), columns below the numerical-zero level
+// they save.  Angles in FP64: two columns are done after one rotation (with FP32 angles after two, 0 to
+// 3 % slower).  Threshold |g| > rows eps sqrt(a b), columns below the numerical-zero level
 // (rows eps)^2 ||B||_F^2 are left alone.  Sraw: column norms of the result.
 __device__ __forceinline__ void jacobi_tiny(double* B, double* V, double* Sraw, int rows, int k, int ldb, int ldv,
                                             double* red, int* s_rot) {
@@ -688,8 +689,12 @@ __device__ __forceinline__ void jacobi_tiny(double* B, double* V, double* Sraw, 
     for (int e = threadIdx.x; e < k * ldb; e += nthreads()) f = fma(B[e], B[e], f);   // (padding zero)
     for (int e = threadIdx.x; e < k * ldv; e += nthreads()) V[e] = e % ldv == e / ldv ? 1.0 : 0.0;
     f = block_sum(f, red);
+    // exact scaling to ||B||_F in [1, 2): squares and products of the norms stay in range
+    const int fe = (__double2hiint(f) >> 20) & 0x7ff, h = fe == 0 || fe == 0x7ff ? 0 : (fe - 1023) >> 1;
+    const double sc = __hiloint2double((1023 - h) << 20, 0), up = __hiloint2double((1023 + h) << 20, 0);
+    for (int e = threadIdx.x; e < k * ldb; e += nthreads()) B[e] *= sc;
     const double tol = (double)rows * DBL_EPSILON;
-    const double tol2 = tol * tol, tiny2 = tol2 * f;
+    const double tol2 = tol * tol, tiny2 = tol2 * (f * sc * sc);
     const int n2 = k + (k & 1);
     const int S = pow2_at_least(rows);
     const int i = lane % S, sg = lane / S;
@@ -723,7 +728,7 @@ __device__ __forceinline__ void jacobi_tiny(double* B, double* V, double* Sraw, 
                 }
                 if (g * g > tol2 * (a * b) && nonneg_key(a) > nonneg_key(tiny2) && nonneg_key(b) > nonneg_key(tiny2)) {
                     double c, s;
-                    jacobi_rotation_fast(a, b, g, &c, &s);
+                    jacobi_rotation(a, b, g, &c, &s);
                     double* Vp = V + min(u, v) * ldv;
                     double* Vq = V + max(u, v) * ldv;
                     if (lane < S && i < rows) {
@@ -750,7 +755,8 @@ __device__ __forceinline__ void jacobi_tiny(double* B, double* V, double* Sraw, 
         const int j = j0 + sg;
         const double x = (j < k && i < rows) ? B[j * ldb + i] : 0.0;
         const double a = seg_sum(x * x, S);
-        if (j < k && i == 0) Sraw[j] = sqrt_via_rsqrt(a);
+        if (j < k && i < rows) B[j * ldb + i] = x * up;
+        if (j < k && i == 0) Sraw[j] = sqrt_via_rsqrt(a) * up;
     }
     __syncthreads();
 }
