@@ -237,10 +237,11 @@ __device__ __forceinline__ double to_double(float f) {
     return __hiloint2double((int)(hi | (u & 0x80000000u)), e ? (int)(u << 29) : 0);
 }
 // Sum over the warp by integer arithmetic: the 32 values as 58-bit fixed-point numbers
-// of a common exponent, added in three limbs by warp reductions (redux), the exact
+// of a common exponent, added in three limbs by warp reductions (redux), their exact
 // sum rounded once.  275 cycles against 605 for five shuffle and FP64 addition
 // steps (about 45 + 75 cycles each here), and no FP64 instruction.  Values outside
-// the middle of the exponent range (and non-finite ones) take the shuffles.
+// the middle of the exponent range (and non-finite ones) take the shuffles.  A term is cut below 2^-57 of
+// the largest one's leading bit, which 32 of them keep within 2^-52 of it: the rounding of the shuffles' additions.
 __device__ __forceinline__ double warp_sum_fixed(double v) {
     const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     const unsigned e = (hi >> 20) & 0x7ff;
@@ -828,12 +829,12 @@ __device__ __forceinline__ float seg8_sum(float v) {
     v += __shfl_xor_sync(0xffffffffu, v, 1);
     return v;
 }
-// Leading dimension of columns of n rows in jacobi_pre(): at n <= 64 columns are
+// Leading dimension of columns of n <= 64 rows in jacobi_pre(): they are
 // padded with zero rows to an odd multiple of 8, so that the 8-lane segments of a
 // warp, which work on neighbouring columns, meet distinct banks (64-byte pieces of
 // columns 64 bytes apart modulo 128), and whole segments of rows need no bounds check.
 __host__ __device__ constexpr int jacobi_ld(int n) {
-    return n > 64 ? n : n <= 8 ? 8 : n <= 24 ? 24 : n <= 40 ? 40 : n <= 56 ? 56 : 72;
+    return n <= 8 ? 8 : n <= 24 ? 24 : n <= 40 ? 40 : n <= 56 ? 56 : 72;
 }
 
 __device__ __forceinline__ float rsqrt_fast(float x) {
@@ -1363,9 +1364,8 @@ __host__ __device__ constexpr int jacobi_scratch(int ldg, int ldv, int k) {
     return f > 2 * k * k ? f : 2 * k * k;
 }
 
-// jacobi_pre() on a square lower triangular G of k <= 64 columns (blockDim as block_for() gives it),
-// else jacobi().  G and V: leading dimension jacobi_ld(k).
-__device__ __forceinline__ void jacobi(double* G, double* V, double* Sraw, int k, double* red, int* s_rot);
+// jacobi_pre() on a square lower triangular G of k <= 64 columns (blockDim as svd_block_for() gives it).
+// G and V: leading dimension jacobi_ld(k).
 __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
                                             SegRot* ring, double* red, int* s_rot) {
     if (k <= 8)
@@ -1380,10 +1380,8 @@ __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, 
         jacobi_pre<5, 5, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else if (k <= 56)
         jacobi_pre<7, 7, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
-    else if (k <= 64)
-        jacobi_pre<8, 8, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
     else
-        jacobi(G, V, Sraw, k, red, s_rot);
+        jacobi_pre<8, 8, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
 }
 
 // One-sided (Hestenes) Jacobi on the columns of G (k x k, column-major) with the

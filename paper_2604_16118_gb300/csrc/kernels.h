@@ -45,7 +45,8 @@ struct QrTask {
     double* R;
     double* tau;
     int M, N;
-    int smem = 0;     // set by launch_qr (1: one CTA in shared memory) and by launch_qr_cluster (reflectors pulled at a time)
+    int smem = 0;     // set by launch_qr: 1 for one CTA in shared memory
+    int pull = 0;     // set by launch_qr_cluster: reflectors pulled at a time
 };
 
 // SVD of an M x N matrix A, k = min(M, N), given in G: A column-major when

@@ -609,7 +609,7 @@ void right_sweep_sitewise(Context* ctx, TruncJob& J) {
         std::vector<int> site_sec, gen_sec;
         for (int ni = 0; ni < nn; ++ni) {
             if (kk[ni] == 0) continue;
-            if (kk[ni] <= kSvdSiteMax && svd_site_fits(bn.dim[ni], c0[ni] + c1[ni]))
+            if (svd_site_fits(bn.dim[ni], c0[ni] + c1[ni]))
                 site_sec.push_back(ni);
             else
                 gen_sec.push_back(ni);

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kQcThreads, 2) k_qr_cluster(const QrTask* __re
     double* taus = Ql + (size_t)nq * M;          // tau_j and v_j(j) of every column
     double* vds = taus + k;                      // (tau_j = 0: -R(j, j)); beta_j < 0 exactly when vds[j] > 0
     double* vb = vds + k;                        // pulled reflectors
-    const int n_pull = tk.smem;
+    const int n_pull = tk.pull;
     const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_loc = rank < N ? (N - 1 - rank) / C + 1 : 0;
     const int nch = M >= kQcLongRows ? 4 : 1;    // warps of the chain
@@ -274,8 +274,8 @@ bool launch_qc(Context* ctx, const std::vector<QrTask>& tasks_in) {
     std::vector<QrTask> tasks = tasks_in;
     for (QrTask& t : tasks) {
         if (qc_smem(t.M, t.N, C) > kQcSmemMax) return false;
-        t.smem = qc_pull(t.M, t.N, C);   // reflectors pulled at a time
-        smem = std::max(smem, qc_smem(t.M, t.N, C) + sizeof(double) * (size_t)(t.smem - 1) * t.M);
+        t.pull = qc_pull(t.M, t.N, C);
+        smem = std::max(smem, qc_smem(t.M, t.N, C) + sizeof(double) * (size_t)(t.pull - 1) * t.M);
     }
     static bool attr = false;
     if (!attr) {

@@ -50,17 +50,16 @@ static_assert(direct_ldb(8) == dev::jacobi_ld(1) && direct_ldb(16) == dev::jacob
 // without a QR step, the padded input, V, the scratch and four vectors.
 __host__ __device__ inline size_t svd_buf(int len, int k) {
     const size_t a = (size_t)len * k, b = (size_t)dev::jacobi_scratch(dev::jacobi_ld(k), dev::jacobi_ld(k), k);
-    return k <= 64 && b > a ? b : a;
+    return b > a ? b : a;
 }
 size_t svd_doubles(int len, int k) {
     return svd_buf(len, k) + (size_t)len * k + 2 * (size_t)k * dev::jacobi_ld(k) + 3 * (size_t)k;
 }
-// Monotone in both sizes: the dynamic sweep sizes its memory by padded column counts and a
-// sector with fewer may take another path.
+// min(M, N) <= 64.  Monotone in both sizes: the dynamic sweep sizes its memory by padded column counts
+// and a sector with fewer may take another path.
 size_t svd_smem(int M, int N) {
     const int k = std::min(M, N), len = std::max(M, N);
     size_t n = svd_doubles(len, k);
-    if (k > 64) n = std::max(n, svd_doubles(len, 64));
     const int rows = std::min(len, kDirectRows), cols = std::min(k, kDirectCols), lb = direct_ldb(rows),
               lv = direct_ldv(rows);
     n = std::max(n, cols * (size_t)(lb + lv) + (size_t)dev::jacobi_scratch(lb, lv, cols) + 4 * (size_t)cols);
@@ -280,7 +279,9 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
     const SvdSiteTask tk = tasks[blockIdx.x];
     const int M = tk.M, N = tk.N, k = tk.k, len = tk.len;
     double* B = sm;
-    const bool direct = len <= 16;   // no more rows than householder() has a segment layout for
+    // Up to 16 rows Jacobi runs without a QR.  17 to 32 keep it here: these sectors run beside the bond's wide
+    // ones, and without it the wide workloads are level (95.3 and 95.4 ms, 20.7 and 20.8, 5.36 and 5.40).
+    const bool direct = len <= 16;
     const int ldb = direct ? direct_ldb(len) : len;
     pad_columns(B, len, ldb, k);
     for (int p = tk.p_beg; p < tk.p_end; ++p) {
@@ -1103,7 +1104,7 @@ bool left_site_fits(int M, int N, int64_t rx_fma) { return left_smem(M, N) <= kS
 
 size_t dyn_svd_smem(int M, int ncols_pad) { return svd_smem(M, ncols_pad); }
 
-bool svd_site_fits(int M, int N) { return std::min(M, N) <= 96 && svd_smem(M, N) <= kSweepSmem; }
+bool svd_site_fits(int M, int N) { return std::min(M, N) <= kSvdSiteMax && svd_smem(M, N) <= kSweepSmem; }
 
 void launch_left_site(Context* ctx, const std::vector<LeftTask>& tasks, const std::vector<LeftSrc>& srcs,
                       const std::vector<LeftX>& xs) {
