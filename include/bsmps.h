@@ -487,15 +487,17 @@ BSMPS_API bsmps_status bsmps_eigensolve_step(bsmps_ctx ctx, bsmps_mpo W, const b
  * rounding relative to max_k |a_ik| max_k |b_kj| K.
  * A (M x K, leading dimension lda), B (K x N, ldb) and C (M x N, ldc) are
  * row-major DEVICE pointers.  The work is ordered on the context stream and the
- * call does not synchronise.  Errors: INVALID_ARG, OOM, CUDA. */
+ * call does not synchronise.  Workspace: 2 bytes per value of A and B and slice (14
+ * with 8 slices), K rounded up to 32.  Errors: INVALID_ARG, OOM, CUDA. */
 /* C = A B (M x N) on the tensor cores in split precision (BSMPS_PREC_TF32X3):
  * every entry of A and B is split into two TF32 values, the three products
  * A_hi B_hi + A_hi B_lo + A_lo B_hi are accumulated in FP32 in tensor memory
  * (tcgen05.mma kind::tf32), and C is stored in FP64.  The error
  * of C_ij is a few units of 2^-21 times sum_k |a_ik| |b_kj| plus the FP32
  * accumulation error.  The paper has no counterpart: this is the contraction
- * kernel of the split-precision MPO application, exposed for testing.  A
- * (M x K, lda), B (K x N, ldb) and C (M x N, ldc) are row-major DEVICE
+ * kernel of the split-precision MPO application, exposed for testing.  Workspace: up
+ * to 8 bytes per value of A and B (K rounded up to 32), none where the device has no
+ * room for it.  A (M x K, lda), B (K x N, ldb) and C (M x N, ldc) are row-major DEVICE
  * pointers; stream-ordered on the context stream, no synchronisation.  A bounded
  * wait that gives up is reported as TIMEOUT at the context's next
  * synchronising call.  Errors: INVALID_ARG, OOM, CUDA. */
@@ -530,7 +532,9 @@ BSMPS_API bsmps_status bsmps_ctx_set_gemm_emulation(bsmps_ctx ctx, int min_log2_
  * G Qp, whose FP64 Jacobi converges in a few sweeps; V = Qp V1.  Every
  * quantity the truncation reads (singular values, vectors) is still the
  * result of the FP64 Jacobi, to FP64 rounding.  min_k = 0 turns it off; the
- * default is 48.  Errors: INVALID_ARG (negative). */
+ * default is 48.  Sectors of at most 64 columns that one SM factorises by itself
+ * start from FP32 whatever min_k > 0 (the rotations orthogonalised by a series),
+ * and in FP64 throughout when min_k = 0.  Errors: INVALID_ARG (negative). */
 BSMPS_API bsmps_status bsmps_ctx_set_jacobi_precond(bsmps_ctx ctx, int min_k);
 
 BSMPS_API bsmps_status bsmps_gemm_ozaki(bsmps_ctx ctx, int M, int N, int K, const double* A, int lda,

@@ -1279,10 +1279,10 @@ __device__ __forceinline__ bool orthogonalise(double* V, int k, double* scr, dou
 // jacobi_ld of max(rows, 8 RG - 7) for G (its padding zero on entry) and of
 // max(k, 8 RV - 7) for V, so that the 8 RG (8 RV) rows a lane segment walks stay
 // within the column.  scr: jacobi_scratch(ldg, ldv, k) shared doubles; del: k of them.
-// Tri: G is lower triangular (rows = k).
+// Tri: G is lower triangular (rows = k).  pre: with the FP32 start.
 template <int RG, int RV, bool Tri>
 __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, int rows, int k, double* scr,
-                                           double* del, SegRot* ring, double* red, int* s_int) {
+                                           double* del, SegRot* ring, double* red, int* s_int, bool pre) {
     const int T = nthreads(), kk = k * k;
     const int ldg = jacobi_ld(max(rows, 8 * RG - 7)), ldv = jacobi_ld(max(k, 8 * RV - 7));   // >= 8 RG, 8 RV
     double f = 0.0;
@@ -1302,11 +1302,14 @@ __device__ __forceinline__ void jacobi_pre(double* G, double* V, double* Sraw, i
     }
     for (int e = threadIdx.x; e < k * ldv; e += T) Vf[e] = e % ldv == e / ldv ? 1.0f : 0.0f;
     __syncthreads();
-    jacobi_f32_segments<RG, RV>(Gf, Vf, k, ldg, ldv, s_int);
-    // V row-major <- P
-    for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
     double own[kOwn];
-    const bool ok = orthogonalise(V, k, scr, own, red);
+    bool ok = false;
+    if (pre) {
+        jacobi_f32_segments<RG, RV>(Gf, Vf, k, ldg, ldv, s_int);
+        // V row-major <- P
+        for (int e = threadIdx.x; e < kk; e += T) V[(e % k) * k + e / k] = to_double(Vf[(e / k) * ldv + e % k]);
+        ok = orthogonalise(V, k, scr, own, red);
+    }
     __syncthreads();
     if (ok) {
         // G <- G Qp, row i to consecutive threads (rows k <= 8 blockDim outputs); V to column-major
@@ -1367,21 +1370,21 @@ __host__ __device__ constexpr int jacobi_scratch(int ldg, int ldv, int k) {
 // jacobi_pre() on a square lower triangular G of k <= 64 columns (blockDim as svd_block_for() gives it).
 // G and V: leading dimension jacobi_ld(k).
 __device__ __forceinline__ void jacobi_auto(double* G, double* V, double* Sraw, int k, double* scr, double* del,
-                                            SegRot* ring, double* red, int* s_rot) {
+                                            SegRot* ring, double* red, int* s_rot, bool pre) {
     if (k <= 8)
-        jacobi_pre<1, 1, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<1, 1, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else if (k <= 16)
-        jacobi_pre<2, 2, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<2, 2, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else if (k <= 24)
-        jacobi_pre<3, 3, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<3, 3, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else if (k <= 32)
-        jacobi_pre<4, 4, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<4, 4, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else if (k <= 40)
-        jacobi_pre<5, 5, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<5, 5, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else if (k <= 56)
-        jacobi_pre<7, 7, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<7, 7, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
     else
-        jacobi_pre<8, 8, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot);
+        jacobi_pre<8, 8, true>(G, V, Sraw, k, k, scr, del, ring, red, s_rot, pre);
 }
 
 // One-sided (Hestenes) Jacobi on the columns of G (k x k, column-major) with the

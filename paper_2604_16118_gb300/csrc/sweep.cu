@@ -215,9 +215,9 @@ __global__ void __launch_bounds__(kSweepThreads) k_left_site(const LeftTask* __r
 // QR, a Jacobi of R^T and Q V, or, with direct (len <= 32, k <= 16; always where len <= 16), a
 // Jacobi on the matrix itself.  Bound by the FP64 warp instructions of the one SM and, below
 // 32 columns, by the latency of the chains.  120 x 60: 947 us (QR 185, FP32 Jacobi 104,
-// orthogonalisation 134, FP64 264, Q V 222, assembly 20), 32 x 20: 126 us.
+// orthogonalisation 134, FP64 264, Q V 222, assembly 20), 32 x 20: 126 us.  pre: with the FP32 start.
 __device__ void svd_core(double* sm, int direct, int M, int N, int k, int len, int wide, double* S, double* US, double* Vt, int ldus,
-                         int ldvt, double* red, int* s_rot, dev::SegRot* ring) {
+                         int ldvt, double* red, int* s_rot, dev::SegRot* ring, bool pre) {
     double* B = sm;
     if (direct) {
         const int ldb = direct_ldb(len), ldv = direct_ldv(len);
@@ -230,11 +230,11 @@ __device__ void svd_core(double* sm, int direct, int M, int N, int k, int len, i
         if (direct == 2)
             dev::jacobi_tiny(B, Vd, Sr, len, k, ldb, ldv, red, s_rot);
         else if (len <= 8)
-            dev::jacobi_pre<1, 1, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+            dev::jacobi_pre<1, 1, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot, pre);
         else if (len <= 16)
-            dev::jacobi_pre<2, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+            dev::jacobi_pre<2, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot, pre);
         else
-            dev::jacobi_pre<4, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot);
+            dev::jacobi_pre<4, 2, false>(B, Vd, Sr, len, k, scr, dl, ring, red, s_rot, pre);
         dev::svd_assemble_direct(B, ldb, Vd, ldv, Sr, rinv, prm, S, US, Vt, M, N, k, wide, ldus, ldvt);
         return;
     }
@@ -255,7 +255,7 @@ __device__ void svd_core(double* sm, int direct, int M, int N, int k, int len, i
     for (int j = threadIdx.x; j < k; j += nthreads()) B[(int64_t)j * len + j] = vd[j];
     __syncthreads();
     double* Sraw = vd;
-    dev::jacobi_auto(G, V, Sraw, k, X, del, ring, red, s_rot);
+    dev::jacobi_auto(G, V, Sraw, k, X, del, ring, red, s_rot, pre);
     for (int e = threadIdx.x; e < len * k; e += nthreads()) {
         const int j = e / len, i = e % len;
         X[e] = i < k ? V[j * ld + i] : 0.0;
@@ -271,7 +271,7 @@ __device__ __forceinline__ void pad_columns(double* B, int len, int ldb, int k) 
 }
 
 __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* __restrict__ tasks,
-                                                       const SvdPart* __restrict__ parts) {
+                                                       const SvdPart* __restrict__ parts, bool pre) {
     extern __shared__ double sm[];
     __shared__ double red[33];
     __shared__ dev::SegRot ring[64];
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_svd_site(const SvdSiteTask* _
         }
     }
     __syncthreads();
-    svd_core(sm, direct, M, N, k, len, tk.wide, tk.S, tk.US, tk.Vt, k, N, red, &s_rot, ring);
+    svd_core(sm, direct, M, N, k, len, tk.wide, tk.S, tk.US, tk.Vt, k, N, red, &s_rot, ring, pre);
 }
 
 __global__ void __launch_bounds__(kThreads) k_right_apply(const RTask* __restrict__ tasks,
@@ -401,7 +401,7 @@ __device__ void right_rank1(const DynTask& tk, const double* v, int len, int wid
 
 template <bool CG>
 __device__ void right_body(const DynTask& tk, double* sm, double* red,
-                           int* s_rot, int* s_cols, dev::SegRot* ring) {
+                           int* s_rot, int* s_cols, dev::SegRot* ring, bool pre) {
     const int np = tk.p_end - tk.p_beg;
     if (threadIdx.x < 2) {
         int c = 0;
@@ -447,17 +447,17 @@ __device__ void right_body(const DynTask& tk, double* sm, double* red,
         right_rank1(tk, B, len, wide, red);
         return;
     }
-    svd_core(sm, direct, M, N, k, len, wide, tk.S, tk.US, tk.Vt, tk.kpad, tk.ncols_pad, red, s_rot, ring);
+    svd_core(sm, direct, M, N, k, len, wide, tk.S, tk.US, tk.Vt, tk.kpad, tk.ncols_pad, red, s_rot, ring, pre);
     if (threadIdx.x == 0) *tk.kact = k;
 }
 
-__global__ void __launch_bounds__(kSweepThreads) k_right_dyn(const DynTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(kSweepThreads) k_right_dyn(const DynTask* __restrict__ tasks, bool pre) {
     extern __shared__ double sm[];
     __shared__ double red[33];
     __shared__ dev::SegRot ring[64];
     __shared__ int s_rot;
     __shared__ int s_cols[2];
-    right_body<false>(tasks[blockIdx.x], sm, red, &s_rot, s_cols, ring);
+    right_body<false>(tasks[blockIdx.x], sm, red, &s_rot, s_cols, ring, pre);
 }
 
 // Pooled cut of one bond (one CTA): stable descending order with ties by
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
                                                           const int* __restrict__ phase_beg,
                                                           const CutTask* __restrict__ cuts,
                                                           const CutSector* __restrict__ secs, int n_phase,
-                                                          int pb_off, GridSync* gs) {
+                                                          int pb_off, GridSync* gs, int pre) {
     extern __shared__ double sm[];
     __shared__ double red[33];
     __shared__ int s_rot;
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_right_sweep(const DynTask* __
             __syncthreads();
             const bool first = ti == pb[p] + (int)blockIdx.x;
             const DynTask& tk = first ? s_task[p & 1] : tasks[ti];
-            right_body<true>(tk, sm, red, &s_rot, s_cols, ring);
+            right_body<true>(tk, sm, red, &s_rot, s_cols, ring, pre);
             // the CTA that completes the last task of this truncation's bond runs its cut
             __syncthreads();
             const CutTask& ct = cuts[tk.cut];
@@ -1162,7 +1162,7 @@ void launch_svd_site(Context* ctx, const std::vector<SvdSiteTask>& tasks, const 
     for (const SvdSiteTask& t : tasks) kmax = std::max(kmax, t.k);
     const cudaStream_t st = on_side ? ctx->fork_side() : ctx->stream;
     k_svd_site<<<(unsigned)tasks.size(), svd_block_for(kmax), smem, st>>>((const SvdSiteTask*)(d + ot),
-                                                                                 (const SvdPart*)(d + op));
+                                                                                 (const SvdPart*)(d + op), ctx->jacobi_precond_min > 0);
     count_launch(ctx);
     pr.done();
 }
@@ -1224,7 +1224,7 @@ int launch_right_dyn(Context* ctx, const std::vector<DynTask>& tasks_in, const s
     Prof pr(ctx, KK_SVD, fl, by);
     allow_smem(k_right_dyn);
     const bool tiny = std::all_of(tasks.begin(), tasks.end(), is_tiny);
-    k_right_dyn<<<(unsigned)tasks.size(), svd_block_for(kmax, tiny), smem, ctx->stream>>>((const DynTask*)(d + ot));
+    k_right_dyn<<<(unsigned)tasks.size(), svd_block_for(kmax, tiny), smem, ctx->stream>>>((const DynTask*)(d + ot), ctx->jacobi_precond_min > 0);
     count_launch(ctx);
     pr.done();
     return ctx->profiling ? (int)ctx->prof.size() - 1 : -1;
@@ -1324,7 +1324,8 @@ bool launch_right_sweep(Context* ctx, const std::vector<DynTask>& tasks_in, cons
     int a4 = n_phase;
     int a5 = (int)pb_off;
     GridSync* a6 = gs;
-    void* args[] = {&a0, &a1, &a2, &a3, &a4, &a5, &a6};
+    int a7 = ctx->jacobi_precond_min > 0;
+    void* args[] = {&a0, &a1, &a2, &a3, &a4, &a5, &a6, &a7};
     Prof pr(ctx, KK_SVD, 0.0, by);   // flops entered by the caller once the ranks are known
     BSM_CUDA(cudaLaunchCooperativeKernel((const void*)k_right_sweep, dim3(grid), dim3(threads), args, smem,
                                          ctx->stream));
