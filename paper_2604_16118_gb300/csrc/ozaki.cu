@@ -189,9 +189,10 @@ __device__ __forceinline__ double oz_round(long long hi, unsigned long long lo, 
 //    products of that diagonal may restart it: the tensor cores wait only for the
 //    first of the eight reads;
 //  - at the end of a tile the two integers are combined and rounded once.
-// Bound by the MMAs' shared-memory operand reads (128 x 16 + 64 x 16 BF16 per MMA,
-// 48 cycles at 128 bytes per cycle, against 32 cycles of multiplication): a wider
-// tile has no room in tensor memory beside eight diagonals.
+// What bounds it is the spacing of the MMAs: at n = 2048 the busiest SMs issue 14336 of 64 columns
+// in 654 us, one per 91 cycles, where the multiplication takes 32 and the operand reads 48 (128 x 16 +
+// 64 x 16 BF16 at 128 bytes per cycle; shared memory 54 % busy, tensor pipe 30 %).  A wider tile has no
+// room in tensor memory beside seven or eight diagonals.
 // Every mbarrier wait is bounded; whoever gives up sets *err and leaves, the
 // others run out of their own waits, and the tensor memory is freed after a
 // bounded wait for the MMAs and copies in flight.
@@ -300,8 +301,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_oz_gemm(const OzProd* __restr
                     tc::fence_after();
                     const uint64_t da = tc::desc_sw64(base + s * kStage);
                     const uint64_t db = tc::desc_sw64(base + s * kStage + kBytesA);
-                    // consecutive MMAs go to kOzWays accumulators in turn: one accumulator takes a new
-                    // product of 64 columns only every 75 cycles, the tensor cores one every 32
+                    // consecutive MMAs go to kOzWays accumulators in turn (4 % faster than one after the
+                    // other: one accumulator takes a new product of 64 columns every 75 cycles)
 #pragma unroll
                     for (int d1 = S - 1; d1 >= 0; d1 -= kOzWays) {
                         const int d0 = d1 - kOzWays + 1 > 0 ? d1 - kOzWays + 1 : 0;
